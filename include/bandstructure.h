@@ -52,7 +52,9 @@ extern "C" {
 #define BS_ESTATE   -6   /* call out of order (e.g. solve before assemble)     */
 
 /* arithmetic of the eigen path */
-#define BS_PREC_FP64   0  /* every step in float64                             */
+#define BS_PREC_FP64   0  /* results to float64 accuracy: every quantity that
+                             enters them is float64 or an exact-slice product of
+                             float64 operands (bs_set_reduction)              */
 #define BS_PREC_MIXED  1  /* FP32 reduction + FP64 Rayleigh-Ritz refinement    */
 
 /* IBZ boundary paths for bs_bands (fractional corner points) */
@@ -256,7 +258,7 @@ int bs_set_iteration_limits(int lobpcg_maxit, int bisect_sweeps);
  * BS_SOLVER_FP64 and its FP64 fallback) reduces C(k) to real tridiagonal
  * form before the Sturm multisection of Eq. (eigenvalueproblem)'s lowest
  * eigenvalues.  The paper leaves the eigensolve to a host library; both
- * modes are unitary similarity transformations, so the eigenvalues agree
+ * reductions are unitary similarity transformations, so the eigenvalues agree
  * to rounding:
  *   BS_REDUCE_ONESTAGE: Householder reflectors column by column, on the
  *     FP64 pipe ((16/3) n^3 flops per k);
@@ -264,7 +266,15 @@ int bs_set_iteration_limits(int lobpcg_maxit, int bisect_sweeps);
  *     QR, the trailing two-sided updates as FP64-exact digit-plane products
  *     on the tensor cores (8 digits of 7 bits per operand), then band ->
  *     tridiagonal by bulge chasing in FP64 (O(n^2) work per k);
- *   BS_REDUCE_AUTO (default): two-stage for n >= 400, one-stage below.
+ *   BS_REDUCE_AUTO (default): solves of at most 22 branches with n >= 200
+ *     take a filtered subspace iteration without a reduction: Chebyshev
+ *     filters of the shifted inverse (FP32) on 32 vectors between float64
+ *     Rayleigh-Ritz steps, until the sum of the squared float64 residuals over
+ *     their distances to the rest of the spectrum bounds the error of every
+ *     eigenvalue by 64 eps64 ||C|| and an inertia count shows that none was
+ *     skipped.  Matrices it does not certify so are reduced (one-stage) in
+ *     the same call, without a wait for the host.  Other solves: two-stage
+ *     for n >= 400, one-stage below.
  * Process-wide; takes effect at the next solve.  The two-stage reduction
  * needs an n x 8 complex panel in shared memory (n up to about 1800 on
  * GB300); larger n use the one-stage reduction in every mode.

@@ -78,6 +78,15 @@ bool bs_use_band(int n) {
   return n >= BS_BAND_AUTO_MIN;
 }
 
+// The filtered iteration takes the solves of few branches: it does a
+// factorisation and some 60 block products where the reductions do n or n/8
+// dependent steps.  A lowered bisection cap (a diagnostic) is meant for the
+// tridiagonal path, so that one runs.
+bool bs_use_filter(int n, int nbands) {
+  return g_reduction.load(std::memory_order_relaxed) == BS_REDUCE_AUTO && bs_bisect_sweeps() == 128 &&
+         bs_filter_fits(n, nbands);
+}
+
 extern "C" int bs_set_reduction(int mode) {
   if (mode != BS_REDUCE_AUTO && mode != BS_REDUCE_ONESTAGE && mode != BS_REDUCE_TWOSTAGE) {
     bs_set_error("bs_set_reduction: mode %d is not BS_REDUCE_AUTO, _ONESTAGE or _TWOSTAGE", mode);
@@ -168,6 +177,11 @@ static void free_workspace(bs_cell* c) {
     bs_band_ws_free(c->band);
     delete c->band;
     c->band = nullptr;
+  }
+  if (c->filt) {
+    bs_filter_ws_free(c->filt);
+    delete c->filt;
+    c->filt = nullptr;
   }
   void* mixed[] = {c->d_C32, c->d_vec32, c->d_part32, c->d_lamT, c->d_scr, c->d_mY, c->d_mphase,
                    c->d_X32, c->d_X64, c->d_CX, c->d_mG, c->d_H, c->d_W, c->d_theta, c->d_beta,
@@ -771,11 +785,23 @@ static int solve_chunk_mixed(bs_cell* c, int kb, int nbands, cudaStream_t s) {
 
 static int solve_chunk(bs_cell* c, int kb, int nbands, cudaStream_t s) {
   if (c->precision == BS_PREC_MIXED) return solve_chunk_mixed(c, kb, nbands, s);
+  const bool filt = bs_use_filter(c->n, nbands);
   bs_phase_begin(c, PH_BUILD, s);
   TRY(bs_launch_builder(c->d_Cm, c->n, c->d_Q, kb, c->q1[0], c->q1[1], c->q2[0], c->q2[1], c->d_C,
-                        s));
+                        s, filt));
   bs_phase_end(c, PH_BUILD, s);
   bs_phase_begin(c, PH_TRID, s);
+  if (filt && !c->filt) c->filt = new FilterWs();
+  // no memory for its workspace: the reductions below need less
+  if (filt && bs_filter_ws_alloc(c->filt, c->n, c->kcap) == BS_OK) {
+    const FilterFallback fb{c->d_vec, c->d_part, c->d_de, c->d_tau, c->d_beta, c->d_count};
+    TRY(bs_launch_eig_filter(c->d_C, c->n, kb, nbands, *c->filt, fb, c->d_w, c->d_stat,
+                             c->d_info + 1, s));
+    c->band_used = false;
+    bs_phase_end(c, PH_TRID, s);
+    c->prof_ready[PH_BISECT] = false;
+    return BS_OK;
+  }
   if (bs_use_band(c->n)) {
     if (!c->band) c->band = new BandWs();
     TRY(bs_band_ws_alloc(c->band, c->n, c->kcap, BS_SLICES_BAND));

@@ -160,6 +160,7 @@ struct BatchGroup {
   zd* vec64;                  // FP64 solver: reduction vectors and partial sums
   zd* part64;
   BandWs* band;               // FP64 solver: two-stage reduction workspace (large n)
+  FilterWs* filt;             // FP64 solver: filtered iteration workspace
   // [0] tensor-core pipeline timeout of a main-stream product, [1] a Gram
   // Cholesky failed, [2] a tensor-core timeout during a cell's assembly
   // (the workers' own flags are reset by every assembly, so each assembly's
@@ -216,6 +217,11 @@ static void free_group(BatchGroup& g) {
     bs_band_ws_free(g.band);
     delete g.band;
     g.band = nullptr;
+  }
+  if (g.filt) {
+    bs_filter_ws_free(g.filt);
+    delete g.filt;
+    g.filt = nullptr;
   }
   for (int w = 0; w < g.nworkers; ++w) {
     if (g.workers[w]) bs_destroy_cell(g.workers[w]);
@@ -460,7 +466,8 @@ static int assemble_chunk(bs_batch* B, BatchGroup& g, int c0, int cn, int p) {
               : bs_cuda_status(cudaGetLastError(), "batch L_R stash");
     if (!r && B->solver == BS_SOLVER_FP64)
       r = bs_launch_builder(wk->d_Cm, n, B->d_Q + (size_t)ci * nk * 2, nk, wk->q1[0], wk->q1[1],
-                            wk->q2[0], wk->q2[1], g.C64 + (size_t)i * nk * nn, ws);
+                            wk->q2[0], wk->q2[1], g.C64 + (size_t)i * nk * nn, ws,
+                            g.filt && bs_use_filter(n, B->nbands));
     else if (!r)
       r = bs_launch_builder_mixed(wk->d_Cm, n, B->d_Q + (size_t)ci * nk * 2, nk, wk->q1[0],
                                   wk->q1[1], wk->q2[0], wk->q2[1], g.C64 + (size_t)i * nk * nn,
@@ -513,8 +520,13 @@ static int reduce_chunk_body(bs_batch* B, BatchGroup& g, int c0, int cn, int p, 
   const int* rows = g.d_rowidx + (size_t)c0 * nk;
   prof_mark(B, s);   // assembly ends, reduction begins
   if (B->solver == BS_SOLVER_FP64) {
-    // the plain FP64 dense path: Householder reduction and Sturm multisection
-    if (g.band) {
+    // the plain FP64 path: filtered iteration, or Householder reduction and
+    // Sturm multisection
+    if (g.filt && bs_use_filter(n, B->nbands)) {
+      const FilterFallback fb{g.vec64, g.part64, g.de, g.tau, g.beta, g.count};
+      TRY_LAUNCH(bs_launch_eig_filter(g.C64, n, K, B->nbands, *g.filt, fb, g.w, g.st, g.d_err, s));
+      prof_mark(B, s);
+    } else if (g.band) {
       BandBisect bis{B->nbands, g.w, g.st};
       TRY_LAUNCH(bs_launch_eig_band(g.C64, n, K, *g.band, g.de, g.d_err, s, &bis));
       prof_mark(B, s);
@@ -867,6 +879,14 @@ extern "C" int bs_batch_set_solver(bs_batch* B, int solver) {
         bs_band_ws_free(g.band);
         delete g.band;
         g.band = nullptr;
+      }
+      // no memory for the filtered iteration: the reductions take the group
+      if (bs_use_filter(g.n, B->nbands)) {
+        if (!g.filt) g.filt = new FilterWs();
+        if (bs_filter_ws_alloc(g.filt, g.n, (int)K) != BS_OK) {
+          delete g.filt;
+          g.filt = nullptr;
+        }
       }
     }
   }

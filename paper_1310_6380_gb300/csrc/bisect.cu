@@ -116,14 +116,18 @@ __device__ void sweep(T& lo, T& hi, int i, int l, unsigned mask, CountFn cnt) {
 __global__ void __launch_bounds__(NTB) bisect_kernel(const double* __restrict__ de, int n,
                                                      int nbands, double* __restrict__ omega,
                                                      int* __restrict__ stat, int want_omega,
-                                                     double stop_rel, int maxsweep) {
+                                                     double stop_rel, int maxsweep,
+                                                     const int* __restrict__ list,
+                                                     const int* __restrict__ nlist) {
   extern __shared__ double sm[];
   double* d = sm;
   double* e2 = sm + n;
   float* d32 = reinterpret_cast<float*>(sm + 2 * n);
   float* e32 = d32 + n;
   __shared__ double red[4];
-  const int b = blockIdx.x, tid = threadIdx.x;
+  // with a list, only its matrices (made on the device, nearly always empty)
+  if (list && (int)blockIdx.x >= *nlist) return;
+  const int b = list ? list[blockIdx.x] : (int)blockIdx.x, tid = threadIdx.x;
   const double* dg = de + (size_t)b * 2 * n;
   for (int k = tid; k < n; k += NTB) {
     d[k] = dg[k];
@@ -209,21 +213,38 @@ __global__ void __launch_bounds__(NTB) bisect_kernel(const double* __restrict__ 
 
 }  // namespace
 
+static int bisect_smem(int n, size_t* smem) {
+  *smem = 2 * (size_t)n * sizeof(double) + 2 * (size_t)n * sizeof(float);
+  if (*smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(bisect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)*smem);
+    if (e != cudaSuccess) return bs_cuda_status(e, "bisect smem");
+  }
+  return BS_OK;
+}
+
 int bs_launch_bisect(const double* de, int n, int batch, int nbands, double* omega, int* stat,
                      cudaStream_t s, bool want_omega, double stop_rel) {
   if (batch < 1 || nbands < 1) return BS_OK;
-  const size_t smem = 2 * (size_t)n * sizeof(double) + 2 * (size_t)n * sizeof(float);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(bisect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return bs_cuda_status(e, "bisect smem");
-  }
+  size_t smem = 0;
+  TRY_LAUNCH(bisect_smem(n, &smem));
   if (stat) {
     const cudaError_t e = cudaMemsetAsync(stat, 0, (size_t)batch * sizeof(int), s);
     if (e != cudaSuccess) return bs_cuda_status(e, "bisect status");
   }
   bisect_kernel<<<dim3(batch, (nbands + EPC - 1) / EPC), NTB, smem, s>>>(
-      de, n, nbands, omega, stat, want_omega ? 1 : 0, stop_rel, bs_bisect_sweeps());
+      de, n, nbands, omega, stat, want_omega ? 1 : 0, stop_rel, bs_bisect_sweeps(), nullptr,
+      nullptr);
+  BS_CHECK_LAUNCH("bisect_kernel");
+  return BS_OK;
+}
+
+int bs_launch_bisect_list(const double* de, int n, int batch, int nbands, double* omega, int* stat,
+                          const int* list, const int* nlist, cudaStream_t s) {
+  size_t smem = 0;
+  TRY_LAUNCH(bisect_smem(n, &smem));
+  bisect_kernel<<<dim3(batch, (nbands + EPC - 1) / EPC), NTB, smem, s>>>(
+      de, n, nbands, omega, stat, 1, 0.0, bs_bisect_sweeps(), list, nlist);
   BS_CHECK_LAUNCH("bisect_kernel");
   return BS_OK;
 }

@@ -76,6 +76,13 @@ __host__ __device__ __forceinline__ zf zfnmac(zf a, zf b, zf acc) {
   acc.y = fmaf(a.x, b.y, acc.y);
   return acc;
 }
+__host__ __device__ __forceinline__ zf zfmac(zf a, zf b, zf acc) {
+  acc.x = fmaf(a.x, b.x, acc.x);
+  acc.x = fmaf(a.y, b.y, acc.x);
+  acc.y = fmaf(a.y, b.x, acc.y);
+  acc.y = fmaf(-a.x, b.y, acc.y);
+  return acc;
+}
 
 // complex type of a real precision
 template <typename R> struct Cplx;
@@ -211,6 +218,7 @@ struct bs_cell {
   // profiling: events around each phase of the last call
   struct BandWs* band;  // two-stage reduction workspace (allocated on first use)
   bool band_used;       // the last FP64 solve took the two-stage reduction
+  struct FilterWs* filt;  // filtered iteration workspace (allocated on first use)
 
   bool prof;
   bool prof_ready[PH_COUNT];
@@ -285,9 +293,11 @@ bool bs_slice_slabs(int S, int Kp, int M, int N, int batch, SliceSlabs* q);
 // (entry, slab) output planes to allocate for any batch up to `batch`
 size_t bs_slice_planes(int S, int Kp, int M, int N, int batch);
 // D[z][q][n][m] = sum_{k < len_q} A[z][m][a0_q + k] B[z][n][b0_q + k] for every
-// slab q of (S, Kp); A: batch x M x S Kp, B: batch x N x S Kp
+// slab q of (S, Kp); A: batch x M x S Kp, B: batch x N x S Kp; entries with a
+// non-zero skip[z] are left out
 int bs_launch_slice_orders(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int S,
-                           int Kp, int batch, int* err, cudaStream_t s);
+                           int Kp, int batch, int* err, cudaStream_t s,
+                           const int* skip = nullptr);
 int bs_launch_fields_tc(bs_cell* c, cudaStream_t s);
 size_t bs_fields_tc_elems(int P, int D, int nf, size_t* nA, size_t* nB, size_t* nD);
 int bs_launch_cx_tc(const zd* C, const zd* X, int n, int b, int kb, uint16_t* sA, uint16_t* sB,
@@ -367,7 +377,7 @@ int bs_launch_band_pack_trail(const zd* A, int n, int o, int m, int kb, uint16_t
                               cudaStream_t s);
 int bs_launch_band_av(int m, const zd* V, int ldv, long sv, int nb, int kb, int S, uint16_t* wA,
                       uint16_t* wB, float* wD, int* eA, int* eB, zd* X, int ldx, long sx,
-                      int* err, cudaStream_t s);
+                      int* err, cudaStream_t s, const int* skip = nullptr);
 int bs_launch_band_pack_rank2(const zd* V, const zd* W, int ld, long sv, const int* dsc, int m,
                               int nb, int kb, int S, uint16_t* wA, uint16_t* wB, int* ex,
                               cudaStream_t s);
@@ -375,9 +385,62 @@ int bs_rank2_column_tiles(int m);
 int bs_launch_rank2_update(const uint16_t* dA, const uint16_t* dB, const int* ex, int m, int kb,
                            zd* A, int n, int o, int ct0, int nct, int* err, cudaStream_t s);
 
+// filter.cu: the lowest branches by filtered subspace iteration (FP32
+// shift-invert operator, FP64 Rayleigh-Ritz, residual and inertia certificate)
+#define BS_FILT_BLOCK 32       // columns of the block
+#define BS_FILT_MAX_BANDS 22   // wanted branches: at least 10 guard vectors remain
+#define BS_FILT_MIN_N 200
+#define BS_FILT_MAXDEG 12      // degrees of one filter
+struct FilterWs {
+  int n = 0, kf = 0;        // order, matrices per chunk
+  zf* A = nullptr;          // kf x np x np scaled matrix, then its LDL^dagger (np: n padded to 64)
+  zf* X = nullptr;          // kf x np x np inverse factor
+  uint16_t* pA = nullptr;   // digit planes of C, of the block, and the digit-order sums
+  uint16_t* pB = nullptr;
+  float* pD = nullptr;
+  int* eA = nullptr;
+  int* eB = nullptr;
+  zd* Xb = nullptr;         // kf x 32 x n block and C times it
+  zd* CX = nullptr;
+  zf* vec = nullptr;        // 5 x kf x 32 x np: R, Lh v, B R, two Chebyshev terms
+  zd* part = nullptr;       // kf x chunks x 2 x 32 x 32 partial Gram matrices
+  float* rpart = nullptr;   // kf x chunks x 2 x 32 partial residual sums
+  double* theta = nullptr;  // kf x 32
+  zd* W = nullptr;          // kf x 32 x 32
+  float* coef = nullptr;    // kf x BS_FILT_MAXDEG x 4 x 32
+  double* shift = nullptr;  // kf
+  double* cmax = nullptr;   // kf
+  double* sigma = nullptr;  // kf
+  int* ord = nullptr;       // kf x 32
+  float* w = nullptr;       // kf x np row scales
+  int* iw = nullptr;        // neg, flag, expected count, list (kf each), list length, fail, done (kf)
+};
+// the buffers of the Householder reduction that takes what is not certified
+struct FilterFallback {
+  zd* vec;
+  zd* part;
+  double* de;
+  double* tau;
+  zd* beta;
+  unsigned* count;
+};
+bool bs_filter_fits(int n, int nbands);
+// whether a solve of nbands branches takes it (BS_REDUCE_AUTO)
+bool bs_use_filter(int n, int nbands);
+int bs_filter_ws_alloc(FilterWs* w, int n, int kb);
+void bs_filter_ws_free(FilterWs* w);
+// C: kb full Hermitian matrices (kept, but for those that take the fallback)
+int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const FilterFallback& fb,
+                         double* omega, int* stat, int* err, cudaStream_t s);
+// tridiag.cu, bisect.cu: the matrices list[0 .. *nlist) of a batch (device list)
+int bs_launch_tridiag_list(zd* A, int n, zd* vec, zd* part, double* de, double* tau, zd* beta,
+                           unsigned* count, const int* list, const int* nlist, cudaStream_t s);
+int bs_launch_bisect_list(const double* de, int n, int batch, int nbands, double* omega, int* stat,
+                          const int* list, const int* nlist, cudaStream_t s);
 
+// full: write the whole Hermitian matrix, else its lower triangle
 int bs_launch_builder(const zd* Cm, int n, const double* Q, int nk, double q1x, double q1y,
-                      double q2x, double q2y, zd* C, cudaStream_t s);
+                      double q2x, double q2y, zd* C, cudaStream_t s, bool full = false);
 
 // tridiag.cu: Householder reduction in precision R (double or float).  On
 // return column j of A below row j+1 holds v_j (v_j[j+1] = 1 implied),

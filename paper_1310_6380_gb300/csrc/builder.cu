@@ -5,7 +5,7 @@
 // K = k + G.  With the six coefficient matrices assembled once per cell,
 //   C(k) = C_1 + k1 C_k1 + k2 C_k2 + k1^2 C_k11 + k1 k2 C_k12 + k2^2 C_k22,
 // so the per-k build is a streaming linear combination (HBM bound) of the
-// lower triangles, written for a whole batch of wavevectors at once so each
+// lower triangles (or the full matrices), written for a whole batch of wavevectors at once so each
 // coefficient element is read once per batch.
 #include "bs_internal.h"
 
@@ -15,11 +15,11 @@ constexpr int KB = 32;   // wavevectors per pass over the coefficients
 
 __global__ void builder_kernel(const zd* __restrict__ Cm, int n, const double* __restrict__ Q,
                                int nk, double q1x, double q1y, double q2x, double q2y,
-                               zd* __restrict__ C) {
+                               zd* __restrict__ C, bool full) {
   __shared__ double coef[KB][6];
   const size_t nn = (size_t)n * n;
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool live = e < nn && (int)(e % n) >= (int)(e / n);
+  const bool live = e < nn && (full || (int)(e % n) >= (int)(e / n));
   zd m[6];
   if (live) {
 #pragma unroll
@@ -55,9 +55,10 @@ __global__ void builder_kernel(const zd* __restrict__ Cm, int n, const double* _
 }  // namespace
 
 int bs_launch_builder(const zd* Cm, int n, const double* Q, int nk, double q1x, double q1y,
-                      double q2x, double q2y, zd* C, cudaStream_t s) {
+                      double q2x, double q2y, zd* C, cudaStream_t s, bool full) {
   const size_t nn = (size_t)n * n;
-  builder_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(Cm, n, Q, nk, q1x, q1y, q2x, q2y, C);
+  builder_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(Cm, n, Q, nk, q1x, q1y, q2x, q2y, C,
+                                                              full);
   BS_CHECK_LAUNCH("builder_kernel");
   return BS_OK;
 }

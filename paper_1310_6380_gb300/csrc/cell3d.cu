@@ -55,6 +55,7 @@ struct bs_cell3 {
   unsigned* d_count;
   int* d_stat;
   BandWs* band;        // two-stage reduction workspace (allocated on first use)
+  FilterWs* filt;      // filtered iteration workspace (allocated on first use)
 };
 
 namespace {
@@ -185,11 +186,11 @@ constexpr int KB3 = 32;
 
 // C(k) = sum_t c_t(k) Cm[t], c = (1, k1, k2, k3, k1^2, k2^2, k3^2, k1 k2, k1 k3, k2 k3)
 __global__ void builder3_kernel(const zd* __restrict__ Cm, int n, const double* __restrict__ Q,
-                                int nk, const double* __restrict__ qv, zd* __restrict__ C) {
+                                int nk, const double* __restrict__ qv, zd* __restrict__ C, bool full) {
   __shared__ double coef[KB3][NMONO];
   const size_t nn = (size_t)n * n;
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool live = e < nn && (int)(e % n) >= (int)(e / n);
+  const bool live = e < nn && (full || (int)(e % n) >= (int)(e / n));
   zd m[NMONO];
   if (live) {
 #pragma unroll
@@ -313,6 +314,11 @@ void free_ws3(bs_cell3* c) {
     bs_band_ws_free(c->band);
     delete c->band;
     c->band = nullptr;
+  }
+  if (c->filt) {
+    bs_filter_ws_free(c->filt);
+    delete c->filt;
+    c->filt = nullptr;
   }
   cudaFree(c->d_C);
   cudaFree(c->d_vec);
@@ -606,15 +612,23 @@ extern "C" int bs_solve_k3(bs_cell3* c, const double* Q, int nk, int nbands, dou
       break;
     }
     const size_t nn = (size_t)n * n;
+    bool filt = bs_use_filter(n, nbands);
+    if (filt && !c->filt) c->filt = new FilterWs();
+    // no memory for its workspace: the reductions below need less
+    filt = filt && bs_filter_ws_alloc(c->filt, n, c->kcap) == BS_OK;
     builder3_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(c->d_Cm, n, c->d_Q, kb, d_qv,
-                                                                 c->d_C);
+                                                                 c->d_C, filt);
     e = cudaGetLastError();
     bs_count_launch();
     if (e != cudaSuccess) {
       r = bs_cuda_status(e, "builder3_kernel");
       break;
     }
-    if (bs_use_band(n)) {
+    if (filt) {
+      const FilterFallback fb{c->d_vec, c->d_part, c->d_de, c->d_tau, c->d_beta, c->d_count};
+      r = bs_launch_eig_filter(c->d_C, n, kb, nbands, *c->filt, fb, c->d_w, c->d_stat,
+                               c->d_info + 1, s);
+    } else if (bs_use_band(n)) {
       if (!c->band) c->band = new BandWs();
       r = bs_band_ws_alloc(c->band, n, c->kcap, BS_SLICES_BAND);
       BandBisect bis{nbands, c->d_w, c->d_stat};
@@ -677,7 +691,7 @@ extern "C" int bs_reduced_matrix3(bs_cell3* c, const double* Q, double* out, voi
   cudaMemcpy(c->d_Q, Qh.data(), 3 * 8, cudaMemcpyHostToDevice);
   const size_t nn = (size_t)c->n * c->n;
   builder3_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(c->d_Cm, c->n, c->d_Q, 1, d_qv,
-                                                               c->d_C);
+                                                               c->d_C, false);
   bs_count_launch();
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)

@@ -1,0 +1,1348 @@
+// The lowest eigenvalues of batched Hermitian matrices C(k) (Eq.
+// (eigenvalueproblem) in standard form) by filtered subspace iteration, for
+// the solves that want a few branches of a large matrix.
+//
+// A reduction to tridiagonal form spends (16/3) n^3 flops per matrix on all n
+// eigenvalues, in n or n/8 dependent steps.  The lowest nb <= 24 need one
+// factorisation and a few dozen products with 32-column blocks:
+//
+//  1. FP32: the LDL^dagger of W (C/s + I) W (s of the size of the wanted
+//     eigenvalues, W = diag(C/s + 1)^-1/2), its triangular inverse, and so
+//     Lh = D^-1/2 L^-1 W with B = Lh^dagger Lh = (C/s + I)^-1 to FP32
+//     accuracy.  The wanted eigenvalues are the largest of B.
+//  2. Rounds: an FP64 Rayleigh-Ritz step on the block X (32 vectors, the
+//     wanted ones and guards) gives theta, X, and the FP64 residual
+//     R = C X - X Theta; then X is filtered by a Chebyshev polynomial T_m of B
+//     that is at most 1 on the unwanted part of the spectrum.  Written for
+//     the change E of X instead of X itself,
+//       T_j(l(B)) x = tau_j (x + E_j),   B x = mu (x - B r / s),  mu = s / (theta + s),
+//     every term is a product of B with the residual: the FP32 operator only
+//     multiplies R, so its rounding shrinks with R and the rounds converge to
+//     the eigenvectors of the FP64 matrix, not of B.
+//  3. Certificate: theta_i is an upper bound of lambda_i; with rho a lower
+//     bound of lambda_{m+1}, Lehmann's bound in its trace form (the residual
+//     Gram matrix replaced by its trace) gives
+//       lambda_i >= theta_i - sum_{c <= m} ||r_c||^2 / (rho - theta_c),  i <= m.
+//     A matrix passes when that sum is at most 64 eps64 max_r C_rr (the
+//     backward error of a reduction to tridiagonal form and its bisection is
+//     of that size; the sum overestimates the error, whose own gap is that to
+//     the eigenvalues outside the block),
+//     and when the inertia of C - sigma I (FP32 LDL^dagger of the scaled
+//     matrix, sigma in a gap above theta_m) counts exactly m eigenvalues
+//     below sigma, so that none was skipped.
+//  4. Matrices that do not pass are reduced by the FP64 Householder reduction
+//     and bisected (tridiag.cu, bisect.cu) in one launch each that returns at
+//     once when there are none; nothing waits for the host.
+//
+// Measured (one GB300, whole FP64 solve with its assembly, the reduction to
+// tridiagonal form before -> this): n = 882, 90 matrices, 18 branches
+// 171 -> 47 ms; n = 1029, 30 matrices, 12 branches 136 -> 35 ms; n = 242,
+// 70 matrices, 18 branches 16.9 -> 9.0 ms.  What bounds it at n = 882 is the
+// FP32 pipe in the products with B and in the factorisations, and the FP64
+// pipe in the Rayleigh-Ritz steps (32-column products at 2 FMA per clock and SM).
+//
+// Everything that enters a result (C X, the Gram matrices, the Ritz values,
+// the residuals) is FP64 or an exact-slice product of FP64 operands.
+#include <float.h>
+#include <math.h>
+
+#include <algorithm>
+#include <atomic>
+
+#include "bs_internal.h"
+
+namespace {
+
+constexpr int FB = BS_FILT_BLOCK;   // columns of the block (32)
+constexpr int TB = 64;              // tile edge of the FP32 factorisation
+constexpr int LDS = TB + 1;         // row stride of the diagonal blocks in shared memory
+constexpr float TINY_PIVOT = 1e-6f; // of the scaled unit diagonal
+constexpr int GR = 64;              // rows per CTA of the Gram and rotation kernels
+
+__device__ __forceinline__ zf cfma(zf a, zf b, zf c) { return zfma(a, b, c); }
+
+// ---------------------------------------------------------------- set-up
+// Per matrix: the FB smallest diagonal entries (the starting vectors are
+// their unit vectors, plane waves in the reduced basis), the shift s, the
+// row scales w_r = (s / (C_rr + s))^1/2 and the largest diagonal entry.
+__global__ void __launch_bounds__(256) filt_prep_kernel(const zd* __restrict__ C, int n, int np,
+                                                        int nb, double sfac,
+                                                        double* __restrict__ shift,
+                                                        double* __restrict__ cmax,
+                                                        int* __restrict__ ord,
+                                                        float* __restrict__ w,
+                                                        int* __restrict__ fail,
+                                                        int* __restrict__ done) {
+  extern __shared__ double dg[];
+  const long long* key = reinterpret_cast<const long long*>(dg);
+  __shared__ int so[FB];
+  __shared__ double red[8];
+  const int k = blockIdx.x, tid = threadIdx.x;
+  const zd* ck = C + (size_t)k * n * n;
+  double cm = 0.0;
+  for (int r = tid; r < n; r += 256) {
+    const double v = ck[(size_t)r * (n + 1)].x;
+    dg[r] = v;
+    cm = fmax(cm, fabs(v));
+  }
+  for (int o = 16; o > 0; o >>= 1) cm = fmax(cm, __shfl_xor_sync(0xffffffffu, cm, o));
+  if ((tid & 31) == 0) red[tid >> 5] = cm;
+  if (tid < FB) so[tid] = tid;
+  __syncthreads();
+  for (int r = tid; r < n; r += 256) {
+    // the diagonal is not negative, so its bit patterns order as its values do
+    const long long v = key[r];
+    int rank = 0;
+    for (int c = 0; c < n; ++c) rank += key[c] < v || (key[c] == v && c < r);
+    if (rank < FB) so[rank] = r;
+  }
+  __syncthreads();
+  double s = sfac * dg[so[nb - 1]];
+  // a zero or non-finite diagonal: any scale will do, the certificate decides
+  if (!(s > 0.0) || !(s < 1e300)) s = 1.0;
+  if (tid < FB) ord[(size_t)k * FB + tid] = so[tid];
+  if (tid == 0) {
+    double v = 0.0;
+    for (int q = 0; q < 8; ++q) v = fmax(v, red[q]);
+    shift[k] = s;
+    cmax[k] = v;
+    fail[k] = 0;
+    done[k] = 0;
+  }
+  const double is = 1.0 / s;
+  for (int r = tid; r < np; r += 256)
+    w[(size_t)k * np + r] = r < n ? rsqrtf(fmaxf((float)(dg[r] * is + 1.0), 1e-30f)) : 0.f;
+}
+
+// (bi, bk), bi >= bk, of the l-th lower-triangular tile (row-major order)
+__device__ __forceinline__ void tile_of(int l, int& bi, int& bk) {
+  int r = (int)((sqrtf(8.0f * (float)l + 1.0f) - 1.0f) * 0.5f);
+  while ((r + 1) * (r + 2) / 2 <= l) ++r;
+  while (r * (r + 1) / 2 > l) --r;
+  bi = r;
+  bk = l - r * (r + 1) / 2;
+}
+
+// A <- W (C / s - beta I) W, lower 64-tiles, FP32, identity in the padding.
+// beta = -1 (the operator) or sigma / s (the inertia check).
+__global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ C, int n, int np,
+                                                         const double* __restrict__ shift,
+                                                         const double* __restrict__ sigma,
+                                                         const float* __restrict__ w,
+                                                         zf* __restrict__ A, int* __restrict__ neg,
+                                                         int* __restrict__ flag) {
+  int bi, bk;
+  tile_of(blockIdx.x, bi, bk);
+  const int k = blockIdx.y, tid = threadIdx.x;
+  const zd* ck = C + (size_t)k * n * n;
+  const float* wk = w + (size_t)k * np;
+  zf* ak = A + (size_t)k * np * np;
+  const double is = 1.0 / shift[k], beta = sigma ? sigma[k] * is : -1.0;
+  if (blockIdx.x == 0 && tid == 0) {
+    neg[k] = 0;
+    flag[k] = 0;
+  }
+  const int r = bi * TB + (tid & 63);
+  const float wr = r < n ? wk[r] : 0.f;
+#pragma unroll 4
+  for (int q = tid >> 6; q < TB; q += 4) {
+    const int c = bk * TB + q;
+    zf v = make_float2(r == c ? 1.f : 0.f, 0.f);
+    if (r < n && c < n) {
+      const zd z = ck[(size_t)c * n + r];
+      const float f = wr * wk[c];
+      v = r == c ? make_float2((float)(z.x * is - beta) * f, 0.f)
+                 : make_float2((float)(z.x * is) * f, (float)(z.y * is) * f);
+    }
+    ak[(size_t)c * np + r] = v;
+  }
+}
+
+// ---------------------------------------------------------------- FP32 LDL^dagger
+// Blocked right-looking factorisation, panels of 64 columns, for a batch of
+// matrices padded to a multiple of 64.  As in the other factorisations of the
+// library each diagonal block is factored and stored by exactly one CTA, in
+// a launch whose other CTAs do not read it: the first by ldl64_diag_kernel,
+// block j + 1 by the CTA of ldl64_update_kernel(j) that has just updated it.
+// That CTA also inverts the unit lower factor (stored in the diagonal block
+// of X), so the block rows below become plain 64 x 64 x 64 products.
+
+// S: the 64 x 64 lower triangle (row-major, stride LDS); on return L D below
+// the diagonal and D on it.  Xs: its inverse unit factor.  One barrier per
+// column: step c reads column c (final) and row c of Xs (final) only.
+__device__ void ldl64_block(zf* S, zf* Xs, float* d, int* bad) {
+  const int tid = threadIdx.x, r = tid & 63, q = tid >> 6;
+  for (int c = q; c < TB; c += 4) Xs[r * LDS + c] = make_float2(r == c ? 1.f : 0.f, 0.f);
+  __syncthreads();
+  for (int c = 0; c < TB; ++c) {
+    float p = S[c * LDS + c].x;
+    if (!(fabsf(p) >= TINY_PIVOT)) {
+      if (tid == 0) *bad = 1;
+      p = p < 0.f ? -TINY_PIVOT : TINY_PIVOT;
+    }
+    if (tid == 0) d[c] = p;
+    if (r > c) {
+      const float inv = 1.f / p;
+      const zf l = zscale(S[r * LDS + c], inv);
+      for (int s = c + 1 + q; s <= r; s += 4) {
+        const zf u = S[s * LDS + c];
+        zf v = S[r * LDS + s];
+        v.x = fmaf(-l.x, u.x, fmaf(-l.y, u.y, v.x));   // - l conj(u)
+        v.y = fmaf(-l.y, u.x, fmaf(l.x, u.y, v.y));
+        S[r * LDS + s] = v;
+      }
+      for (int s = q; s <= c; s += 4) {
+        const zf u = Xs[c * LDS + s];
+        zf v = Xs[r * LDS + s];
+        v.x = fmaf(-l.x, u.x, fmaf(l.y, u.y, v.x));    // - l u
+        v.y = fmaf(-l.x, u.y, fmaf(-l.y, u.x, v.y));
+        Xs[r * LDS + s] = v;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// factor the diagonal block at j0 held in S and store L (unit), D, X
+__device__ void ldl64_diag(zf* a, zf* x, int np, int j0, int k, zf* S, zf* Xs, float* d, int* bad,
+                           int* neg, int* flag) {
+  const int tid = threadIdx.x, r = tid & 63;
+  if (tid == 0) *bad = 0;
+  __syncthreads();
+  ldl64_block(S, Xs, d, bad);
+  for (int c = tid >> 6; c < TB; c += 4) {
+    zf v = make_float2(0.f, 0.f);
+    if (r > c) v = zscale(S[r * LDS + c], 1.f / d[c]);
+    if (r == c) v.x = d[c];
+    if (r >= c) a[(size_t)(j0 + c) * np + j0 + r] = v;
+    x[(size_t)(j0 + c) * np + j0 + r] = r >= c ? Xs[r * LDS + c] : make_float2(0.f, 0.f);
+  }
+  if (tid == 0) {
+    int cnt = 0;
+    for (int c = 0; c < TB; ++c) cnt += d[c] < 0.f;
+    neg[k] += cnt;   // one CTA per matrix and launch, launches in order
+    if (*bad) flag[k] = 1;
+  }
+}
+
+__global__ void __launch_bounds__(256) ldl64_diag_kernel(zf* __restrict__ A, zf* __restrict__ X,
+                                                         int np, int* __restrict__ neg,
+                                                         int* __restrict__ flag) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ float d[TB];
+  __shared__ int bad;
+  zf* S = reinterpret_cast<zf*>(dsm);
+  zf* Xs = S + TB * LDS;
+  const int k = blockIdx.x, tid = threadIdx.x, r = tid & 63;
+  zf* a = A + (size_t)k * np * np;
+  for (int c = tid >> 6; c < TB; c += 4)
+    if (r >= c) S[r * LDS + c] = a[(size_t)c * np + r];
+  __syncthreads();
+  ldl64_diag(a, X + (size_t)k * np * np, np, 0, k, S, Xs, d, &bad, neg, flag);
+}
+
+// 64 x 64 x 64 product on 256 threads, 4 x 4 complex per thread:
+// acc[i][j] += sum_t As[t][tx + 16 i] op(B[t][ty + 16 j])
+template <bool CONJB>
+__device__ __forceinline__ void mm64(const zf* __restrict__ As, const zf* __restrict__ Bs, int bs_t,
+                                     int bs_c, zf (&acc)[4][4]) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll 8
+  for (int t = 0; t < TB; ++t) {
+    zf a[4], b[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = As[t * TB + tx + 16 * i];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) b[j] = Bs[t * bs_t + (ty + 16 * j) * bs_c];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = CONJB ? zfmac(a[i], b[j], acc[i][j])
+                                                    : zfma(a[i], b[j], acc[i][j]);
+  }
+}
+
+// a 64 x 64 tile of a column-major matrix into dst[t * 64 + r] (t = column)
+__device__ __forceinline__ void load_tile(zf* dst, const zf* src, int np) {
+  float4* d4 = reinterpret_cast<float4*>(dst);
+  for (int e = threadIdx.x; e < TB * TB / 2; e += 256) {
+    const int t = e >> 5, r2 = e & 31;
+    d4[t * 32 + r2] = *reinterpret_cast<const float4*>(src + (size_t)t * np + 2 * r2);
+  }
+}
+
+// block row i = j + 1 + blockIdx.x: L_i1 = A_i1 L11^-dagger D1^-1
+__global__ void __launch_bounds__(256) ldl64_panel_kernel(zf* __restrict__ A,
+                                                          const zf* __restrict__ X, int np,
+                                                          int j0) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  zf* As = reinterpret_cast<zf*>(dsm);
+  zf* Bs = As + TB * TB;
+  __shared__ float di[TB];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  zf* a = A + (size_t)blockIdx.y * np * np;
+  const int i0 = j0 + TB * (blockIdx.x + 1);
+  zf* ai = a + (size_t)j0 * np + i0;
+  load_tile(As, ai, np);
+  load_tile(Bs, X + (size_t)blockIdx.y * np * np + (size_t)j0 * np + j0, np);
+  if (tid < TB) di[tid] = 1.f / a[(size_t)(j0 + tid) * (np + 1)].x;
+  __syncthreads();
+  zf acc[4][4] = {};
+  mm64<true>(As, Bs, TB, 1, acc);   // Y[r][c] = sum_t A[r][t] conj(L11^-1[c][t])
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = ty + 16 * j;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ai[(size_t)c * np + tx + 16 * i] = zscale(acc[i][j], di[c]);
+  }
+}
+
+// trailing update A_ik -= L_i1 D1 L_k1^dagger; the first tile's CTA factors
+// the next diagonal block
+__global__ void __launch_bounds__(256) ldl64_update_kernel(zf* __restrict__ A, zf* __restrict__ X,
+                                                           int np, int j0, int* __restrict__ neg,
+                                                           int* __restrict__ flag) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  zf* As = reinterpret_cast<zf*>(dsm);
+  zf* Bs = As + TB * LDS;
+  __shared__ float d[TB];
+  __shared__ int bad;
+  int bi, bk;
+  tile_of(blockIdx.x, bi, bk);
+  zf* a = A + (size_t)blockIdx.y * np * np;
+  const int i0 = j0 + TB * (bi + 1), k0 = j0 + TB * (bk + 1);
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  if (tid < TB) d[tid] = a[(size_t)(j0 + tid) * (np + 1)].x;
+  load_tile(Bs, a + (size_t)j0 * np + k0, np);
+  __syncthreads();
+  {
+    float4* d4 = reinterpret_cast<float4*>(As);
+    const zf* src = a + (size_t)j0 * np + i0;
+    for (int e = tid; e < TB * TB / 2; e += 256) {
+      const int t = e >> 5, r2 = e & 31;
+      float4 v = *reinterpret_cast<const float4*>(src + (size_t)t * np + 2 * r2);
+      const float dt = d[t];
+      v.x *= dt;
+      v.y *= dt;
+      v.z *= dt;
+      v.w *= dt;
+      d4[t * 32 + r2] = v;
+    }
+  }
+  __syncthreads();
+  zf acc[4][4] = {};
+  mm64<true>(As, Bs, TB, 1, acc);
+  const bool first = blockIdx.x == 0;
+  if (first) __syncthreads();   // As is reused for the block below
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = ty + 16 * j;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = tx + 16 * i;
+      zf* o = a + (size_t)(k0 + c) * np + i0 + r;
+      if (bi == bk && r < c) continue;
+      zf v = zsub(*o, acc[i][j]);
+      if (first) As[r * LDS + c] = v;
+      else *o = v;
+    }
+  }
+  if (first) {
+    __syncthreads();
+    ldl64_diag(a, X + (size_t)blockIdx.y * np * np, np, i0, blockIdx.y, As, Bs, d, &bad, neg, flag);
+  }
+}
+
+// X_ij = -X_ii sum_{k=j}^{i-1} L_ik X_kj for block diagonal i - j = dd
+__global__ void __launch_bounds__(256) trinv64_kernel(const zf* __restrict__ A, zf* __restrict__ X,
+                                                      int np, int dd) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  zf* As = reinterpret_cast<zf*>(dsm);
+  zf* Bs = As + TB * TB;   // [col][t], stride LDS
+  const int bj = blockIdx.x, bi = bj + dd;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const zf* l = A + (size_t)blockIdx.y * np * np;
+  zf* x = X + (size_t)blockIdx.y * np * np;
+  zf acc[4][4] = {};
+  for (int bk = bj; bk < bi; ++bk) {
+    __syncthreads();
+    load_tile(As, l + (size_t)bk * TB * np + bi * TB, np);
+    for (int e = tid; e < TB * TB; e += 256) {
+      const int c = e >> 6, t = e & 63;
+      Bs[c * LDS + t] = x[(size_t)(bj * TB + c) * np + bk * TB + t];
+    }
+    __syncthreads();
+    mm64<false>(As, Bs, 1, LDS, acc);
+  }
+  __syncthreads();
+  load_tile(As, x + (size_t)bi * TB * np + bi * TB, np);
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      Bs[(ty + 16 * j) * LDS + tx + 16 * i] = acc[i][j];
+      acc[i][j] = make_float2(0.f, 0.f);
+    }
+  __syncthreads();
+  mm64<false>(As, Bs, 1, LDS, acc);
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      x[(size_t)(bj * TB + ty + 16 * j) * np + bi * TB + tx + 16 * i] =
+          make_float2(-acc[i][j].x, -acc[i][j].y);
+}
+
+// Lh = D^-1/2 X W in place on the lower tiles
+__global__ void __launch_bounds__(256) filt_lhat_kernel(const zf* __restrict__ A,
+                                                        zf* __restrict__ X, int np,
+                                                        const float* __restrict__ w) {
+  int bi, bk;
+  tile_of(blockIdx.x, bi, bk);
+  const int k = blockIdx.y, r = bi * TB + (threadIdx.x & 63);
+  zf* x = X + (size_t)k * np * np;
+  const float dr = rsqrtf(fabsf(A[(size_t)k * np * np + (size_t)r * (np + 1)].x));
+#pragma unroll 4
+  for (int q = threadIdx.x >> 6; q < TB; q += 4) {
+    const int c = bk * TB + q;
+    zf* p = x + (size_t)c * np + r;
+    *p = zscale(*p, dr * w[(size_t)k * np + c]);
+  }
+}
+
+// ---------------------------------------------------------------- B products
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src));
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src));
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N));
+}
+
+// One block row (64) of Lh V (FWD) or Lh^dagger V, V: 32 columns of np; 128
+// threads, 4 x 4 complex each, K in chunks of 32 through a two-stage
+// cp.async ring.  The backward product's epilogue forms the next Chebyshev
+// term (coefficients per column: cf[0] B E + cf[1] E + cf[2] E_prev + cf[3] g,
+// written over E_prev), or g = B R and E_1 = cf[3] g when E is null.
+constexpr int KC = 32;
+constexpr int AP_SMEM = 2 * (KC * (TB + 2) + KC * (FB + 1) + 8) * (int)sizeof(zf);
+
+template <bool FWD>
+__global__ void __launch_bounds__(128) filt_apply_kernel(
+    const zf* __restrict__ Lh, const zf* __restrict__ V, int np, zf* __restrict__ out,
+    const float* __restrict__ coef, int cstride, const zf* __restrict__ E, zf* __restrict__ Ep,
+    zf* __restrict__ g, const int* __restrict__ done) {
+  if (done[blockIdx.y]) return;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  constexpr int ASZ = KC * (TB + 2), BSZ = KC * (FB + 1) + 8;
+  zf* As[2] = {reinterpret_cast<zf*>(dsm), reinterpret_cast<zf*>(dsm) + ASZ};
+  zf* Bs[2] = {reinterpret_cast<zf*>(dsm) + 2 * ASZ, reinterpret_cast<zf*>(dsm) + 2 * ASZ + BSZ};
+  const int k = blockIdx.y, nt = np / TB;
+  // the longest block rows first
+  const int b = FWD ? nt - 1 - (int)blockIdx.x : (int)blockIdx.x;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const zf* l = Lh + (size_t)k * np * np;
+  const zf* v = V + (size_t)k * FB * np;
+  const int kbeg = FWD ? 0 : b * TB, nch = (FWD ? (b + 1) * TB : np - b * TB) / KC;
+  auto load = [&](int st, int k0) {
+    if (FWD) {
+      for (int e = tid; e < KC * TB / 2; e += 128) {
+        const int t = e >> 5, r2 = e & 31;
+        cp_async16(As[st] + t * TB + 2 * r2, l + (size_t)(k0 + t) * np + b * TB + 2 * r2);
+      }
+    } else {
+      for (int e = tid; e < KC * TB; e += 128) {
+        const int r = e >> 5, t = e & 31;
+        cp_async8(As[st] + r * (KC + 1) + t, l + (size_t)(b * TB + r) * np + k0 + t);
+      }
+    }
+    for (int e = tid; e < KC * FB; e += 128) {
+      const int c = e >> 5, t = e & 31;
+      cp_async8(Bs[st] + c * (KC + 1) + t, v + (size_t)c * np + k0 + t);
+    }
+    cp_commit();
+  };
+  zf acc[4][4] = {};
+  load(0, kbeg);
+  for (int ch = 0; ch < nch; ++ch) {
+    if (ch + 1 < nch) {
+      load((ch + 1) & 1, kbeg + (ch + 1) * KC);
+      cp_wait<1>();
+    } else {
+      cp_wait<0>();
+    }
+    __syncthreads();
+    const zf* a_ = As[ch & 1];
+    const zf* b_ = Bs[ch & 1];
+#pragma unroll 8
+    for (int t = 0; t < KC; ++t) {
+      zf a[4], bb[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        a[i] = FWD ? a_[t * TB + tx + 16 * i] : a_[(tx + 16 * i) * (KC + 1) + t];
+        if (!FWD) a[i].y = -a[i].y;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) bb[j] = b_[(ty + 8 * j) * (KC + 1) + t];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = cfma(a[i], bb[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+  const size_t base = (size_t)k * FB * np;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = ty + 8 * j;
+    float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
+    if (!FWD) {
+      const float* cf = coef + (size_t)k * cstride + c;
+      c0 = cf[0];
+      c1 = cf[FB];
+      c2 = cf[2 * FB];
+      c3 = cf[3 * FB];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const size_t o = base + (size_t)c * np + b * TB + tx + 16 * i;
+      const zf y = acc[i][j];
+      if (FWD) {
+        out[o] = y;
+      } else if (!E) {
+        g[o] = y;
+        Ep[o] = zscale(y, c3);
+      } else {
+        const zf e = E[o], gg = g[o];
+        const zf p = c2 != 0.f ? Ep[o] : make_float2(0.f, 0.f);
+        Ep[o] = make_float2(c0 * y.x + c1 * e.x + c2 * p.x + c3 * gg.x,
+                            c0 * y.y + c1 * e.y + c2 * p.y + c3 * gg.y);
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------- Rayleigh-Ritz
+// X = unit vectors at ord, CX = the columns of C (full Hermitian storage)
+__global__ void filt_start_kernel(const zd* __restrict__ C, int n, const int* __restrict__ ord,
+                                  zd* __restrict__ X, zd* __restrict__ CX) {
+  const int k = blockIdx.z, i = blockIdx.y, r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= n) return;
+  const int o = ord[(size_t)k * FB + i];
+  const size_t q = ((size_t)k * FB + i) * n + r;
+  X[q] = zmake(r == o ? 1.0 : 0.0, 0.0);
+  CX[q] = C[(size_t)k * n * n + (size_t)o * n + r];
+}
+
+// X += E
+__global__ void filt_add_kernel(zd* __restrict__ X, const zf* __restrict__ E, int n, int np,
+                                const int* __restrict__ done) {
+  const int k = blockIdx.z, i = blockIdx.y, r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= n || done[k]) return;
+  zd* x = X + ((size_t)k * FB + i) * n + r;
+  const zf e = E[((size_t)k * FB + i) * np + r];
+  *x = zmake(x->x + (double)e.x, x->y + (double)e.y);
+}
+
+template <typename R>
+struct RrSmem {   // rows of X and C X in the arithmetic of the step
+  typename Cplx<R>::T X[GR][FB + 1], Y[GR][FB + 1];
+};
+
+template <typename R>
+__device__ __forceinline__ void rr_load(RrSmem<R>& sm, const zd* X, const zd* CX, int n, int r0,
+                                        int nthreads) {
+  typedef typename Cplx<R>::T T;
+  for (int e = threadIdx.x; e < GR * FB; e += nthreads) {
+    const int c = e / GR, r = e % GR;
+    T x = Cplx<R>::make((R)0, (R)0), y = x;
+    if (r0 + r < n) {
+      const zd a = X[(size_t)c * n + r0 + r], b = CX[(size_t)c * n + r0 + r];
+      x = Cplx<R>::make((R)a.x, (R)a.y);
+      y = Cplx<R>::make((R)b.x, (R)b.y);
+    }
+    sm.X[r][c] = x;
+    sm.Y[r][c] = y;
+  }
+}
+
+// Partial Gram matrices over 64 rows: G = X^dagger X and H = X^dagger C X, lower
+// triangle in 2 x 2 blocks, one per thread (2 x 136 of 288 threads).
+constexpr int GT = 288;
+template <typename R>
+__global__ void __launch_bounds__(GT) filt_gram_kernel(const zd* __restrict__ X,
+                                                       const zd* __restrict__ CX, int n,
+                                                       zd* __restrict__ part,
+                                                       const int* __restrict__ done) {
+  if (done[blockIdx.y]) return;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  typedef typename Cplx<R>::T T;
+  RrSmem<R>& sm = *reinterpret_cast<RrSmem<R>*>(dsm);
+  const int k = blockIdx.y, ch = blockIdx.x, tid = threadIdx.x;
+  rr_load(sm, X + (size_t)k * FB * n, CX + (size_t)k * FB * n, n, ch * GR, GT);
+  __syncthreads();
+  if (tid >= 272) return;
+  const int mat = tid >= 136;
+  int bi, bj;
+  tile_of(mat ? tid - 136 : tid, bi, bj);
+  T acc[2][2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) acc[i][j] = Cplx<R>::make((R)0, (R)0);
+  const int rows = min(GR, n - ch * GR);
+#pragma unroll 4
+  for (int r = 0; r < rows; ++r) {
+    const T a0 = sm.X[r][2 * bi], a1 = sm.X[r][2 * bi + 1];
+    const T b0 = mat ? sm.Y[r][2 * bj] : sm.X[r][2 * bj];
+    const T b1 = mat ? sm.Y[r][2 * bj + 1] : sm.X[r][2 * bj + 1];
+    acc[0][0] = zfmac(b0, a0, acc[0][0]);   // conj(a) b
+    acc[0][1] = zfmac(b1, a0, acc[0][1]);
+    acc[1][0] = zfmac(b0, a1, acc[1][0]);
+    acc[1][1] = zfmac(b1, a1, acc[1][1]);
+  }
+  zd* p = part + (((size_t)k * gridDim.x + ch) * 2 + mat) * FB * FB;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      p[(2 * bi + i) * FB + 2 * bj + j] = zmake((double)acc[i][j].x, (double)acc[i][j].y);
+}
+
+// X <- X W, R / s = (C X W - X W Theta) / s in FP32 (zero in the padding) and
+// the sums of its squares per column (one partial per warp of rows)
+template <typename R>
+__global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
+                                                          const zd* __restrict__ CX, int n, int np,
+                                                          const zd* __restrict__ W,
+                                                          const double* __restrict__ theta,
+                                                          const double* __restrict__ shift,
+                                                          zf* __restrict__ Rr,
+                                                          float* __restrict__ rpart,
+                                                          const int* __restrict__ done) {
+  if (done[blockIdx.y]) return;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  typedef typename Cplx<R>::T T;
+  RrSmem<R>& sm = *reinterpret_cast<RrSmem<R>*>(dsm);
+  T* Ws = reinterpret_cast<T*>(dsm + sizeof(RrSmem<R>));   // [l][c]
+  const int k = blockIdx.y, ch = blockIdx.x, tid = threadIdx.x;
+  zd* xk = X + (size_t)k * FB * n;
+  rr_load(sm, xk, CX + (size_t)k * FB * n, n, ch * GR, 256);
+  for (int e = tid; e < FB * FB; e += 256) {
+    const zd w = W[(size_t)k * FB * FB + e];   // column-major: l + c FB
+    Ws[(e % FB) * FB + e / FB] = Cplx<R>::make((R)w.x, (R)w.y);
+  }
+  __syncthreads();
+  const int r = tid & 63, c0 = (tid >> 6) * 8;
+  const int row = ch * GR + r;
+  const double is = 1.0 / shift[k];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {   // two passes of four columns
+    T xa[4], ya[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) xa[j] = ya[j] = Cplx<R>::make((R)0, (R)0);
+#pragma unroll 4
+    for (int l = 0; l < FB; ++l) {
+      const T xv = sm.X[r][l], yv = sm.Y[r][l];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const T w = Ws[l * FB + c0 + 4 * h + j];
+        xa[j] = zfma(xv, w, xa[j]);
+        ya[j] = zfma(yv, w, ya[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int c = c0 + 4 * h + j;
+      const double t = theta[(size_t)k * FB + c];
+      zf rv = make_float2(0.f, 0.f);
+      if (row < n) {
+        xk[(size_t)c * n + row] = zmake((double)xa[j].x, (double)xa[j].y);
+        rv = make_float2((float)(((double)ya[j].x - t * (double)xa[j].x) * is),
+                         (float)(((double)ya[j].y - t * (double)xa[j].y) * is));
+      }
+      if (row < np) Rr[((size_t)k * FB + c) * np + row] = rv;
+      float q = rv.x * rv.x + rv.y * rv.y;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      if ((tid & 31) == 0)
+        rpart[(((size_t)k * gridDim.x + ch) * 2 + ((tid >> 5) & 1)) * FB + c] = q;
+    }
+  }
+}
+
+// cyclic Jacobi of the 32 x 32 Hermitian matrix A (shared, stride FB + 1) with
+// the round-robin pairing: one thread per pair of index pairs applies both
+// sides' rotations to its 2 x 2 block (the blocks partition A), two threads'
+// worth of work per pair and row rotate V.  256 threads.
+template <typename R>
+__device__ void jacobi32(typename Cplx<R>::T (*A)[FB + 1], typename Cplx<R>::T (*V)[FB + 1],
+                         R offtol, int maxsweep, R* red) {
+  typedef typename Cplx<R>::T T;
+  __shared__ R cs_[FB / 2], sn_[FB / 2];
+  __shared__ T ph_[FB / 2];
+  const int tid = threadIdx.x;
+  const int u = tid >> 4, v = tid & 15;
+  for (int sweep = 0; sweep < maxsweep; ++sweep) {
+    R o = 0, t = 0;
+    for (int e = tid; e < FB * FB; e += 256) {
+      const int r = e >> 5, c = e & 31;
+      const T a = A[r][c];
+      const R m2 = a.x * a.x + a.y * a.y;
+      t += m2;
+      if (r != c) o += m2;
+    }
+    for (int sh = 16; sh > 0; sh >>= 1) {
+      o += __shfl_xor_sync(0xffffffffu, o, sh);
+      t += __shfl_xor_sync(0xffffffffu, t, sh);
+    }
+    if ((tid & 31) == 0) {
+      red[2 * (tid >> 5)] = o;
+      red[2 * (tid >> 5) + 1] = t;
+    }
+    __syncthreads();
+    R so = 0, stt = 0;
+    for (int q = 0; q < 8; ++q) {
+      so += red[2 * q];
+      stt += red[2 * q + 1];
+    }
+    if (!(so > offtol * stt)) break;   // also ends on NaN
+    const R skip = offtol * stt / (R)(FB * FB);   // pairs already below the stopping size
+    for (int rd = 0; rd < FB - 1; ++rd) {
+      auto pair = [&](int m, int& p, int& q) {
+        if (m == 0) {
+          p = rd;
+          q = FB - 1;
+        } else {
+          p = rd + m;
+          if (p >= FB - 1) p -= FB - 1;
+          q = rd - m;
+          if (q < 0) q += FB - 1;
+        }
+        if (p > q) {
+          const int w = p;
+          p = q;
+          q = w;
+        }
+      };
+      int act = 0;
+      if (tid < FB / 2) {
+        int p, q;
+        pair(tid, p, q);
+        const T c = A[p][q];
+        const R c2 = c.x * c.x + c.y * c.y;
+        R cs = 1, sn = 0;
+        T ph = Cplx<R>::make((R)1, (R)0);
+        if (c2 > skip * (R)0.25) {
+          act = 1;
+          const R ica = rsqrt(c2), ca = c2 * ica;
+          ph = Cplx<R>::make(c.x * ica, c.y * ica);
+          const R zeta = (A[q][q].x - A[p][p].x) * (R)0.5 / ca;
+          const R az = zeta < 0 ? -zeta : zeta;
+          // beyond 1e9 (FP32: 1e6) the rotation is 1 / (2 zeta) to rounding
+          R tt = (R)1 / (az + sqrt((R)1 + az * az));
+          if (zeta < 0) tt = -tt;
+          cs = rsqrt((R)1 + tt * tt);
+          sn = tt * cs;
+        }
+        cs_[tid] = cs;
+        sn_[tid] = sn;
+        ph_[tid] = ph;
+      }
+      if (!__syncthreads_or(act)) continue;
+      // J = [[cs, sn], [-sn conj(ph), cs conj(ph)]] on columns (p, q); A <- J_u^dagger A J_v
+      {
+        int pu, qu, pv, qv;
+        pair(u, pu, qu);
+        pair(v, pv, qv);
+        const R cu = cs_[u], su = sn_[u], cv = cs_[v], sv = sn_[v];
+        const T fu = ph_[u], fv = zconj(ph_[v]);
+        const T a00 = A[pu][pv], a01 = zmul(A[pu][qv], fv);
+        const T a10 = zmul(A[qu][pv], fu), a11 = zmul(zmul(A[qu][qv], fv), fu);
+        const T b00 = zsub(zscale(a00, cv), zscale(a01, sv));
+        const T b01 = zadd(zscale(a00, sv), zscale(a01, cv));
+        const T b10 = zsub(zscale(a10, cv), zscale(a11, sv));
+        const T b11 = zadd(zscale(a10, sv), zscale(a11, cv));
+        A[pu][pv] = zsub(zscale(b00, cu), zscale(b10, su));
+        A[pu][qv] = zsub(zscale(b01, cu), zscale(b11, su));
+        A[qu][pv] = zadd(zscale(b00, su), zscale(b10, cu));
+        A[qu][qv] = zadd(zscale(b01, su), zscale(b11, cu));
+        // rows of V: pair v, rows u and u + 16
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = u + 16 * h;
+          const T vp = V[r][pv], vq = zmul(V[r][qv], fv);
+          V[r][pv] = zsub(zscale(vp, cv), zscale(vq, sv));
+          V[r][qv] = zadd(zscale(vp, sv), zscale(vq, cv));
+        }
+      }
+      __syncthreads();
+    }
+  }
+  __syncthreads();
+}
+
+// H w = theta G w per matrix from the Gram partials: FP64 Cholesky of the
+// unit-diagonal G and its inverse factor (one barrier per column, as
+// ldl64_block), A = L^-1 H L^-dagger, Jacobi in R, W = S L^-dagger V.  fail: G not
+// positive definite.
+//
+// The FP64 Jacobi starts from the FP32 one: a sweep of 31 rotation rounds is
+// bound by the SM's FP64 pipe (2 FMA per clock), so the FP32 eigenvectors, made
+// orthonormal to 1e-12 by one Newton-Schulz step, first make A diagonal to
+// 1e-6, and one or two FP64 sweeps finish it; the vectors' norms are divided out.
+typedef zd Zd32[FB][FB + 1];
+struct EigSmem {
+  Zd32 G, H, Li, V;
+  zf A32[FB][FB + 1], V32[FB][FB + 1];
+};
+
+// D = op(A) B (op: conjugate transpose when CT), lower triangle only when herm
+template <bool CT>
+__device__ __forceinline__ void mul32(const Zd32& A, const Zd32& B, Zd32& D, bool herm) {
+  for (int e = threadIdx.x; e < FB * FB; e += 256) {
+    const int r = e / FB, c = e % FB;
+    if (herm && r < c) continue;
+    zd s = zmake(0.0, 0.0);
+    for (int t = 0; t < FB; ++t) s = CT ? zfmac(B[t][c], A[t][r], s) : zfma(A[r][t], B[t][c], s);
+    if (herm) {
+      if (r == c) s.y = 0.0;
+      D[c][r] = zconj(s);
+    }
+    D[r][c] = s;
+  }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ part, int nch,
+                                                       double* __restrict__ theta,
+                                                       zd* __restrict__ W,
+                                                       int* __restrict__ fail,
+                                                       const int* __restrict__ done) {
+  if (done[blockIdx.x]) return;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  EigSmem& sm = *reinterpret_cast<EigSmem*>(dsm);
+  __shared__ double sc[FB], ev[FB], sc_top;
+  __shared__ double red[16];
+  __shared__ int rank[FB], bad, out[FB];
+  // a pivot of the unit-diagonal G below the rounding of its entries
+  constexpr double kTiny = sizeof(R) == 8 ? 1e-13 : 1e-5;
+  const int k = blockIdx.x, tid = threadIdx.x;
+  if (tid == 0) bad = 0;
+  for (int e = tid; e < FB * FB; e += 256) {
+    const int r = e / FB, c = e % FB;
+    if (r < c) continue;
+    zd g = zmake(0.0, 0.0), h = g;
+    for (int q = 0; q < nch; ++q) {
+      const zd* p = part + ((size_t)k * nch + q) * 2 * FB * FB + e;
+      g = zadd(g, p[0]);
+      h = zadd(h, p[FB * FB]);
+    }
+    if (r == c) g.y = h.y = 0.0;
+    sm.G[r][c] = g;
+    sm.H[r][c] = h;
+    sm.H[c][r] = zconj(h);
+  }
+  __syncthreads();
+  if (tid < FB) {
+    const double g = sm.G[tid][tid].x;
+    sc[tid] = g > 0.0 ? rsqrt(g) : 0.0;
+    out[tid] = 0;
+  }
+  __syncthreads();
+  for (int e = tid; e < FB * FB; e += 256) {
+    const int r = e / FB, c = e % FB;
+    const double f = sc[r] * sc[c];
+    if (r >= c) sm.G[r][c] = zscale(sm.G[r][c], f);
+    sm.H[r][c] = zscale(sm.H[r][c], f);
+    sm.Li[r][c] = zmake(r == c ? 1.0 : 0.0, 0.0);
+    sm.V32[r][c] = make_float2(r == c ? 1.f : 0.f, 0.f);
+  }
+  __syncthreads();
+  {
+    // unit L and pivots: G = L D L^dagger; Li accumulates L^-1
+    const int r = tid & 31, q = tid >> 5;
+    for (int c = 0; c < FB; ++c) {
+      double p = sm.G[c][c].x;
+      if (!(p > kTiny)) {
+        if (tid == 0) {
+          bad = 1;
+          out[c] = 1;
+        }
+        p = 1.0;
+      }
+      const double inv = 1.0 / p;
+      if (r > c) {
+        const zd l = zscale(sm.G[r][c], inv);
+        for (int s = c + 1 + q; s <= r; s += 8) sm.G[r][s] = zfnmac(l, sm.G[s][c], sm.G[r][s]);
+        for (int s = q; s <= c; s += 8) sm.Li[r][s] = zfnma(l, sm.Li[c][s], sm.Li[r][s]);
+      }
+      __syncthreads();
+    }
+    if (tid == 0) fail[k] = bad;
+    if (tid < FB) {
+      const double p = sm.G[tid][tid].x;
+      ev[tid] = p > kTiny ? rsqrt(p) : 1.0;
+    }
+    __syncthreads();
+    for (int e = tid; e < FB * FB; e += 256) {
+      const int rr = e / FB, c = e % FB;
+      sm.Li[rr][c] = rr >= c ? zscale(sm.Li[rr][c], ev[rr]) : zmake(0.0, 0.0);
+    }
+    __syncthreads();
+  }
+  // G <- Li H, then H <- (Li H) Li^dagger (lower triangle, mirrored)
+  for (int e = tid; e < FB * FB; e += 256) {
+    const int r = e / FB, c = e % FB;
+    zd s = zmake(0.0, 0.0);
+    for (int t = 0; t <= r; ++t) s = zfma(sm.Li[r][t], sm.H[t][c], s);
+    sm.G[r][c] = s;
+  }
+  __syncthreads();
+  for (int e = tid; e < FB * FB; e += 256) {
+    const int r = e / FB, c = e % FB;
+    if (r < c) continue;
+    zd s = zmake(0.0, 0.0);
+    for (int t = 0; t <= c; ++t) s = zfmac(sm.G[r][t], sm.Li[c][t], s);
+    if (r == c) s.y = 0.0;
+    sm.H[r][c] = s;
+    sm.H[c][r] = zconj(s);
+    sm.A32[r][c] = make_float2((float)s.x, (float)s.y);
+    sm.A32[c][r] = make_float2((float)s.x, (float)-s.y);
+  }
+  __syncthreads();
+  if (bad) {
+    // vectors that depend on the others: decoupled, at the top of the spectrum
+    if (tid < 32) {
+      double m = out[tid] ? 0.0 : sm.H[tid][tid].x;
+      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (tid == 0) sc_top = m;
+    }
+    __syncthreads();
+    for (int e = tid; e < FB * FB; e += 256) {
+      const int r = e / FB, c = e % FB;
+      if (!out[r] && !out[c]) continue;
+      sm.H[r][c] = zmake(r == c ? sc_top : 0.0, 0.0);
+      sm.A32[r][c] = make_float2(r == c ? (float)sc_top : 0.f, 0.f);
+    }
+    __syncthreads();
+  }
+  // FP32: off-diagonal norm below 1e-6 of the whole
+  jacobi32<float>(sm.A32, sm.V32, 1e-12f, 12, reinterpret_cast<float*>(red));
+  for (int e = tid; e < FB * FB; e += 256) {
+    const zf v = sm.V32[e / FB][e % FB];
+    sm.V[e / FB][e % FB] = zmake((double)v.x, (double)v.y);
+  }
+  __syncthreads();
+  if (sizeof(R) == 8) {
+    mul32<true>(sm.V, sm.V, sm.G, true);
+    __syncthreads();
+    for (int e = tid; e < FB * FB; e += 256) {   // (3 I - V^dagger V) / 2
+      const int r = e / FB, c = e % FB;
+      const zd g = sm.G[r][c];
+      sm.G[r][c] = zmake((r == c ? 1.5 : 0.0) - 0.5 * g.x, -0.5 * g.y);
+    }
+    __syncthreads();
+    // the corrected V goes where the FP32 matrices lay (they are done with)
+    Zd32& V = *reinterpret_cast<Zd32*>(&sm.A32[0][0]);
+    mul32<false>(sm.V, sm.G, V, false);
+    __syncthreads();
+    mul32<false>(sm.H, V, sm.G, false);
+    __syncthreads();
+    mul32<true>(V, sm.G, sm.H, true);
+    __syncthreads();
+    // off-diagonal norm below 1e-10 of the whole: the Ritz values then carry
+    // (1e-10 ||H||)^2 / gap
+    jacobi32<double>(sm.H, V, 1e-20, 12, red);
+    // columns of V to unit length
+    const int c = tid >> 3, q = tid & 7;
+    double v2 = 0.0;
+    for (int r = q; r < FB; r += 8) v2 = fma(V[r][c].x, V[r][c].x, fma(V[r][c].y, V[r][c].y, v2));
+    for (int o = 4; o > 0; o >>= 1) v2 += __shfl_xor_sync(0xffffffffu, v2, o);
+    __syncthreads();
+    const double iv = rsqrt(v2);
+    if (q == 0) ev[c] = sm.H[c][c].x * iv * iv;
+    for (int r = q; r < FB; r += 8) sm.V[r][c] = zscale(V[r][c], iv);
+  } else {
+    if (tid < FB) ev[tid] = (double)sm.A32[tid][tid].x;
+  }
+  __syncthreads();
+  if (tid < FB) {
+    const double x = ev[tid];
+    int rk = 0;
+    for (int c = 0; c < FB; ++c) rk += ev[c] < x || (ev[c] == x && c < tid);
+    if (!(x == x)) rk = tid;
+    rank[tid] = rk;
+  }
+  __syncthreads();
+  for (int e = tid; e < FB * FB; e += 256) {
+    const int r = e % FB, c = e / FB;   // W[r][rank(c)] = sc_r sum_t conj(Li[t][r]) V[t][c]
+    zd s = zmake(0.0, 0.0);
+    for (int t = r; t < FB; ++t) s = zfmac(sm.V[t][c], sm.Li[t][r], s);
+    W[(size_t)k * FB * FB + r + (size_t)rank[c] * FB] = zscale(s, sc[r]);
+    if (r == 0) theta[(size_t)k * FB + rank[c]] = ev[c];
+  }
+}
+
+// After a Rayleigh-Ritz step, one warp per matrix, lane c = column c: the
+// residual norms and the coefficients of a degree-m filter.  The polynomial
+// is T_j(l(mu)), l(mu) = 2 mu / mu_cut - 1 with mu_cut that of the last guard
+// vector, so l >= 1 on the block.  A column stops at the last degree whose
+// growth relative to it, tau_j(l_0) / tau_j(l_c) (the lowest branch grows
+// most), times what the residual holds of the other branches stays below 0.1:
+// 6e-8 of itself (FP32 rounding), `couple` of the block's largest Ritz value
+// (the off-diagonal the Jacobi sweeps left) and the rounding of C X.  Beyond,
+// the column would turn into the lowest branches and the block lose rank.
+__global__ void __launch_bounds__(128) filt_coef_kernel(const double* __restrict__ theta,
+                                                        const float* __restrict__ rpart, int nch,
+                                                        const double* __restrict__ shift, int kb,
+                                                        const double* __restrict__ cmax,
+                                                        double couple, int m,
+                                                        float* __restrict__ coef,
+                                                        const int* __restrict__ done) {
+  const int k = blockIdx.x * 4 + (threadIdx.x >> 5), c = threadIdx.x & 31;
+  if (k >= kb || done[k]) return;
+  float rn = 0.f;
+  for (int q = 0; q < 2 * nch; ++q) rn += rpart[((size_t)k * 2 * nch + q) * FB + c];
+  const double t = fmax(theta[(size_t)k * FB + c] / shift[k], 0.0);
+  const double cut = __shfl_sync(0xffffffffu, t, 31);
+  const double mu = 1.0 / (t + 1.0), imuc = cut + 1.0;
+  const double l = fmax(2.0 * mu * imuc - 1.0, 1.0), f = 2.0 * mu * imuc;
+  const double lim = 0.1 / (6e-8 * (double)sqrtf(rn) + couple * cut +
+                            4.0 * DBL_EPSILON * cmax[k] / shift[k]);
+  float* cf = coef + (size_t)k * BS_FILT_MAXDEG * 4 * FB + c;
+  double t0 = 1.0, t1 = l;   // tau_{j-1}, tau_j
+  bool stop = __shfl_sync(0xffffffffu, t1, 0) > lim * t1;
+  // step 0 (from g): E_1 = -(f / tau_1) g
+  cf[0] = cf[FB] = cf[2 * FB] = 0.f;
+  cf[3 * FB] = stop ? 0.f : (float)(-f / t1);
+  for (int j = 1; j < m; ++j) {
+    const double t2 = 2.0 * l * t1 - t0;
+    const double g2 = __shfl_sync(0xffffffffu, t2, 0);
+    stop = stop || g2 > lim * t2;
+    const double s1 = t1 / t2, s0 = t0 / t2;
+    cf += 4 * FB;
+    cf[0] = stop ? 0.f : (float)(4.0 * imuc * s1);
+    cf[FB] = stop ? 1.f : (float)(-2.0 * s1);
+    cf[2 * FB] = stop || j == 1 ? 0.f : (float)(-s0);   // E_0 = 0
+    cf[3 * FB] = stop ? 0.f : (float)(-2.0 * s1 * f);
+    t0 = t1;
+    t1 = t2;
+  }
+}
+
+// Certificate of the last Rayleigh-Ritz step, one warp per matrix: the cut
+// (a gap of at least 2e-3 above a Ritz value i >= nb - 1, sigma in it) with the
+// smallest error sum; omega; sigma and the count it has to have (-1: the
+// sum is too large or there is no gap).  The inertia of the scaled matrix in
+// FP32 is exact for a matrix within a relative 1e-4 of C in the form sense
+// (n 2^-24 of the scaled diagonal, doubled), so rho is sigma less that.
+__global__ void __launch_bounds__(128) filt_cert_kernel(
+    const double* __restrict__ theta, const float* __restrict__ rpart, int nch,
+    const double* __restrict__ shift, const double* __restrict__ cmax, int kb, int nb,
+    const int* __restrict__ fail, double* __restrict__ omega, double* __restrict__ sigma,
+    int* __restrict__ expect, int* __restrict__ done) {
+  const int k = blockIdx.x * 4 + (threadIdx.x >> 5), c = threadIdx.x & 31;
+  if (k >= kb || done[k]) return;
+  const double s = shift[k];
+  float q32 = 0.f;
+  for (int q = 0; q < 2 * nch; ++q) q32 += rpart[((size_t)k * 2 * nch + q) * FB + c];
+  const double t = theta[(size_t)k * FB + c];
+  const double r2 = 1.001 * (double)q32 * s * s;   // 0.1 % for the FP32 sum
+  const double tn = __shfl_down_sync(0xffffffffu, t, 1);
+  // lane i: the cut above Ritz value i
+  const double gap = tn - t, at = fmax(t, 1e-3 * s);
+  const double sig = t + 0.5 * fmin(gap, 0.02 * at);
+  const double rho = sig - 1e-4 * at;
+  double err = 0.0;
+  for (int i = 0; i < FB; ++i) {
+    const double ti = __shfl_sync(0xffffffffu, t, i), ri = __shfl_sync(0xffffffffu, r2, i);
+    if (i <= c) err += ri / (rho - ti);
+  }
+  const bool usable = c >= nb - 1 && c < FB - 1 && gap >= 2e-3 * fmax(tn, 1e-3 * s) && rho > t &&
+                      err >= 0.0;
+  double best = usable ? err : INFINITY;
+  int at_i = c;
+  for (int o = 16; o > 0; o >>= 1) {
+    const double e2 = __shfl_xor_sync(0xffffffffu, best, o);
+    const int i2 = __shfl_xor_sync(0xffffffffu, at_i, o);
+    if (e2 < best || (e2 == best && i2 < at_i)) {
+      best = e2;
+      at_i = i2;
+    }
+  }
+  const double sg = __shfl_sync(0xffffffffu, sig, at_i);
+  const bool ok = best <= 64.0 * DBL_EPSILON * cmax[k] && !fail[k];
+  if (c < nb) omega[(size_t)k * nb + c] = sqrt(fmax(t, 0.0));
+  if (c == 0) {
+    done[k] = ok;
+    sigma[k] = ok ? sg : 0.0;
+    expect[k] = ok ? at_i + 1 : -1;
+  }
+}
+
+// the matrices that did not pass, in order; one CTA
+__global__ void __launch_bounds__(1024) filt_decide_kernel(const int* __restrict__ neg,
+                                                           const int* __restrict__ flag,
+                                                           const int* __restrict__ expect, int kb,
+                                                           int* __restrict__ stat,
+                                                           int* __restrict__ list,
+                                                           int* __restrict__ nlist) {
+  __shared__ int cnt[32], base;
+  const int tid = threadIdx.x;
+  if (tid == 0) base = 0;
+  for (int k0 = 0; k0 < kb; k0 += 1024) {
+    const int k = k0 + tid;
+    const bool bad = k < kb && (expect[k] < 0 || flag[k] || neg[k] != expect[k]);
+    const unsigned m = __ballot_sync(0xffffffffu, bad);
+    if ((tid & 31) == 0) cnt[tid >> 5] = __popc(m);
+    __syncthreads();
+    int off = base;
+    for (int w = 0; w < (tid >> 5); ++w) off += cnt[w];
+    if (bad) list[off + __popc(m & ((1u << (tid & 31)) - 1u))] = k;
+    if (k < kb) stat[k] = 0;
+    __syncthreads();
+    if (tid == 0)
+      for (int w = 0; w < 32; ++w) base += cnt[w];
+    __syncthreads();
+  }
+  if (tid == 0) *nlist = base;
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------- host side
+// Largest number of branches, and the sizes, that the filtered iteration
+// takes: at least 10 guard vectors beside the wanted ones, diagonals that fit
+// the set-up kernel's shared memory, and an order from which its some 200
+// launches take less than the reduction's n dependent steps also for a
+// single matrix (ms of one solve, iteration / reduction, 1 and 64 matrices:
+// n = 98 3.9 / 2.4 and 4.2 / 3.6, n = 162 4.4 / 4.1 and 5.8 / 7.4,
+// n = 242 4.8 / 6.3 and 6.8 / 14.5, n = 578 8.1 / 40.5 and 18.2 / 61.8).
+bool bs_filter_fits(int n, int nbands) {
+  return nbands >= 1 && nbands <= BS_FILT_MAX_BANDS && n >= BS_FILT_MIN_N && n <= 2048;
+}
+
+void bs_filter_ws_free(FilterWs* w) {
+  void* p[] = {w->A, w->X, w->pA, w->pB, w->pD, w->eA, w->eB, w->Xb, w->CX, w->vec, w->part,
+               w->rpart, w->theta, w->W, w->coef, w->shift, w->cmax, w->sigma, w->ord, w->w, w->iw};
+  for (void* q : p) cudaFree(q);
+  *w = FilterWs();
+}
+
+// bytes of workspace per matrix (the digit planes of C and the two FP32
+// factors are most of it)
+static size_t filter_bytes(int n) {
+  const size_t np = (n + TB - 1) / TB * TB, Kp = (2 * (size_t)n + 63) / 64 * 64;
+  return 2 * np * np * sizeof(zf) + (size_t)n * 8 * Kp * 2 + 2 * FB * 8 * Kp * 2 +
+         (size_t)24 * 2 * FB * n * 4 + 2 * (size_t)FB * n * sizeof(zd) +
+         5 * FB * np * sizeof(zf) + 65536;
+}
+
+int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
+  // chunks of at most about 8 GB of workspace, and of the slab launches' grid limit
+  const int cap = (int)std::max<size_t>(1, std::min<size_t>(1000, ((size_t)8 << 30) / filter_bytes(n)));
+  const int kf = std::min(kb, cap);
+  if (w->n == n && w->kf >= kf) return BS_OK;
+  bs_filter_ws_free(w);
+  const size_t np = (n + TB - 1) / TB * TB, Kp = (2 * (size_t)n + 63) / 64 * 64;
+  const size_t nch = (n + GR - 1) / GR;
+  const size_t k = kf;
+  struct Item { void** p; size_t bytes; } items[] = {
+      {(void**)&w->A, k * np * np * sizeof(zf)},
+      {(void**)&w->X, k * np * np * sizeof(zf)},
+      {(void**)&w->pA, k * n * 8 * Kp * 2},
+      {(void**)&w->pB, k * 2 * FB * 8 * Kp * 2},
+      {(void**)&w->pD, bs_slice_planes(8, (int)Kp, n, 2 * FB, kf) * n * 2 * FB * sizeof(float)},
+      {(void**)&w->eA, k * n * sizeof(int)},
+      {(void**)&w->eB, k * FB * sizeof(int)},
+      {(void**)&w->Xb, k * FB * n * sizeof(zd)},
+      {(void**)&w->CX, k * FB * n * sizeof(zd)},
+      {(void**)&w->vec, 5 * k * FB * np * sizeof(zf)},
+      {(void**)&w->part, k * nch * 2 * FB * FB * sizeof(zd)},
+      {(void**)&w->rpart, k * nch * 2 * FB * sizeof(float)},
+      {(void**)&w->theta, k * FB * sizeof(double)},
+      {(void**)&w->W, k * FB * FB * sizeof(zd)},
+      {(void**)&w->coef, k * BS_FILT_MAXDEG * 4 * FB * sizeof(float)},
+      {(void**)&w->shift, k * sizeof(double)},
+      {(void**)&w->cmax, k * sizeof(double)},
+      {(void**)&w->sigma, k * sizeof(double)},
+      {(void**)&w->ord, k * FB * sizeof(int)},
+      {(void**)&w->w, k * np * sizeof(float)},
+      {(void**)&w->iw, (6 * k + 1) * sizeof(int)},
+  };
+  for (auto& it : items) {
+    if (cudaMalloc(it.p, it.bytes) != cudaSuccess) {
+      cudaGetLastError();
+      bs_filter_ws_free(w);
+      bs_set_error("out of device memory (filtered iteration, %zu bytes)", it.bytes);
+      return BS_ENOMEM;
+    }
+  }
+  w->n = n;
+  w->kf = kf;
+  return BS_OK;
+}
+
+// shared-memory opt-ins, per device
+static int filter_attrs() {
+  static std::atomic<bool> attr[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+  if (attr[dev].load(std::memory_order_acquire)) return BS_OK;
+  struct { const void* f; int bytes; } fs[] = {
+      {(const void*)ldl64_diag_kernel, 2 * TB * LDS * (int)sizeof(zf)},
+      {(const void*)ldl64_panel_kernel, 2 * TB * TB * (int)sizeof(zf)},
+      {(const void*)ldl64_update_kernel, 2 * TB * LDS * (int)sizeof(zf)},
+      {(const void*)trinv64_kernel, (TB * TB + TB * LDS) * (int)sizeof(zf)},
+      {(const void*)filt_apply_kernel<true>, AP_SMEM},
+      {(const void*)filt_apply_kernel<false>, AP_SMEM},
+      {(const void*)filt_gram_kernel<double>, (int)sizeof(RrSmem<double>)},
+      {(const void*)filt_rotate_kernel<double>,
+       (int)(sizeof(RrSmem<double>) + FB * FB * sizeof(zd))},
+      {(const void*)filt_gram_kernel<float>, (int)sizeof(RrSmem<float>)},
+      {(const void*)filt_rotate_kernel<float>, (int)(sizeof(RrSmem<float>) + FB * FB * sizeof(zf))},
+      {(const void*)filt_eig_kernel<double>, (int)sizeof(EigSmem)},
+      {(const void*)filt_eig_kernel<float>, (int)sizeof(EigSmem)},
+  };
+  for (auto& f : fs) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(f.f, cudaFuncAttributeMaxDynamicSharedMemorySize, f.bytes);
+    if (e != cudaSuccess) return bs_cuda_status(e, "filtered iteration smem");
+  }
+  attr[dev].store(true, std::memory_order_release);
+  return BS_OK;
+}
+
+// factor A (kf matrices); with_x: also the full inverse factor
+static int filter_factor(FilterWs& w, int np, int kf, bool inverse, cudaStream_t s) {
+  const int nt = np / TB;
+  int* neg = w.iw;
+  int* flag = w.iw + w.kf;
+  ldl64_diag_kernel<<<kf, 256, 2 * TB * LDS * sizeof(zf), s>>>(w.A, w.X, np, neg, flag);
+  BS_CHECK_LAUNCH("ldl64_diag_kernel");
+  for (int j = 0; j + 1 < nt; ++j) {
+    const int rem = nt - j - 1;
+    ldl64_panel_kernel<<<dim3(rem, kf), 256, 2 * TB * TB * sizeof(zf), s>>>(w.A, w.X, np, j * TB);
+    BS_CHECK_LAUNCH("ldl64_panel_kernel");
+    ldl64_update_kernel<<<dim3(rem * (rem + 1) / 2, kf), 256, 2 * TB * LDS * sizeof(zf), s>>>(
+        w.A, w.X, np, j * TB, neg, flag);
+    BS_CHECK_LAUNCH("ldl64_update_kernel");
+  }
+  if (!inverse) return BS_OK;
+  for (int d = 1; d < nt; ++d) {
+    trinv64_kernel<<<dim3(nt - d, kf), 256, (TB * TB + TB * LDS) * sizeof(zf), s>>>(w.A, w.X, np, d);
+    BS_CHECK_LAUNCH("trinv64_kernel");
+  }
+  filt_lhat_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(w.A, w.X, np, w.w);
+  BS_CHECK_LAUNCH("filt_lhat_kernel");
+  return BS_OK;
+}
+
+template <typename R>
+static int filter_ritz(FilterWs& w, int n, int np, int kf, cudaStream_t s) {
+  const int nch = (n + GR - 1) / GR;
+  int *fail = w.iw + 4 * w.kf + 1, *done = fail + w.kf;
+  filt_gram_kernel<R><<<dim3(nch, kf), GT, sizeof(RrSmem<R>), s>>>(w.Xb, w.CX, n, w.part,
+                                                                      done);
+  BS_CHECK_LAUNCH("filt_gram_kernel");
+  filt_eig_kernel<R><<<kf, 256, sizeof(EigSmem), s>>>(w.part, nch, w.theta, w.W,
+                                                         fail, done);
+  BS_CHECK_LAUNCH("filt_eig_kernel");
+  // the rotation covers the padded rows as well (np <= nch GR)
+  filt_rotate_kernel<R><<<dim3(nch, kf), 256,
+                          sizeof(RrSmem<R>) + FB * FB * sizeof(typename Cplx<R>::T), s>>>(
+      w.Xb, w.CX, n, np, w.W, w.theta, w.shift, w.vec, w.rpart, done);
+  BS_CHECK_LAUNCH("filt_rotate_kernel");
+  return BS_OK;
+}
+
+int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const FilterFallback& fb,
+                         double* omega, int* stat, int* err, cudaStream_t s) {
+  static_assert(TB == GR, "padded rows are covered by the row chunks");
+  // filter degrees of the rounds: the first Ritz values come from plane
+  // waves and misplace the cut, so the first filters are short; the later ones
+  // are long because a Rayleigh-Ritz step costs as much as several products.
+  // Matrices certified after the fourth round skip the others.
+  static const int degs[] = {4, 6, 8, 8, 8, 8};
+  constexpr int rounds = sizeof(degs) / sizeof(degs[0]), base = 4;
+  if (w.n != n || w.kf < 1 || !bs_filter_fits(n, nbands)) {
+    bs_set_error("filtered iteration: workspace for n = %d not set up", n);
+    return BS_EINVAL;
+  }
+  TRY_LAUNCH(filter_attrs());
+  const int np = (n + TB - 1) / TB * TB, nt = np / TB, nch = (n + GR - 1) / GR;
+  for (int k0 = 0; k0 < kb; k0 += w.kf) {
+    const int kf = std::min(w.kf, kb - k0);
+    zd* Ck = C + (size_t)k0 * n * n;
+    int *neg = w.iw, *flag = w.iw + w.kf, *expect = w.iw + 2 * w.kf, *list = w.iw + 3 * w.kf,
+        *nlist = w.iw + 4 * w.kf, *fail = nlist + 1, *done = fail + w.kf;
+    filt_prep_kernel<<<kf, 256, n * sizeof(double), s>>>(Ck, n, np, nbands, 0.2, w.shift, w.cmax,
+                                                         w.ord, w.w, fail, done);
+    BS_CHECK_LAUNCH("filt_prep_kernel");
+    filt_scale_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(Ck, n, np, w.shift, nullptr, w.w,
+                                                                  w.A, neg, flag);
+    BS_CHECK_LAUNCH("filt_scale_kernel");
+    TRY_LAUNCH(filter_factor(w, np, kf, true, s));
+    TRY_LAUNCH(bs_launch_band_pack_trail(Ck, n, 0, n, kf, w.pA, w.eA, s));
+    const dim3 cg((n + 255) / 256, FB, kf);
+    filt_start_kernel<<<cg, 256, 0, s>>>(Ck, n, w.ord, w.Xb, w.CX);
+    BS_CHECK_LAUNCH("filt_start_kernel");
+    const size_t vb = (size_t)w.kf * FB * np;
+    zf *Rr = w.vec, *Tv = w.vec + vb, *g = w.vec + 2 * vb, *E[2] = {w.vec + 3 * vb, w.vec + 4 * vb};
+    const int cstride = BS_FILT_MAXDEG * 4 * FB;
+    for (int rd = 0; rd <= rounds; ++rd) {
+      // the first three steps only steer the iteration: FP32 products of the block
+      if (rd < 3) TRY_LAUNCH(filter_ritz<float>(w, n, np, kf, s));
+      else TRY_LAUNCH(filter_ritz<double>(w, n, np, kf, s));
+      if (rd >= base) {
+        filt_cert_kernel<<<(kf + 3) / 4, 128, 0, s>>>(w.theta, w.rpart, nch, w.shift, w.cmax, kf,
+                                                      nbands, fail, omega + (size_t)k0 * nbands,
+                                                      w.sigma, expect, done);
+        BS_CHECK_LAUNCH("filt_cert_kernel");
+      }
+      if (rd == rounds) break;
+      const int m = degs[rd];
+      filt_coef_kernel<<<(kf + 3) / 4, 128, 0, s>>>(w.theta, w.rpart, nch, w.shift, kf, w.cmax,
+                                                    rd < 3 ? 1e-6 : 1e-10, m, w.coef, done);
+      BS_CHECK_LAUNCH("filt_coef_kernel");
+      const dim3 ag(nt, kf);
+      for (int j = 0; j < m; ++j) {
+        // j = 0: g = B R, E_1; then E_{j+1} from E_j and E_{j-1}
+        const zf* in = j == 0 ? Rr : E[(j - 1) & 1];
+        filt_apply_kernel<true><<<ag, 128, AP_SMEM, s>>>(w.X, in, np, Tv, nullptr, 0, nullptr,
+                                                         nullptr, nullptr, done);
+        BS_CHECK_LAUNCH("filt_apply_kernel");
+        filt_apply_kernel<false><<<ag, 128, AP_SMEM, s>>>(
+            w.X, Tv, np, nullptr, w.coef + (size_t)j * 4 * FB, cstride,
+            j == 0 ? nullptr : E[(j - 1) & 1], E[j & 1], g, done);
+        BS_CHECK_LAUNCH("filt_apply_kernel");
+      }
+      filt_add_kernel<<<cg, 256, 0, s>>>(w.Xb, E[(m - 1) & 1], n, np, done);
+      BS_CHECK_LAUNCH("filt_add_kernel");
+      TRY_LAUNCH(bs_launch_band_av(n, w.Xb, n, (long)FB * n, FB, kf, 8, w.pA, w.pB, w.pD, w.eA,
+                                   w.eB, w.CX, n, (long)FB * n, err, s, done));
+    }
+    filt_scale_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(Ck, n, np, w.shift, w.sigma, w.w,
+                                                                  w.A, neg, flag);
+    BS_CHECK_LAUNCH("filt_scale_kernel");
+    TRY_LAUNCH(filter_factor(w, np, kf, false, s));
+    filt_decide_kernel<<<1, 1024, 0, s>>>(neg, flag, expect, kf, stat + k0, list, nlist);
+    BS_CHECK_LAUNCH("filt_decide_kernel");
+    TRY_LAUNCH(bs_launch_tridiag_list(Ck, n, fb.vec + (size_t)k0 * bs_tridiag_vec_elems(n),
+                                      fb.part + (size_t)k0 * bs_tridiag_part_elems(n),
+                                      fb.de + (size_t)k0 * 2 * n, fb.tau + (size_t)k0 * n,
+                                      fb.beta + (size_t)k0 * n, fb.count + k0, list, nlist, s));
+    TRY_LAUNCH(bs_launch_bisect_list(fb.de + (size_t)k0 * 2 * n, n, kf, nbands,
+                                     omega + (size_t)k0 * nbands, stat + k0, list, nlist, s));
+  }
+  return BS_OK;
+}

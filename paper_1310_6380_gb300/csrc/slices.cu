@@ -525,9 +525,10 @@ __global__ void pack_trail_kernel(const zd* __restrict__ A, int n, int o, int m,
 // grid (nb, kb), block 128
 __global__ void pack_panel_kernel(const zd* __restrict__ V, int ldv, long sv, int m, int nb,
                                   int S, int Kp, uint16_t* __restrict__ out,
-                                  int* __restrict__ ex) {
+                                  int* __restrict__ ex, const int* __restrict__ skip) {
   __shared__ double sh[4];
   const int i = blockIdx.x, k = blockIdx.y;
+  if (skip && skip[k]) return;
   const zd* x = V + (size_t)k * sv + (size_t)i * ldv;
   double mx = 0.0;
   for (int r = threadIdx.x; r < m; r += 128) mx = fmax(mx, fmax(fabs(x[r].x), fabs(x[r].y)));
@@ -552,8 +553,10 @@ __global__ void pack_panel_kernel(const zd* __restrict__ V, int ldv, long sv, in
 // X[k][r + i ldx] = 2^(eA + eB) sum_u 2^(-12-7u) (slabs of order u)[(i, part)][r]
 __global__ void recombine_panel_kernel(const float* __restrict__ Dm, const SliceSlabs sl,
                                        const int* __restrict__ eA, const int* __restrict__ eB,
-                                       int m, int nb, zd* __restrict__ X, int ldx, long sx) {
+                                       int m, int nb, zd* __restrict__ X, int ldx, long sx,
+                                       const int* __restrict__ skip) {
   const int k = blockIdx.y;
+  if (skip && skip[k]) return;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= m * nb) return;
   const int r = idx % m, i = idx / m;
@@ -655,18 +658,18 @@ int bs_launch_band_pack_trail(const zd* A, int n, int o, int m, int kb, uint16_t
 // X = A22 V from the trailing block's digit planes (bs_launch_band_pack_trail)
 int bs_launch_band_av(int m, const zd* V, int ldv, long sv, int nb, int kb, int S, uint16_t* wA,
                       uint16_t* wB, float* wD, int* eA, int* eB, zd* X, int ldx, long sx,
-                      int* err, cudaStream_t s) {
+                      int* err, cudaStream_t s, const int* skip) {
   const int Kp = (2 * m + 63) / 64 * 64;
   SliceSlabs sl;
   if (S != 8 || !bs_slice_slabs(S, Kp, m, 2 * nb, kb, &sl)) {
     bs_set_error("band reduction: m = %d gives too many digit slabs", m);
     return BS_EINVAL;
   }
-  pack_panel_kernel<<<dim3(nb, kb), 128, 0, s>>>(V, ldv, sv, m, nb, S, Kp, wB, eB);
+  pack_panel_kernel<<<dim3(nb, kb), 128, 0, s>>>(V, ldv, sv, m, nb, S, Kp, wB, eB, skip);
   BS_CHECK_LAUNCH("pack_panel_kernel");
-  TRY_LAUNCH(bs_launch_slice_orders(wA, wB, wD, m, 2 * nb, S, Kp, kb, err, s));
+  TRY_LAUNCH(bs_launch_slice_orders(wA, wB, wD, m, 2 * nb, S, Kp, kb, err, s, skip));
   recombine_panel_kernel<<<dim3((m * nb + 255) / 256, kb), 256, 0, s>>>(wD, sl, eA, eB, m, nb, X,
-                                                                       ldx, sx);
+                                                                       ldx, sx, skip);
   BS_CHECK_LAUNCH("recombine_panel_kernel");
   return BS_OK;
 }

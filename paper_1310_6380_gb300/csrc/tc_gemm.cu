@@ -106,7 +106,8 @@ __global__ void __launch_bounds__(128, 2)
     slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                       const __grid_constant__ CUtensorMap tmB, float* __restrict__ D, int M,
                       int N, long ldd, long strideD, const SliceSlabs slabs,
-                      int* __restrict__ err) {
+                      int* __restrict__ err, const int* __restrict__ skip) {
+  if (skip && skip[blockIdx.z / slabs.nq]) return;
   constexpr int TILE_B = tile_b(BN);
   constexpr uint32_t IDESC = idesc(BN);
   extern __shared__ uint8_t smem_raw[];
@@ -466,7 +467,7 @@ static int pick_bn(int N) {
 template <int BN>
 static int launch_bn(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int K,
                      int batch, long sA, long sB, long ldd, long sD, const SliceSlabs& slabs,
-                     int* err, cudaStream_t s) {
+                     int* err, cudaStream_t s, const int* skip) {
   CUtensorMap ta, tb;
   int r = make_map(&ta, A, K, M, batch, sA, BM);
   if (!r) r = make_map(&tb, B, K, N, batch, sB, BN);
@@ -483,20 +484,21 @@ static int launch_bn(const uint16_t* A, const uint16_t* B, float* D, int M, int 
     attr[dev].store(true, std::memory_order_release);
   }
   dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN, batch * slabs.nq);
-  slice_gemm_kernel<BN><<<grid, 128, smem_bytes(BN), s>>>(ta, tb, D, M, N, ldd, sD, slabs, err);
+  slice_gemm_kernel<BN><<<grid, 128, smem_bytes(BN), s>>>(ta, tb, D, M, N, ldd, sD, slabs, err,
+                                                           skip);
   BS_CHECK_LAUNCH("slice_gemm_kernel");
   return BS_OK;
 }
 
 static int dispatch_bn(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int K,
                        int batch, long sA, long sB, long ldd, long sD, const SliceSlabs& slabs,
-                       int* err, cudaStream_t s) {
+                       int* err, cudaStream_t s, const int* skip) {
   switch (pick_bn(N)) {
-    case 64: return launch_bn<64>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s);
-    case 80: return launch_bn<80>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s);
-    case 96: return launch_bn<96>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s);
-    case 112: return launch_bn<112>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s);
-    default: return launch_bn<128>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s);
+    case 64: return launch_bn<64>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
+    case 80: return launch_bn<80>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
+    case 96: return launch_bn<96>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
+    case 112: return launch_bn<112>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
+    default: return launch_bn<128>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
   }
 }
 
@@ -571,11 +573,11 @@ int bs_launch_slice_gemm(const uint16_t* A, const uint16_t* B, float* D, int M, 
   one.order[0] = 0;
   one.a0[0] = one.b0[0] = 0;
   one.len[0] = K;
-  return dispatch_bn(A, B, D, M, N, K, batch, sA, sB, ldd, sD, one, err, s);
+  return dispatch_bn(A, B, D, M, N, K, batch, sA, sB, ldd, sD, one, err, s, nullptr);
 }
 
 int bs_launch_slice_orders(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int S,
-                           int Kp, int batch, int* err, cudaStream_t s) {
+                           int Kp, int batch, int* err, cudaStream_t s, const int* skip) {
   SliceSlabs sl;
   if (Kp % 64 != 0 || S < 1 || ((uintptr_t)A & 15) || ((uintptr_t)B & 15) || M < 1 || N < 1 ||
       batch < 1 || !bs_slice_slabs(S, Kp, M, N, batch, &sl) || (long)batch * sl.nq > 65535) {
@@ -585,7 +587,7 @@ int bs_launch_slice_orders(const uint16_t* A, const uint16_t* B, float* D, int M
   }
   const int K = S * Kp;
   return dispatch_bn(A, B, D, M, N, K, batch, (long)M * K, (long)N * K, M, (long)M * N, sl, err,
-                     s);
+                     s, skip);
 }
 
 // A22 (m x m at offset o of each n x n matrix) -= X Y^dagger from the digit

@@ -14,6 +14,8 @@
 // and builds the next reflector.  In FP64 the loop is bound by the FP64
 // pipe of GB300, so it is written for FP64 issue: 16 FMAs per element and
 // one shared-memory reduction of the row and column partials per tile.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "bs_internal.h"
@@ -93,16 +95,12 @@ __device__ void householder(typename Cplx<R>::T* a, int n, int c, typename Cplx<
 }
 
 template <typename R>
-__global__ void __launch_bounds__(NT) tridiag_init_kernel(typename Cplx<R>::T* __restrict__ A,
-                                                          int n,
-                                                          typename Cplx<R>::T* __restrict__ vec,
-                                                          double* __restrict__ de,
-                                                          double* __restrict__ tau,
-                                                          zd* __restrict__ beta,
-                                                          unsigned* __restrict__ count) {
+__device__ void tridiag_begin(typename Cplx<R>::T* __restrict__ A, int n,
+                              typename Cplx<R>::T* __restrict__ vec, double* __restrict__ de,
+                              double* __restrict__ tau, zd* __restrict__ beta,
+                              unsigned* __restrict__ count, int b) {
   typedef typename Cplx<R>::T C;
   __shared__ double sh[NT / 32 + 1];
-  const int b = blockIdx.x;
   C* a = A + (size_t)b * n * n;
   C* vb = vec + (size_t)b * 3 * n;
   for (int r = threadIdx.x; r < 3 * n; r += NT) vb[r] = Cplx<R>::make((R)0, (R)0);
@@ -117,6 +115,17 @@ __global__ void __launch_bounds__(NT) tridiag_init_kernel(typename Cplx<R>::T* _
   if (n > 1) householder<R>(a, n, 0, vb, tau + (size_t)b * n, beta + (size_t)b * n, d + n, sh);
 }
 
+template <typename R>
+__global__ void __launch_bounds__(NT) tridiag_init_kernel(typename Cplx<R>::T* __restrict__ A,
+                                                          int n,
+                                                          typename Cplx<R>::T* __restrict__ vec,
+                                                          double* __restrict__ de,
+                                                          double* __restrict__ tau,
+                                                          zd* __restrict__ beta,
+                                                          unsigned* __restrict__ count) {
+  tridiag_begin<R>(A, n, vec, de, tau, beta, count, blockIdx.x);
+}
+
 // (bi, bk) with bi >= bk of the l-th lower-triangular tile, row-major;
 // FP32 square root (FP64 square root is a long sequence on GB300), then
 // exact integer correction
@@ -128,18 +137,14 @@ __device__ __forceinline__ void tri_index(int l, int& bi, int& bk) {
   bk = l - r * (r + 1) / 2;
 }
 
-// FP32: 3 CTAs per SM (memory latency needs warps); FP64: 2 (its pipe is the limit).
-// TS = 64 (4 x 4 elements per thread) or 32 (2 x 2): the tile edge is tuned per n.
+// One tile of step j of matrix b (tile: its index among the ntl lower tiles).
 template <typename R, int TS>
-__global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) tridiag_step_kernel(typename Cplx<R>::T* __restrict__ A,
-                                                             int n, int j,
-                                                             typename Cplx<R>::T* __restrict__ vec,
-                                                             typename Cplx<R>::T* __restrict__ part,
-                                                             double* __restrict__ de,
-                                                             double* __restrict__ tau,
-                                                             zd* __restrict__ beta,
-                                                             unsigned* __restrict__ count,
-                                                             int ntl) {
+__device__ __forceinline__ void tridiag_tile(typename Cplx<R>::T* __restrict__ A, int n, int j,
+                                             typename Cplx<R>::T* __restrict__ vec,
+                                             typename Cplx<R>::T* __restrict__ part,
+                                             double* __restrict__ de, double* __restrict__ tau,
+                                             zd* __restrict__ beta, unsigned* __restrict__ count,
+                                             int ntl, int b, int tile) {
   typedef typename Cplx<R>::T C;
   // Thread (tx, ty) owns rows R*TS + tx + 16v and columns S*TS + ty + 16u,
   // u, v < EPT: its EPT^2 elements give EPT row and EPT column partials of p,
@@ -151,7 +156,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) tridiag_step_kerne
   __shared__ double sh[NT / 32 + 1];
   __shared__ int is_last;
 
-  const int b = blockIdx.y, tid = threadIdx.x;
+  const int tid = threadIdx.x;
   const int tx = tid % 16, ty = tid / 16;
   const int nt = (n + TS - 1) / TS, t0 = (j + 1) / TS, r0 = j + 1;   // TS: template
   const C zero = Cplx<R>::make((R)0, (R)0);
@@ -163,7 +168,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) tridiag_step_kerne
   C* pt = part + (size_t)b * nt * n;
 
   int bi, bk;
-  tri_index(blockIdx.x, bi, bk);
+  tri_index(tile, bi, bk);
   const int Rt = t0 + bi, St = t0 + bk;
   const int rbase = Rt * TS, sbase = St * TS;
 
@@ -294,7 +299,64 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) tridiag_step_kerne
                    d + n + r0, sh);
 }
 
+// FP32: 3 CTAs per SM (memory latency needs warps); FP64: 2 (its pipe is the limit).
+// TS = 64 (4 x 4 elements per thread) or 32 (2 x 2): the tile edge is tuned per n.
+template <typename R, int TS>
+__global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2)
+    tridiag_step_kernel(typename Cplx<R>::T* __restrict__ A, int n, int j,
+                        typename Cplx<R>::T* __restrict__ vec,
+                        typename Cplx<R>::T* __restrict__ part, double* __restrict__ de,
+                        double* __restrict__ tau, zd* __restrict__ beta,
+                        unsigned* __restrict__ count, int ntl) {
+  tridiag_tile<R, TS>(A, n, j, vec, part, de, tau, beta, count, ntl, blockIdx.y, blockIdx.x);
+}
+
+// The same reduction of the matrices list[0 .. *nlist) of a batch, in one
+// cooperative launch: the tiles of a step go round the CTAs, a grid barrier
+// separates the steps.  The list is made on the device (the matrices an
+// iterative solve did not certify) and is nearly always empty: the launch
+// then returns at once, where n step launches would cost their launch gaps.
+__global__ void __launch_bounds__(NT, 2)
+    tridiag_list_kernel(zd* __restrict__ A, int n, zd* __restrict__ vec, zd* __restrict__ part,
+                        double* __restrict__ de, double* __restrict__ tau, zd* __restrict__ beta,
+                        unsigned* __restrict__ count, const int* __restrict__ list,
+                        const int* __restrict__ nlist) {
+  const int nf = *nlist;
+  if (nf == 0) return;   // the same for every CTA
+  cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+  for (int f = blockIdx.x; f < nf; f += gridDim.x) {
+    tridiag_begin<double>(A, n, vec, de, tau, beta, count, list[f]);
+    __syncthreads();
+  }
+  grid.sync();
+  const int nt = (n + 63) / 64;
+  for (int j = 0; j + 1 < n; ++j) {
+    const int m = nt - (j + 1) / 64, ntl = m * (m + 1) / 2;
+    const long items = (long)nf * ntl;
+    for (long it = blockIdx.x; it < items; it += gridDim.x) {
+      tridiag_tile<double, 64>(A, n, j, vec, part, de, tau, beta, count, ntl, list[it / ntl],
+                               (int)(it % ntl));
+      __syncthreads();
+    }
+    grid.sync();
+  }
+}
+
 }  // namespace
+
+int bs_launch_tridiag_list(zd* A, int n, zd* vec, zd* part, double* de, double* tau, zd* beta,
+                           unsigned* count, const int* list, const int* nlist, cudaStream_t s) {
+  int per = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tridiag_list_kernel, NT, 0);
+  if (e != cudaSuccess) return bs_cuda_status(e, "tridiag_list_kernel");
+  const int grid = std::max(1, per) * bs_sm_count();
+  void* args[] = {&A, &n, &vec, &part, &de, &tau, &beta, &count, (void*)&list, (void*)&nlist};
+  e = cudaLaunchCooperativeKernel((const void*)tridiag_list_kernel, dim3(grid), dim3(NT), args, 0,
+                                  s);
+  if (e != cudaSuccess) return bs_cuda_status(e, "tridiag_list_kernel");
+  BS_CHECK_LAUNCH("tridiag_list_kernel");
+  return BS_OK;
+}
 
 size_t bs_tridiag_vec_elems(int n) { return 3 * (size_t)n; }
 size_t bs_tridiag_part_elems(int n) { return (size_t)((n + TSMIN - 1) / TSMIN) * n; }
