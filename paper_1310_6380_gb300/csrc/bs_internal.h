@@ -7,6 +7,8 @@
 
 #include <string>
 
+#include <cuda_bf16.h>
+
 #include "bandstructure.h"
 
 // ------------------------------------------------------------------ complex
@@ -318,6 +320,33 @@ int bs_launch_zgemm_tc_rect(const zd* A, int lda, long sA, const double* sc, con
                             cudaStream_t s);
 
 // builder.cu
+// x = hi + lo, two BF16 terms (2^-17 relative)
+__device__ __forceinline__ void bs_bf16_split(float x, uint16_t& hi, uint16_t& lo) {
+  const __nv_bfloat16 h = __float2bfloat16_rn(x);
+  hi = __bfloat16_as_ushort(h);
+  lo = __bfloat16_as_ushort(__float2bfloat16_rn(x - __bfloat162float(h)));
+}
+// entry r of a complex column as an operand of bs_launch_filter_product: v
+// points at entry r of the column's first row, rows [Re | -Im], [Im | Re], hi
+// then lo, each block np wide
+__device__ __forceinline__ void bs_store_block_split(uint16_t* v, int np, zf y) {
+  uint16_t rh, rl, ih, il;
+  bs_bf16_split(y.x, rh, rl);
+  bs_bf16_split(y.y, ih, il);
+  v[0] = rh;
+  v[np] = ih ^ 0x8000;
+  v[2 * np] = rl;
+  v[3 * np] = il ^ 0x8000;
+  v += 4 * (size_t)np;
+  v[0] = ih;
+  v[np] = rh;
+  v[2 * np] = il;
+  v[3 * np] = rl;
+}
+// tc_gemm.cu: one term of the filter's recurrence (B, V: BF16 splits)
+int bs_launch_filter_product(const uint16_t* B, const uint16_t* V, int np, int batch,
+                             const float* coef, int cstride, const zf* E, zf* Ep, zf* g,
+                             uint16_t* Vout, const int* skip, int* err, cudaStream_t s);
 // ---- two-stage reduction to tridiagonal form (band.cu)
 #define BS_BAND_NB 8        // half-width of the intermediate band
 #define BS_SLICES_BAND 8    // digit planes per operand in its contractions (~2^-53)
@@ -393,8 +422,10 @@ int bs_launch_rank2_update(const uint16_t* dA, const uint16_t* dB, const int* ex
 #define BS_FILT_MAXDEG 12      // degrees of one filter
 struct FilterWs {
   int n = 0, kf = 0;        // order, matrices per chunk
-  zf* A = nullptr;          // kf x np x np scaled matrix, then its LDL^dagger (np: n padded to 64)
+  zf* A = nullptr;          // kf x np x np scaled matrix, then its LDL^dagger (np: n padded to
+                            // 64), then the BF16 split of the operator B (np x 4 np)
   zf* X = nullptr;          // kf x np x np inverse factor
+  float* d = nullptr;       // kf x np pivots
   uint16_t* pA = nullptr;   // digit planes of C, of the block, and the digit-order sums
   uint16_t* pB = nullptr;
   float* pD = nullptr;
@@ -402,7 +433,8 @@ struct FilterWs {
   int* eB = nullptr;
   zd* Xb = nullptr;         // kf x 32 x n block and C times it
   zd* CX = nullptr;
-  zf* vec = nullptr;        // 5 x kf x 32 x np: R, Lh v, B R, two Chebyshev terms
+  zf* vec = nullptr;        // 3 x kf x 32 x np: B R, two Chebyshev terms
+  uint16_t* vs = nullptr;   // 2 x kf x 64 x 4 np: BF16 splits of the residual and the terms
   zd* part = nullptr;       // kf x chunks x 2 x 32 x 32 partial Gram matrices
   float* rpart = nullptr;   // kf x chunks x 2 x 32 partial residual sums
   double* theta = nullptr;  // kf x 32

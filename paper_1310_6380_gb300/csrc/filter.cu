@@ -8,16 +8,16 @@
 //
 //  1. FP32: the LDL^dagger of W (C/s + I) W (s of the size of the wanted
 //     eigenvalues, W = diag(C/s + 1)^-1/2), its triangular inverse, and so
-//     Lh = D^-1/2 L^-1 W with B = Lh^dagger Lh = (C/s + I)^-1 to FP32
-//     accuracy.  The wanted eigenvalues are the largest of B.
+//     B = W L^-dagger D^-1 L^-1 W = (C/s + I)^-1 to FP32 accuracy, stored as two
+//     BF16 terms (2^-17).  The wanted eigenvalues are the largest of B.
 //  2. Rounds: an FP64 Rayleigh-Ritz step on the block X (32 vectors, the
 //     wanted ones and guards) gives theta, X, and the FP64 residual
 //     R = C X - X Theta; then X is filtered by a Chebyshev polynomial T_m of B
 //     that is at most 1 on the unwanted part of the spectrum.  Written for
 //     the change E of X instead of X itself,
 //       T_j(l(B)) x = tau_j (x + E_j),   B x = mu (x - B r / s),  mu = s / (theta + s),
-//     every term is a product of B with the residual: the FP32 operator only
-//     multiplies R, so its rounding shrinks with R and the rounds converge to
+//     every term is a product of B (on the tensor cores) with the residual: the operator only
+//     multiplies R, so its error shrinks with R and the rounds converge to
 //     the eigenvectors of the FP64 matrix, not of B.
 //  3. Certificate: theta_i is an upper bound of lambda_i; with rho a lower
 //     bound of lambda_{m+1}, Lehmann's bound in its trace form (the residual
@@ -36,10 +36,10 @@
 //
 // Measured (one GB300, whole FP64 solve with its assembly, the reduction to
 // tridiagonal form before -> this): n = 882, 90 matrices, 18 branches
-// 171 -> 47 ms; n = 1029, 30 matrices, 12 branches 136 -> 35 ms; n = 242,
-// 70 matrices, 18 branches 16.9 -> 9.0 ms.  What bounds it at n = 882 is the
-// FP32 pipe in the products with B and in the factorisations, and the FP64
-// pipe in the Rayleigh-Ritz steps (32-column products at 2 FMA per clock and SM).
+// 171 -> 36 ms; n = 1029, 30 matrices, 12 branches 136 -> 25 ms; n = 242,
+// 70 matrices, 18 branches 16.9 -> 7.9 ms.  What bounds it at n = 882 is the
+// FP32 pipe in the factorisations and the FP64 pipe in the Rayleigh-Ritz steps
+// (32-column products at 2 FMA per clock and SM).
 //
 // Everything that enters a result (C X, the Gram matrices, the Ritz values,
 // the residuals) is FP64 or an exact-slice product of FP64 operands.
@@ -58,8 +58,6 @@ constexpr int TB = 64;              // tile edge of the FP32 factorisation
 constexpr int LDS = TB + 1;         // row stride of the diagonal blocks in shared memory
 constexpr float TINY_PIVOT = 1e-6f; // of the scaled unit diagonal
 constexpr int GR = 64;              // rows per CTA of the Gram and rotation kernels
-
-__device__ __forceinline__ zf cfma(zf a, zf b, zf c) { return zfma(a, b, c); }
 
 // ---------------------------------------------------------------- set-up
 // Per matrix: the FB smallest diagonal entries (the starting vectors are
@@ -204,8 +202,8 @@ __device__ void ldl64_block(zf* S, zf* Xs, float* d, int* bad) {
 }
 
 // factor the diagonal block at j0 held in S and store L (unit), D, X
-__device__ void ldl64_diag(zf* a, zf* x, int np, int j0, int k, zf* S, zf* Xs, float* d, int* bad,
-                           int* neg, int* flag) {
+__device__ void ldl64_diag(zf* a, zf* x, float* dk, int np, int j0, int k, zf* S, zf* Xs, float* d,
+                           int* bad, int* neg, int* flag) {
   const int tid = threadIdx.x, r = tid & 63;
   if (tid == 0) *bad = 0;
   __syncthreads();
@@ -217,6 +215,7 @@ __device__ void ldl64_diag(zf* a, zf* x, int np, int j0, int k, zf* S, zf* Xs, f
     if (r >= c) a[(size_t)(j0 + c) * np + j0 + r] = v;
     x[(size_t)(j0 + c) * np + j0 + r] = r >= c ? Xs[r * LDS + c] : make_float2(0.f, 0.f);
   }
+  if (tid < TB) dk[j0 + tid] = d[tid];
   if (tid == 0) {
     int cnt = 0;
     for (int c = 0; c < TB; ++c) cnt += d[c] < 0.f;
@@ -226,7 +225,8 @@ __device__ void ldl64_diag(zf* a, zf* x, int np, int j0, int k, zf* S, zf* Xs, f
 }
 
 __global__ void __launch_bounds__(256) ldl64_diag_kernel(zf* __restrict__ A, zf* __restrict__ X,
-                                                         int np, int* __restrict__ neg,
+                                                         int np, float* __restrict__ dv,
+                                                         int* __restrict__ neg,
                                                          int* __restrict__ flag) {
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ float d[TB];
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(256) ldl64_diag_kernel(zf* __restrict__ A, zf*
   for (int c = tid >> 6; c < TB; c += 4)
     if (r >= c) S[r * LDS + c] = a[(size_t)c * np + r];
   __syncthreads();
-  ldl64_diag(a, X + (size_t)k * np * np, np, 0, k, S, Xs, d, &bad, neg, flag);
+  ldl64_diag(a, X + (size_t)k * np * np, dv + (size_t)k * np, np, 0, k, S, Xs, d, &bad, neg, flag);
 }
 
 // 64 x 64 x 64 product on 256 threads, 4 x 4 complex per thread:
@@ -300,7 +300,8 @@ __global__ void __launch_bounds__(256) ldl64_panel_kernel(zf* __restrict__ A,
 // trailing update A_ik -= L_i1 D1 L_k1^dagger; the first tile's CTA factors
 // the next diagonal block
 __global__ void __launch_bounds__(256) ldl64_update_kernel(zf* __restrict__ A, zf* __restrict__ X,
-                                                           int np, int j0, int* __restrict__ neg,
+                                                           int np, int j0, float* __restrict__ dv,
+                                                           int* __restrict__ neg,
                                                            int* __restrict__ flag) {
   extern __shared__ __align__(16) unsigned char dsm[];
   zf* As = reinterpret_cast<zf*>(dsm);
@@ -349,7 +350,7 @@ __global__ void __launch_bounds__(256) ldl64_update_kernel(zf* __restrict__ A, z
   }
   if (first) {
     __syncthreads();
-    ldl64_diag(a, X + (size_t)blockIdx.y * np * np, np, i0, blockIdx.y, As, Bs, d, &bad, neg, flag);
+    ldl64_diag(a, X + (size_t)blockIdx.y * np * np, dv + (size_t)blockIdx.y * np, np, i0, blockIdx.y, As, Bs, d, &bad, neg, flag);
   }
 }
 
@@ -393,139 +394,73 @@ __global__ void __launch_bounds__(256) trinv64_kernel(const zf* __restrict__ A, 
           make_float2(-acc[i][j].x, -acc[i][j].y);
 }
 
-// Lh = D^-1/2 X W in place on the lower tiles
-__global__ void __launch_bounds__(256) filt_lhat_kernel(const zf* __restrict__ A,
-                                                        zf* __restrict__ X, int np,
-                                                        const float* __restrict__ w) {
+// B = W X^dagger D^-1 X W (X = L^-1), 64-tiles (bi, bk) and their mirrors,
+// straight to the BF16 split [Re | Im] hi, [Re | Im] lo of rows of 4 np.  The
+// tile sums over the block rows t >= bi; the longest sums come first.
+__global__ void __launch_bounds__(256) filt_operator_kernel(const zf* __restrict__ X,
+                                                            const float* __restrict__ d, int np,
+                                                            const float* __restrict__ w,
+                                                            uint16_t* __restrict__ Bp) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  zf* As = reinterpret_cast<zf*>(dsm);   // [column][t], stride LDS
+  zf* Bs = As + TB * LDS;
   int bi, bk;
   tile_of(blockIdx.x, bi, bk);
-  const int k = blockIdx.y, r = bi * TB + (threadIdx.x & 63);
-  zf* x = X + (size_t)k * np * np;
-  const float dr = rsqrtf(fabsf(A[(size_t)k * np * np + (size_t)r * (np + 1)].x));
-#pragma unroll 4
-  for (int q = threadIdx.x >> 6; q < TB; q += 4) {
-    const int c = bk * TB + q;
-    zf* p = x + (size_t)c * np + r;
-    *p = zscale(*p, dr * w[(size_t)k * np + c]);
-  }
-}
-
-// ---------------------------------------------------------------- B products
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                   (uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src));
-}
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
-                   (uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src));
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N));
-}
-
-// One block row (64) of Lh V (FWD) or Lh^dagger V, V: 32 columns of np; 128
-// threads, 4 x 4 complex each, K in chunks of 32 through a two-stage
-// cp.async ring.  The backward product's epilogue forms the next Chebyshev
-// term (coefficients per column: cf[0] B E + cf[1] E + cf[2] E_prev + cf[3] g,
-// written over E_prev), or g = B R and E_1 = cf[3] g when E is null.
-constexpr int KC = 32;
-constexpr int AP_SMEM = 2 * (KC * (TB + 2) + KC * (FB + 1) + 8) * (int)sizeof(zf);
-
-template <bool FWD>
-__global__ void __launch_bounds__(128) filt_apply_kernel(
-    const zf* __restrict__ Lh, const zf* __restrict__ V, int np, zf* __restrict__ out,
-    const float* __restrict__ coef, int cstride, const zf* __restrict__ E, zf* __restrict__ Ep,
-    zf* __restrict__ g, const int* __restrict__ done) {
-  if (done[blockIdx.y]) return;
-  extern __shared__ __align__(16) unsigned char dsm[];
-  constexpr int ASZ = KC * (TB + 2), BSZ = KC * (FB + 1) + 8;
-  zf* As[2] = {reinterpret_cast<zf*>(dsm), reinterpret_cast<zf*>(dsm) + ASZ};
-  zf* Bs[2] = {reinterpret_cast<zf*>(dsm) + 2 * ASZ, reinterpret_cast<zf*>(dsm) + 2 * ASZ + BSZ};
-  const int k = blockIdx.y, nt = np / TB;
-  // the longest block rows first
-  const int b = FWD ? nt - 1 - (int)blockIdx.x : (int)blockIdx.x;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const zf* l = Lh + (size_t)k * np * np;
-  const zf* v = V + (size_t)k * FB * np;
-  const int kbeg = FWD ? 0 : b * TB, nch = (FWD ? (b + 1) * TB : np - b * TB) / KC;
-  auto load = [&](int st, int k0) {
-    if (FWD) {
-      for (int e = tid; e < KC * TB / 2; e += 128) {
-        const int t = e >> 5, r2 = e & 31;
-        cp_async16(As[st] + t * TB + 2 * r2, l + (size_t)(k0 + t) * np + b * TB + 2 * r2);
-      }
-    } else {
-      for (int e = tid; e < KC * TB; e += 128) {
-        const int r = e >> 5, t = e & 31;
-        cp_async8(As[st] + r * (KC + 1) + t, l + (size_t)(b * TB + r) * np + k0 + t);
-      }
-    }
-    for (int e = tid; e < KC * FB; e += 128) {
-      const int c = e >> 5, t = e & 31;
-      cp_async8(Bs[st] + c * (KC + 1) + t, v + (size_t)c * np + k0 + t);
-    }
-    cp_commit();
-  };
+  const int k = blockIdx.y, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const zf* x = X + (size_t)k * np * np;
+  const float* dk = d + (size_t)k * np;
+  const float* wk = w + (size_t)k * np;
   zf acc[4][4] = {};
-  load(0, kbeg);
-  for (int ch = 0; ch < nch; ++ch) {
-    if (ch + 1 < nch) {
-      load((ch + 1) & 1, kbeg + (ch + 1) * KC);
-      cp_wait<1>();
-    } else {
-      cp_wait<0>();
+  for (int t0 = bi * TB; t0 < np; t0 += TB) {
+    __syncthreads();
+    const float di = 1.f / dk[t0 + (tid & 63)];
+    for (int c = tid >> 6; c < TB; c += 4) {
+      const int t = tid & 63;
+      As[c * LDS + t] = zscale(x[(size_t)(bi * TB + c) * np + t0 + t], di);
+      Bs[c * LDS + t] = x[(size_t)(bk * TB + c) * np + t0 + t];
     }
     __syncthreads();
-    const zf* a_ = As[ch & 1];
-    const zf* b_ = Bs[ch & 1];
 #pragma unroll 8
-    for (int t = 0; t < KC; ++t) {
-      zf a[4], bb[4];
+    for (int t = 0; t < TB; ++t) {
+      zf a[4], b[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        a[i] = FWD ? a_[t * TB + tx + 16 * i] : a_[(tx + 16 * i) * (KC + 1) + t];
-        if (!FWD) a[i].y = -a[i].y;
-      }
+      for (int i = 0; i < 4; ++i) a[i] = As[(tx + 16 * i) * LDS + t];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = b_[(ty + 8 * j) * (KC + 1) + t];
+      for (int j = 0; j < 4; ++j) b[j] = Bs[(ty + 16 * j) * LDS + t];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = cfma(a[i], bb[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) acc[i][j] = zfmac(b[j], a[i], acc[i][j]);   // conj(a) b
     }
-    __syncthreads();
   }
-  const size_t base = (size_t)k * FB * np;
+  __syncthreads();
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const int c = ty + 8 * j;
-    float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
-    if (!FWD) {
-      const float* cf = coef + (size_t)k * cstride + c;
-      c0 = cf[0];
-      c1 = cf[FB];
-      c2 = cf[2 * FB];
-      c3 = cf[3 * FB];
-    }
+    const float wc = wk[bk * TB + ty + 16 * j];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const size_t o = base + (size_t)c * np + b * TB + tx + 16 * i;
-      const zf y = acc[i][j];
-      if (FWD) {
-        out[o] = y;
-      } else if (!E) {
-        g[o] = y;
-        Ep[o] = zscale(y, c3);
-      } else {
-        const zf e = E[o], gg = g[o];
-        const zf p = c2 != 0.f ? Ep[o] : make_float2(0.f, 0.f);
-        Ep[o] = make_float2(c0 * y.x + c1 * e.x + c2 * p.x + c3 * gg.x,
-                            c0 * y.y + c1 * e.y + c2 * p.y + c3 * gg.y);
+    for (int i = 0; i < 4; ++i)
+      As[(tx + 16 * i) * LDS + ty + 16 * j] = zscale(acc[i][j], wk[bi * TB + tx + 16 * i] * wc);
+  }
+  __syncthreads();
+  uint16_t* b = Bp + (size_t)k * np * 4 * np;
+  for (int h = 0; h < (bi == bk ? 1 : 2); ++h) {
+    // h = 0: rows of bi, columns of bk; h = 1: the conjugate mirror
+    const int r0 = (h ? bk : bi) * TB, c0 = (h ? bi : bk) * TB;
+    for (int e = tid; e < TB * TB / 2; e += 256) {
+      const int r = e >> 5, c = (e & 31) * 2;
+      uint32_t v[4];
+      uint16_t q[2][4];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const zf y = h ? zconj(As[(c + u) * LDS + r]) : As[r * LDS + c + u];
+        bs_bf16_split(y.x, q[u][0], q[u][2]);
+        bs_bf16_split(y.y, q[u][1], q[u][3]);
       }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) v[m] = (uint32_t)q[0][m] | ((uint32_t)q[1][m] << 16);
+      uint16_t* o = b + (size_t)(r0 + r) * 4 * np + c0 + c;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) *reinterpret_cast<uint32_t*>(o + (size_t)m * np) = v[m];
     }
   }
 }
@@ -617,7 +552,7 @@ __global__ void __launch_bounds__(GT) filt_gram_kernel(const zd* __restrict__ X,
       p[(2 * bi + i) * FB + 2 * bj + j] = zmake((double)acc[i][j].x, (double)acc[i][j].y);
 }
 
-// X <- X W, R / s = (C X W - X W Theta) / s in FP32 (zero in the padding) and
+// X <- X W, the split of R / s = (C X W - X W Theta) / s (zero in the padding) and
 // the sums of its squares per column (one partial per warp of rows)
 template <typename R>
 __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
@@ -625,7 +560,7 @@ __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
                                                           const zd* __restrict__ W,
                                                           const double* __restrict__ theta,
                                                           const double* __restrict__ shift,
-                                                          zf* __restrict__ Rr,
+                                                          uint16_t* __restrict__ Rs,
                                                           float* __restrict__ rpart,
                                                           const int* __restrict__ done) {
   if (done[blockIdx.y]) return;
@@ -669,7 +604,8 @@ __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
         rv = make_float2((float)(((double)ya[j].x - t * (double)xa[j].x) * is),
                          (float)(((double)ya[j].y - t * (double)xa[j].y) * is));
       }
-      if (row < np) Rr[((size_t)k * FB + c) * np + row] = rv;
+      if (row < np)
+        bs_store_block_split(Rs + ((size_t)k * 2 * FB + 2 * c) * 4 * np + row, np, rv);
       float q = rv.x * rv.x + rv.y * rv.y;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
@@ -998,7 +934,7 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
 // vector, so l >= 1 on the block.  A column stops at the last degree whose
 // growth relative to it, tau_j(l_0) / tau_j(l_c) (the lowest branch grows
 // most), times what the residual holds of the other branches stays below 0.1:
-// 6e-8 of itself (FP32 rounding), `couple` of the block's largest Ritz value
+// 4e-6 of itself (the split operands), `couple` of the block's largest Ritz value
 // (the off-diagonal the Jacobi sweeps left) and the rounding of C X.  Beyond,
 // the column would turn into the lowest branches and the block lose rank.
 __global__ void __launch_bounds__(128) filt_coef_kernel(const double* __restrict__ theta,
@@ -1016,7 +952,7 @@ __global__ void __launch_bounds__(128) filt_coef_kernel(const double* __restrict
   const double cut = __shfl_sync(0xffffffffu, t, 31);
   const double mu = 1.0 / (t + 1.0), imuc = cut + 1.0;
   const double l = fmax(2.0 * mu * imuc - 1.0, 1.0), f = 2.0 * mu * imuc;
-  const double lim = 0.1 / (6e-8 * (double)sqrtf(rn) + couple * cut +
+  const double lim = 0.1 / (4e-6 * (double)sqrtf(rn) + couple * cut +
                             4.0 * DBL_EPSILON * cmax[k] / shift[k]);
   float* cf = coef + (size_t)k * BS_FILT_MAXDEG * 4 * FB + c;
   double t0 = 1.0, t1 = l;   // tau_{j-1}, tau_j
@@ -1132,7 +1068,7 @@ bool bs_filter_fits(int n, int nbands) {
 }
 
 void bs_filter_ws_free(FilterWs* w) {
-  void* p[] = {w->A, w->X, w->pA, w->pB, w->pD, w->eA, w->eB, w->Xb, w->CX, w->vec, w->part,
+  void* p[] = {w->A, w->X, w->pA, w->pB, w->pD, w->eA, w->eB, w->Xb, w->CX, w->vec, w->vs, w->d, w->part,
                w->rpart, w->theta, w->W, w->coef, w->shift, w->cmax, w->sigma, w->ord, w->w, w->iw};
   for (void* q : p) cudaFree(q);
   *w = FilterWs();
@@ -1144,7 +1080,7 @@ static size_t filter_bytes(int n) {
   const size_t np = (n + TB - 1) / TB * TB, Kp = (2 * (size_t)n + 63) / 64 * 64;
   return 2 * np * np * sizeof(zf) + (size_t)n * 8 * Kp * 2 + 2 * FB * 8 * Kp * 2 +
          (size_t)24 * 2 * FB * n * 4 + 2 * (size_t)FB * n * sizeof(zd) +
-         5 * FB * np * sizeof(zf) + 65536;
+         7 * FB * np * sizeof(zf) + 65536;
 }
 
 int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
@@ -1166,7 +1102,9 @@ int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
       {(void**)&w->eB, k * FB * sizeof(int)},
       {(void**)&w->Xb, k * FB * n * sizeof(zd)},
       {(void**)&w->CX, k * FB * n * sizeof(zd)},
-      {(void**)&w->vec, 5 * k * FB * np * sizeof(zf)},
+      {(void**)&w->vec, 3 * k * FB * np * sizeof(zf)},
+      {(void**)&w->vs, 2 * k * 2 * FB * 4 * np * sizeof(uint16_t)},
+      {(void**)&w->d, k * np * sizeof(float)},
       {(void**)&w->part, k * nch * 2 * FB * FB * sizeof(zd)},
       {(void**)&w->rpart, k * nch * 2 * FB * sizeof(float)},
       {(void**)&w->theta, k * FB * sizeof(double)},
@@ -1203,8 +1141,7 @@ static int filter_attrs() {
       {(const void*)ldl64_panel_kernel, 2 * TB * TB * (int)sizeof(zf)},
       {(const void*)ldl64_update_kernel, 2 * TB * LDS * (int)sizeof(zf)},
       {(const void*)trinv64_kernel, (TB * TB + TB * LDS) * (int)sizeof(zf)},
-      {(const void*)filt_apply_kernel<true>, AP_SMEM},
-      {(const void*)filt_apply_kernel<false>, AP_SMEM},
+      {(const void*)filt_operator_kernel, 2 * TB * LDS * (int)sizeof(zf)},
       {(const void*)filt_gram_kernel<double>, (int)sizeof(RrSmem<double>)},
       {(const void*)filt_rotate_kernel<double>,
        (int)(sizeof(RrSmem<double>) + FB * FB * sizeof(zd))},
@@ -1222,19 +1159,20 @@ static int filter_attrs() {
   return BS_OK;
 }
 
-// factor A (kf matrices); with_x: also the full inverse factor
+// factor A (kf matrices); inverse: then the operator B, whose split replaces A
 static int filter_factor(FilterWs& w, int np, int kf, bool inverse, cudaStream_t s) {
   const int nt = np / TB;
   int* neg = w.iw;
   int* flag = w.iw + w.kf;
-  ldl64_diag_kernel<<<kf, 256, 2 * TB * LDS * sizeof(zf), s>>>(w.A, w.X, np, neg, flag);
+  ldl64_diag_kernel<<<kf, 256, 2 * TB * LDS * sizeof(zf), s>>>(w.A, w.X, np, w.d, neg,
+                                                                   flag);
   BS_CHECK_LAUNCH("ldl64_diag_kernel");
   for (int j = 0; j + 1 < nt; ++j) {
     const int rem = nt - j - 1;
     ldl64_panel_kernel<<<dim3(rem, kf), 256, 2 * TB * TB * sizeof(zf), s>>>(w.A, w.X, np, j * TB);
     BS_CHECK_LAUNCH("ldl64_panel_kernel");
     ldl64_update_kernel<<<dim3(rem * (rem + 1) / 2, kf), 256, 2 * TB * LDS * sizeof(zf), s>>>(
-        w.A, w.X, np, j * TB, neg, flag);
+        w.A, w.X, np, j * TB, w.d, neg, flag);
     BS_CHECK_LAUNCH("ldl64_update_kernel");
   }
   if (!inverse) return BS_OK;
@@ -1242,8 +1180,9 @@ static int filter_factor(FilterWs& w, int np, int kf, bool inverse, cudaStream_t
     trinv64_kernel<<<dim3(nt - d, kf), 256, (TB * TB + TB * LDS) * sizeof(zf), s>>>(w.A, w.X, np, d);
     BS_CHECK_LAUNCH("trinv64_kernel");
   }
-  filt_lhat_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(w.A, w.X, np, w.w);
-  BS_CHECK_LAUNCH("filt_lhat_kernel");
+  filt_operator_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 2 * TB * LDS * sizeof(zf), s>>>(
+      w.X, w.d, np, w.w, reinterpret_cast<uint16_t*>(w.A));
+  BS_CHECK_LAUNCH("filt_operator_kernel");
   return BS_OK;
 }
 
@@ -1260,7 +1199,7 @@ static int filter_ritz(FilterWs& w, int n, int np, int kf, cudaStream_t s) {
   // the rotation covers the padded rows as well (np <= nch GR)
   filt_rotate_kernel<R><<<dim3(nch, kf), 256,
                           sizeof(RrSmem<R>) + FB * FB * sizeof(typename Cplx<R>::T), s>>>(
-      w.Xb, w.CX, n, np, w.W, w.theta, w.shift, w.vec, w.rpart, done);
+      w.Xb, w.CX, n, np, w.W, w.theta, w.shift, w.vs, w.rpart, done);
   BS_CHECK_LAUNCH("filt_rotate_kernel");
   return BS_OK;
 }
@@ -1297,7 +1236,10 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
     filt_start_kernel<<<cg, 256, 0, s>>>(Ck, n, w.ord, w.Xb, w.CX);
     BS_CHECK_LAUNCH("filt_start_kernel");
     const size_t vb = (size_t)w.kf * FB * np;
-    zf *Rr = w.vec, *Tv = w.vec + vb, *g = w.vec + 2 * vb, *E[2] = {w.vec + 3 * vb, w.vec + 4 * vb};
+    zf *g = w.vec, *E[2] = {w.vec + vb, w.vec + 2 * vb};
+    // the split of the residual and of even terms, and of odd terms
+    uint16_t* vs[2] = {w.vs, w.vs + 8 * vb};
+    const uint16_t* Bp = reinterpret_cast<const uint16_t*>(w.A);
     const int cstride = BS_FILT_MAXDEG * 4 * FB;
     for (int rd = 0; rd <= rounds; ++rd) {
       // the first three steps only steer the iteration: FP32 products of the block
@@ -1314,18 +1256,11 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
       filt_coef_kernel<<<(kf + 3) / 4, 128, 0, s>>>(w.theta, w.rpart, nch, w.shift, kf, w.cmax,
                                                     rd < 3 ? 1e-6 : 1e-10, m, w.coef, done);
       BS_CHECK_LAUNCH("filt_coef_kernel");
-      const dim3 ag(nt, kf);
-      for (int j = 0; j < m; ++j) {
+      for (int j = 0; j < m; ++j)
         // j = 0: g = B R, E_1; then E_{j+1} from E_j and E_{j-1}
-        const zf* in = j == 0 ? Rr : E[(j - 1) & 1];
-        filt_apply_kernel<true><<<ag, 128, AP_SMEM, s>>>(w.X, in, np, Tv, nullptr, 0, nullptr,
-                                                         nullptr, nullptr, done);
-        BS_CHECK_LAUNCH("filt_apply_kernel");
-        filt_apply_kernel<false><<<ag, 128, AP_SMEM, s>>>(
-            w.X, Tv, np, nullptr, w.coef + (size_t)j * 4 * FB, cstride,
-            j == 0 ? nullptr : E[(j - 1) & 1], E[j & 1], g, done);
-        BS_CHECK_LAUNCH("filt_apply_kernel");
-      }
+        TRY_LAUNCH(bs_launch_filter_product(Bp, vs[j & 1], np, kf, w.coef + (size_t)j * 4 * FB,
+                                            cstride, j == 0 ? nullptr : E[(j - 1) & 1], E[j & 1], g,
+                                            vs[(j + 1) & 1], done, err, s));
       filt_add_kernel<<<cg, 256, 0, s>>>(w.Xb, E[(m - 1) & 1], n, np, done);
       BS_CHECK_LAUNCH("filt_add_kernel");
       TRY_LAUNCH(bs_launch_band_av(n, w.Xb, n, (long)FB * n, FB, kf, 8, w.pA, w.pB, w.pD, w.eA,

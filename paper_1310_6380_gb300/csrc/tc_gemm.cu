@@ -410,6 +410,164 @@ __global__ void __launch_bounds__(NT, MINB)
   }
 }
 
+// ---- products of the filtered iteration (filter.cu): Y = B V for the
+// Hermitian operator B (np x np) and a block V of 32 complex columns, both
+// split into two BF16 terms, x = hi + lo + O(2^-17 |x|), of which the products
+// hi hi + hi lo + lo hi are summed in one FP32 accumulator.  A rows r
+// [Re B | Im B] (hi then lo), B rows (i, part) [Re V; -Im V], [Im V; Re V] (hi
+// then lo), so a 64-column accumulator holds the 32 complex columns.  The
+// epilogue forms the next term of the filter's recurrence in FP32 and stores
+// it with its BF16 split, the operand of the next product.
+// Bound: the operator's 8 np^2 bytes per matrix are read once per product
+// (90 x 896^2: 578 MB); two CTAs of two 48 KB stages share an SM so that one's
+// epilogue runs beside the other's loads.  Measured, 90 x 896^2: 0.60 ms as two
+// FP32 products with the triangular factor of the inverse, 0.13 ms here
+// (4.4 TB/s of the operator), for 2 ms to form the operator once.
+constexpr int FP_STAGES = 2, FP_BN = 64;
+constexpr int FP_STAGE = 2 * TILE_A + 2 * tile_b(FP_BN);
+
+__global__ void __launch_bounds__(128, 2)
+    filter_product_kernel(const __grid_constant__ CUtensorMap tmB,
+                          const __grid_constant__ CUtensorMap tmV, int np,
+                          const float* __restrict__ coef, int cstride, const zf* __restrict__ E,
+                          zf* __restrict__ Ep, zf* __restrict__ g, uint16_t* __restrict__ Vout,
+                          const int* __restrict__ skip, int* __restrict__ err) {
+  constexpr uint32_t IDESC = idesc(FP_BN);
+  constexpr int TB_V = tile_b(FP_BN);
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full[FP_STAGES], empty[FP_STAGES], done;
+  __shared__ uint32_t tmem_base;
+  __shared__ float cf[4][32];
+  const int z = blockIdx.y, m0 = blockIdx.x * BM;
+  if (skip[z]) return;
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int K2 = 2 * np, nk = K2 / BK;   // np % 64 == 0
+  cf[warp][lane] = coef[(size_t)z * cstride + threadIdx.x];
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < FP_STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(&done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_base)),
+                 "r"(FP_BN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_base;
+
+  if (warp == 0 && lane == 0) {
+    for (int kb = 0; kb < nk; ++kb) {
+      const int s = kb % FP_STAGES;
+      const uint32_t ph = (uint32_t)(kb / FP_STAGES) & 1u;
+      if (kb >= FP_STAGES && !mbar_wait(&empty[s], ph ^ 1u, err)) break;
+      uint8_t* st = smem + s * FP_STAGE;
+      mbar_expect_tx(&full[s], FP_STAGE);
+      tma_load_3d(st, &tmB, kb * BK, m0, z, &full[s]);
+      tma_load_3d(st + TILE_A, &tmB, K2 + kb * BK, m0, z, &full[s]);
+      tma_load_3d(st + 2 * TILE_A, &tmV, kb * BK, 0, z, &full[s]);
+      tma_load_3d(st + 2 * TILE_A + TB_V, &tmV, K2 + kb * BK, 0, z, &full[s]);
+    }
+  } else if (warp == 1 && lane == 0) {
+    for (int kb = 0; kb < nk; ++kb) {
+      const int s = kb % FP_STAGES;
+      const uint32_t ph = (uint32_t)(kb / FP_STAGES) & 1u;
+      if (!mbar_wait(&full[s], ph, err)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t ah = smem_u32(smem + s * FP_STAGE), al = ah + TILE_A;
+      const uint32_t vh = al + TILE_A, vl = vh + TB_V;
+#pragma unroll
+      for (int kk = 0; kk < BK / 16; ++kk) {
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {   // hi hi, hi lo, lo hi
+          const uint64_t ad = sdesc((t == 2 ? al : ah) + kk * 32);
+          const uint64_t bd = sdesc((t == 1 ? vl : vh) + kk * 32);
+          const uint32_t acc = (kb > 0 || kk > 0 || t > 0) ? 1u : 0u;
+          asm volatile(
+              "{\n\t.reg .pred p;\n\t"
+              "setp.ne.b32 p, %4, 0;\n\t"
+              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+              "l"(ad), "l"(bd), "r"(IDESC), "r"(acc));
+        }
+      }
+      asm volatile(
+          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+              smem_u32(&empty[s]))
+          : "memory");
+    }
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+            smem_u32(&done))
+        : "memory");
+  }
+  __syncwarp();
+  const int r = m0 + warp * 32 + lane;
+  const bool live = r < np;
+  const size_t base = (size_t)z * 32 * np + r;
+  const bool ok = __all_sync(0xffffffffu, mbar_wait(&done, 0u, err));
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (ok) {
+    uint16_t* vo = Vout + (size_t)z * 64 * 4 * np + r;
+#pragma unroll 1
+    for (int c0 = 0; c0 < 32; c0 += 8) {
+      // the recurrence's terms of these columns, fetched before the TMEM wait
+      zf e[8], p[8], gg[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const size_t o = base + (size_t)(c0 + j) * np;
+        e[j] = p[j] = gg[j] = make_float2(0.f, 0.f);
+        if (live && E) {
+          e[j] = E[o];
+          gg[j] = g[o];
+          if (cf[2][c0 + j] != 0.f) p[j] = Ep[o];
+        }
+      }
+      uint32_t v[16];
+      const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(2 * c0);
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+          "%11, %12, %13, %14, %15}, [%16];"
+          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+            "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+            "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+          : "r"(ta));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      if (live) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int c = c0 + j;
+          const size_t o = base + (size_t)c * np;
+          const float yr = __uint_as_float(v[2 * j]), yi = __uint_as_float(v[2 * j + 1]);
+          zf y;
+          if (E) {
+            const float k0 = cf[0][c], k1 = cf[1][c], k2 = cf[2][c], k3 = cf[3][c];
+            y = make_float2(k0 * yr + k1 * e[j].x + k2 * p[j].x + k3 * gg[j].x,
+                            k0 * yi + k1 * e[j].y + k2 * p[j].y + k3 * gg[j].y);
+          } else {
+            g[o] = make_float2(yr, yi);
+            y = make_float2(cf[3][c] * yr, cf[3][c] * yi);
+          }
+          Ep[o] = y;
+          bs_store_block_split(vo + (size_t)c * 8 * np, np, y);
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(FP_BN));
+  }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
@@ -631,5 +789,34 @@ int bs_launch_rank2_update(const uint16_t* dA, const uint16_t* dB, const int* ex
   rank2_update_kernel<BN, R2_STAGES, MINB, NT><<<grid, NT, smem, s>>>(ta, tb, ex, m, A, n, o,
                                                                        ct0, err);
   BS_CHECK_LAUNCH("rank2_update_kernel");
+  return BS_OK;
+}
+
+// E_{j+1} (over E_{j-1}) and its split from E_j: Y = B V, see filter_product_kernel;
+// E null: g = Y and E_1 = coef[3] g
+int bs_launch_filter_product(const uint16_t* B, const uint16_t* V, int np, int batch,
+                             const float* coef, int cstride, const zf* E, zf* Ep, zf* g,
+                             uint16_t* Vout, const int* skip, int* err, cudaStream_t s) {
+  if (np % 64 || ((uintptr_t)B & 15) || ((uintptr_t)V & 15) || batch < 1 || batch > 65535) {
+    bs_set_error("filter product: bad operands (np = %d, batch = %d)", np, batch);
+    return BS_EINVAL;
+  }
+  CUtensorMap tb, tv;
+  int r = make_map(&tb, B, 4 * np, np, batch, (long)np * 4 * np, BM);
+  if (!r) r = make_map(&tv, V, 4 * np, 64, batch, (long)64 * 4 * np, FP_BN);
+  if (r) return r;
+  constexpr int smem = FP_STAGES * FP_STAGE + 1024;
+  static std::atomic<bool> attr[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+  if (!attr[dev].load(std::memory_order_acquire)) {
+    cudaError_t e = cudaFuncSetAttribute(filter_product_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return bs_cuda_status(e, "filter product smem");
+    attr[dev].store(true, std::memory_order_release);
+  }
+  filter_product_kernel<<<dim3((np + BM - 1) / BM, batch), 128, smem, s>>>(
+      tb, tv, np, coef, cstride, E, Ep, g, Vout, skip, err);
+  BS_CHECK_LAUNCH("filter_product_kernel");
   return BS_OK;
 }
