@@ -78,6 +78,13 @@ __host__ __device__ __forceinline__ zf zfnmac(zf a, zf b, zf acc) {
   acc.y = fmaf(a.x, b.y, acc.y);
   return acc;
 }
+__host__ __device__ __forceinline__ zf zfnma(zf a, zf b, zf acc) {
+  acc.x = fmaf(-a.x, b.x, acc.x);
+  acc.x = fmaf(a.y, b.y, acc.x);
+  acc.y = fmaf(-a.x, b.y, acc.y);
+  acc.y = fmaf(-a.y, b.x, acc.y);
+  return acc;
+}
 __host__ __device__ __forceinline__ zf zfmac(zf a, zf b, zf acc) {
   acc.x = fmaf(a.x, b.x, acc.x);
   acc.x = fmaf(a.y, b.y, acc.x);
@@ -296,10 +303,10 @@ bool bs_slice_slabs(int S, int Kp, int M, int N, int batch, SliceSlabs* q);
 size_t bs_slice_planes(int S, int Kp, int M, int N, int batch);
 // D[z][q][n][m] = sum_{k < len_q} A[z][m][a0_q + k] B[z][n][b0_q + k] for every
 // slab q of (S, Kp); A: batch x M x S Kp, B: batch x N x S Kp; entries with a
-// non-zero skip[z] are left out
+// non-zero skip[z] are left out; SA > S: the rows of A hold SA digits
 int bs_launch_slice_orders(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int S,
                            int Kp, int batch, int* err, cudaStream_t s,
-                           const int* skip = nullptr);
+                           const int* skip = nullptr, int SA = 0);
 int bs_launch_fields_tc(bs_cell* c, cudaStream_t s);
 size_t bs_fields_tc_elems(int P, int D, int nf, size_t* nA, size_t* nB, size_t* nD);
 int bs_launch_cx_tc(const zd* C, const zd* X, int n, int b, int kb, uint16_t* sA, uint16_t* sB,

@@ -36,8 +36,8 @@
 //
 // Measured (one GB300, whole FP64 solve with its assembly, the reduction to
 // tridiagonal form before -> this): n = 882, 90 matrices, 18 branches
-// 171 -> 36 ms; n = 1029, 30 matrices, 12 branches 136 -> 25 ms; n = 242,
-// 70 matrices, 18 branches 16.9 -> 7.9 ms.  What bounds it at n = 882 is the
+// 171 -> 34 ms; n = 1029, 30 matrices, 12 branches 136 -> 23 ms; n = 242,
+// 70 matrices, 18 branches 16.9 -> 5.8 ms.  What bounds it at n = 882 is the
 // FP32 pipe in the factorisations and the FP64 pipe in the Rayleigh-Ritz steps
 // (32-column products at 2 FMA per clock and SM).
 //
@@ -58,6 +58,7 @@ constexpr int TB = 64;              // tile edge of the FP32 factorisation
 constexpr int LDS = TB + 1;         // row stride of the diagonal blocks in shared memory
 constexpr float TINY_PIVOT = 1e-6f; // of the scaled unit diagonal
 constexpr int GR = 64;              // rows per CTA of the Gram and rotation kernels
+constexpr int STEER_DIGITS = 5;     // of C X in the steps that only steer (34 bits)
 
 // ---------------------------------------------------------------- set-up
 // Per matrix: the FB smallest diagonal entries (the starting vectors are
@@ -615,147 +616,152 @@ __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
   }
 }
 
-// cyclic Jacobi of the 32 x 32 Hermitian matrix A (shared, stride FB + 1) with
-// the round-robin pairing: one thread per pair of index pairs applies both
-// sides' rotations to its 2 x 2 block (the blocks partition A), two threads'
-// worth of work per pair and row rotate V.  256 threads.
-template <typename R>
-__device__ void jacobi32(typename Cplx<R>::T (*A)[FB + 1], typename Cplx<R>::T (*V)[FB + 1],
-                         R offtol, int maxsweep, R* red) {
-  typedef typename Cplx<R>::T T;
-  __shared__ R cs_[FB / 2], sn_[FB / 2];
-  __shared__ T ph_[FB / 2];
-  const int tid = threadIdx.x;
-  const int u = tid >> 4, v = tid & 15;
+// Cyclic Jacobi of a 32 x 32 Hermitian matrix with the round-robin pairing,
+// 256 threads.  The off-diagonal entries and the vectors are FP32, the
+// diagonal is a sum hi + lo of two FP32 numbers (48 bits): the rotations take
+// differences of the diagonal and shifts t |c| of it, both exact to FP32
+// relative to the off-diagonal entry c, so the error left is FP32 rounding of
+// the off-diagonal part alone (1e-7 of what the block is away from diagonal
+// when the step begins, squared in the Ritz values).  A full FP64 sweep is
+// bound by the SM's FP64 pipe (31 rounds of 8 us); the FP64 step's kernel took
+// 1120 us with FP64 sweeps alone, 560 us with one behind FP32 ones, 270 us so
+// (90 matrices of n = 882).  Thread (u, v) applies both
+// sides' rotations to the 2 x 2 block of the index pairs u, v (the blocks
+// partition the matrix) from one copy of A to the other and rotates V's
+// columns of pair v in rows u and u + 16: one barrier per round.
+struct JacobiSmem {
+  zf A[2][FB][FB + 1], V[FB][FB + 1];
+  float2 D[2][FB];   // diagonal, hi + lo
+  float red[16];
+};
+
+// (hi, lo) + x, renormalised
+__device__ __forceinline__ float2 dd_add(float2 a, float x) {
+  const float s = a.x + x, b = s - a.x;
+  const float e = (a.x - (s - b)) + (x - b) + a.y;
+  const float h = s + e;
+  return make_float2(h, e - (h - s));
+}
+
+// rotation of the pair with off-diagonal entry c and diagonal difference
+// dq - dp: cs, sn, the phase c / |c| and the shift t |c|
+__device__ __forceinline__ void rotation(zf c, float diff, float skip, float& cs, float& sn, zf& ph,
+                                         float& shift) {
+  const float c2 = c.x * c.x + c.y * c.y;
+  cs = 1.f;
+  sn = shift = 0.f;
+  ph = make_float2(1.f, 0.f);
+  if (c2 > skip) {
+    const float ica = rsqrtf(c2), ca = c2 * ica;
+    ph = make_float2(c.x * ica, c.y * ica);
+    const float zeta = 0.5f * diff * ica, az = fabsf(zeta);
+    // t = 1 / (|zeta| + sqrt(1 + zeta^2)), for large zeta without its square
+    float t = az > 1e4f ? __fdividef(0.5f, az)
+                        : __fdividef(1.f, az + (1.f + az * az) * rsqrtf(1.f + az * az));
+    t = copysignf(t, zeta);
+    cs = rsqrtf(1.f + t * t);
+    sn = t * cs;
+    shift = t * ca;
+  }
+}
+
+// returns the copy of D that holds the result
+__device__ int jacobi32(JacobiSmem& sm, float offtol, int maxsweep) {
+  const int tid = threadIdx.x, u = tid >> 4, v = tid & 15;
+  int cur = 0;
   for (int sweep = 0; sweep < maxsweep; ++sweep) {
-    R o = 0, t = 0;
+    float o = 0.f, t = 0.f;
     for (int e = tid; e < FB * FB; e += 256) {
       const int r = e >> 5, c = e & 31;
-      const T a = A[r][c];
-      const R m2 = a.x * a.x + a.y * a.y;
-      t += m2;
-      if (r != c) o += m2;
+      const zf a = sm.A[cur][r][c];
+      if (r != c) o += a.x * a.x + a.y * a.y;
+      else t += sm.D[cur][r].x * sm.D[cur][r].x;
     }
     for (int sh = 16; sh > 0; sh >>= 1) {
       o += __shfl_xor_sync(0xffffffffu, o, sh);
       t += __shfl_xor_sync(0xffffffffu, t, sh);
     }
     if ((tid & 31) == 0) {
-      red[2 * (tid >> 5)] = o;
-      red[2 * (tid >> 5) + 1] = t;
+      sm.red[2 * (tid >> 5)] = o;
+      sm.red[2 * (tid >> 5) + 1] = t;
     }
     __syncthreads();
-    R so = 0, stt = 0;
+    float so = 0.f, st = 0.f;
     for (int q = 0; q < 8; ++q) {
-      so += red[2 * q];
-      stt += red[2 * q + 1];
+      so += sm.red[2 * q];
+      st += sm.red[2 * q + 1];
     }
-    if (!(so > offtol * stt)) break;   // also ends on NaN
-    const R skip = offtol * stt / (R)(FB * FB);   // pairs already below the stopping size
+    st += so;
+    if (!(so > offtol * st)) break;   // also ends on NaN
+    const float skip = 0.25f * offtol * st / (FB * FB);   // below the stopping size
     for (int rd = 0; rd < FB - 1; ++rd) {
       auto pair = [&](int m, int& p, int& q) {
-        if (m == 0) {
-          p = rd;
-          q = FB - 1;
-        } else {
-          p = rd + m;
-          if (p >= FB - 1) p -= FB - 1;
-          q = rd - m;
-          if (q < 0) q += FB - 1;
-        }
-        if (p > q) {
-          const int w = p;
-          p = q;
-          q = w;
-        }
+        p = rd + m;
+        if (p >= FB - 1) p -= FB - 1;
+        q = rd - m;
+        if (q < 0) q += FB - 1;
+        if (m == 0) q = FB - 1;
+        const int lo = min(p, q);
+        q = max(p, q);
+        p = lo;
       };
-      int act = 0;
-      if (tid < FB / 2) {
-        int p, q;
-        pair(tid, p, q);
-        const T c = A[p][q];
-        const R c2 = c.x * c.x + c.y * c.y;
-        R cs = 1, sn = 0;
-        T ph = Cplx<R>::make((R)1, (R)0);
-        if (c2 > skip * (R)0.25) {
-          act = 1;
-          const R ica = rsqrt(c2), ca = c2 * ica;
-          ph = Cplx<R>::make(c.x * ica, c.y * ica);
-          const R zeta = (A[q][q].x - A[p][p].x) * (R)0.5 / ca;
-          const R az = zeta < 0 ? -zeta : zeta;
-          // beyond 1e9 (FP32: 1e6) the rotation is 1 / (2 zeta) to rounding
-          R tt = (R)1 / (az + sqrt((R)1 + az * az));
-          if (zeta < 0) tt = -tt;
-          cs = rsqrt((R)1 + tt * tt);
-          sn = tt * cs;
-        }
-        cs_[tid] = cs;
-        sn_[tid] = sn;
-        ph_[tid] = ph;
-      }
-      if (!__syncthreads_or(act)) continue;
+      int pu, qu, pv, qv;
+      pair(u, pu, qu);
+      pair(v, pv, qv);
+      zf(*A)[FB + 1] = sm.A[cur];
+      zf(*B)[FB + 1] = sm.A[cur ^ 1];
+      const float2 dpu = sm.D[cur][pu], dqu = sm.D[cur][qu];
+      const float2 dpv = sm.D[cur][pv], dqv = sm.D[cur][qv];
+      float cu, su, shu, cv, sv, shv;
+      zf fu, fv;
+      rotation(A[pu][qu], (dqu.x - dpu.x) + (dqu.y - dpu.y), skip, cu, su, fu, shu);
+      rotation(A[pv][qv], (dqv.x - dpv.x) + (dqv.y - dpv.y), skip, cv, sv, fv, shv);
+      fv = zconj(fv);
       // J = [[cs, sn], [-sn conj(ph), cs conj(ph)]] on columns (p, q); A <- J_u^dagger A J_v
-      {
-        int pu, qu, pv, qv;
-        pair(u, pu, qu);
-        pair(v, pv, qv);
-        const R cu = cs_[u], su = sn_[u], cv = cs_[v], sv = sn_[v];
-        const T fu = ph_[u], fv = zconj(ph_[v]);
-        const T a00 = A[pu][pv], a01 = zmul(A[pu][qv], fv);
-        const T a10 = zmul(A[qu][pv], fu), a11 = zmul(zmul(A[qu][qv], fv), fu);
-        const T b00 = zsub(zscale(a00, cv), zscale(a01, sv));
-        const T b01 = zadd(zscale(a00, sv), zscale(a01, cv));
-        const T b10 = zsub(zscale(a10, cv), zscale(a11, sv));
-        const T b11 = zadd(zscale(a10, sv), zscale(a11, cv));
-        A[pu][pv] = zsub(zscale(b00, cu), zscale(b10, su));
-        A[pu][qv] = zsub(zscale(b01, cu), zscale(b11, su));
-        A[qu][pv] = zadd(zscale(b00, su), zscale(b10, cu));
-        A[qu][qv] = zadd(zscale(b01, su), zscale(b11, cu));
-        // rows of V: pair v, rows u and u + 16
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int r = u + 16 * h;
-          const T vp = V[r][pv], vq = zmul(V[r][qv], fv);
-          V[r][pv] = zsub(zscale(vp, cv), zscale(vq, sv));
-          V[r][qv] = zadd(zscale(vp, sv), zscale(vq, cv));
-        }
+      if (u == v) {
+        // the pair itself: the shifted diagonal and a zero (or the skipped entry)
+        sm.D[cur ^ 1][pu] = dd_add(dpu, -shu);
+        sm.D[cur ^ 1][qu] = dd_add(dqu, shu);
+        const zf c = su != 0.f ? make_float2(0.f, 0.f) : A[pu][qu];
+        B[pu][qu] = c;
+        B[qu][pu] = zconj(c);
+      } else {
+        const zf a00 = A[pu][pv], a01 = zmul(A[pu][qv], fv);
+        const zf a10 = zmul(A[qu][pv], fu), a11 = zmul(zmul(A[qu][qv], fv), fu);
+        const zf b00 = zsub(zscale(a00, cv), zscale(a01, sv));
+        const zf b01 = zadd(zscale(a00, sv), zscale(a01, cv));
+        const zf b10 = zsub(zscale(a10, cv), zscale(a11, sv));
+        const zf b11 = zadd(zscale(a10, sv), zscale(a11, cv));
+        B[pu][pv] = zsub(zscale(b00, cu), zscale(b10, su));
+        B[pu][qv] = zsub(zscale(b01, cu), zscale(b11, su));
+        B[qu][pv] = zadd(zscale(b00, su), zscale(b10, cu));
+        B[qu][qv] = zadd(zscale(b01, su), zscale(b11, cu));
       }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = u + 16 * h;
+        const zf vp = sm.V[r][pv], vq = zmul(sm.V[r][qv], fv);
+        sm.V[r][pv] = zsub(zscale(vp, cv), zscale(vq, sv));
+        sm.V[r][qv] = zadd(zscale(vp, sv), zscale(vq, cv));
+      }
+      cur ^= 1;
       __syncthreads();
     }
   }
-  __syncthreads();
+  return cur;
 }
 
-// H w = theta G w per matrix from the Gram partials: FP64 Cholesky of the
+// H w = theta G w per matrix from the Gram partials: Cholesky of the
 // unit-diagonal G and its inverse factor (one barrier per column, as
-// ldl64_block), A = L^-1 H L^-dagger, Jacobi in R, W = S L^-dagger V.  fail: G not
-// positive definite.
-//
-// The FP64 Jacobi starts from the FP32 one: a sweep of 31 rotation rounds is
-// bound by the SM's FP64 pipe (2 FMA per clock), so the FP32 eigenvectors, made
-// orthonormal to 1e-12 by one Newton-Schulz step, first make A diagonal to
-// 1e-6, and one or two FP64 sweeps finish it; the vectors' norms are divided out.
-typedef zd Zd32[FB][FB + 1];
+// ldl64_block), A = L^-1 H L^-dagger, Jacobi, W = S L^-dagger V, all but the
+// Jacobi in R (FP64 throughout but in the steps that only steer).  In FP64 a
+// Newton-Schulz step makes the FP32 vectors orthonormal to 1e-12 and their
+// norms are divided out.  fail: G not positive definite.
+template <typename R>
 struct EigSmem {
-  Zd32 G, H, Li, V;
-  zf A32[FB][FB + 1], V32[FB][FB + 1];
+  typename Cplx<R>::T G[FB][FB + 1], H[FB][FB + 1], Li[FB][FB + 1], V[FB][FB + 1];
+  JacobiSmem J;
 };
-
-// D = op(A) B (op: conjugate transpose when CT), lower triangle only when herm
-template <bool CT>
-__device__ __forceinline__ void mul32(const Zd32& A, const Zd32& B, Zd32& D, bool herm) {
-  for (int e = threadIdx.x; e < FB * FB; e += 256) {
-    const int r = e / FB, c = e % FB;
-    if (herm && r < c) continue;
-    zd s = zmake(0.0, 0.0);
-    for (int t = 0; t < FB; ++t) s = CT ? zfmac(B[t][c], A[t][r], s) : zfma(A[r][t], B[t][c], s);
-    if (herm) {
-      if (r == c) s.y = 0.0;
-      D[c][r] = zconj(s);
-    }
-    D[r][c] = s;
-  }
-}
 
 template <typename R>
 __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ part, int nch,
@@ -765,12 +771,14 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
                                                        const int* __restrict__ done) {
   if (done[blockIdx.x]) return;
   extern __shared__ __align__(16) unsigned char dsm[];
-  EigSmem& sm = *reinterpret_cast<EigSmem*>(dsm);
-  __shared__ double sc[FB], ev[FB], sc_top;
-  __shared__ double red[16];
+  typedef typename Cplx<R>::T T;
+  EigSmem<R>& sm = *reinterpret_cast<EigSmem<R>*>(dsm);
+  __shared__ double ev[FB];
+  __shared__ R sc[FB], pinv[FB], sc_top;
   __shared__ int rank[FB], bad, out[FB];
   // a pivot of the unit-diagonal G below the rounding of its entries
-  constexpr double kTiny = sizeof(R) == 8 ? 1e-13 : 1e-5;
+  constexpr R kTiny = sizeof(R) == 8 ? (R)1e-13 : (R)1e-5;
+  const T zero = Cplx<R>::make((R)0, (R)0);
   const int k = blockIdx.x, tid = threadIdx.x;
   if (tid == 0) bad = 0;
   for (int e = tid; e < FB * FB; e += 256) {
@@ -783,62 +791,63 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
       h = zadd(h, p[FB * FB]);
     }
     if (r == c) g.y = h.y = 0.0;
-    sm.G[r][c] = g;
-    sm.H[r][c] = h;
-    sm.H[c][r] = zconj(h);
+    sm.G[r][c] = Cplx<R>::make((R)g.x, (R)g.y);
+    sm.H[r][c] = Cplx<R>::make((R)h.x, (R)h.y);
+    sm.H[c][r] = Cplx<R>::make((R)h.x, (R)-h.y);
   }
   __syncthreads();
   if (tid < FB) {
-    const double g = sm.G[tid][tid].x;
-    sc[tid] = g > 0.0 ? rsqrt(g) : 0.0;
+    const R g = sm.G[tid][tid].x;
+    sc[tid] = g > (R)0 ? rsqrt(g) : (R)0;
     out[tid] = 0;
   }
   __syncthreads();
   for (int e = tid; e < FB * FB; e += 256) {
     const int r = e / FB, c = e % FB;
-    const double f = sc[r] * sc[c];
+    const R f = sc[r] * sc[c];
     if (r >= c) sm.G[r][c] = zscale(sm.G[r][c], f);
     sm.H[r][c] = zscale(sm.H[r][c], f);
-    sm.Li[r][c] = zmake(r == c ? 1.0 : 0.0, 0.0);
-    sm.V32[r][c] = make_float2(r == c ? 1.f : 0.f, 0.f);
+    sm.Li[r][c] = Cplx<R>::make(r == c ? (R)1 : (R)0, (R)0);
+    sm.J.V[r][c] = make_float2(r == c ? 1.f : 0.f, 0.f);
   }
   __syncthreads();
   {
-    // unit L and pivots: G = L D L^dagger; Li accumulates L^-1
+    // unit L and pivots: G = L D L^dagger; Li accumulates L^-1.  The lane that
+    // finishes a pivot also inverts it, so the other warps issue no division.
     const int r = tid & 31, q = tid >> 5;
-    for (int c = 0; c < FB; ++c) {
-      double p = sm.G[c][c].x;
+    auto pivot = [&](int c) {
+      R p = sm.G[c][c].x;
       if (!(p > kTiny)) {
-        if (tid == 0) {
-          bad = 1;
-          out[c] = 1;
-        }
-        p = 1.0;
+        bad = 1;
+        out[c] = 1;
+        p = (R)1;
       }
-      const double inv = 1.0 / p;
+      pinv[c] = (R)1 / p;
+    };
+    if (tid == 0) pivot(0);
+    __syncthreads();
+    for (int c = 0; c < FB; ++c) {
       if (r > c) {
-        const zd l = zscale(sm.G[r][c], inv);
+        const T l = zscale(sm.G[r][c], pinv[c]);
         for (int s = c + 1 + q; s <= r; s += 8) sm.G[r][s] = zfnmac(l, sm.G[s][c], sm.G[r][s]);
+        if (q == 0 && r == c + 1) pivot(r);
         for (int s = q; s <= c; s += 8) sm.Li[r][s] = zfnma(l, sm.Li[c][s], sm.Li[r][s]);
       }
       __syncthreads();
     }
     if (tid == 0) fail[k] = bad;
-    if (tid < FB) {
-      const double p = sm.G[tid][tid].x;
-      ev[tid] = p > kTiny ? rsqrt(p) : 1.0;
-    }
+    if (tid < FB) pinv[tid] = sqrt(pinv[tid]);
     __syncthreads();
     for (int e = tid; e < FB * FB; e += 256) {
       const int rr = e / FB, c = e % FB;
-      sm.Li[rr][c] = rr >= c ? zscale(sm.Li[rr][c], ev[rr]) : zmake(0.0, 0.0);
+      sm.Li[rr][c] = rr >= c ? zscale(sm.Li[rr][c], pinv[rr]) : zero;
     }
     __syncthreads();
   }
   // G <- Li H, then H <- (Li H) Li^dagger (lower triangle, mirrored)
   for (int e = tid; e < FB * FB; e += 256) {
     const int r = e / FB, c = e % FB;
-    zd s = zmake(0.0, 0.0);
+    T s = zero;
     for (int t = 0; t <= r; ++t) s = zfma(sm.Li[r][t], sm.H[t][c], s);
     sm.G[r][c] = s;
   }
@@ -846,71 +855,73 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
   for (int e = tid; e < FB * FB; e += 256) {
     const int r = e / FB, c = e % FB;
     if (r < c) continue;
-    zd s = zmake(0.0, 0.0);
+    T s = zero;
     for (int t = 0; t <= c; ++t) s = zfmac(sm.G[r][t], sm.Li[c][t], s);
-    if (r == c) s.y = 0.0;
+    if (r == c) s.y = (R)0;
     sm.H[r][c] = s;
-    sm.H[c][r] = zconj(s);
-    sm.A32[r][c] = make_float2((float)s.x, (float)s.y);
-    sm.A32[c][r] = make_float2((float)s.x, (float)-s.y);
   }
   __syncthreads();
-  if (bad) {
+  if (bad && tid < 32) {
     // vectors that depend on the others: decoupled, at the top of the spectrum
-    if (tid < 32) {
-      double m = out[tid] ? 0.0 : sm.H[tid][tid].x;
-      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (tid == 0) sc_top = m;
+    R m = out[tid] ? (R)0 : sm.H[tid][tid].x;
+    for (int o = 16; o > 0; o >>= 1) {
+      const R x = __shfl_xor_sync(0xffffffffu, m, o);
+      m = x > m ? x : m;
+    }
+    if (tid == 0) sc_top = m;
+  }
+  __syncthreads();
+  for (int e = tid; e < FB * FB; e += 256) {
+    const int r = e / FB, c = e % FB;
+    if (r < c) continue;
+    T s = sm.H[r][c];
+    if (bad && (out[r] || out[c])) s = Cplx<R>::make(r == c ? sc_top : (R)0, (R)0);
+    if (r == c) {
+      const float h = (float)s.x;
+      sm.J.D[0][r] = make_float2(h, (float)(s.x - (R)h));
+      sm.J.A[0][r][r] = make_float2(0.f, 0.f);
+      sm.J.A[1][r][r] = make_float2(0.f, 0.f);
+    } else {
+      sm.J.A[0][r][c] = make_float2((float)s.x, (float)s.y);
+      sm.J.A[0][c][r] = make_float2((float)s.x, (float)-s.y);
+    }
+  }
+  __syncthreads();
+  // off-diagonal norm below 3e-10 of the whole (3e-7 in the steps that steer)
+  const int cur = jacobi32(sm.J, sizeof(R) == 8 ? 1e-19f : 1e-13f, 10);
+  for (int e = tid; e < FB * FB; e += 256) {
+    const zf v = sm.J.V[e / FB][e % FB];
+    sm.V[e / FB][e % FB] = Cplx<R>::make((R)v.x, (R)v.y);
+  }
+  if (tid < FB) ev[tid] = (double)sm.J.D[cur][tid].x + (double)sm.J.D[cur][tid].y;
+  __syncthreads();
+  if (sizeof(R) == 8) {
+    // G <- (3 I - V^dagger V) / 2, H <- V G, columns to unit length
+    for (int e = tid; e < FB * FB; e += 256) {
+      const int r = e / FB, c = e % FB;
+      if (r < c) continue;
+      T s = zero;
+      for (int t = 0; t < FB; ++t) s = zfmac(sm.V[t][c], sm.V[t][r], s);   // conj(V_tr) V_tc
+      s = Cplx<R>::make((r == c ? (R)1.5 : (R)0) - (R)0.5 * s.x, r == c ? (R)0 : (R)-0.5 * s.y);
+      sm.G[r][c] = s;
+      sm.G[c][r] = zconj(s);
     }
     __syncthreads();
     for (int e = tid; e < FB * FB; e += 256) {
       const int r = e / FB, c = e % FB;
-      if (!out[r] && !out[c]) continue;
-      sm.H[r][c] = zmake(r == c ? sc_top : 0.0, 0.0);
-      sm.A32[r][c] = make_float2(r == c ? (float)sc_top : 0.f, 0.f);
+      T s = zero;
+      for (int t = 0; t < FB; ++t) s = zfma(sm.V[r][t], sm.G[t][c], s);
+      sm.H[r][c] = s;
     }
     __syncthreads();
-  }
-  // FP32: off-diagonal norm below 1e-6 of the whole
-  jacobi32<float>(sm.A32, sm.V32, 1e-12f, 12, reinterpret_cast<float*>(red));
-  for (int e = tid; e < FB * FB; e += 256) {
-    const zf v = sm.V32[e / FB][e % FB];
-    sm.V[e / FB][e % FB] = zmake((double)v.x, (double)v.y);
-  }
-  __syncthreads();
-  if (sizeof(R) == 8) {
-    mul32<true>(sm.V, sm.V, sm.G, true);
-    __syncthreads();
-    for (int e = tid; e < FB * FB; e += 256) {   // (3 I - V^dagger V) / 2
-      const int r = e / FB, c = e % FB;
-      const zd g = sm.G[r][c];
-      sm.G[r][c] = zmake((r == c ? 1.5 : 0.0) - 0.5 * g.x, -0.5 * g.y);
-    }
-    __syncthreads();
-    // the corrected V goes where the FP32 matrices lay (they are done with)
-    Zd32& V = *reinterpret_cast<Zd32*>(&sm.A32[0][0]);
-    mul32<false>(sm.V, sm.G, V, false);
-    __syncthreads();
-    mul32<false>(sm.H, V, sm.G, false);
-    __syncthreads();
-    mul32<true>(V, sm.G, sm.H, true);
-    __syncthreads();
-    // off-diagonal norm below 1e-10 of the whole: the Ritz values then carry
-    // (1e-10 ||H||)^2 / gap
-    jacobi32<double>(sm.H, V, 1e-20, 12, red);
-    // columns of V to unit length
     const int c = tid >> 3, q = tid & 7;
-    double v2 = 0.0;
-    for (int r = q; r < FB; r += 8) v2 = fma(V[r][c].x, V[r][c].x, fma(V[r][c].y, V[r][c].y, v2));
+    R v2 = (R)0;
+    for (int r = q; r < FB; r += 8) v2 += sm.H[r][c].x * sm.H[r][c].x + sm.H[r][c].y * sm.H[r][c].y;
     for (int o = 4; o > 0; o >>= 1) v2 += __shfl_xor_sync(0xffffffffu, v2, o);
+    const R iv = rsqrt(v2);
+    for (int r = q; r < FB; r += 8) sm.V[r][c] = zscale(sm.H[r][c], iv);
     __syncthreads();
-    const double iv = rsqrt(v2);
-    if (q == 0) ev[c] = sm.H[c][c].x * iv * iv;
-    for (int r = q; r < FB; r += 8) sm.V[r][c] = zscale(V[r][c], iv);
-  } else {
-    if (tid < FB) ev[tid] = (double)sm.A32[tid][tid].x;
   }
-  __syncthreads();
   if (tid < FB) {
     const double x = ev[tid];
     int rk = 0;
@@ -920,10 +931,11 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
   }
   __syncthreads();
   for (int e = tid; e < FB * FB; e += 256) {
-    const int r = e % FB, c = e / FB;   // W[r][rank(c)] = sc_r sum_t conj(Li[t][r]) V[t][c]
-    zd s = zmake(0.0, 0.0);
+    const int r = e / FB, c = e % FB;   // W[r][rank(c)] = sc_r sum_t conj(Li[t][r]) V[t][c]
+    T s = zero;
     for (int t = r; t < FB; ++t) s = zfmac(sm.V[t][c], sm.Li[t][r], s);
-    W[(size_t)k * FB * FB + r + (size_t)rank[c] * FB] = zscale(s, sc[r]);
+    s = zscale(s, sc[r]);
+    W[(size_t)k * FB * FB + r + (size_t)rank[c] * FB] = zmake((double)s.x, (double)s.y);
     if (r == 0) theta[(size_t)k * FB + rank[c]] = ev[c];
   }
 }
@@ -933,15 +945,17 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
 // is T_j(l(mu)), l(mu) = 2 mu / mu_cut - 1 with mu_cut that of the last guard
 // vector, so l >= 1 on the block.  A column stops at the last degree whose
 // growth relative to it, tau_j(l_0) / tau_j(l_c) (the lowest branch grows
-// most), times what the residual holds of the other branches stays below 0.1:
-// 4e-6 of itself (the split operands), `couple` of the block's largest Ritz value
-// (the off-diagonal the Jacobi sweeps left) and the rounding of C X.  Beyond,
-// the column would turn into the lowest branches and the block lose rank.
+// most), times what the residual holds of the other branches stays below
+// `allow`: 4e-6 of itself (the split operands), `couple` of the column's Ritz
+// value (the rounding of the Rayleigh-Ritz step, and what its Jacobi sweeps
+// left, of the largest one) and the rounding of C X.  Beyond, the column
+// would turn into the lowest branches; allow is what the Gram matrix of the
+// next step can separate again (3 in FP32, 100 in FP64, 1 before the last).
 __global__ void __launch_bounds__(128) filt_coef_kernel(const double* __restrict__ theta,
                                                         const float* __restrict__ rpart, int nch,
                                                         const double* __restrict__ shift, int kb,
                                                         const double* __restrict__ cmax,
-                                                        double couple, int m,
+                                                        double couple, double allow, int m,
                                                         float* __restrict__ coef,
                                                         const int* __restrict__ done) {
   const int k = blockIdx.x * 4 + (threadIdx.x >> 5), c = threadIdx.x & 31;
@@ -952,8 +966,8 @@ __global__ void __launch_bounds__(128) filt_coef_kernel(const double* __restrict
   const double cut = __shfl_sync(0xffffffffu, t, 31);
   const double mu = 1.0 / (t + 1.0), imuc = cut + 1.0;
   const double l = fmax(2.0 * mu * imuc - 1.0, 1.0), f = 2.0 * mu * imuc;
-  const double lim = 0.1 / (4e-6 * (double)sqrtf(rn) + couple * cut +
-                            4.0 * DBL_EPSILON * cmax[k] / shift[k]);
+  const double lim = allow / (4e-6 * (double)sqrtf(rn) + couple * (t + 0.1 * cut) +
+                              4.0 * DBL_EPSILON * cmax[k] / shift[k]);
   float* cf = coef + (size_t)k * BS_FILT_MAXDEG * 4 * FB + c;
   double t0 = 1.0, t1 = l;   // tau_{j-1}, tau_j
   bool stop = __shfl_sync(0xffffffffu, t1, 0) > lim * t1;
@@ -1097,7 +1111,10 @@ int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
       {(void**)&w->X, k * np * np * sizeof(zf)},
       {(void**)&w->pA, k * n * 8 * Kp * 2},
       {(void**)&w->pB, k * 2 * FB * 8 * Kp * 2},
-      {(void**)&w->pD, bs_slice_planes(8, (int)Kp, n, 2 * FB, kf) * n * 2 * FB * sizeof(float)},
+      // fewer digits can be cut into more slabs: room for either
+      {(void**)&w->pD, std::max(bs_slice_planes(8, (int)Kp, n, 2 * FB, kf),
+                                bs_slice_planes(STEER_DIGITS, (int)Kp, n, 2 * FB, kf)) *
+                           n * 2 * FB * sizeof(float)},
       {(void**)&w->eA, k * n * sizeof(int)},
       {(void**)&w->eB, k * FB * sizeof(int)},
       {(void**)&w->Xb, k * FB * n * sizeof(zd)},
@@ -1147,8 +1164,8 @@ static int filter_attrs() {
        (int)(sizeof(RrSmem<double>) + FB * FB * sizeof(zd))},
       {(const void*)filt_gram_kernel<float>, (int)sizeof(RrSmem<float>)},
       {(const void*)filt_rotate_kernel<float>, (int)(sizeof(RrSmem<float>) + FB * FB * sizeof(zf))},
-      {(const void*)filt_eig_kernel<double>, (int)sizeof(EigSmem)},
-      {(const void*)filt_eig_kernel<float>, (int)sizeof(EigSmem)},
+      {(const void*)filt_eig_kernel<double>, (int)sizeof(EigSmem<double>)},
+      {(const void*)filt_eig_kernel<float>, (int)sizeof(EigSmem<float>)},
   };
   for (auto& f : fs) {
     const cudaError_t e =
@@ -1193,7 +1210,7 @@ static int filter_ritz(FilterWs& w, int n, int np, int kf, cudaStream_t s) {
   filt_gram_kernel<R><<<dim3(nch, kf), GT, sizeof(RrSmem<R>), s>>>(w.Xb, w.CX, n, w.part,
                                                                       done);
   BS_CHECK_LAUNCH("filt_gram_kernel");
-  filt_eig_kernel<R><<<kf, 256, sizeof(EigSmem), s>>>(w.part, nch, w.theta, w.W,
+  filt_eig_kernel<R><<<kf, 256, sizeof(EigSmem<R>), s>>>(w.part, nch, w.theta, w.W,
                                                          fail, done);
   BS_CHECK_LAUNCH("filt_eig_kernel");
   // the rotation covers the padded rows as well (np <= nch GR)
@@ -1254,7 +1271,8 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
       if (rd == rounds) break;
       const int m = degs[rd];
       filt_coef_kernel<<<(kf + 3) / 4, 128, 0, s>>>(w.theta, w.rpart, nch, w.shift, kf, w.cmax,
-                                                    rd < 3 ? 1e-6 : 1e-10, m, w.coef, done);
+                                                    rd < 3 ? 3e-7 : 1e-9,
+                                                    rd < 2 ? 3.0 : rd == 2 ? 100.0 : 1.0, m, w.coef, done);
       BS_CHECK_LAUNCH("filt_coef_kernel");
       for (int j = 0; j < m; ++j)
         // j = 0: g = B R, E_1; then E_{j+1} from E_j and E_{j-1}
@@ -1263,7 +1281,8 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
                                             vs[(j + 1) & 1], done, err, s));
       filt_add_kernel<<<cg, 256, 0, s>>>(w.Xb, E[(m - 1) & 1], n, np, done);
       BS_CHECK_LAUNCH("filt_add_kernel");
-      TRY_LAUNCH(bs_launch_band_av(n, w.Xb, n, (long)FB * n, FB, kf, 8, w.pA, w.pB, w.pD, w.eA,
+      TRY_LAUNCH(bs_launch_band_av(n, w.Xb, n, (long)FB * n, FB, kf, rd < 2 ? STEER_DIGITS : 8,
+                                   w.pA, w.pB, w.pD, w.eA,
                                    w.eB, w.CX, n, (long)FB * n, err, s, done));
     }
     filt_scale_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(Ck, n, np, w.shift, w.sigma, w.w,

@@ -655,19 +655,20 @@ int bs_launch_band_pack_trail(const zd* A, int n, int o, int m, int kb, uint16_t
   return BS_OK;
 }
 
-// X = A22 V from the trailing block's digit planes (bs_launch_band_pack_trail)
+// X = A22 V from the trailing block's eight digit planes (bs_launch_band_pack_trail)
+// and the first S digits of both (S = 8: all of FP64)
 int bs_launch_band_av(int m, const zd* V, int ldv, long sv, int nb, int kb, int S, uint16_t* wA,
                       uint16_t* wB, float* wD, int* eA, int* eB, zd* X, int ldx, long sx,
                       int* err, cudaStream_t s, const int* skip) {
   const int Kp = (2 * m + 63) / 64 * 64;
   SliceSlabs sl;
-  if (S != 8 || !bs_slice_slabs(S, Kp, m, 2 * nb, kb, &sl)) {
+  if (S < 1 || S > 8 || !bs_slice_slabs(S, Kp, m, 2 * nb, kb, &sl)) {
     bs_set_error("band reduction: m = %d gives too many digit slabs", m);
     return BS_EINVAL;
   }
   pack_panel_kernel<<<dim3(nb, kb), 128, 0, s>>>(V, ldv, sv, m, nb, S, Kp, wB, eB, skip);
   BS_CHECK_LAUNCH("pack_panel_kernel");
-  TRY_LAUNCH(bs_launch_slice_orders(wA, wB, wD, m, 2 * nb, S, Kp, kb, err, s, skip));
+  TRY_LAUNCH(bs_launch_slice_orders(wA, wB, wD, m, 2 * nb, S, Kp, kb, err, s, skip, 8));
   recombine_panel_kernel<<<dim3((m * nb + 255) / 256, kb), 256, 0, s>>>(wD, sl, eA, eB, m, nb, X,
                                                                        ldx, sx, skip);
   BS_CHECK_LAUNCH("recombine_panel_kernel");

@@ -625,9 +625,9 @@ static int pick_bn(int N) {
 template <int BN>
 static int launch_bn(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int K,
                      int batch, long sA, long sB, long ldd, long sD, const SliceSlabs& slabs,
-                     int* err, cudaStream_t s, const int* skip) {
+                     int* err, cudaStream_t s, const int* skip, int KA) {
   CUtensorMap ta, tb;
-  int r = make_map(&ta, A, K, M, batch, sA, BM);
+  int r = make_map(&ta, A, KA, M, batch, sA, BM);
   if (!r) r = make_map(&tb, B, K, N, batch, sB, BN);
   if (r) return r;
   // the shared-memory opt-in is a per-device attribute of the kernel
@@ -650,13 +650,13 @@ static int launch_bn(const uint16_t* A, const uint16_t* B, float* D, int M, int 
 
 static int dispatch_bn(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int K,
                        int batch, long sA, long sB, long ldd, long sD, const SliceSlabs& slabs,
-                       int* err, cudaStream_t s, const int* skip) {
+                       int* err, cudaStream_t s, const int* skip, int KA) {
   switch (pick_bn(N)) {
-    case 64: return launch_bn<64>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
-    case 80: return launch_bn<80>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
-    case 96: return launch_bn<96>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
-    case 112: return launch_bn<112>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
-    default: return launch_bn<128>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip);
+    case 64: return launch_bn<64>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip, KA);
+    case 80: return launch_bn<80>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip, KA);
+    case 96: return launch_bn<96>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip, KA);
+    case 112: return launch_bn<112>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip, KA);
+    default: return launch_bn<128>(A, B, D, M, N, K, batch, sA, sB, ldd, sD, slabs, err, s, skip, KA);
   }
 }
 
@@ -731,11 +731,12 @@ int bs_launch_slice_gemm(const uint16_t* A, const uint16_t* B, float* D, int M, 
   one.order[0] = 0;
   one.a0[0] = one.b0[0] = 0;
   one.len[0] = K;
-  return dispatch_bn(A, B, D, M, N, K, batch, sA, sB, ldd, sD, one, err, s, nullptr);
+  return dispatch_bn(A, B, D, M, N, K, batch, sA, sB, ldd, sD, one, err, s, nullptr, K);
 }
 
 int bs_launch_slice_orders(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int S,
-                           int Kp, int batch, int* err, cudaStream_t s, const int* skip) {
+                           int Kp, int batch, int* err, cudaStream_t s, const int* skip,
+                           int SA) {
   SliceSlabs sl;
   if (Kp % 64 != 0 || S < 1 || ((uintptr_t)A & 15) || ((uintptr_t)B & 15) || M < 1 || N < 1 ||
       batch < 1 || !bs_slice_slabs(S, Kp, M, N, batch, &sl) || (long)batch * sl.nq > 65535) {
@@ -743,9 +744,9 @@ int bs_launch_slice_orders(const uint16_t* A, const uint16_t* B, float* D, int M
                  BS_SLAB_MAX);
     return BS_EINVAL;
   }
-  const int K = S * Kp;
-  return dispatch_bn(A, B, D, M, N, K, batch, (long)M * K, (long)N * K, M, (long)M * N, sl, err,
-                     s, skip);
+  const int K = S * Kp, KA = (SA ? SA : S) * Kp;
+  return dispatch_bn(A, B, D, M, N, K, batch, (long)M * KA, (long)N * K, M, (long)M * N, sl, err,
+                     s, skip, KA);
 }
 
 // A22 (m x m at offset o of each n x n matrix) -= X Y^dagger from the digit
