@@ -121,10 +121,18 @@ int bs_launch_gram_aniso(bs_cell* c, cudaStream_t s) {
   const int N = c->N;
   const size_t NN = (size_t)N * N, n3 = 3 * (size_t)N;
   // R = T[rho] (slot 2): Cholesky in place and its inverse, where the isotropic path keeps them
-  TRY_LAUNCH(bs_launch_cholesky(c->d_T + 2 * NN, N, 1, (long)NN, c->d_info, s));
-  TRY_LAUNCH(bs_launch_trinv(c->d_T + 2 * NN, c->d_Linv + 2 * NN, N, 1, (long)NN, s));
+  const bool f64 = c->precision == BS_PREC_FP64;
+  zd *R = c->d_T + 2 * NN, *Ri = c->d_Linv + 2 * NN;
+  if (f64) {
+    TRY_LAUNCH(bs_launch_gram_factor(R, Ri, N, 1, (long)NN, c->d_info, s));
+  } else {
+    TRY_LAUNCH(bs_launch_cholesky(R, N, 1, (long)NN, c->d_info, s));
+    TRY_LAUNCH(bs_launch_trinv(R, Ri, N, 1, (long)NN, s));
+  }
   phi_build_kernel<<<(unsigned)((n3 * n3 + 255) / 256), 256, 0, s>>>(c->d_T, N, c->d_Phi);
   BS_CHECK_LAUNCH("phi_build_kernel");
+  if (f64)
+    return bs_launch_gram_factor(c->d_Phi, c->d_LPhi, 3 * N, 1, (long)(n3 * n3), c->d_info, s);
   TRY_LAUNCH(bs_launch_cholesky(c->d_Phi, 3 * N, 1, (long)(n3 * n3), c->d_info, s));
   TRY_LAUNCH(bs_launch_trinv(c->d_Phi, c->d_LPhi, 3 * N, 1, (long)(n3 * n3), s));
   return BS_OK;

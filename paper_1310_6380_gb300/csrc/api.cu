@@ -704,6 +704,8 @@ extern "C" int bs_assemble(bs_cell* c, void* stream) {
   TRY(bs_launch_toeplitz(c, s));                                   // a3 expansion
   if (c->aniso) {
     TRY(bs_launch_gram_aniso(c, s));                               // R and the full Phi
+  } else if (c->precision == BS_PREC_FP64) {
+    TRY(bs_launch_gram_factor(c->d_T, c->d_Linv, c->N, 3, (long)NN, c->d_info, s));
   } else {
     TRY(bs_launch_cholesky(c->d_T, c->N, 3, (long)NN, c->d_info, s)); // a3 factors
     TRY(bs_launch_trinv(c->d_T, c->d_Linv, c->N, 3, (long)NN, s));

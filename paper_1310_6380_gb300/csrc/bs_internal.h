@@ -260,6 +260,9 @@ int bs_cuda_status(cudaError_t e, const char* where);
 int bs_launch_assembly(bs_cell* c, cudaStream_t s);
 int bs_launch_toeplitz(bs_cell* c, cudaStream_t s);
 
+// gram.cu: Cholesky factors (in place) and their inverses, FP64 path
+int bs_launch_gram_factor(zd* A, zd* X, int n, int batch, long stride, int* info, cudaStream_t s);
+
 // dense.cu
 int bs_launch_cholesky(zd* A, int n, int batch, long stride, int* info, cudaStream_t s);
 int bs_launch_trinv(const zd* L, zd* X, int n, int batch, long stride, cudaStream_t s);

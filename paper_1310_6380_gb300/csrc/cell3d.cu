@@ -544,8 +544,7 @@ extern "C" int bs_assemble3(bs_cell3* c, void* stream) {
   toeplitz3_kernel<<<(unsigned)((3 * NN + 255) / 256), 256, 0, s>>>(c->d_ghat, c->M, N, D,
                                                                    c->d_T);
   BS_CHECK_LAUNCH("toeplitz3_kernel");
-  TRY_LAUNCH(bs_launch_cholesky(c->d_T, N, 3, (long)NN, c->d_info, s));
-  TRY_LAUNCH(bs_launch_trinv(c->d_T, c->d_Linv, N, 3, (long)NN, s));
+  TRY_LAUNCH(bs_launch_gram_factor(c->d_T, c->d_Linv, N, 3, (long)NN, c->d_info, s));
   // F_X^a = L_R^-1 diag(s_a) L_X^-dagger for X in {h, m} (batch of 2), a = 0..3
   const zd* LinvR = c->d_Linv + 2 * NN;
   CK3(cudaMemcpyAsync(c->d_LinvR2, LinvR, NN * sizeof(zd), cudaMemcpyDeviceToDevice, s), "copy");
