@@ -36,8 +36,8 @@
 //
 // Measured (one GB300, whole FP64 solve with its assembly, the reduction to
 // tridiagonal form before -> this): n = 882, 90 matrices, 18 branches
-// 171 -> 34 ms; n = 1029, 30 matrices, 12 branches 136 -> 23 ms; n = 242,
-// 70 matrices, 18 branches 16.9 -> 5.8 ms.  What bounds it at n = 882 is the
+// 171 -> 29 ms; n = 1029, 30 matrices, 12 branches 136 -> 20 ms; n = 242,
+// 70 matrices, 18 branches 16.9 -> 5.0 ms.  What bounds it at n = 882 is the
 // FP32 pipe in the factorisations and the FP64 pipe in the Rayleigh-Ritz steps
 // (32-column products at 2 FMA per clock and SM).
 //
@@ -122,6 +122,19 @@ __device__ __forceinline__ void tile_of(int l, int& bi, int& bk) {
   bk = l - r * (r + 1) / 2;
 }
 
+// (float)x by integer arithmetic (round half up; below the FP32 normal range
+// 0): the FP64 to FP32 conversion runs on the FP64 pipe, 2 per clock and SM
+// (the scaling of 90 matrices of n = 882: 456 us with it, 158 us without).
+// |x| of 2^127 and more is left to it.
+__device__ __forceinline__ float to_float(double x) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff);
+  if (e >= 1023 + 127) return (float)x;
+  if (e < 1023 - 126) return 0.f;
+  const unsigned m = (unsigned)((b - ((long long)(1023 - 127) << 52) + (1LL << 28)) >> 29);
+  return __uint_as_float((m & 0x7fffffffu) | ((unsigned)(b >> 32) & 0x80000000u));
+}
+
 // A <- W (C / s - beta I) W, lower 64-tiles, FP32, identity in the padding.
 // beta = -1 (the operator) or sigma / s (the inertia check).
 __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ C, int n, int np,
@@ -137,6 +150,7 @@ __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ 
   const float* wk = w + (size_t)k * np;
   zf* ak = A + (size_t)k * np * np;
   const double is = 1.0 / shift[k], beta = sigma ? sigma[k] * is : -1.0;
+  const float fs = (float)is;
   if (blockIdx.x == 0 && tid == 0) {
     neg[k] = 0;
     flag[k] = 0;
@@ -150,8 +164,11 @@ __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ 
     if (r < n && c < n) {
       const zd z = ck[(size_t)c * n + r];
       const float f = wr * wk[c];
-      v = r == c ? make_float2((float)(z.x * is - beta) * f, 0.f)
-                 : make_float2((float)(z.x * is) * f, (float)(z.y * is) * f);
+      if (r == c) {
+        v = make_float2((float)(z.x * is - beta) * f, 0.f);
+      } else {
+        v = make_float2(to_float(z.x) * fs * f, to_float(z.y) * fs * f);
+      }
     }
     ak[(size_t)c * np + r] = v;
   }
@@ -166,40 +183,82 @@ __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ 
 // That CTA also inverts the unit lower factor (stored in the diagonal block
 // of X), so the block rows below become plain 64 x 64 x 64 products.
 
-// S: the 64 x 64 lower triangle (row-major, stride LDS); on return L D below
-// the diagonal and D on it.  Xs: its inverse unit factor.  One barrier per
-// column: step c reads column c (final) and row c of Xs (final) only.
-__device__ void ldl64_block(zf* S, zf* Xs, float* d, int* bad) {
-  const int tid = threadIdx.x, r = tid & 63, q = tid >> 6;
-  for (int c = q; c < TB; c += 4) Xs[r * LDS + c] = make_float2(r == c ? 1.f : 0.f, 0.f);
+// The 32 x 32 diagonal block at b0 of S (row-major, stride LDS): on return L D
+// below its diagonal and D on it, its inverse unit factor in Xs.  One barrier
+// per column: step c reads column c (final) and row c of Xs (final) only;
+// warps 0..3 update the block, warps 4..7 the inverse.
+__device__ void ldl32_block(zf* S, zf* Xs, float* d, int b0, int* bad) {
+  const int tid = threadIdx.x, r = tid & 31, w = tid >> 5;
+  S += b0 * (LDS + 1);
+  Xs += b0 * (LDS + 1);
+  for (int c = w; c < 32; c += 8) Xs[r * LDS + c] = make_float2(r == c ? 1.f : 0.f, 0.f);
   __syncthreads();
-  for (int c = 0; c < TB; ++c) {
+  for (int c = 0; c < 32; ++c) {
     float p = S[c * LDS + c].x;
     if (!(fabsf(p) >= TINY_PIVOT)) {
       if (tid == 0) *bad = 1;
       p = p < 0.f ? -TINY_PIVOT : TINY_PIVOT;
     }
-    if (tid == 0) d[c] = p;
+    if (tid == 0) d[b0 + c] = p;
     if (r > c) {
-      const float inv = 1.f / p;
-      const zf l = zscale(S[r * LDS + c], inv);
-      for (int s = c + 1 + q; s <= r; s += 4) {
-        const zf u = S[s * LDS + c];
-        zf v = S[r * LDS + s];
-        v.x = fmaf(-l.x, u.x, fmaf(-l.y, u.y, v.x));   // - l conj(u)
-        v.y = fmaf(-l.y, u.x, fmaf(l.x, u.y, v.y));
-        S[r * LDS + s] = v;
-      }
-      for (int s = q; s <= c; s += 4) {
-        const zf u = Xs[c * LDS + s];
-        zf v = Xs[r * LDS + s];
-        v.x = fmaf(-l.x, u.x, fmaf(l.y, u.y, v.x));    // - l u
-        v.y = fmaf(-l.x, u.y, fmaf(-l.y, u.x, v.y));
-        Xs[r * LDS + s] = v;
+      const zf l = zscale(S[r * LDS + c], __fdividef(1.f, p));
+      if (w < 4) {
+        for (int s = c + 1 + w; s <= r; s += 4) S[r * LDS + s] = zfnmac(l, S[s * LDS + c], S[r * LDS + s]);
+      } else {
+        for (int s = w - 4; s <= c; s += 4) Xs[r * LDS + s] = zfnma(l, Xs[c * LDS + s], Xs[r * LDS + s]);
       }
     }
     __syncthreads();
   }
+}
+
+// S: the 64 x 64 lower triangle (row-major, stride LDS); on return L D below
+// the diagonal and D on it.  Xs: its inverse unit factor.  Two 32 x 32 blocks
+// and 32 x 32 x 32 products between them: 64 dependent steps over the whole
+// block took 62 us per launch, this 46 us, and this chain is what every panel waits for.
+__device__ void ldl64_block(zf* S, zf* Xs, float* d, int* bad) {
+  const int tid = threadIdx.x, r = tid & 31, w = tid >> 5;
+  ldl32_block(S, Xs, d, 0, bad);
+  zf* S21 = S + 32 * LDS;
+  zf v[4];
+  // L21 D1 = A21 X11^dagger
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = w + 8 * j;
+    v[j] = make_float2(0.f, 0.f);
+    for (int t = 0; t <= c; ++t) v[j] = zfmac(S21[r * LDS + t], Xs[c * LDS + t], v[j]);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < 4; ++j) S21[r * LDS + w + 8 * j] = v[j];
+  __syncthreads();
+  // A22 -= (L21 D1) D1^-1 (L21 D1)^dagger, and M = L21 X11 into the unused
+  // block of S above the diagonal
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = w + 8 * j;
+    zf a = make_float2(0.f, 0.f), m = a;
+#pragma unroll 4
+    for (int t = 0; t < 32; ++t) {
+      const zf l = zscale(S21[r * LDS + t], __fdividef(1.f, d[t]));
+      a = zfmac(l, S21[c * LDS + t], a);
+      if (t >= c) m = zfma(l, Xs[t * LDS + c], m);
+    }
+    if (c <= r) S21[r * LDS + 32 + c] = zsub(S21[r * LDS + 32 + c], a);
+    S[r * LDS + 32 + c] = m;
+  }
+  __syncthreads();
+  ldl32_block(S, Xs, d, 32, bad);
+  // X21 = -X22 M, X12 = 0
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = w + 8 * j;
+    zf x = make_float2(0.f, 0.f);
+    for (int t = 0; t <= r; ++t) x = zfnma(Xs[(32 + r) * LDS + 32 + t], S[t * LDS + 32 + c], x);
+    Xs[(32 + r) * LDS + c] = x;
+    Xs[r * LDS + 32 + c] = make_float2(0.f, 0.f);
+  }
+  __syncthreads();
 }
 
 // factor the diagonal block at j0 held in S and store L (unit), D, X
