@@ -36,8 +36,8 @@
 //
 // Measured (one GB300, whole FP64 solve with its assembly, the reduction to
 // tridiagonal form before -> this): n = 882, 90 matrices, 18 branches
-// 171 -> 29 ms; n = 1029, 30 matrices, 12 branches 136 -> 20 ms; n = 242,
-// 70 matrices, 18 branches 16.9 -> 5.0 ms.  What bounds it at n = 882 is the
+// 171 -> 27 ms; n = 1029, 30 matrices, 12 branches 136 -> 19 ms; n = 242,
+// 70 matrices, 18 branches 16.9 -> 4.3 ms.  What bounds it at n = 882 is the
 // FP32 pipe in the factorisations and the FP64 pipe in the Rayleigh-Ritz steps
 // (32-column products at 2 FMA per clock and SM).
 //
@@ -183,42 +183,105 @@ __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ 
 // That CTA also inverts the unit lower factor (stored in the diagonal block
 // of X), so the block rows below become plain 64 x 64 x 64 products.
 
-// The 32 x 32 diagonal block at b0 of S (row-major, stride LDS): on return L D
-// below its diagonal and D on it, its inverse unit factor in Xs.  One barrier
-// per column: step c reads column c (final) and row c of Xs (final) only;
-// warps 0..3 update the block, warps 4..7 the inverse.
-__device__ void ldl32_block(zf* S, zf* Xs, float* d, int b0, int* bad) {
-  const int tid = threadIdx.x, r = tid & 31, w = tid >> 5;
-  S += b0 * (LDS + 1);
-  Xs += b0 * (LDS + 1);
-  for (int c = w; c < 32; c += 8) Xs[r * LDS + c] = make_float2(r == c ? 1.f : 0.f, 0.f);
+// 1 / p by the hardware approximation and, in FP64, one cubic correction
+// (1 + e + e^2, e = 1 - p r below 2^-22; plain division outside the FP32 range)
+__device__ __forceinline__ float quick_rcp(float p) { return __fdividef(1.f, p); }
+__device__ __forceinline__ double quick_rcp(double p) {
+  if (!(p > 1e-36 && p < 1e36)) return 1.0 / p;
+  float rf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"((float)p));
+  const double r = (double)rf, e = fma(-p, r, 1.0);
+  return fma(fma(e, e, e), r, r);
+}
+
+// LDL^dagger of the 32 x 32 lower triangle S and its inverse unit factor X (row
+// strides LD; X's strict upper part is not written), 256 threads: on return
+// L D below the diagonal of S, the pivots on it and 1 / pivot in pinv.  ok(p, c)
+// passes a pivot or replaces it.  Thread t owns up to three entries (r, s) of
+// the lower triangle: step c < s updates S[r][s] -= l conj(S[s][c]), step
+// c >= s X[r][s] -= l X[c][s] (kept in a register until row r is next), so the
+// three are independent, loads need no branches, and rows that are done leave
+// the pipe (FP64 issues a warp in 16 cycles).  One barrier per step; the
+// thread that finishes a pivot inverts it, so no other issues a division.
+template <typename R, int LD, typename Ok>
+__device__ __forceinline__ void ldl32_inverse(typename Cplx<R>::T* S, typename Cplx<R>::T* X,
+                                              R* pinv, Ok ok) {
+  typedef typename Cplx<R>::T T;
+  const int tid = threadIdx.x;
+  int er[3], es[3];
+  T x[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int e = tid + 256 * q;
+    int r = 0, c = 0;   // (0, 0) is never updated
+    if (e < 32 * 33 / 2) tile_of(e, r, c);
+    er[q] = r;
+    es[q] = c;
+    x[q] = Cplx<R>::make(r == c ? (R)1 : (R)0, (R)0);
+    X[r * LD + c] = x[q];
+  }
+  if (tid == 0) {
+    const R p = ok(S[0].x, 0);
+    S[0] = Cplx<R>::make(p, (R)0);
+    pinv[0] = quick_rcp(p);
+  }
   __syncthreads();
   for (int c = 0; c < 32; ++c) {
-    float p = S[c * LDS + c].x;
-    if (!(fabsf(p) >= TINY_PIVOT)) {
-      if (tid == 0) *bad = 1;
-      p = p < 0.f ? -TINY_PIVOT : TINY_PIVOT;
+    T l[3], u[3], v[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int r = er[q], s = es[q];
+      const bool f = s > c;
+      l[q] = S[r * LD + c];
+      const T* up = f ? S + s * LD + c : X + c * LD + s;
+      u[q] = *up;
+      const T sv = S[r * LD + s];
+      v[q] = f ? sv : x[q];
+      u[q].y = f ? -u[q].y : u[q].y;
     }
-    if (tid == 0) d[b0 + c] = p;
-    if (r > c) {
-      const zf l = zscale(S[r * LDS + c], __fdividef(1.f, p));
-      if (w < 4) {
-        for (int s = c + 1 + w; s <= r; s += 4) S[r * LDS + s] = zfnmac(l, S[s * LDS + c], S[r * LDS + s]);
+    const R inv = pinv[c];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int r = er[q], s = es[q];
+      if (r <= c) continue;
+      T w = zfnma(zscale(l[q], inv), u[q], v[q]);
+      if (s > c) {
+        if (s == c + 1 && r == s) {
+          const R p = ok(w.x, r);
+          w = Cplx<R>::make(p, (R)0);
+          pinv[r] = quick_rcp(p);
+        }
+        S[r * LD + s] = w;
       } else {
-        for (int s = w - 4; s <= c; s += 4) Xs[r * LDS + s] = zfnma(l, Xs[c * LDS + s], Xs[r * LDS + s]);
+        x[q] = w;
+        if (r == c + 1) X[r * LD + s] = w;   // the row is final: the next steps read it
       }
     }
     __syncthreads();
   }
 }
 
+// The 32 x 32 diagonal block at b0 of the 64 x 64 block: see ldl32_inverse
+__device__ __forceinline__ void ldl32_block(zf* S, zf* Xs, float* d, float* pinv, int b0, int* bad) {
+  ldl32_inverse<float, LDS>(S + b0 * (LDS + 1), Xs + b0 * (LDS + 1), pinv + b0,
+                       [&](float p, int c) {
+                         if (!(fabsf(p) >= TINY_PIVOT)) {
+                           *bad = 1;
+                           p = p < 0.f ? -TINY_PIVOT : TINY_PIVOT;
+                         }
+                         d[b0 + c] = p;
+                         return p;
+                       });
+}
+
 // S: the 64 x 64 lower triangle (row-major, stride LDS); on return L D below
 // the diagonal and D on it.  Xs: its inverse unit factor.  Two 32 x 32 blocks
 // and 32 x 32 x 32 products between them: 64 dependent steps over the whole
-// block took 62 us per launch, this 46 us, and this chain is what every panel waits for.
-__device__ void ldl64_block(zf* S, zf* Xs, float* d, int* bad) {
+// block took 62 us per launch, this 39 us, and this chain is what every panel waits for.
+__device__ __forceinline__ void ldl64_block(zf* S, zf* Xs, float* d, int* bad) {
+  __shared__ float pinv[TB];
   const int tid = threadIdx.x, r = tid & 31, w = tid >> 5;
-  ldl32_block(S, Xs, d, 0, bad);
+  ldl32_block(S, Xs, d, pinv, 0, bad);
   zf* S21 = S + 32 * LDS;
   zf v[4];
   // L21 D1 = A21 X11^dagger
@@ -240,7 +303,7 @@ __device__ void ldl64_block(zf* S, zf* Xs, float* d, int* bad) {
     zf a = make_float2(0.f, 0.f), m = a;
 #pragma unroll 4
     for (int t = 0; t < 32; ++t) {
-      const zf l = zscale(S21[r * LDS + t], __fdividef(1.f, d[t]));
+      const zf l = zscale(S21[r * LDS + t], pinv[t]);
       a = zfmac(l, S21[c * LDS + t], a);
       if (t >= c) m = zfma(l, Xs[t * LDS + c], m);
     }
@@ -248,7 +311,7 @@ __device__ void ldl64_block(zf* S, zf* Xs, float* d, int* bad) {
     S[r * LDS + 32 + c] = m;
   }
   __syncthreads();
-  ldl32_block(S, Xs, d, 32, bad);
+  ldl32_block(S, Xs, d, pinv, 32, bad);
   // X21 = -X22 M, X12 = 0
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -262,7 +325,7 @@ __device__ void ldl64_block(zf* S, zf* Xs, float* d, int* bad) {
 }
 
 // factor the diagonal block at j0 held in S and store L (unit), D, X
-__device__ void ldl64_diag(zf* a, zf* x, float* dk, int np, int j0, int k, zf* S, zf* Xs, float* d,
+__device__ __forceinline__ void ldl64_diag(zf* a, zf* x, float* dk, int np, int j0, int k, zf* S, zf* Xs, float* d,
                            int* bad, int* neg, int* flag) {
   const int tid = threadIdx.x, r = tid & 63;
   if (tid == 0) *bad = 0;
@@ -561,8 +624,13 @@ __device__ __forceinline__ void rr_load(RrSmem<R>& sm, const zd* X, const zd* CX
     T x = Cplx<R>::make((R)0, (R)0), y = x;
     if (r0 + r < n) {
       const zd a = X[(size_t)c * n + r0 + r], b = CX[(size_t)c * n + r0 + r];
-      x = Cplx<R>::make((R)a.x, (R)a.y);
-      y = Cplx<R>::make((R)b.x, (R)b.y);
+      if constexpr (sizeof(R) == 8) {
+        x = a;
+        y = b;
+      } else {
+        x = make_float2(to_float(a.x), to_float(a.y));
+        y = make_float2(to_float(b.x), to_float(b.y));
+      }
     }
     sm.X[r][c] = x;
     sm.Y[r][c] = y;
@@ -582,18 +650,18 @@ __global__ void __launch_bounds__(GT) filt_gram_kernel(const zd* __restrict__ X,
   typedef typename Cplx<R>::T T;
   RrSmem<R>& sm = *reinterpret_cast<RrSmem<R>*>(dsm);
   const int k = blockIdx.y, ch = blockIdx.x, tid = threadIdx.x;
-  rr_load(sm, X + (size_t)k * FB * n, CX + (size_t)k * FB * n, n, ch * GR, GT);
-  __syncthreads();
-  if (tid >= 272) return;
   const int mat = tid >= 136;
   int bi, bj;
-  tile_of(mat ? tid - 136 : tid, bi, bj);
+  tile_of(mat ? min(tid - 136, 135) : tid, bi, bj);
   T acc[2][2];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j) acc[i][j] = Cplx<R>::make((R)0, (R)0);
-  const int rows = min(GR, n - ch * GR);
+  const int r0 = ch * GR, rows = min(GR, n - r0);
+  rr_load(sm, X + (size_t)k * FB * n, CX + (size_t)k * FB * n, n, r0, GT);
+  __syncthreads();
+  if (tid >= 272) return;
 #pragma unroll 4
   for (int r = 0; r < rows; ++r) {
     const T a0 = sm.X[r][2 * bi], a1 = sm.X[r][2 * bi + 1];
@@ -612,8 +680,50 @@ __global__ void __launch_bounds__(GT) filt_gram_kernel(const zd* __restrict__ X,
       p[(2 * bi + i) * FB + 2 * bj + j] = zmake((double)acc[i][j].x, (double)acc[i][j].y);
 }
 
+// A real number as two FP32 terms, and acc += a b with it: the product's high
+// part exactly (one FMA gives its rounding), the cross terms, a two-sum.  48
+// bits at 11 FP32 operations, where an FP64 FMA costs 64 times an FP32 one.
+struct df {
+  float h, l;
+};
+// the upper 24 bits of the mantissa are an FP32 number as they stand, so one
+// FP64 subtraction is all that the split takes from the FP64 pipe
+__device__ __forceinline__ df df_of(double x) {
+  const double xh = __longlong_as_double(__double_as_longlong(x) & ~0x1FFFFFFFLL);
+  return {to_float(xh), to_float(x - xh)};
+}
+__device__ __forceinline__ void df_fma(df a, df b, df& acc) {
+  const float p = a.h * b.h;
+  const float e = fmaf(a.h, b.h, -p);
+  const float s = acc.h + p, bb = s - acc.h;
+  const float t = (acc.h - (s - bb)) + (p - bb);
+  acc.h = s;
+  acc.l += fmaf(a.h, b.l, fmaf(a.l, b.h, e + t));
+}
+__device__ __forceinline__ df df_neg(df a) { return {-a.h, -a.l}; }
+
+// operands of the rotation: FP32, or two FP32 terms (re, im) high, (re, im) low
+template <typename R> struct RotSmem;
+template <> struct RotSmem<float> {
+  zf W[FB][FB], X[FB][GR], Y[FB][GR];
+  static __device__ __forceinline__ void put(zf& o, zd v) {
+    o = make_float2(to_float(v.x), to_float(v.y));
+  }
+};
+template <> struct RotSmem<double> {
+  float4 W[FB][FB], X[FB][GR], Y[FB][GR];
+  static __device__ __forceinline__ void put(float4& o, zd v) {
+    const df a = df_of(v.x), b = df_of(v.y);
+    o = make_float4(a.h, b.h, a.l, b.l);
+  }
+};
+
 // X <- X W, the split of R / s = (C X W - X W Theta) / s (zero in the padding) and
-// the sums of its squares per column (one partial per warp of rows)
+// the sums of its squares per column (one partial per warp of rows).  R =
+// float: FP32 products; double: products in two FP32 terms (48 bits), which
+// leave 1e-14 of C X in a residual that is compared with 1e-12 of it; the
+// Ritz values themselves come from the FP64 Gram matrices.  (90 matrices of
+// n = 882: 1.19 ms in FP64, 0.43 ms so.)  A thread owns a row and eight columns.
 template <typename R>
 __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
                                                           const zd* __restrict__ CX, int n, int np,
@@ -624,54 +734,76 @@ __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
                                                           float* __restrict__ rpart,
                                                           const int* __restrict__ done) {
   if (done[blockIdx.y]) return;
+  constexpr bool D = sizeof(R) == 8;
   extern __shared__ __align__(16) unsigned char dsm[];
-  typedef typename Cplx<R>::T T;
-  RrSmem<R>& sm = *reinterpret_cast<RrSmem<R>*>(dsm);
-  T* Ws = reinterpret_cast<T*>(dsm + sizeof(RrSmem<R>));   // [l][c]
+  RotSmem<R>& sm = *reinterpret_cast<RotSmem<R>*>(dsm);
   const int k = blockIdx.y, ch = blockIdx.x, tid = threadIdx.x;
   zd* xk = X + (size_t)k * FB * n;
-  rr_load(sm, xk, CX + (size_t)k * FB * n, n, ch * GR, 256);
-  for (int e = tid; e < FB * FB; e += 256) {
-    const zd w = W[(size_t)k * FB * FB + e];   // column-major: l + c FB
-    Ws[(e % FB) * FB + e / FB] = Cplx<R>::make((R)w.x, (R)w.y);
+  const zd* yk = CX + (size_t)k * FB * n;
+  for (int e = tid; e < FB * FB; e += 256)   // column-major: l + c FB
+    RotSmem<R>::put(sm.W[e % FB][e / FB], W[(size_t)k * FB * FB + e]);
+  for (int e = tid; e < GR * FB; e += 256) {
+    const int l = e / GR, r = e % GR, row = ch * GR + r;
+    const bool ok = row < n;
+    RotSmem<R>::put(sm.X[l][r], ok ? xk[(size_t)l * n + row] : zmake(0.0, 0.0));
+    RotSmem<R>::put(sm.Y[l][r], ok ? yk[(size_t)l * n + row] : zmake(0.0, 0.0));
   }
   __syncthreads();
   const int r = tid & 63, c0 = (tid >> 6) * 8;
   const int row = ch * GR + r;
+  const bool live = row < n;
+  df xr[8], xi[8], yr[8], yi[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) xr[j] = xi[j] = yr[j] = yi[j] = {0.f, 0.f};
+#pragma unroll 2
+  for (int l = 0; l < FB; ++l) {
+    if constexpr (D) {
+      const float4 xv = sm.X[l][r], yv = sm.Y[l][r];
+      const df ax = {xv.x, xv.z}, bx = {xv.y, xv.w}, ay = {yv.x, yv.z}, by = {yv.y, yv.w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float4 w4 = sm.W[l][c0 + j];
+        const df wr = {w4.x, w4.z}, wi = {w4.y, w4.w};
+        df_fma(ax, wr, xr[j]);
+        df_fma(df_neg(bx), wi, xr[j]);
+        df_fma(ax, wi, xi[j]);
+        df_fma(bx, wr, xi[j]);
+        df_fma(ay, wr, yr[j]);
+        df_fma(df_neg(by), wi, yr[j]);
+        df_fma(ay, wi, yi[j]);
+        df_fma(by, wr, yi[j]);
+      }
+    } else {
+      const zf xv = sm.X[l][r], yv = sm.Y[l][r];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const zf w = sm.W[l][c0 + j];
+        xr[j].h = fmaf(xv.x, w.x, fmaf(-xv.y, w.y, xr[j].h));
+        xi[j].h = fmaf(xv.x, w.y, fmaf(xv.y, w.x, xi[j].h));
+        yr[j].h = fmaf(yv.x, w.x, fmaf(-yv.y, w.y, yr[j].h));
+        yi[j].h = fmaf(yv.x, w.y, fmaf(yv.y, w.x, yi[j].h));
+      }
+    }
+  }
   const double is = 1.0 / shift[k];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {   // two passes of four columns
-    T xa[4], ya[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) xa[j] = ya[j] = Cplx<R>::make((R)0, (R)0);
-#pragma unroll 4
-    for (int l = 0; l < FB; ++l) {
-      const T xv = sm.X[r][l], yv = sm.Y[r][l];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const T w = Ws[l * FB + c0 + 4 * h + j];
-        xa[j] = zfma(xv, w, xa[j]);
-        ya[j] = zfma(yv, w, ya[j]);
-      }
+  for (int j = 0; j < 8; ++j) {
+    const int c = c0 + j;
+    const double t = theta[(size_t)k * FB + c];
+    zf rv = make_float2(0.f, 0.f);
+    if (live) {
+      const zd x = zmake((double)xr[j].h + (double)xr[j].l, (double)xi[j].h + (double)xi[j].l);
+      const zd y = zmake((double)yr[j].h + (double)yr[j].l, (double)yi[j].h + (double)yi[j].l);
+      xk[(size_t)c * n + row] = x;
+      rv = make_float2((float)(fma(-t, x.x, y.x) * is), (float)(fma(-t, x.y, y.y) * is));
     }
+    if (row < np)
+      bs_store_block_split(Rs + ((size_t)k * 2 * FB + 2 * c) * 4 * np + row, np, rv);
+    float q = rv.x * rv.x + rv.y * rv.y;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = c0 + 4 * h + j;
-      const double t = theta[(size_t)k * FB + c];
-      zf rv = make_float2(0.f, 0.f);
-      if (row < n) {
-        xk[(size_t)c * n + row] = zmake((double)xa[j].x, (double)xa[j].y);
-        rv = make_float2((float)(((double)ya[j].x - t * (double)xa[j].x) * is),
-                         (float)(((double)ya[j].y - t * (double)xa[j].y) * is));
-      }
-      if (row < np)
-        bs_store_block_split(Rs + ((size_t)k * 2 * FB + 2 * c) * 4 * np + row, np, rv);
-      float q = rv.x * rv.x + rv.y * rv.y;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-      if ((tid & 31) == 0)
-        rpart[(((size_t)k * gridDim.x + ch) * 2 + ((tid >> 5) & 1)) * FB + c] = q;
-    }
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if ((tid & 31) == 0)
+      rpart[(((size_t)k * gridDim.x + ch) * 2 + ((tid >> 5) & 1)) * FB + c] = q;
   }
 }
 
@@ -687,7 +819,9 @@ __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
 // (90 matrices of n = 882).  Thread (u, v) applies both
 // sides' rotations to the 2 x 2 block of the index pairs u, v (the blocks
 // partition the matrix) from one copy of A to the other and rotates V's
-// columns of pair v in rows u and u + 16: one barrier per round.
+// columns of pair v in rows u and u + 16: one barrier per round, a lane
+// computes the rotation of its v and takes that of its u from the lane with
+// that v.
 struct JacobiSmem {
   zf A[2][FB][FB + 1], V[FB][FB + 1];
   float2 D[2][FB];   // diagonal, hi + lo
@@ -702,6 +836,17 @@ __device__ __forceinline__ float2 dd_add(float2 a, float x) {
   return make_float2(h, e - (h - s));
 }
 
+__device__ __forceinline__ float frsqrt(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float frcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // rotation of the pair with off-diagonal entry c and diagonal difference
 // dq - dp: cs, sn, the phase c / |c| and the shift t |c|
 __device__ __forceinline__ void rotation(zf c, float diff, float skip, float& cs, float& sn, zf& ph,
@@ -710,22 +855,22 @@ __device__ __forceinline__ void rotation(zf c, float diff, float skip, float& cs
   cs = 1.f;
   sn = shift = 0.f;
   ph = make_float2(1.f, 0.f);
+  const float ica = frsqrt(c2), ca = c2 * ica;
+  const float zeta = 0.5f * diff * ica, az = fabsf(zeta);
+  // t = 1 / (|zeta| + sqrt(1 + zeta^2)); for large zeta 1 / (2 |zeta|)
+  const float z2 = 1.f + az * az;
+  float t = frcp(az > 1e4f ? 2.f * az : az + z2 * frsqrt(z2));
+  t = copysignf(t, zeta);
   if (c2 > skip) {
-    const float ica = rsqrtf(c2), ca = c2 * ica;
     ph = make_float2(c.x * ica, c.y * ica);
-    const float zeta = 0.5f * diff * ica, az = fabsf(zeta);
-    // t = 1 / (|zeta| + sqrt(1 + zeta^2)), for large zeta without its square
-    float t = az > 1e4f ? __fdividef(0.5f, az)
-                        : __fdividef(1.f, az + (1.f + az * az) * rsqrtf(1.f + az * az));
-    t = copysignf(t, zeta);
-    cs = rsqrtf(1.f + t * t);
+    cs = frsqrt(1.f + t * t);
     sn = t * cs;
     shift = t * ca;
   }
 }
 
 // returns the copy of D that holds the result
-__device__ int jacobi32(JacobiSmem& sm, float offtol, int maxsweep) {
+__device__ __forceinline__ int jacobi32(JacobiSmem& sm, float offtol, int maxsweep) {
   const int tid = threadIdx.x, u = tid >> 4, v = tid & 15;
   int cur = 0;
   for (int sweep = 0; sweep < maxsweep; ++sweep) {
@@ -767,41 +912,43 @@ __device__ int jacobi32(JacobiSmem& sm, float offtol, int maxsweep) {
       int pu, qu, pv, qv;
       pair(u, pu, qu);
       pair(v, pv, qv);
-      zf(*A)[FB + 1] = sm.A[cur];
+      const zf(*A)[FB + 1] = sm.A[cur];
       zf(*B)[FB + 1] = sm.A[cur ^ 1];
-      const float2 dpu = sm.D[cur][pu], dqu = sm.D[cur][qu];
-      const float2 dpv = sm.D[cur][pv], dqv = sm.D[cur][qv];
-      float cu, su, shu, cv, sv, shv;
-      zf fu, fv;
-      rotation(A[pu][qu], (dqu.x - dpu.x) + (dqu.y - dpu.y), skip, cu, su, fu, shu);
-      rotation(A[pv][qv], (dqv.x - dpv.x) + (dqv.y - dpv.y), skip, cv, sv, fv, shv);
+      // everything the round reads, before its stores
+      const zf apq = A[pv][qv];
+      const float2 dp = sm.D[cur][pv], dq = sm.D[cur][qv];
+      const zf a00 = A[pu][pv], a01 = A[pu][qv], a10 = A[qu][pv], a11 = A[qu][qv];
+      const zf v0p = sm.V[u][pv], v0q = sm.V[u][qv], v1p = sm.V[u + 16][pv], v1q = sm.V[u + 16][qv];
+      float cv, sv, shv;
+      zf fv;
+      rotation(apq, (dq.x - dp.x) + (dq.y - dp.y), skip, cv, sv, fv, shv);
+      // the rotation of pair u is that of the lane whose v is u
+      const float cu = __shfl_sync(0xffffffffu, cv, u), su = __shfl_sync(0xffffffffu, sv, u);
+      const zf fu = make_float2(__shfl_sync(0xffffffffu, fv.x, u), __shfl_sync(0xffffffffu, fv.y, u));
       fv = zconj(fv);
       // J = [[cs, sn], [-sn conj(ph), cs conj(ph)]] on columns (p, q); A <- J_u^dagger A J_v
+      const zf w0 = zmul(v0q, fv), w1 = zmul(v1q, fv);
+      sm.V[u][pv] = zsub(zscale(v0p, cv), zscale(w0, sv));
+      sm.V[u][qv] = zadd(zscale(v0p, sv), zscale(w0, cv));
+      sm.V[u + 16][pv] = zsub(zscale(v1p, cv), zscale(w1, sv));
+      sm.V[u + 16][qv] = zadd(zscale(v1p, sv), zscale(w1, cv));
       if (u == v) {
         // the pair itself: the shifted diagonal and a zero (or the skipped entry)
-        sm.D[cur ^ 1][pu] = dd_add(dpu, -shu);
-        sm.D[cur ^ 1][qu] = dd_add(dqu, shu);
-        const zf c = su != 0.f ? make_float2(0.f, 0.f) : A[pu][qu];
-        B[pu][qu] = c;
-        B[qu][pu] = zconj(c);
+        sm.D[cur ^ 1][pv] = dd_add(dp, -shv);
+        sm.D[cur ^ 1][qv] = dd_add(dq, shv);
+        const zf c = sv != 0.f ? make_float2(0.f, 0.f) : apq;
+        B[pv][qv] = c;
+        B[qv][pv] = zconj(c);
       } else {
-        const zf a00 = A[pu][pv], a01 = zmul(A[pu][qv], fv);
-        const zf a10 = zmul(A[qu][pv], fu), a11 = zmul(zmul(A[qu][qv], fv), fu);
-        const zf b00 = zsub(zscale(a00, cv), zscale(a01, sv));
-        const zf b01 = zadd(zscale(a00, sv), zscale(a01, cv));
-        const zf b10 = zsub(zscale(a10, cv), zscale(a11, sv));
-        const zf b11 = zadd(zscale(a10, sv), zscale(a11, cv));
+        const zf c01 = zmul(a01, fv), c10 = zmul(a10, fu), c11 = zmul(zmul(a11, fv), fu);
+        const zf b00 = zsub(zscale(a00, cv), zscale(c01, sv));
+        const zf b01 = zadd(zscale(a00, sv), zscale(c01, cv));
+        const zf b10 = zsub(zscale(c10, cv), zscale(c11, sv));
+        const zf b11 = zadd(zscale(c10, sv), zscale(c11, cv));
         B[pu][pv] = zsub(zscale(b00, cu), zscale(b10, su));
         B[pu][qv] = zsub(zscale(b01, cu), zscale(b11, su));
         B[qu][pv] = zadd(zscale(b00, su), zscale(b10, cu));
         B[qu][qv] = zadd(zscale(b01, su), zscale(b11, cu));
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int r = u + 16 * h;
-        const zf vp = sm.V[r][pv], vq = zmul(sm.V[r][qv], fv);
-        sm.V[r][pv] = zsub(zscale(vp, cv), zscale(vq, sv));
-        sm.V[r][qv] = zadd(zscale(vp, sv), zscale(vq, cv));
       }
       cur ^= 1;
       __syncthreads();
@@ -840,69 +987,56 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
   const T zero = Cplx<R>::make((R)0, (R)0);
   const int k = blockIdx.x, tid = threadIdx.x;
   if (tid == 0) bad = 0;
-  for (int e = tid; e < FB * FB; e += 256) {
-    const int r = e / FB, c = e % FB;
-    if (r < c) continue;
+  constexpr int NT2 = FB * (FB + 1) / 2;   // entries of a lower triangle
+  for (int e = tid; e < NT2; e += 256) {
+    int r, c;
+    tile_of(e, r, c);
     zd g = zmake(0.0, 0.0), h = g;
+    const zd* p = part + (size_t)k * nch * 2 * FB * FB + r * FB + c;
+#pragma unroll 4
     for (int q = 0; q < nch; ++q) {
-      const zd* p = part + ((size_t)k * nch + q) * 2 * FB * FB + e;
-      g = zadd(g, p[0]);
-      h = zadd(h, p[FB * FB]);
+      g = zadd(g, p[(size_t)q * 2 * FB * FB]);
+      h = zadd(h, p[(size_t)(q * 2 + 1) * FB * FB]);
     }
     if (r == c) g.y = h.y = 0.0;
     sm.G[r][c] = Cplx<R>::make((R)g.x, (R)g.y);
     sm.H[r][c] = Cplx<R>::make((R)h.x, (R)h.y);
-    sm.H[c][r] = Cplx<R>::make((R)h.x, (R)-h.y);
+    if (r == c) {
+      sc[r] = g.x > 0.0 ? (R)rsqrt((R)g.x) : (R)0;
+      out[r] = 0;
+    }
   }
   __syncthreads();
-  if (tid < FB) {
-    const R g = sm.G[tid][tid].x;
-    sc[tid] = g > (R)0 ? rsqrt(g) : (R)0;
-    out[tid] = 0;
-  }
-  __syncthreads();
-  for (int e = tid; e < FB * FB; e += 256) {
-    const int r = e / FB, c = e % FB;
+  for (int e = tid; e < NT2; e += 256) {
+    int r, c;
+    tile_of(e, r, c);
     const R f = sc[r] * sc[c];
-    if (r >= c) sm.G[r][c] = zscale(sm.G[r][c], f);
-    sm.H[r][c] = zscale(sm.H[r][c], f);
-    sm.Li[r][c] = Cplx<R>::make(r == c ? (R)1 : (R)0, (R)0);
-    sm.J.V[r][c] = make_float2(r == c ? 1.f : 0.f, 0.f);
+    sm.G[r][c] = zscale(sm.G[r][c], f);
+    const T h = zscale(sm.H[r][c], f);
+    sm.H[r][c] = h;
+    sm.H[c][r] = zconj(h);
+  }
+  for (int e = tid; e < FB * FB; e += 256)
+    sm.J.V[e / FB][e % FB] = make_float2(e / FB == e % FB ? 1.f : 0.f, 0.f);
+  __syncthreads();
+  // unit L and pivots: G = L D L^dagger, Li = L^-1, then scaled to the Cholesky factor's
+  ldl32_inverse<R, FB + 1>(&sm.G[0][0], &sm.Li[0][0], pinv, [&](R p, int c) {
+    if (!(p > kTiny)) {
+      bad = 1;
+      out[c] = 1;
+      p = (R)1;
+    }
+    return p;
+  });
+  if (tid == 0) fail[k] = bad;
+  if (tid < FB) pinv[tid] = sqrt(pinv[tid]);
+  __syncthreads();
+  for (int e = tid; e < NT2; e += 256) {
+    int r, c;
+    tile_of(e, r, c);
+    sm.Li[r][c] = zscale(sm.Li[r][c], pinv[r]);
   }
   __syncthreads();
-  {
-    // unit L and pivots: G = L D L^dagger; Li accumulates L^-1.  The lane that
-    // finishes a pivot also inverts it, so the other warps issue no division.
-    const int r = tid & 31, q = tid >> 5;
-    auto pivot = [&](int c) {
-      R p = sm.G[c][c].x;
-      if (!(p > kTiny)) {
-        bad = 1;
-        out[c] = 1;
-        p = (R)1;
-      }
-      pinv[c] = (R)1 / p;
-    };
-    if (tid == 0) pivot(0);
-    __syncthreads();
-    for (int c = 0; c < FB; ++c) {
-      if (r > c) {
-        const T l = zscale(sm.G[r][c], pinv[c]);
-        for (int s = c + 1 + q; s <= r; s += 8) sm.G[r][s] = zfnmac(l, sm.G[s][c], sm.G[r][s]);
-        if (q == 0 && r == c + 1) pivot(r);
-        for (int s = q; s <= c; s += 8) sm.Li[r][s] = zfnma(l, sm.Li[c][s], sm.Li[r][s]);
-      }
-      __syncthreads();
-    }
-    if (tid == 0) fail[k] = bad;
-    if (tid < FB) pinv[tid] = sqrt(pinv[tid]);
-    __syncthreads();
-    for (int e = tid; e < FB * FB; e += 256) {
-      const int rr = e / FB, c = e % FB;
-      sm.Li[rr][c] = rr >= c ? zscale(sm.Li[rr][c], pinv[rr]) : zero;
-    }
-    __syncthreads();
-  }
   // G <- Li H, then H <- (Li H) Li^dagger (lower triangle, mirrored)
   for (int e = tid; e < FB * FB; e += 256) {
     const int r = e / FB, c = e % FB;
@@ -911,9 +1045,9 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
     sm.G[r][c] = s;
   }
   __syncthreads();
-  for (int e = tid; e < FB * FB; e += 256) {
-    const int r = e / FB, c = e % FB;
-    if (r < c) continue;
+  for (int e = tid; e < NT2; e += 256) {
+    int r, c;
+    tile_of(e, r, c);
     T s = zero;
     for (int t = 0; t <= c; ++t) s = zfmac(sm.G[r][t], sm.Li[c][t], s);
     if (r == c) s.y = (R)0;
@@ -956,10 +1090,11 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
   __syncthreads();
   if (sizeof(R) == 8) {
     // G <- (3 I - V^dagger V) / 2, H <- V G, columns to unit length
-    for (int e = tid; e < FB * FB; e += 256) {
-      const int r = e / FB, c = e % FB;
-      if (r < c) continue;
+    for (int e = tid; e < NT2; e += 256) {
+      int r, c;
+      tile_of(e, r, c);
       T s = zero;
+#pragma unroll 8
       for (int t = 0; t < FB; ++t) s = zfmac(sm.V[t][c], sm.V[t][r], s);   // conj(V_tr) V_tc
       s = Cplx<R>::make((r == c ? (R)1.5 : (R)0) - (R)0.5 * s.x, r == c ? (R)0 : (R)-0.5 * s.y);
       sm.G[r][c] = s;
@@ -969,6 +1104,7 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
     for (int e = tid; e < FB * FB; e += 256) {
       const int r = e / FB, c = e % FB;
       T s = zero;
+#pragma unroll 8
       for (int t = 0; t < FB; ++t) s = zfma(sm.V[r][t], sm.G[t][c], s);
       sm.H[r][c] = s;
     }
@@ -1048,9 +1184,8 @@ __global__ void __launch_bounds__(128) filt_coef_kernel(const double* __restrict
   }
 }
 
-// Certificate of the last Rayleigh-Ritz step, one warp per matrix: the cut
-// (a gap of at least 2e-3 above a Ritz value i >= nb - 1, sigma in it) with the
-// smallest error sum; omega; sigma and the count it has to have (-1: the
+// Certificate of a Rayleigh-Ritz step, one warp per matrix: a cut (a gap of at
+// least 2e-3 above a Ritz value i >= nb - 1, sigma in it) whose error sum is small; omega; sigma and the count it has to have (-1: the
 // sum is too large or there is no gap).  The inertia of the scaled matrix in
 // FP32 is exact for a matrix within a relative 1e-4 of C in the form sense
 // (n 2^-24 of the scaled diagonal, doubled), so rho is sigma less that.
@@ -1078,7 +1213,10 @@ __global__ void __launch_bounds__(128) filt_cert_kernel(
   }
   const bool usable = c >= nb - 1 && c < FB - 1 && gap >= 2e-3 * fmax(tn, 1e-3 * s) && rho > t &&
                       err >= 0.0;
-  double best = usable ? err : INFINITY;
+  // of the cuts whose sum is small enough the one with the widest gap (where
+  // the FP32 count is safest), else the one with the smallest sum
+  const double tol = 64.0 * DBL_EPSILON * cmax[k];
+  double best = !usable ? INFINITY : err <= tol ? -gap / at : err;
   int at_i = c;
   for (int o = 16; o > 0; o >>= 1) {
     const double e2 = __shfl_xor_sync(0xffffffffu, best, o);
@@ -1089,7 +1227,7 @@ __global__ void __launch_bounds__(128) filt_cert_kernel(
     }
   }
   const double sg = __shfl_sync(0xffffffffu, sig, at_i);
-  const bool ok = best <= 64.0 * DBL_EPSILON * cmax[k] && !fail[k];
+  const bool ok = best <= tol && !fail[k];
   if (c < nb) omega[(size_t)k * nb + c] = sqrt(fmax(t, 0.0));
   if (c == 0) {
     done[k] = ok;
@@ -1219,10 +1357,9 @@ static int filter_attrs() {
       {(const void*)trinv64_kernel, (TB * TB + TB * LDS) * (int)sizeof(zf)},
       {(const void*)filt_operator_kernel, 2 * TB * LDS * (int)sizeof(zf)},
       {(const void*)filt_gram_kernel<double>, (int)sizeof(RrSmem<double>)},
-      {(const void*)filt_rotate_kernel<double>,
-       (int)(sizeof(RrSmem<double>) + FB * FB * sizeof(zd))},
       {(const void*)filt_gram_kernel<float>, (int)sizeof(RrSmem<float>)},
-      {(const void*)filt_rotate_kernel<float>, (int)(sizeof(RrSmem<float>) + FB * FB * sizeof(zf))},
+      {(const void*)filt_rotate_kernel<double>, (int)sizeof(RotSmem<double>)},
+      {(const void*)filt_rotate_kernel<float>, (int)sizeof(RotSmem<float>)},
       {(const void*)filt_eig_kernel<double>, (int)sizeof(EigSmem<double>)},
       {(const void*)filt_eig_kernel<float>, (int)sizeof(EigSmem<float>)},
   };
@@ -1266,16 +1403,14 @@ template <typename R>
 static int filter_ritz(FilterWs& w, int n, int np, int kf, cudaStream_t s) {
   const int nch = (n + GR - 1) / GR;
   int *fail = w.iw + 4 * w.kf + 1, *done = fail + w.kf;
-  filt_gram_kernel<R><<<dim3(nch, kf), GT, sizeof(RrSmem<R>), s>>>(w.Xb, w.CX, n, w.part,
-                                                                      done);
+  filt_gram_kernel<R><<<dim3(nch, kf), GT, sizeof(RrSmem<R>), s>>>(w.Xb, w.CX, n, w.part, done);
   BS_CHECK_LAUNCH("filt_gram_kernel");
   filt_eig_kernel<R><<<kf, 256, sizeof(EigSmem<R>), s>>>(w.part, nch, w.theta, w.W,
                                                          fail, done);
   BS_CHECK_LAUNCH("filt_eig_kernel");
   // the rotation covers the padded rows as well (np <= nch GR)
-  filt_rotate_kernel<R><<<dim3(nch, kf), 256,
-                          sizeof(RrSmem<R>) + FB * FB * sizeof(typename Cplx<R>::T), s>>>(
-      w.Xb, w.CX, n, np, w.W, w.theta, w.shift, w.vs, w.rpart, done);
+  filt_rotate_kernel<R><<<dim3(nch, kf), 256, sizeof(RotSmem<R>), s>>>(w.Xb, w.CX, n, np, w.W, w.theta, w.shift,
+                                                       w.vs, w.rpart, done);
   BS_CHECK_LAUNCH("filt_rotate_kernel");
   return BS_OK;
 }
