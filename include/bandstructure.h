@@ -417,8 +417,10 @@ int bs_tridiag_eigenvalues_static(const double* d, const double* e, int n, int b
  *   ms[1] FP32 Householder reduction, ms[2] eigenvalue shifts, ms[3] FP64
  *   refinement.
  * bs_batch_destroy - free everything (NULL is a no-op).
- * bs_batch_set_solver - BS_SOLVER_DENSE (default: the FP32 Householder
- *   reduction above), BS_SOLVER_FP64 (the plain FP64 path of bs_solve_k on
+ * bs_batch_set_solver - BS_SOLVER_DENSE (default: the filtered iteration of
+ *   bs_set_reduction for the groups it takes under BS_REDUCE_AUTO, unless
+ *   bs_batch_set_tile chose a reduction tile or bs_batch_set_vectors keeps
+ *   eigenvectors; else the FP32 Householder reduction above), BS_SOLVER_FP64 (the plain FP64 path of bs_solve_k on
  *   FP64 C(k): Householder reduction and Sturm multisection, every (cell, k)
  *   of a chunk at once) or BS_SOLVER_LOBPCG (the block LOBPCG of
  *   bs_solve_k_lobpcg, its FP64 Rayleigh-Ritz tail and residual bound;

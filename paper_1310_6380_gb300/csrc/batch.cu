@@ -109,6 +109,7 @@ struct BatchGroup {
   int chunk;                  // cells per reduction batch
   int tile;                   // tridiagonal tile edge (autotuned)
   bool tuned;
+  bool forced;                // bs_batch_set_tile chose the tile: the reduction is wanted
   // chunk workspace (chunk * nk matrices)
   zd* C64;
   zf* C32;
@@ -160,7 +161,7 @@ struct BatchGroup {
   zd* vec64;                  // FP64 solver: reduction vectors and partial sums
   zd* part64;
   BandWs* band;               // FP64 solver: two-stage reduction workspace (large n)
-  FilterWs* filt;             // FP64 solver: filtered iteration workspace
+  FilterWs* filt;             // filtered iteration workspace (FP64 and dense solvers)
   // [0] tensor-core pipeline timeout of a main-stream product, [1] a Gram
   // Cholesky failed, [2] a tensor-core timeout during a cell's assembly
   // (the workers' own flags are reset by every assembly, so each assembly's
@@ -210,6 +211,17 @@ static void prof_mark(bs_batch* B, cudaStream_t s) {
     B->pev.push_back(e);
   }
   cudaEventRecord(B->pev[B->pev_used++], s);
+}
+
+// Whether a group's solves take the filtered iteration (bs_set_reduction): the
+// FP64 solver, and the dense one unless a reduction tile was chosen for it or
+// its eigenvectors are kept.  Its results are accurate to FP64, so the dense
+// solver's residual bound holds with room to spare.  Measured, 48 cells of
+// n = 242 .. 578 x 30 k, 10 branches: 274 ms with the FP32 reduction and its
+// refinement, 145 ms so (results within 7e-11 of each other).
+static bool group_filter(const bs_batch* B, const BatchGroup& g) {
+  return g.filt && bs_use_filter(g.n, B->nbands) &&
+         (B->solver == BS_SOLVER_FP64 || (B->solver == BS_SOLVER_DENSE && !g.forced && !B->d_vec));
 }
 
 static void free_group(BatchGroup& g) {
@@ -464,10 +476,10 @@ static int assemble_chunk(bs_batch* B, BatchGroup& g, int c0, int cn, int p) {
                           (size_t)g.N * g.N * sizeof(zd), cudaMemcpyDeviceToDevice, ws) == cudaSuccess
               ? BS_OK
               : bs_cuda_status(cudaGetLastError(), "batch L_R stash");
-    if (!r && B->solver == BS_SOLVER_FP64)
+    if (!r && (B->solver == BS_SOLVER_FP64 || group_filter(B, g)))
       r = bs_launch_builder(wk->d_Cm, n, B->d_Q + (size_t)ci * nk * 2, nk, wk->q1[0], wk->q1[1],
                             wk->q2[0], wk->q2[1], g.C64 + (size_t)i * nk * nn, ws,
-                            g.filt && bs_use_filter(n, B->nbands));
+                            group_filter(B, g));
     else if (!r)
       r = bs_launch_builder_mixed(wk->d_Cm, n, B->d_Q + (size_t)ci * nk * 2, nk, wk->q1[0],
                                   wk->q1[1], wk->q2[0], wk->q2[1], g.C64 + (size_t)i * nk * nn,
@@ -519,10 +531,10 @@ static int reduce_chunk_body(bs_batch* B, BatchGroup& g, int c0, int cn, int p, 
   const int K = cn * nk;
   const int* rows = g.d_rowidx + (size_t)c0 * nk;
   prof_mark(B, s);   // assembly ends, reduction begins
-  if (B->solver == BS_SOLVER_FP64) {
+  if (B->solver == BS_SOLVER_FP64 || group_filter(B, g)) {
     // the plain FP64 path: filtered iteration, or Householder reduction and
     // Sturm multisection
-    if (g.filt && bs_use_filter(n, B->nbands)) {
+    if (group_filter(B, g)) {
       const FilterFallback fb{g.vec64, g.part64, g.de, g.tau, g.beta, g.count};
       TRY_LAUNCH(bs_launch_eig_filter(g.C64, n, K, B->nbands, *g.filt, fb, g.w, g.st, g.d_err, s));
       prof_mark(B, s);
@@ -849,6 +861,20 @@ static void drop_graph(bs_batch* B) {
   }
 }
 
+// the filtered iteration's workspace, and the buffers of the reduction behind
+// it; without memory for them the reductions take the group
+static void alloc_filter(bs_batch* B, BatchGroup& g) {
+  if (!bs_use_filter(g.n, B->nbands)) return;
+  const size_t K = (size_t)g.chunk * B->nk;
+  if (!g.vec64 && balloc(&g.vec64, K * bs_tridiag_vec_elems(g.n), "batch FP64 vectors")) return;
+  if (!g.part64 && balloc(&g.part64, K * bs_tridiag_part_elems(g.n), "batch FP64 partials")) return;
+  if (!g.filt) g.filt = new FilterWs();
+  if (bs_filter_ws_alloc(g.filt, g.n, (int)K) != BS_OK) {
+    delete g.filt;
+    g.filt = nullptr;
+  }
+}
+
 extern "C" int bs_batch_set_solver(bs_batch* B, int solver) {
   if (!B || (solver != BS_SOLVER_DENSE && solver != BS_SOLVER_LOBPCG && solver != BS_SOLVER_FP64)) {
     bs_set_error("bs_batch_set_solver: NULL batch or unknown solver");
@@ -880,14 +906,7 @@ extern "C" int bs_batch_set_solver(bs_batch* B, int solver) {
         delete g.band;
         g.band = nullptr;
       }
-      // no memory for the filtered iteration: the reductions take the group
-      if (bs_use_filter(g.n, B->nbands)) {
-        if (!g.filt) g.filt = new FilterWs();
-        if (bs_filter_ws_alloc(g.filt, g.n, (int)K) != BS_OK) {
-          delete g.filt;
-          g.filt = nullptr;
-        }
-      }
+      alloc_filter(B, g);
     }
   }
   if (solver != B->solver) drop_graph(B);
@@ -1058,6 +1077,7 @@ extern "C" int bs_batch_set_tile(bs_batch* B, int tile) {
   }
   drop_graph(B);
   for (auto& g : B->groups) {
+    g.forced = tile != -1;
     if (tile == -1) {
       g.tuned = false;
     } else {
@@ -1231,7 +1251,8 @@ extern "C" int bs_batch_solve(bs_batch* B, const double* Q, double* omega_out, i
   const bool prof = B->prof;
   B->prof = false;   // not while tuning or recording a graph
   for (auto& g : B->groups) {
-    if (g.tuned || B->solver != BS_SOLVER_DENSE) continue;
+    if (B->solver == BS_SOLVER_DENSE && !g.forced && !B->d_vec && !g.filt) alloc_filter(B, g);
+    if (g.tuned || B->solver != BS_SOLVER_DENSE || group_filter(B, g)) continue;
     const auto key = tile_key(B, g);
     {
       std::lock_guard<std::mutex> lk(g_tile_mu);
