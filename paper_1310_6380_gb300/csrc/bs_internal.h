@@ -301,7 +301,9 @@ struct SliceSlabs {
 // the slabs of S digits of width Kp for an M x N product over `batch`
 // entries (cut finer while the launch would have fewer than two CTAs per
 // SM); false when they do not fit BS_SLAB_MAX
-bool bs_slice_slabs(int S, int Kp, int M, int N, int batch, SliceSlabs* q);
+// extra: orders S .. S + extra - 1 too, for operands whose entries are far below
+// their row's largest (an order left out weighs 2^-7 of the one before it)
+bool bs_slice_slabs(int S, int Kp, int M, int N, int batch, SliceSlabs* q, int extra = 0);
 // (entry, slab) output planes to allocate for any batch up to `batch`
 size_t bs_slice_planes(int S, int Kp, int M, int N, int batch);
 // D[z][q][n][m] = sum_{k < len_q} A[z][m][a0_q + k] B[z][n][b0_q + k] for every
@@ -309,7 +311,7 @@ size_t bs_slice_planes(int S, int Kp, int M, int N, int batch);
 // non-zero skip[z] are left out; SA > S: the rows of A hold SA digits
 int bs_launch_slice_orders(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int S,
                            int Kp, int batch, int* err, cudaStream_t s,
-                           const int* skip = nullptr, int SA = 0);
+                           const int* skip = nullptr, int SA = 0, int extra = 0);
 int bs_launch_fields_tc(bs_cell* c, cudaStream_t s);
 size_t bs_fields_tc_elems(int P, int D, int nf, size_t* nA, size_t* nB, size_t* nD);
 int bs_launch_cx_tc(const zd* C, const zd* X, int n, int b, int kb, uint16_t* sA, uint16_t* sB,
@@ -416,10 +418,15 @@ int bs_launch_band_pack_trail(const zd* A, int n, int o, int m, int kb, uint16_t
                               cudaStream_t s);
 int bs_launch_band_av(int m, const zd* V, int ldv, long sv, int nb, int kb, int S, uint16_t* wA,
                       uint16_t* wB, float* wD, int* eA, int* eB, zd* X, int ldx, long sx,
-                      int* err, cudaStream_t s, const int* skip = nullptr);
+                      int* err, cudaStream_t s, const int* skip = nullptr, int extra = 0);
 int bs_launch_band_pack_rank2(const zd* V, const zd* W, int ld, long sv, const int* dsc, int m,
                               int nb, int kb, int S, uint16_t* wA, uint16_t* wB, int* ex,
                               cudaStream_t s);
+// digit planes of the rows of A or of A^dagger (n x n, eight digits), and the
+// sizes of the operands of bs_launch_band_av for nc columns and one matrix
+void bs_zgemm_tc_cols_elems(int n, int nc, size_t* nA, size_t* nB, size_t* nD);
+size_t bs_slice_col_elems(int S, int Kp, int M, int N, int extra);
+int bs_launch_pack_rows8(const zd* A, bool dagger, int n, uint16_t* wA, int* eA, cudaStream_t s);
 int bs_rank2_column_tiles(int m);
 int bs_launch_rank2_update(const uint16_t* dA, const uint16_t* dB, const int* ex, int m, int kb,
                            zd* A, int n, int o, int ct0, int nct, int* err, cudaStream_t s);
@@ -643,8 +650,16 @@ int bs_launch_bisect(const double* de, int n, int batch, int nbands, double* ome
 
 // modes.cu: stress coefficients and plane-wave fields on a grid
 void bs_free_mode_workspace(bs_cell* c);
+// digit-plane buffers of the Gram solves (null: FP64 products)
+struct StressDigits {
+  int cols = 0;             // columns per product
+  uint16_t *wA = nullptr, *wB = nullptr;
+  float* wD = nullptr;
+  int *eA = nullptr, *eB = nullptr;
+  int* err = nullptr;
+};
 int bs_launch_stress(bs_cell* c, const zd* U, const double* Q, int kc, int nvec, zd* Zk, zd* Zm,
-                     zd* Y, zd* S, cudaStream_t s);
+                     zd* Y, zd* S, const StressDigits& dg, cudaStream_t s);
 int bs_launch_mode_field(const zd* coef, const double* Q, long kbase, int nkt, long f0, long nf,
                          int fpk, int M, int G, zf* E, zf* out, cudaStream_t s);
 

@@ -12,8 +12,14 @@
 // where T_X^-1 = L_X^-dagger L_X^-1 uses the triangular inverses that the
 // assembly keeps.  On a mesh cell the centroid rule does not make the plane
 // waves orthogonal, H = i I1 diag(K) with I1 = int conj(f_a) f_b, and V u
-// becomes I1 u in the right-hand sides.  All of it is FP64: two complex products per Gram solve,
-// every (k, mode) a column of one batched product.
+// becomes I1 u in the right-hand sides.  All of it is accurate to FP64: two
+// complex products per Gram solve, every (k, mode) a column of one product.
+// The products run as exact-slice contractions on the tensor cores with eight
+// digits per operand (all 53 bits of every entry within a factor 4 of its row's
+// or column's largest) and nine digit orders (eight left an error up to 1.4 times
+// that of the FP64 products, the entries of a mode lying far below its largest):
+// the FP64 pipe bounded them (2 FMA per clock and SM; 90 x 12 modes of N = 441:
+// 7.3 ms in FP64, 1.0 ms so).
 //
 // Fields (Eq. (approximation2d)): F(x_pq) = sum_a c_a exp(i K_a . x_pq) at
 // x_pq = ((p + 1/2)/G) h1 + ((q + 1/2)/G) h2.  With K_a = (Q1 + alpha) q^1 +
@@ -24,8 +30,12 @@
 // contractions run in FP32 (the output is complex64).  Each CTA owns one
 // field: every thread keeps the column T[.][q] of the first contraction in
 // registers, so the second streams rows p with shared-memory broadcasts of
-// Ep and coalesced stores along q.  The kernel is bound by its stores and
-// the FP32 pipe, not by any read.
+// Ep and coalesced stores along q.  Rows p and G - 1 - p lie at x and 1 - x, so
+// Ep[alpha][G - 1 - p] = e^{2 pi i Q1} conj(Ep[alpha][p]): with the real sums
+// A = sum_a T[a] Re Ep, B = sum_a T[a] Im Ep the two rows are A + i B and
+// e^{2 pi i Q1} (A - i B), for half the multiply-adds.  The kernel is bound by
+// the FP32 pipe and its stores, not by any read (5400 fields of M = 10,
+// G = 256: 1.96 ms with every row summed by itself, 1.08 ms in pairs).
 #include <algorithm>
 #include <vector>
 
@@ -61,13 +71,52 @@ __global__ void field_table_kernel(const double* __restrict__ Q, int nk, int M, 
   E[i] = make_float2((float)c, (float)s);
 }
 
+// The same table with the phase split into exp(i pi Q (2p + 1)/G), once per point,
+// and exp(i pi a (2p + 1)/G), a root of unity of order 2G: an FP64 sincospi for
+// every entry bounds the kernel above (99 us for 90 wavevectors of M = 10,
+// G = 256; 21 us here), so this one evaluates 2G + G of them per CTA, in
+// shared memory, and multiplies.  One CTA per wavevector and direction;
+// 2G <= ROOTS.
+constexpr int ROOTS = 2048;
+__global__ void __launch_bounds__(256) field_roots_kernel(const double* __restrict__ Q, int M,
+                                                          int WP, int G, zf* __restrict__ E) {
+  extern __shared__ __align__(16) zd root[];
+  const int k = blockIdx.x, dir = blockIdx.y, twoG = 2 * G;
+  for (int j = threadIdx.x; j < twoG; j += 256) {
+    double s, c;
+    sincospi((double)j / (double)G, &s, &c);
+    root[j] = zmake(c, s);
+  }
+  __syncthreads();
+  zf* e = E + ((size_t)k * 2 + dir) * WP * G;
+  const double q = Q[2 * k + dir];
+  for (int p = threadIdx.x; p < G; p += 256) {
+    const int odd = 2 * p + 1;
+    double s, c;
+    sincospi(fmod(q * (double)odd / (double)G, 2.0), &s, &c);
+    const zd b = zmake(c, s);
+    int m = (int)((-(long long)M * odd) % twoG);
+    if (m < 0) m += twoG;
+    for (int a = 0; a < WP; ++a) {
+      zf v = make_float2(0.f, 0.f);
+      if (a < 2 * M + 1) {
+        const zd x = zmul(root[m], b);
+        v = make_float2((float)x.x, (float)x.y);
+        m += odd;
+        if (m >= twoG) m -= twoG;
+      }
+      e[(size_t)a * G + p] = v;
+    }
+  }
+}
+
 // out[j][p][q] for field j of the chunk, global field f0 + j of wavevector
 // (f0 + j) / fpk; the table holds wavevectors kbase, kbase + 1, ...
 // WP >= 2M + 1, WP % 4 == 0; rows of four outputs per thread for independent chains
 template <int WP>
 __global__ void __launch_bounds__(FT, 2)
 field_kernel(const zd* __restrict__ coef, int M, int N, int G, long f0, int fpk, long kbase,
-             const zf* __restrict__ E, zf* __restrict__ out) {
+             const double* __restrict__ Q, const zf* __restrict__ E, zf* __restrict__ out) {
   __shared__ __align__(16) zf Ct[WP * WP];     // Ct[b][a] = c[a][b]
   __shared__ __align__(16) zf Es[PB][WP];
   const long f = f0 + blockIdx.x;
@@ -87,6 +136,12 @@ field_kernel(const zd* __restrict__ coef, int M, int N, int G, long f0, int fpk,
   const zf* Ep = E + (size_t)k * 2 * WP * G;
   const zf* Eq = Ep + (size_t)WP * G;
   zf* o = out + (size_t)blockIdx.x * G * G;
+  zf turn;   // e^{2 pi i Q1}
+  {
+    double sn, cs;
+    sincospi(2.0 * fmod(Q[2 * k], 1.0), &sn, &cs);
+    turn = make_float2((float)cs, (float)sn);
+  }
   for (int q0 = 0; q0 < G; q0 += blockDim.x) {
     const int q = q0 + tid;
     const bool act = q < G;
@@ -106,33 +161,46 @@ field_kernel(const zd* __restrict__ coef, int M, int N, int G, long f0, int fpk,
         T[a + 1] = zfma(make_float2(v.z, v.w), eb, T[a + 1]);
       }
     }
-    // second contraction, PB rows per staging pass, four rows at a time
-    for (int p0 = 0; p0 < G; p0 += PB) {
+    // second contraction, PB row pairs per staging pass, four pairs at a time
+    const int H = (G + 1) / 2;   // rows of the first half (the middle row of an odd G with it)
+    for (int p0 = 0; p0 < H; p0 += PB) {
       __syncthreads();
       for (int e = tid; e < PB * WP; e += blockDim.x) {
         const int r = e / WP, a = e % WP;
-        Es[r][a] = p0 + r < G ? Ep[(size_t)a * G + p0 + r] : make_float2(0.f, 0.f);
+        Es[r][a] = p0 + r < H ? Ep[(size_t)a * G + p0 + r] : make_float2(0.f, 0.f);
       }
       __syncthreads();
       if (act) {
-        const int rows = min(PB, G - p0);
+        const int rows = min(PB, H - p0);
 #pragma unroll
         for (int r = 0; r < PB; r += 4) {
-          zf acc[4];
+          zf A[4], B[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.f, 0.f);
+          for (int i = 0; i < 4; ++i) A[i] = B[i] = make_float2(0.f, 0.f);
 #pragma unroll
           for (int a = 0; a < WP; a += 2) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const float4 v = reinterpret_cast<const float4*>(&Es[r + i][0])[a / 2];
-              acc[i] = zfma(make_float2(v.x, v.y), T[a], acc[i]);
-              acc[i] = zfma(make_float2(v.z, v.w), T[a + 1], acc[i]);
+              A[i].x = fmaf(v.x, T[a].x, A[i].x);
+              A[i].y = fmaf(v.x, T[a].y, A[i].y);
+              B[i].x = fmaf(v.y, T[a].x, B[i].x);
+              B[i].y = fmaf(v.y, T[a].y, B[i].y);
+              A[i].x = fmaf(v.z, T[a + 1].x, A[i].x);
+              A[i].y = fmaf(v.z, T[a + 1].y, A[i].y);
+              B[i].x = fmaf(v.w, T[a + 1].x, B[i].x);
+              B[i].y = fmaf(v.w, T[a + 1].y, B[i].y);
             }
           }
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            if (r + i < rows) o[(size_t)(p0 + r + i) * G + q] = acc[i];
+            if (r + i < rows) {
+              const int p = p0 + r + i;
+              o[(size_t)p * G + q] = make_float2(A[i].x - B[i].y, A[i].y + B[i].x);
+              if (G - 1 - p != p)
+                o[(size_t)(G - 1 - p) * G + q] =
+                    zmul(turn, make_float2(A[i].x + B[i].y, A[i].y - B[i].x));
+            }
         }
       }
     }
@@ -213,11 +281,11 @@ int mode_ws(bs_cell* c, size_t bytes) {
 
 template <int WP>
 int launch_field(const zd* coef, long nf, int M, int N, int G, long f0, int fpk, long kbase,
-                 const zf* E, zf* out, cudaStream_t s) {
+                 const double* Q, const zf* E, zf* out, cudaStream_t s) {
   const int chunks = (G + FT - 1) / FT;
   const int per = (G + chunks - 1) / chunks;
   const int threads = std::min(FT, (per + 31) / 32 * 32);
-  field_kernel<WP><<<(unsigned)nf, threads, 0, s>>>(coef, M, N, G, f0, fpk, kbase, E, out);
+  field_kernel<WP><<<(unsigned)nf, threads, 0, s>>>(coef, M, N, G, f0, fpk, kbase, Q, E, out);
   BS_CHECK_LAUNCH("field_kernel");
   return BS_OK;
 }
@@ -236,24 +304,53 @@ int bs_launch_mode_field(const zd* coef, const double* Q, long kbase, int nkt, l
                          int fpk, int M, int G, zf* E, zf* out, cudaStream_t s) {
   const int W = 2 * M + 1, WP = (W + 3) / 4 * 4, N = W * W;
   const size_t te = (size_t)nkt * 2 * WP * G;
-  field_table_kernel<<<(unsigned)((te + 255) / 256), 256, 0, s>>>(Q + 2 * kbase, nkt, M, WP, G, E);
-  BS_CHECK_LAUNCH("field_table_kernel");
+  const double* Qt = Q + 2 * kbase;   // the table's wavevectors
+  if (2 * G <= ROOTS) {
+    field_roots_kernel<<<dim3(nkt, 2), 256, 2 * G * sizeof(zd), s>>>(Qt, M, WP, G, E);
+    BS_CHECK_LAUNCH("field_roots_kernel");
+  } else {
+    field_table_kernel<<<(unsigned)((te + 255) / 256), 256, 0, s>>>(Qt, nkt, M, WP, G, E);
+    BS_CHECK_LAUNCH("field_table_kernel");
+  }
   switch (WP) {
-    case 4: return launch_field<4>(coef, nf, M, N, G, f0, fpk, kbase, E, out, s);
-    case 8: return launch_field<8>(coef, nf, M, N, G, f0, fpk, kbase, E, out, s);
-    case 12: return launch_field<12>(coef, nf, M, N, G, f0, fpk, kbase, E, out, s);
-    case 16: return launch_field<16>(coef, nf, M, N, G, f0, fpk, kbase, E, out, s);
-    case 20: return launch_field<20>(coef, nf, M, N, G, f0, fpk, kbase, E, out, s);
-    case 24: return launch_field<24>(coef, nf, M, N, G, f0, fpk, kbase, E, out, s);
-    case 28: return launch_field<28>(coef, nf, M, N, G, f0, fpk, kbase, E, out, s);
-    case 32: return launch_field<32>(coef, nf, M, N, G, f0, fpk, kbase, E, out, s);
+    case 4: return launch_field<4>(coef, nf, M, N, G, f0, fpk, kbase, Qt, E, out, s);
+    case 8: return launch_field<8>(coef, nf, M, N, G, f0, fpk, kbase, Qt, E, out, s);
+    case 12: return launch_field<12>(coef, nf, M, N, G, f0, fpk, kbase, Qt, E, out, s);
+    case 16: return launch_field<16>(coef, nf, M, N, G, f0, fpk, kbase, Qt, E, out, s);
+    case 20: return launch_field<20>(coef, nf, M, N, G, f0, fpk, kbase, Qt, E, out, s);
+    case 24: return launch_field<24>(coef, nf, M, N, G, f0, fpk, kbase, Qt, E, out, s);
+    case 28: return launch_field<28>(coef, nf, M, N, G, f0, fpk, kbase, Qt, E, out, s);
+    case 32: return launch_field<32>(coef, nf, M, N, G, f0, fpk, kbase, Qt, E, out, s);
   }
   bs_set_error("mode field: truncation M = %d outside [0, 15]", M);
   return BS_EINVAL;
 }
 
+// X = L^-1 Z, then Z = L^-dagger X for nc columns (Li: L^-1)
+static int gram_solve(const zd* Li, int N, int nc, zd* Z, zd* X, const StressDigits& d,
+                      cudaStream_t s) {
+  const zd one = zmake(1.0, 0.0);
+  if (!d.wA) {
+    TRY_LAUNCH(bs_launch_zgemm(false, false, N, nc, N, one, Li, N, 0, Z, N, 0, nullptr, 0, X, N, 0,
+                               1, 1, s));
+    return bs_launch_zgemm(true, false, N, nc, N, one, Li, N, 0, X, N, 0, nullptr, 0, Z, N, 0, 1, 4,
+                           s);
+  }
+  for (int h = 0; h < 2; ++h) {
+    TRY_LAUNCH(bs_launch_pack_rows8(Li, h == 1, N, d.wA, d.eA, s));
+    const zd* in = h ? X : Z;
+    zd* out = h ? Z : X;
+    for (int j = 0; j < nc; j += d.cols) {
+      const int nb = std::min(d.cols, nc - j);
+      TRY_LAUNCH(bs_launch_band_av(N, in + (size_t)j * N, N, 0, nb, 1, 8, d.wA, d.wB, d.wD, d.eA,
+                                   d.eB, out + (size_t)j * N, N, 0, d.err, s, nullptr, 1));
+    }
+  }
+  return BS_OK;
+}
+
 int bs_launch_stress(bs_cell* c, const zd* U, const double* Q, int kc, int nvec, zd* Zk, zd* Zm,
-                     zd* Y, zd* S, cudaStream_t s) {
+                     zd* Y, zd* S, const StressDigits& dg, cudaStream_t s) {
   const int N = c->N, m = kc * nvec;
   const size_t NN = (size_t)N * N, tot = (size_t)N * m;
   const zd one = zmake(1.0, 0.0);
@@ -267,17 +364,9 @@ int bs_launch_stress(bs_cell* c, const zd* U, const double* Q, int kc, int nvec,
   stress_rhs_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(
       Uin, Q, c->d_G, N, nvec, m, c->q1[0], c->q1[1], c->q2[0], c->q2[1], Zk, Zm);
   BS_CHECK_LAUNCH("stress_rhs_kernel");
-  const zd* Lk = c->d_Linv;
-  const zd* Lm = c->d_Linv + NN;
-  // T_k^-1 Zk = L_k^-dagger (L_k^-1 Zk): Y = L^-1 Z (lower), then Zk = L^-dagger Y
-  TRY_LAUNCH(bs_launch_zgemm(false, false, N, m, N, one, Lk, N, 0, Zk, N, 0, nullptr, 0, Y, N, 0,
-                             1, 1, s));
-  TRY_LAUNCH(bs_launch_zgemm(true, false, N, m, N, one, Lk, N, 0, Y, N, 0, nullptr, 0, Zk, N, 0,
-                             1, 4, s));
-  TRY_LAUNCH(bs_launch_zgemm(false, false, N, 2 * m, N, one, Lm, N, 0, Zm, N, 0, nullptr, 0, Y,
-                             N, 0, 1, 1, s));
-  TRY_LAUNCH(bs_launch_zgemm(true, false, N, 2 * m, N, one, Lm, N, 0, Y, N, 0, nullptr, 0, Zm, N,
-                             0, 1, 4, s));
+  // T_X^-1 Z = L_X^-dagger (L_X^-1 Z)
+  TRY_LAUNCH(gram_solve(c->d_Linv, N, m, Zk, Y, dg, s));
+  TRY_LAUNCH(gram_solve(c->d_Linv + NN, N, 2 * m, Zm, Y, dg, s));
   stress_combine_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(Zk, Zm, N, m,
                                                                      c->mesh ? 1.0 : c->V, S);
   BS_CHECK_LAUNCH("stress_combine_kernel");
@@ -305,6 +394,26 @@ extern "C" int bs_stress_coefficients(bs_cell* c, const double* Q, int nk, int n
   const size_t m = (size_t)kc * nvec;
   const size_t zq = 2 * (size_t)kc, zu = 2 * (size_t)N * m, zs = 3 * (size_t)N * m;
   const size_t need = (zq + 2 * (6 * (size_t)N * m + zu + zs)) * sizeof(double);
+  // digit planes of the Gram solves behind the FP64 blocks; below 32 plane
+  // waves a product has no work to speed up, and without memory for the
+  // planes the FP64 products take it
+  StressDigits dg;
+  size_t nA = 0, nB = 0, nD = 0;
+  if (!c->aniso && N >= 32) {
+    dg.cols = (int)std::min<size_t>(2 * m, 2048);
+    bs_zgemm_tc_cols_elems(N, dg.cols, &nA, &nB, &nD);
+    const size_t a = (need + 255) / 256 * 256, b = a + (nA + nB) * 2;
+    const size_t d0 = (b + 255) / 256 * 256, e = d0 + (nD + N + dg.cols) * 4;
+    if (mode_ws(c, e) == BS_OK) {
+      char* p = (char*)c->d_mode;
+      dg.wA = (uint16_t*)(p + a);
+      dg.wB = dg.wA + nA;
+      dg.wD = (float*)(p + d0);
+      dg.eA = (int*)(dg.wD + nD);
+      dg.eB = dg.eA + N;
+      dg.err = c->d_info + 1;
+    }
+  }
   TRY_LAUNCH(mode_ws(c, need));
   double* dQ = c->d_mode;
   zd* Zk = (zd*)(dQ + zq);             // Zk, Zm: 3 N m contiguous (R3 of the anisotropic path)
@@ -334,13 +443,23 @@ extern "C" int bs_stress_coefficients(bs_cell* c, const double* Q, int nk, int n
       }
       TRY_LAUNCH(bs_launch_stress_aniso(c, ui, dQ, kb, nvec, Zk, Y, sk, s));
     } else {
-      TRY_LAUNCH(bs_launch_stress(c, uk, dQ, kb, nvec, Zk, Zm, Y, sk, s));
+      TRY_LAUNCH(bs_launch_stress(c, uk, dQ, kb, nvec, Zk, Zm, Y, sk, dg, s));
     }
     if (!s_dev)
       MCK(cudaMemcpyAsync((zd*)S_out + (size_t)k0 * nvec * 3 * N, dS, mb * 3 * N * sizeof(zd),
                           cudaMemcpyDeviceToHost, s),
           "bs_stress_coefficients S");
-    if (!u_dev || !s_dev) MCK(cudaStreamSynchronize(s), "bs_stress_coefficients sync");
+    if (!u_dev || !s_dev) {
+      int late = 0;   // a tensor-core wait that reached its limit
+      if (dg.wA)
+        MCK(cudaMemcpyAsync(&late, dg.err, sizeof(int), cudaMemcpyDeviceToHost, s),
+            "bs_stress_coefficients sync");
+      MCK(cudaStreamSynchronize(s), "bs_stress_coefficients sync");
+      if (late) {
+        bs_set_error("a tensor-core pipeline wait reached its limit");
+        return BS_ECUDA;
+      }
+    }
   }
   return BS_OK;
 }

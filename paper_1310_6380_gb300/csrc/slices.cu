@@ -28,6 +28,7 @@
 // (shorter slabs when the product is too small to fill the SMs otherwise).
 // The recombination adds the slabs of each order as exact 32-bit integers
 // and combines the S orders in FP64 with exactly constructed powers of two.
+#include <math_constants.h>
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stddef.h>
@@ -199,6 +200,7 @@ __device__ __forceinline__ unsigned long long warp_umax(unsigned long long v) {
   return v;
 }
 // block-wide: blockDim.x == 32 * nw, sh holds nw entries
+constexpr int NONFINITE_EXP = 2047 - 1022;   // of a row with an infinity or NaN: no digits hold it
 __device__ int row_exp_bits(unsigned long long v, unsigned long long* sh, int nw) {
   v = warp_umax(v);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
@@ -540,13 +542,17 @@ __global__ void pack_trail_kernel(const zd* __restrict__ A, int n, int o, int m,
 __global__ void pack_panel_kernel(const zd* __restrict__ V, int ldv, long sv, int m, int nb,
                                   int S, int Kp, uint16_t* __restrict__ out,
                                   int* __restrict__ ex, const int* __restrict__ skip) {
-  __shared__ double sh[4];
+  __shared__ unsigned long long sh[4];
   const int i = blockIdx.x, k = blockIdx.y;
   if (skip && skip[k]) return;
   const zd* x = V + (size_t)k * sv + (size_t)i * ldv;
-  double mx = 0.0;
-  for (int r = threadIdx.x; r < m; r += 128) mx = fmax(mx, fmax(fabs(x[r].x), fabs(x[r].y)));
-  const int e = row_exp(row_max(mx, sh));
+  unsigned long long mx = 0;
+  for (int r = threadIdx.x; r < m; r += 128) {
+    const unsigned long long a = abs_bits(x[r].x), b = abs_bits(x[r].y);
+    mx = a > mx ? a : mx;
+    mx = b > mx ? b : mx;
+  }
+  const int e = row_exp_bits(mx, sh, 4);
   uint16_t* base0 = out + ((size_t)k * 2 * nb + 2 * i) * S * Kp + (size_t)(S - 1) * Kp;
   uint16_t* base1 = base0 + (size_t)S * Kp;
   for (int c = threadIdx.x; c < Kp; c += 128) {
@@ -578,6 +584,7 @@ __global__ void recombine_panel_kernel(const float* __restrict__ Dm, const Slice
   const float* dk = Dm + (size_t)k * sl.nq * Nn * M;
   double xr, xi;
   order_sums(dk, Nn * M, (2 * (size_t)i) * M + r, (2 * (size_t)i + 1) * M + r, sl, &xr, &xi);
+  if (eB[(size_t)k * nb + i] == NONFINITE_EXP) xr = xi = CUDART_NAN;
   const int e = eA[(size_t)k * m + r] + eB[(size_t)k * nb + i];
   X[(size_t)k * sx + (size_t)i * ldx + r] = zmake(ldexp(xr, e), ldexp(xi, e));
 }
@@ -673,16 +680,17 @@ int bs_launch_band_pack_trail(const zd* A, int n, int o, int m, int kb, uint16_t
 // and the first S digits of both (S = 8: all of FP64)
 int bs_launch_band_av(int m, const zd* V, int ldv, long sv, int nb, int kb, int S, uint16_t* wA,
                       uint16_t* wB, float* wD, int* eA, int* eB, zd* X, int ldx, long sx,
-                      int* err, cudaStream_t s, const int* skip) {
+                      int* err, cudaStream_t s, const int* skip, int extra) {
   const int Kp = (2 * m + 63) / 64 * 64;
   SliceSlabs sl;
-  if (S < 1 || S > 8 || !bs_slice_slabs(S, Kp, m, 2 * nb, kb, &sl)) {
+  if (S < 1 || S > 8 || !bs_slice_slabs(S, Kp, m, 2 * nb, kb, &sl, extra)) {
     bs_set_error("band reduction: m = %d gives too many digit slabs", m);
     return BS_EINVAL;
   }
   pack_panel_kernel<<<dim3(nb, kb), 128, 0, s>>>(V, ldv, sv, m, nb, S, Kp, wB, eB, skip);
   BS_CHECK_LAUNCH("pack_panel_kernel");
-  TRY_LAUNCH(bs_launch_slice_orders(wA, wB, wD, m, 2 * nb, S, Kp, kb, err, s, skip, 8));
+  TRY_LAUNCH(bs_launch_slice_orders(wA, wB, wD, m, 2 * nb, S, Kp, kb, err, s, skip, 8,
+                                    extra));
   recombine_panel_kernel<<<dim3((m * nb + 255) / 256, kb), 256, 0, s>>>(wD, sl, eA, eB, m, nb, X,
                                                                        ldx, sx, skip);
   BS_CHECK_LAUNCH("recombine_panel_kernel");
@@ -699,5 +707,23 @@ int bs_launch_band_pack_rank2(const zd* V, const zd* W, int ld, long sv, const i
   }
   pack_rank2_kernel<<<dim3(m, kb), 64, 0, s>>>(V, W, ld, sv, dsc, m, nb, S, wA, wB, ex);
   BS_CHECK_LAUNCH("pack_rank2_kernel");
+  return BS_OK;
+}
+
+// X = A V or A^dagger V for a column-major n x n A and n x nc blocks V and X,
+// eight digits per operand (the whole FP64 mantissa) and nine orders: the digit
+// planes of A, then bs_launch_band_av on the columns
+void bs_zgemm_tc_cols_elems(int n, int nc, size_t* nA, size_t* nB, size_t* nD) {
+  const int Kp = (2 * n + 63) / 64 * 64;
+  *nA = (size_t)n * 8 * Kp;
+  *nB = (size_t)2 * nc * 8 * Kp;
+  *nD = bs_slice_col_elems(8, Kp, n, 2 * nc, 1);
+}
+
+int bs_launch_pack_rows8(const zd* A, bool dagger, int n, uint16_t* wA, int* eA, cudaStream_t s) {
+  const int Kp = (2 * n + 63) / 64 * 64;
+  if (dagger) return bs_launch_band_pack_trail(A, n, 0, n, 1, wA, eA, s);
+  pack_zrows_kernel<<<dim3(n, 1), 128, 0, s>>>(A, n, 0, nullptr, n, n, 8, Kp, 1, 0, wA, eA);
+  BS_CHECK_LAUNCH("pack_zrows_kernel");
   return BS_OK;
 }

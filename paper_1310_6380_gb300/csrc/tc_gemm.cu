@@ -22,6 +22,7 @@
 // parameters and blockIdx.z picks the slab.  The FP64 recombination of the
 // orders u < S reproduces the FP64 contraction to about 2^-46 of |A||B|
 // (seven digits) on the BF16 tensor pipe.
+#include <algorithm>
 #include <atomic>
 
 #include <cuda.h>
@@ -662,17 +663,19 @@ static int dispatch_bn(const uint16_t* A, const uint16_t* B, float* D, int M, in
 
 }  // namespace
 
-// slabs of at most L terms (L % 64 == 0); false when there are more than BS_SLAB_MAX
-static bool cut_slabs(int S, int Kp, int L, SliceSlabs* sl) {
+// slabs of at most L terms (L % 64 == 0) of the orders u < S + extra; false when
+// there are more than BS_SLAB_MAX
+static bool cut_slabs(int S, int Kp, int L, int extra, SliceSlabs* sl) {
   sl->nq = 0;
-  for (int u = 0; u < S; ++u) {
-    const int len = (u + 1) * Kp;
+  for (int u = 0; u < S + extra; ++u) {
+    // u >= S: the digits u - S + 1 .. S - 1 of both operands
+    const int first = u < S ? 0 : u - S + 1, len = (u < S ? u + 1 : 2 * S - 1 - u) * Kp;
     for (int k0 = 0; k0 < len; k0 += L) {
       if (sl->nq == BS_SLAB_MAX) return false;
       const int q = sl->nq++;
       sl->order[q] = u;
-      sl->a0[q] = k0;
-      sl->b0[q] = (S - 1 - u) * Kp + k0;
+      sl->a0[q] = first * Kp + k0;
+      sl->b0[q] = (u < S ? S - 1 - u : 0) * Kp + k0;
       sl->len[q] = len - k0 < L ? len - k0 : L;
     }
   }
@@ -684,16 +687,16 @@ static bool cut_slabs(int S, int Kp, int L, SliceSlabs* sl) {
 // per SM, the slabs are halved (down to 128 terms), which trades a serial K
 // loop for parallel CTAs.  Small contractions (one cell's form factors) need
 // this; batched ones keep the longest slabs.
-bool bs_slice_slabs(int S, int Kp, int M, int N, int batch, SliceSlabs* sl) {
+bool bs_slice_slabs(int S, int Kp, int M, int N, int batch, SliceSlabs* sl, int extra) {
   const int bn = pick_bn(N);
   const long tiles = (long)((M + BM - 1) / BM) * ((N + bn - 1) / bn) * batch;
   const long want = 2L * bs_sm_count();
   int L = BS_SLAB_K;
-  if (!cut_slabs(S, Kp, L, sl)) return false;
+  if (!cut_slabs(S, Kp, L, extra, sl)) return false;
   while (tiles * sl->nq < want && L > 128) {
     const int L2 = (L / 2) / 64 * 64 < 128 ? 128 : (L / 2) / 64 * 64;
     SliceSlabs t;
-    if (!cut_slabs(S, Kp, L2, &t)) break;
+    if (!cut_slabs(S, Kp, L2, extra, &t)) break;
     *sl = t;
     L = L2;
   }
@@ -704,7 +707,7 @@ size_t bs_slice_planes(int S, int Kp, int M, int N, int batch) {
   // a smaller batch may cut its slabs finer: take the largest count of
   // (entry, slab) output planes over every batch size up to `batch`
   SliceSlabs full, sl;
-  if (!cut_slabs(S, Kp, BS_SLAB_K, &full)) return (size_t)BS_SLAB_MAX * batch;
+  if (!cut_slabs(S, Kp, BS_SLAB_K, 0, &full)) return (size_t)BS_SLAB_MAX * batch;
   const int bn = pick_bn(N);
   const long t1 = (long)((M + BM - 1) / BM) * ((N + bn - 1) / bn);
   size_t best = (size_t)full.nq * batch;
@@ -716,6 +719,15 @@ size_t bs_slice_planes(int S, int Kp, int M, int N, int batch) {
     if (v > best) best = v;
   }
   return best;
+}
+
+size_t bs_slice_col_elems(int S, int Kp, int M, int N, int extra) {
+  // uncut slabs for all N columns, or up to BS_SLAB_MAX while the tiles are too
+  // few to fill the SMs (N below about 128 want / (row tiles x slabs))
+  SliceSlabs full;
+  if (!cut_slabs(S, Kp, BS_SLAB_K, extra, &full)) return (size_t)BS_SLAB_MAX * M * N;
+  const long rows = (M + BM - 1) / BM, few = 128L * (2L * bs_sm_count()) / (rows * full.nq) + 128;
+  return (size_t)M * std::max<size_t>((size_t)full.nq * N, (size_t)BS_SLAB_MAX * std::min<long>(N, few));
 }
 
 int bs_launch_slice_gemm(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int K,
@@ -736,10 +748,10 @@ int bs_launch_slice_gemm(const uint16_t* A, const uint16_t* B, float* D, int M, 
 
 int bs_launch_slice_orders(const uint16_t* A, const uint16_t* B, float* D, int M, int N, int S,
                            int Kp, int batch, int* err, cudaStream_t s, const int* skip,
-                           int SA) {
+                           int SA, int extra) {
   SliceSlabs sl;
   if (Kp % 64 != 0 || S < 1 || ((uintptr_t)A & 15) || ((uintptr_t)B & 15) || M < 1 || N < 1 ||
-      batch < 1 || !bs_slice_slabs(S, Kp, M, N, batch, &sl) || (long)batch * sl.nq > 65535) {
+      batch < 1 || !bs_slice_slabs(S, Kp, M, N, batch, &sl, extra) || (long)batch * sl.nq > 65535) {
     bs_set_error("slice orders: need Kp %% 64 == 0, 16-byte aligned operands, at most %d slabs",
                  BS_SLAB_MAX);
     return BS_EINVAL;
