@@ -435,7 +435,7 @@ int bs_launch_rank2_update(const uint16_t* dA, const uint16_t* dB, const int* ex
 // shift-invert operator, FP64 Rayleigh-Ritz, residual and inertia certificate)
 #define BS_FILT_BLOCK 32       // columns of the block
 #define BS_FILT_MAX_BANDS 22   // wanted branches: at least 10 guard vectors remain
-#define BS_FILT_MIN_N 200
+#define BS_FILT_MIN_N 96
 #define BS_FILT_MAXDEG 12      // degrees of one filter
 struct FilterWs {
   int n = 0, kf = 0;        // order, matrices per chunk

@@ -36,8 +36,9 @@
 //
 // Measured (one GB300, whole FP64 solve with its assembly, the reduction to
 // tridiagonal form before -> this): n = 882, 90 matrices, 18 branches
-// 171 -> 27 ms; n = 1029, 30 matrices, 12 branches 136 -> 19 ms; n = 242,
-// 70 matrices, 18 branches 16.9 -> 4.3 ms.  What bounds it at n = 882 is the
+// 171 -> 26 ms; n = 1029, 30 matrices, 12 branches 136 -> 18.3 ms; n = 242,
+// 70 matrices, 18 branches 16.9 -> 4.3 ms; n = 98, 65 matrices, 18 branches
+// 3.86 -> 2.52 ms.  What bounds it at n = 882 is the
 // FP32 pipe in the factorisations and the FP64 pipe in the Rayleigh-Ritz steps
 // (32-column products at 2 FMA per clock and SM).
 //
@@ -58,7 +59,8 @@ constexpr int TB = 64;              // tile edge of the FP32 factorisation
 constexpr int LDS = TB + 1;         // row stride of the diagonal blocks in shared memory
 constexpr float TINY_PIVOT = 1e-6f; // of the scaled unit diagonal
 constexpr int GR = 64;              // rows per CTA of the Gram and rotation kernels
-constexpr int STEER_DIGITS = 5;     // of C X in the steps that only steer (34 bits)
+constexpr int STEER_DIGITS = 5;     // of C X in the steps that only steer (34 bits),
+constexpr int LAST_STEER_DIGITS = 6;// and in the step before the first that can certify (41)
 
 // ---------------------------------------------------------------- set-up
 // Per matrix: the FB smallest diagonal entries (the starting vectors are
@@ -365,18 +367,26 @@ __global__ void __launch_bounds__(256) ldl64_diag_kernel(zf* __restrict__ A, zf*
 }
 
 // 64 x 64 x 64 product on 256 threads, 4 x 4 complex per thread:
-// acc[i][j] += sum_t As[t][tx + 16 i] op(B[t][ty + 16 j])
-template <bool CONJB>
-__device__ __forceinline__ void mm64(const zf* __restrict__ As, const zf* __restrict__ Bs, int bs_t,
-                                     int bs_c, zf (&acc)[4][4]) {
+// acc[i][j] += sum_t As[t][row(i)] op(Bs[t][col(j)]), rows 2 tx + {0, 1, 32, 33} and
+// columns 2 ty + {0, 1, 32, 33}, so that two 16-byte loads fetch each operand
+// (eight 8-byte ones kept the shared-memory pipe half busy: 205 -> 183 us per
+// update launch of 90 x 896^2).  Rows t of the tiles are LA, LB apart.
+__device__ __forceinline__ int own(int x, int i) { return 2 * x + (i & 1) + 32 * (i >> 1); }
+
+template <bool CONJB, int LA = TB, int LB = TB>
+__device__ __forceinline__ void mm64(const zf* __restrict__ As, const zf* __restrict__ Bs,
+                                     zf (&acc)[4][4]) {
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const float4* A4 = reinterpret_cast<const float4*>(As) + tx;
+  const float4* B4 = reinterpret_cast<const float4*>(Bs) + ty;
 #pragma unroll 8
   for (int t = 0; t < TB; ++t) {
-    zf a[4], b[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = As[t * TB + tx + 16 * i];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = Bs[t * bs_t + (ty + 16 * j) * bs_c];
+    const float4 a0 = A4[t * (LA / 2)], a1 = A4[t * (LA / 2) + 16];
+    const float4 b0 = B4[t * (LB / 2)], b1 = B4[t * (LB / 2) + 16];
+    const zf a[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
+                     make_float2(a1.z, a1.w)};
+    const zf b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                     make_float2(b1.z, b1.w)};
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -391,6 +401,23 @@ __device__ __forceinline__ void load_tile(zf* dst, const zf* src, int np) {
   for (int e = threadIdx.x; e < TB * TB / 2; e += 256) {
     const int t = e >> 5, r2 = e & 31;
     d4[t * 32 + r2] = *reinterpret_cast<const float4*>(src + (size_t)t * np + 2 * r2);
+  }
+}
+
+// the transpose of a 64 x 64 tile: dst[t * LDT + c] = src[t + c np], scaled by
+// sc[t] (optional).  A warp takes eight columns of eight rows t: 64-byte segments
+// of global memory, two-way conflicts in shared memory.
+constexpr int LDT = TB + 4;
+__device__ __forceinline__ void load_tile_t(zf* dst, const zf* src, int np,
+                                            const float* sc = nullptr) {
+  const int tid = threadIdx.x, t2 = (tid & 3) * 2, c0 = tid >> 2;   // 64 columns, 8 rows a pass
+#pragma unroll 4
+  for (int t0 = 0; t0 < TB; t0 += 8) {
+    const int t = t0 + t2;
+    const float4 v = *reinterpret_cast<const float4*>(src + (size_t)c0 * np + t);
+    const float f0 = sc ? sc[t] : 1.f, f1 = sc ? sc[t + 1] : 1.f;
+    dst[t * LDT + c0] = make_float2(v.x * f0, v.y * f0);
+    dst[(t + 1) * LDT + c0] = make_float2(v.z * f1, v.w * f1);
   }
 }
 
@@ -411,12 +438,15 @@ __global__ void __launch_bounds__(256) ldl64_panel_kernel(zf* __restrict__ A,
   if (tid < TB) di[tid] = 1.f / a[(size_t)(j0 + tid) * (np + 1)].x;
   __syncthreads();
   zf acc[4][4] = {};
-  mm64<true>(As, Bs, TB, 1, acc);   // Y[r][c] = sum_t A[r][t] conj(L11^-1[c][t])
+  mm64<true>(As, Bs, acc);   // Y[r][c] = sum_t A[r][t] conj(L11^-1[c][t])
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const int c = ty + 16 * j;
+    const int c = own(ty, j);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) ai[(size_t)c * np + tx + 16 * i] = zscale(acc[i][j], di[c]);
+    for (int i = 0; i < 4; i += 2) {
+      const zf u = zscale(acc[i][j], di[c]), v = zscale(acc[i + 1][j], di[c]);
+      *reinterpret_cast<float4*>(ai + (size_t)c * np + own(tx, i)) = make_float4(u.x, u.y, v.x, v.y);
+    }
   }
 }
 
@@ -455,20 +485,28 @@ __global__ void __launch_bounds__(256) ldl64_update_kernel(zf* __restrict__ A, z
   }
   __syncthreads();
   zf acc[4][4] = {};
-  mm64<true>(As, Bs, TB, 1, acc);
+  mm64<true>(As, Bs, acc);
   const bool first = blockIdx.x == 0;
   if (first) __syncthreads();   // As is reused for the block below
+  // (entries above the diagonal of a diagonal tile are written too: nothing reads them)
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const int c = ty + 16 * j;
+    const int c = own(ty, j);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = tx + 16 * i;
-      zf* o = a + (size_t)(k0 + c) * np + i0 + r;
-      if (bi == bk && r < c) continue;
-      zf v = zsub(*o, acc[i][j]);
-      if (first) As[r * LDS + c] = v;
-      else *o = v;
+    for (int i = 0; i < 4; i += 2) {
+      const int r = own(tx, i);
+      float4* o = reinterpret_cast<float4*>(a + (size_t)(k0 + c) * np + i0 + r);
+      float4 v = *o;
+      v.x -= acc[i][j].x;
+      v.y -= acc[i][j].y;
+      v.z -= acc[i + 1][j].x;
+      v.w -= acc[i + 1][j].y;
+      if (first) {
+        As[r * LDS + c] = make_float2(v.x, v.y);
+        As[(r + 1) * LDS + c] = make_float2(v.z, v.w);
+      } else {
+        *o = v;
+      }
     }
   }
   if (first) {
@@ -482,7 +520,7 @@ __global__ void __launch_bounds__(256) trinv64_kernel(const zf* __restrict__ A, 
                                                       int np, int dd) {
   extern __shared__ __align__(16) unsigned char dsm[];
   zf* As = reinterpret_cast<zf*>(dsm);
-  zf* Bs = As + TB * TB;   // [col][t], stride LDS
+  zf* Bs = As + TB * TB;   // [t][col], stride LDT
   const int bj = blockIdx.x, bi = bj + dd;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const zf* l = A + (size_t)blockIdx.y * np * np;
@@ -491,12 +529,9 @@ __global__ void __launch_bounds__(256) trinv64_kernel(const zf* __restrict__ A, 
   for (int bk = bj; bk < bi; ++bk) {
     __syncthreads();
     load_tile(As, l + (size_t)bk * TB * np + bi * TB, np);
-    for (int e = tid; e < TB * TB; e += 256) {
-      const int c = e >> 6, t = e & 63;
-      Bs[c * LDS + t] = x[(size_t)(bj * TB + c) * np + bk * TB + t];
-    }
+    load_tile_t(Bs, x + (size_t)bj * TB * np + bk * TB, np);
     __syncthreads();
-    mm64<false>(As, Bs, 1, LDS, acc);
+    mm64<false, TB, LDT>(As, Bs, acc);
   }
   __syncthreads();
   load_tile(As, x + (size_t)bi * TB * np + bi * TB, np);
@@ -504,17 +539,17 @@ __global__ void __launch_bounds__(256) trinv64_kernel(const zf* __restrict__ A, 
   for (int j = 0; j < 4; ++j)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      Bs[(ty + 16 * j) * LDS + tx + 16 * i] = acc[i][j];
+      Bs[own(tx, i) * LDT + own(ty, j)] = acc[i][j];
       acc[i][j] = make_float2(0.f, 0.f);
     }
   __syncthreads();
-  mm64<false>(As, Bs, 1, LDS, acc);
+  mm64<false, TB, LDT>(As, Bs, acc);
 #pragma unroll
   for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      x[(size_t)(bj * TB + ty + 16 * j) * np + bi * TB + tx + 16 * i] =
-          make_float2(-acc[i][j].x, -acc[i][j].y);
+    for (int i = 0; i < 4; i += 2)
+      *reinterpret_cast<float4*>(x + (size_t)(bj * TB + own(ty, j)) * np + bi * TB + own(tx, i)) =
+          make_float4(-acc[i][j].x, -acc[i][j].y, -acc[i + 1][j].x, -acc[i + 1][j].y);
 }
 
 // B = W X^dagger D^-1 X W (X = L^-1), 64-tiles (bi, bk) and their mirrors,
@@ -525,44 +560,33 @@ __global__ void __launch_bounds__(256) filt_operator_kernel(const zf* __restrict
                                                             const float* __restrict__ w,
                                                             uint16_t* __restrict__ Bp) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  zf* As = reinterpret_cast<zf*>(dsm);   // [column][t], stride LDS
-  zf* Bs = As + TB * LDS;
+  zf* As = reinterpret_cast<zf*>(dsm);   // [t][column], stride LDT
+  zf* Bs = As + TB * LDT;
+  __shared__ float di[TB];
   int bi, bk;
   tile_of(blockIdx.x, bi, bk);
   const int k = blockIdx.y, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const zf* x = X + (size_t)k * np * np;
   const float* dk = d + (size_t)k * np;
   const float* wk = w + (size_t)k * np;
-  zf acc[4][4] = {};
+  zf acc[4][4] = {};   // conj(B_rc): the columns' conjugates times the rows
   for (int t0 = bi * TB; t0 < np; t0 += TB) {
     __syncthreads();
-    const float di = 1.f / dk[t0 + (tid & 63)];
-    for (int c = tid >> 6; c < TB; c += 4) {
-      const int t = tid & 63;
-      As[c * LDS + t] = zscale(x[(size_t)(bi * TB + c) * np + t0 + t], di);
-      Bs[c * LDS + t] = x[(size_t)(bk * TB + c) * np + t0 + t];
-    }
+    if (tid < TB) di[tid] = 1.f / dk[t0 + tid];
+    load_tile_t(Bs, x + (size_t)bk * TB * np + t0, np);
     __syncthreads();
-#pragma unroll 8
-    for (int t = 0; t < TB; ++t) {
-      zf a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[(tx + 16 * i) * LDS + t];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[(ty + 16 * j) * LDS + t];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = zfmac(b[j], a[i], acc[i][j]);   // conj(a) b
-    }
+    load_tile_t(As, x + (size_t)bi * TB * np + t0, np, di);
+    __syncthreads();
+    mm64<true, LDT, LDT>(As, Bs, acc);   // sum_t x_tr conj(x_tc) / d_t
   }
   __syncthreads();
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const float wc = wk[bk * TB + ty + 16 * j];
+    const float wc = wk[bk * TB + own(ty, j)];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      As[(tx + 16 * i) * LDS + ty + 16 * j] = zscale(acc[i][j], wk[bi * TB + tx + 16 * i] * wc);
+      As[own(tx, i) * LDS + own(ty, j)] =
+          zscale(zconj(acc[i][j]), wk[bi * TB + own(tx, i)] * wc);
   }
   __syncthreads();
   uint16_t* b = Bp + (size_t)k * np * 4 * np;
@@ -1272,8 +1296,8 @@ __global__ void __launch_bounds__(1024) filt_decide_kernel(const int* __restrict
 // the set-up kernel's shared memory, and an order from which its some 200
 // launches take less than the reduction's n dependent steps also for a
 // single matrix (ms of one solve, iteration / reduction, 1 and 64 matrices:
-// n = 98 3.9 / 2.4 and 4.2 / 3.6, n = 162 4.4 / 4.1 and 5.8 / 7.4,
-// n = 242 4.8 / 6.3 and 6.8 / 14.5, n = 578 8.1 / 40.5 and 18.2 / 61.8).
+// n = 50 1.7 / 1.2 and 1.9 / 1.5, n = 98 1.9 / 2.4 and 2.2 / 3.6,
+// n = 162 2.2 / 4.1 and 2.9 / 7.5, n = 338 2.8 / 9.2 and 5.2 / 28.5).
 bool bs_filter_fits(int n, int nbands) {
   return nbands >= 1 && nbands <= BS_FILT_MAX_BANDS && n >= BS_FILT_MIN_N && n <= 2048;
 }
@@ -1310,7 +1334,8 @@ int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
       {(void**)&w->pB, k * 2 * FB * 8 * Kp * 2},
       // fewer digits can be cut into more slabs: room for either
       {(void**)&w->pD, std::max(bs_slice_planes(8, (int)Kp, n, 2 * FB, kf),
-                                bs_slice_planes(STEER_DIGITS, (int)Kp, n, 2 * FB, kf)) *
+                                std::max(bs_slice_planes(STEER_DIGITS, (int)Kp, n, 2 * FB, kf),
+                                         bs_slice_planes(LAST_STEER_DIGITS, (int)Kp, n, 2 * FB, kf))) *
                            n * 2 * FB * sizeof(float)},
       {(void**)&w->eA, k * n * sizeof(int)},
       {(void**)&w->eB, k * FB * sizeof(int)},
@@ -1354,8 +1379,8 @@ static int filter_attrs() {
       {(const void*)ldl64_diag_kernel, 2 * TB * LDS * (int)sizeof(zf)},
       {(const void*)ldl64_panel_kernel, 2 * TB * TB * (int)sizeof(zf)},
       {(const void*)ldl64_update_kernel, 2 * TB * LDS * (int)sizeof(zf)},
-      {(const void*)trinv64_kernel, (TB * TB + TB * LDS) * (int)sizeof(zf)},
-      {(const void*)filt_operator_kernel, 2 * TB * LDS * (int)sizeof(zf)},
+      {(const void*)trinv64_kernel, (TB * TB + TB * LDT) * (int)sizeof(zf)},
+      {(const void*)filt_operator_kernel, 2 * TB * LDT * (int)sizeof(zf)},
       {(const void*)filt_gram_kernel<double>, (int)sizeof(RrSmem<double>)},
       {(const void*)filt_gram_kernel<float>, (int)sizeof(RrSmem<float>)},
       {(const void*)filt_rotate_kernel<double>, (int)sizeof(RotSmem<double>)},
@@ -1390,10 +1415,10 @@ static int filter_factor(FilterWs& w, int np, int kf, bool inverse, cudaStream_t
   }
   if (!inverse) return BS_OK;
   for (int d = 1; d < nt; ++d) {
-    trinv64_kernel<<<dim3(nt - d, kf), 256, (TB * TB + TB * LDS) * sizeof(zf), s>>>(w.A, w.X, np, d);
+    trinv64_kernel<<<dim3(nt - d, kf), 256, (TB * TB + TB * LDT) * sizeof(zf), s>>>(w.A, w.X, np, d);
     BS_CHECK_LAUNCH("trinv64_kernel");
   }
-  filt_operator_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 2 * TB * LDS * sizeof(zf), s>>>(
+  filt_operator_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 2 * TB * LDT * sizeof(zf), s>>>(
       w.X, w.d, np, w.w, reinterpret_cast<uint16_t*>(w.A));
   BS_CHECK_LAUNCH("filt_operator_kernel");
   return BS_OK;
@@ -1475,7 +1500,7 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
                                             vs[(j + 1) & 1], done, err, s));
       filt_add_kernel<<<cg, 256, 0, s>>>(w.Xb, E[(m - 1) & 1], n, np, done);
       BS_CHECK_LAUNCH("filt_add_kernel");
-      TRY_LAUNCH(bs_launch_band_av(n, w.Xb, n, (long)FB * n, FB, kf, rd < 2 ? STEER_DIGITS : 8,
+      TRY_LAUNCH(bs_launch_band_av(n, w.Xb, n, (long)FB * n, FB, kf, rd < 2 ? STEER_DIGITS : rd == 2 ? LAST_STEER_DIGITS : 8,
                                    w.pA, w.pB, w.pD, w.eA,
                                    w.eB, w.CX, n, (long)FB * n, err, s, done));
     }

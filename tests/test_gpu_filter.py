@@ -119,3 +119,12 @@ def test_batch_fp64_solver():
     for i, c in enumerate(cl):
         _, ref, n, cmax = solve2(c["cell"], c["M"], np.ascontiguousarray(Q[i]), 10)
         assert np.abs(w[i] ** 2 - ref ** 2).max() <= (n + 128) * EPS * cmax
+
+
+@pytest.mark.parametrize("M,nb,nk", [(3, 1, 1), (3, 22, 40), (3, 9, 13), (4, 22, 1), (4, 10, 25)])
+def test_smallest_matrices(M, nb, nk):
+    """n = 98 and 162, the smallest that take the iteration (two and three tiles)."""
+    for cell in (cells.circle_cell(32, 0.3), cells.voronoi_cell(32, 9, seed=2, lattice="hex")):
+        Q = cells.ibz_path(cell.lattice, max(nk, 2), cell.h1, cell.h2)[:nk].copy()
+        a, b, n, cmax = solve2(cell, M, Q, nb)
+        assert np.abs(a ** 2 - b ** 2).max() <= (n + 128) * EPS * cmax
