@@ -38,124 +38,179 @@ const int COUT[NCONV] = {16, 32, 32, 32};
 const int SIDE[NCONV] = {64, 32, 16, 8};   // input side of conv l (output side equal, then pooled)
 
 // ------------------------------------------------------------ convolution (3x3, circular)
-// out[b][co][y][x] = relu(bias[co] + sum_ci,dy,dx w[co][ci][dy][dx] in[b][ci][y+dy-1][x+dx-1])
-constexpr int CO_T = 8;   // output channels per thread
-__global__ void conv_fwd_kernel(const float* __restrict__ in, const float* __restrict__ w,
-                                const float* __restrict__ bias, int cin, int cout, int S,
-                                float* __restrict__ out) {
-  extern __shared__ float wsh[];   // CO_T x cin x 9
-  const int b = blockIdx.z, co0 = blockIdx.y * CO_T;
-  const int npix = S * S, p = blockIdx.x * blockDim.x + threadIdx.x;
-  for (int e = threadIdx.x; e < CO_T * cin * 9; e += blockDim.x) {
-    const int co = co0 + e / (cin * 9);
-    wsh[e] = co < cout ? w[(size_t)co * cin * 9 + e % (cin * 9)] : 0.f;
+// forward: out[b][o][y][x] = relu(bias[o] + sum_i,dy,dx w[o][i][dy][dx] in[b][i][y+dy-1][x+dx-1])
+// and its 2 x 2 means; data gradient (the taps reversed, the channels of w exchanged):
+// out[b][o][y][x] = sum_i,dy,dx w[i][o][dy][dx] in[b][i][y-dy+1][x-dx+1].
+//
+// A thread owns a 2 x 2 quad of pixels and CT output channels: 16 loads of the
+// input and 9 CT / 4 wide broadcast loads of the weights feed 36 CT multiply-adds
+// per input channel, so the FP32 pipe bounds it and not the load unit (one pixel
+// and scalar weights per thread took a shared load per multiply-add: 170 -> 84 us
+// for the four forward layers of 64 cells, their pooling included, 129 -> 71 us
+// for the three data gradients).  Every output sums its terms in the order of
+// (i, dy, dx), whatever CT is.  S is a power of two.
+template <int CT, bool BWD>
+__global__ void __launch_bounds__(128) conv_kernel(const float* __restrict__ in,
+                                                   const float* __restrict__ w,
+                                                   const float* __restrict__ bias, int ni, int no,
+                                                   int S, int lgh, int nquad,
+                                                   float* __restrict__ out,
+                                                   float* __restrict__ pooled) {
+  extern __shared__ __align__(16) float wsh[];   // ni x 9 x CT
+  const int o0 = blockIdx.y * CT;
+  for (int e = threadIdx.x; e < ni * 9 * CT; e += blockDim.x) {
+    const int t = e % CT, d = (e / CT) % 9, i = e / (9 * CT);
+    wsh[e] = BWD ? w[((size_t)i * no + o0 + t) * 9 + d] : w[((size_t)(o0 + t) * ni + i) * 9 + d];
   }
   __syncthreads();
-  if (p >= npix) return;
-  const int y = p / S, x = p % S;
-  float acc[CO_T];
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= nquad) return;
+  const int h = S / 2, npix = S * S;
+  const int x = 2 * (q & (h - 1)), y = 2 * ((q >> lgh) & (h - 1)), b = q >> (2 * lgh);
+  float acc[4][CT];
 #pragma unroll
-  for (int t = 0; t < CO_T; ++t) acc[t] = co0 + t < cout ? bias[co0 + t] : 0.f;
-  const float* ib = in + (size_t)b * cin * npix;
-  for (int ci = 0; ci < cin; ++ci) {
-    const float* ic = ib + (size_t)ci * npix;
-    float v[9];
+  for (int t = 0; t < CT; ++t) {
+    const float v = BWD ? 0.f : bias[o0 + t];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) acc[f][t] = v;
+  }
+  const float* ic = in + (size_t)b * ni * npix;
+  int ro[4], co[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    ro[r] = ((y + r - 1) & (S - 1)) * S;
+    co[r] = (x + r - 1) & (S - 1);
+  }
+#pragma unroll 2
+  for (int i = 0; i < ni; ++i, ic += npix) {
+    float P[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) P[r][c] = ic[ro[r] + co[c]];
+    const float* wi = wsh + i * 9 * CT;
 #pragma unroll
     for (int d = 0; d < 9; ++d) {
-      const int yy = (y + d / 3 - 1 + S) % S, xx = (x + d % 3 - 1 + S) % S;
-      v[d] = ic[yy * S + xx];
-    }
+      float wt[CT];
 #pragma unroll
-    for (int t = 0; t < CO_T; ++t) {
-      const float* wt = wsh + (t * cin + ci) * 9;
+      for (int t = 0; t < CT; t += 2) {
+        if constexpr (CT >= 4) {
+          if (t % 4 == 0) {
+            const float4 f = *reinterpret_cast<const float4*>(wi + d * CT + t);
+            wt[t] = f.x;
+            wt[t + 1] = f.y;
+            wt[t + 2] = f.z;
+            wt[t + 3] = f.w;
+          }
+        } else {
+          const float2 f = *reinterpret_cast<const float2*>(wi + d * CT + t);
+          wt[t] = f.x;
+          wt[t + 1] = f.y;
+        }
+      }
+      const int dy = BWD ? 2 - d / 3 : d / 3, dx = BWD ? 2 - d % 3 : d % 3;
 #pragma unroll
-      for (int d = 0; d < 9; ++d) acc[t] = fmaf(wt[d], v[d], acc[t]);
-    }
-  }
+      for (int f = 0; f < 4; ++f)
 #pragma unroll
-  for (int t = 0; t < CO_T; ++t)
-    if (co0 + t < cout) out[((size_t)b * cout + co0 + t) * npix + p] = fmaxf(acc[t], 0.f);
-}
-
-// gin[b][ci][y][x] = sum_co,dy,dx w[co][ci][dy][dx] g[b][co][y-dy+1][x-dx+1]
-constexpr int CI_T = 8;
-__global__ void conv_bwd_data_kernel(const float* __restrict__ g, const float* __restrict__ w,
-                                     int cin, int cout, int S, float* __restrict__ gin) {
-  extern __shared__ float wsh[];   // CI_T x cout x 9, [t][co][d]
-  const int b = blockIdx.z, ci0 = blockIdx.y * CI_T;
-  const int npix = S * S, p = blockIdx.x * blockDim.x + threadIdx.x;
-  for (int e = threadIdx.x; e < CI_T * cout * 9; e += blockDim.x) {
-    const int t = e / (cout * 9), co = (e / 9) % cout, d = e % 9;
-    wsh[e] = ci0 + t < cin ? w[((size_t)co * cin + ci0 + t) * 9 + d] : 0.f;
-  }
-  __syncthreads();
-  if (p >= npix) return;
-  const int y = p / S, x = p % S;
-  float acc[CI_T];
-#pragma unroll
-  for (int t = 0; t < CI_T; ++t) acc[t] = 0.f;
-  const float* gb = g + (size_t)b * cout * npix;
-  for (int co = 0; co < cout; ++co) {
-    const float* gc = gb + (size_t)co * npix;
-    float v[9];
-#pragma unroll
-    for (int d = 0; d < 9; ++d) {
-      const int yy = (y - d / 3 + 1 + S) % S, xx = (x - d % 3 + 1 + S) % S;
-      v[d] = gc[yy * S + xx];
-    }
-#pragma unroll
-    for (int t = 0; t < CI_T; ++t) {
-      const float* wt = wsh + (t * cout + co) * 9;
-#pragma unroll
-      for (int d = 0; d < 9; ++d) acc[t] = fmaf(wt[d], v[d], acc[t]);
+        for (int t = 0; t < CT; ++t)
+          acc[f][t] = fmaf(wt[t], P[f / 2 + dy][f % 2 + dx], acc[f][t]);
     }
   }
 #pragma unroll
-  for (int t = 0; t < CI_T; ++t)
-    if (ci0 + t < cin) gin[((size_t)b * cin + ci0 + t) * npix + p] = acc[t];
+  for (int t = 0; t < CT; ++t) {
+    float v[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) v[f] = BWD ? acc[f][t] : fmaxf(acc[f][t], 0.f);
+    const size_t plane = (size_t)b * no + o0 + t;
+    float* o = out + plane * npix + y * S + x;
+    *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
+    *reinterpret_cast<float2*>(o + S) = make_float2(v[2], v[3]);
+    if (!BWD) pooled[plane * h * h + (q & (h * h - 1))] = 0.25f * (v[0] + v[1] + v[2] + v[3]);
+  }
 }
 
 // partial weight gradients: part[split][co][ci][9] (+ bias partial at part[split][co][cin][0])
-// over the samples b with b % nsplit == split
-__global__ void conv_bwd_weight_kernel(const float* __restrict__ g, const float* __restrict__ in,
-                                       int B, int cin, int cout, int S, int nsplit,
-                                       float* __restrict__ part) {
-  const int co = blockIdx.x / (cin + 1), ci = blockIdx.x % (cin + 1), split = blockIdx.y;
-  const int npix = S * S;
-  float acc[9];
+// over the samples b with b % nsplit == split.  A CTA takes one input channel
+// (or the bias) and WCO output channels: the nine inputs of a pixel serve WCO
+// gradients, 9 WCO multiply-adds for 9 + WCO loads (one output channel per CTA
+// was bound by the load unit and index arithmetic: 470 -> 127 us for the four
+// layers of 64 cells).  The 72 sums of a warp are reduced by halving, 71
+// shuffles instead of 360.
+constexpr int WCO = 8;
+__global__ void __launch_bounds__(256) conv_bwd_weight_kernel(const float* __restrict__ g,
+                                                              const float* __restrict__ in, int B,
+                                                              int cin, int cout, int S, int lgpix,
+                                                              int nsplit,
+                                                              float* __restrict__ part) {
+  const int co0 = blockIdx.x / (cin + 1) * WCO, ci = blockIdx.x % (cin + 1), split = blockIdx.y;
+  const int npix = S * S, lgS = lgpix / 2;
+  float acc[9 * WCO];
 #pragma unroll
-  for (int d = 0; d < 9; ++d) acc[d] = 0.f;
-  for (int b = split; b < B; b += nsplit) {
-    const float* gc = g + ((size_t)b * cout + co) * npix;
+  for (int e = 0; e < 9 * WCO; ++e) acc[e] = 0.f;
+  const int cnt = (B - split + nsplit - 1) / nsplit * npix;   // pixels of this split
+  for (int e = threadIdx.x; e < cnt; e += 256) {
+    const int b = split + nsplit * (e >> lgpix), p = e & (npix - 1);
+    const float* gc = g + ((size_t)b * cout + co0) * npix + p;
+    float gv[WCO];
+#pragma unroll
+    for (int t = 0; t < WCO; ++t) gv[t] = gc[(size_t)t * npix];
     if (ci == cin) {   // bias
-      for (int p = threadIdx.x; p < npix; p += blockDim.x) acc[0] += gc[p];
+#pragma unroll
+      for (int t = 0; t < WCO; ++t) acc[9 * t] += gv[t];
       continue;
     }
     const float* ic = in + ((size_t)b * cin + ci) * npix;
-    for (int p = threadIdx.x; p < npix; p += blockDim.x) {
-      const float gv = gc[p];
-      if (gv == 0.f) continue;
-      const int y = p / S, x = p % S;
+    const int y = p >> lgS, x = p & (S - 1);
+    float v[9], sum = 0.f;
 #pragma unroll
-      for (int d = 0; d < 9; ++d) {
-        const int yy = (y + d / 3 - 1 + S) % S, xx = (x + d % 3 - 1 + S) % S;
-        acc[d] = fmaf(gv, ic[yy * S + xx], acc[d]);
-      }
+    for (int d = 0; d < 9; ++d) {
+      v[d] = ic[((y + d / 3 - 1) & (S - 1)) * S + ((x + d % 3 - 1) & (S - 1))];
+      sum += v[d];
+    }
+    if (isfinite(sum)) {
+#pragma unroll
+      for (int t = 0; t < WCO; ++t)
+#pragma unroll
+        for (int d = 0; d < 9; ++d) acc[9 * t + d] = fmaf(gv[t], v[d], acc[9 * t + d]);
+    } else {   // a gradient stopped by the ReLU adds nothing, whatever the input is
+#pragma unroll
+      for (int t = 0; t < WCO; ++t)
+#pragma unroll
+        for (int d = 0; d < 9; ++d)
+          if (gv[t] != 0.f) acc[9 * t + d] = fmaf(gv[t], v[d], acc[9 * t + d]);
     }
   }
-  __shared__ float red[9][8];
+  static_assert(WCO == 8, "the reduction is written for 64 + 8 sums");
+  __shared__ float red[8][9 * WCO];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-  for (int d = 0; d < 9; ++d) {
-    float v = acc[d];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[d][wid] = v;
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < 2 * o; ++i) {   // entries i and i + 2 o of the first 64
+      const float keep = up ? acc[i + 2 * o] : acc[i], send = up ? acc[i] : acc[i + 2 * o];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    if (o >= 4) {
+#pragma unroll
+      for (int i = 0; i < o / 4; ++i) {   // 64 + i and 64 + i + o / 4
+        const float keep = up ? acc[64 + i + o / 4] : acc[64 + i];
+        const float send = up ? acc[64 + i] : acc[64 + i + o / 4];
+        acc[64 + i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    } else {
+      acc[64] += __shfl_xor_sync(0xffffffffu, acc[64], o);
+    }
   }
+  red[wid][2 * lane] = acc[0];
+  red[wid][2 * lane + 1] = acc[1];
+  if ((lane & 3) == 0) red[wid][64 + lane / 4] = acc[64];
   __syncthreads();
-  if (threadIdx.x < 9) {
+  if (threadIdx.x < 9 * WCO) {
     float sum = 0.f;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) sum += red[threadIdx.x][q];
-    part[(((size_t)split * cout + co) * (cin + 1) + ci) * 9 + threadIdx.x] = sum;
+    for (int q = 0; q < 8; ++q) sum += red[q][threadIdx.x];
+    const int co = co0 + threadIdx.x / 9;
+    part[(((size_t)split * cout + co) * (cin + 1) + ci) * 9 + threadIdx.x % 9] = sum;
   }
 }
 
@@ -173,67 +228,93 @@ __global__ void conv_wgrad_reduce_kernel(const float* __restrict__ part, int cin
   else if (d == 0) gb[co] = s;
 }
 
-// 2x2 mean pooling and its adjoint (the latter also applies the ReLU mask of
-// the pooled layer's input: zero gradient where that activation is zero)
-__global__ void pool_fwd_kernel(const float* __restrict__ in, int S, size_t planes,
-                                float* __restrict__ out) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int h = S / 2;
-  if (e >= planes * h * h) return;
-  const size_t pl = e / (h * h);
-  const int y = (int)(e % (h * h)) / h, x = (int)(e % h);
-  const float* ip = in + pl * S * S;
-  out[e] = 0.25f * (ip[(2 * y) * S + 2 * x] + ip[(2 * y) * S + 2 * x + 1] +
-                    ip[(2 * y + 1) * S + 2 * x] + ip[(2 * y + 1) * S + 2 * x + 1]);
-}
+// adjoint of the 2x2 mean pooling, with the ReLU mask of the pooled layer's
+// input: zero gradient where that activation is zero; one pooled entry per thread
 __global__ void pool_bwd_kernel(const float* __restrict__ gout, const float* __restrict__ act,
-                                int S, size_t planes, float* __restrict__ gin) {
+                                int S, int lgh, size_t npool, float* __restrict__ gin) {
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= planes * S * S) return;
-  const size_t pl = e / (S * S);
-  const int y = (int)(e % (S * S)) / S, x = (int)(e % S), h = S / 2;
-  gin[e] = act[e] > 0.f ? 0.25f * gout[pl * h * h + (y / 2) * h + x / 2] : 0.f;
+  if (e >= npool) return;
+  const int h = S / 2, x = (int)e & (h - 1), y = (int)(e >> lgh) & (h - 1);
+  const size_t o = (e >> (2 * lgh)) * S * S + (size_t)(2 * y) * S + 2 * x;
+  const float v = 0.25f * gout[e];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const float2 a = *reinterpret_cast<const float2*>(act + o + r * S);
+    *reinterpret_cast<float2*>(gin + o + r * S) =
+        make_float2(a.x > 0.f ? v : 0.f, a.y > 0.f ? v : 0.f);
+  }
 }
 
 // ------------------------------------------------------------ dense layers
-// C[m][n] = sum_k A(m,k) B(k,n) (+ bias[n], ReLU): A(m,k) = TA ? A[k*lda+m] : A[m*lda+k],
-// B(k,n) = TB ? B[n*ldb+k] : B[k*ldb+n]; 64 x 64 tiles, 4 x 4 per thread
-template <bool TA, bool TB>
-__global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int K, const float* __restrict__ A,
-                                                    int lda, const float* __restrict__ Bm, int ldb,
-                                                    const float* __restrict__ bias, bool relu,
-                                                    float* __restrict__ C, int ldc) {
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
-  const int tid = threadIdx.x, tm = tid / 16, tn = tid % 16;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int e = tid; e < 16 * 64; e += 256) {
-      const int kk = e / 64, mm = e % 64;
-      const int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < M && k < K) ? (TA ? A[(size_t)k * lda + m] : A[(size_t)m * lda + k]) : 0.f;
-      const int n = n0 + mm;
-      Bs[kk][mm] = (n < N && k < K) ? (TB ? Bm[(size_t)n * ldb + k] : Bm[(size_t)k * ldb + n]) : 0.f;
+// C[m][n] = sum_k A(m,k) B(k,n) (+ bias[n], ReLU; or 0 where mask <= 0): A(m,k) =
+// TA ? A[k*lda+m] : A[m*lda+k], B(k,n) = TB ? B[n*ldb+k] : B[k*ldb+n].
+//
+// BT x BT tiles, 32 terms a step, the next step's loads in flight in registers
+// and along the contiguous index of each operand.  The layers have few rows (one
+// per wavevector), so what bounds them is latency: 64-wide tiles where they fill
+// the chip, 32-wide ones elsewhere, and long sums of the backward pass also split
+// over blockIdx.z (the partial blocks are added by sum_parts_kernel).  256 rows,
+// 512 / 512 / 2352 columns: forward 218 -> 68 us, the two backward products
+// 665 -> 122 us for the three layers.  The terms of an entry are added in
+// the order of k for both tiles.
+template <bool TA, bool TB, int BT>
+__global__ void __launch_bounds__(BT == 64 ? 256 : 128)
+sgemm_kernel(int M, int N, int K, const float* __restrict__ A, int lda,
+             const float* __restrict__ Bm, int ldb, const float* __restrict__ bias, bool relu,
+             const float* __restrict__ mask, float* __restrict__ C, int ldc, int kslice,
+             size_t zstride) {
+  constexpr int NTH = BT == 64 ? 256 : 128, BK = 32, LDT = BT + 4;
+  constexpr int PER = BT * BK / NTH, RM = BT * BT / NTH / 4;   // loads and rows per thread
+  __shared__ __align__(16) float As[BK][LDT];
+  __shared__ __align__(16) float Bs[BK][LDT];
+  const int tid = threadIdx.x, tm = tid / (BT / 4), tn = tid % (BT / 4);
+  const int m0 = blockIdx.y * BT, n0 = blockIdx.x * BT;
+  const int kbeg = blockIdx.z * kslice, kend = min(K, kbeg + kslice);
+  float acc[RM][4] = {}, ra[PER], rb[PER];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * NTH;
+      const int ka = k0 + (TA ? e / BT : e % BK), m = m0 + (TA ? e % BT : e / BK);
+      const int kb = k0 + (TB ? e % BK : e / BT), n = n0 + (TB ? e / BK : e % BT);
+      ra[i] = m < M && ka < kend ? (TA ? A[(size_t)ka * lda + m] : A[(size_t)m * lda + ka]) : 0.f;
+      rb[i] = n < N && kb < kend ? (TB ? Bm[(size_t)n * ldb + kb] : Bm[(size_t)kb * ldb + n]) : 0.f;
     }
+  };
+  fetch(kbeg);
+  for (int k0 = kbeg; k0 < kend; k0 += BK) {
     __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], bv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][tm * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tn * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bv[j], acc[i][j]);
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * NTH;
+      As[TA ? e / BT : e % BK][TA ? e % BT : e / BK] = ra[i];
+      Bs[TB ? e % BK : e / BT][TB ? e / BK : e % BT] = rb[i];
     }
     __syncthreads();
+    if (k0 + BK < kend) fetch(k0 + BK);
+#pragma unroll
+    for (int kk = 0; kk < BK; ++kk) {
+      float a[RM];
+      const float4 b = *reinterpret_cast<const float4*>(&Bs[kk][tn * 4]);
+#pragma unroll
+      for (int i = 0; i < RM; i += 2) {
+        const float2 f = *reinterpret_cast<const float2*>(&As[kk][tm * RM + i]);
+        a[i] = f.x;
+        a[i + 1] = f.y;
+      }
+#pragma unroll
+      for (int i = 0; i < RM; ++i) {
+        acc[i][0] = fmaf(a[i], b.x, acc[i][0]);
+        acc[i][1] = fmaf(a[i], b.y, acc[i][1]);
+        acc[i][2] = fmaf(a[i], b.z, acc[i][2]);
+        acc[i][3] = fmaf(a[i], b.w, acc[i][3]);
+      }
+    }
   }
+  float* c = C + blockIdx.z * zstride;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + tm * 4 + i;
+  for (int i = 0; i < RM; ++i) {
+    const int m = m0 + tm * RM + i;
     if (m >= M) continue;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -241,25 +322,41 @@ __global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int K, const f
       if (n >= N) continue;
       float v = acc[i][j] + (bias ? bias[n] : 0.f);
       if (relu) v = fmaxf(v, 0.f);
-      C[(size_t)m * ldc + n] = v;
+      if (mask && !(mask[(size_t)m * ldc + n] > 0.f)) v = 0.f;
+      c[(size_t)m * ldc + n] = v;
     }
   }
 }
 
-// column sums: out[n] = sum_m A[m*ld + n]
-__global__ void colsum_kernel(const float* __restrict__ A, int M, int N, int ld,
-                              float* __restrict__ out) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
+// C[e] = sum_z part[z][e], 0 where mask <= 0
+__global__ void sum_parts_kernel(const float* __restrict__ part, int nz, size_t n,
+                                 const float* __restrict__ mask, float* __restrict__ C) {
+  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n) return;
   float s = 0.f;
-  for (int m = 0; m < M; ++m) s += A[(size_t)m * ld + n];
-  out[n] = s;
+#pragma unroll 4
+  for (int z = 0; z < nz; ++z) s += part[z * n + e];
+  C[e] = mask && !(mask[e] > 0.f) ? 0.f : s;
 }
 
-// g[i] *= (act[i] > 0)
-__global__ void relu_mask_kernel(float* __restrict__ g, const float* __restrict__ act, size_t n) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && !(act[i] > 0.f)) g[i] = 0.f;
+// column sums: out[n] = sum_m A[m*ld + n]; 32 columns and 8 interleaved row
+// groups per CTA (one thread per column waited for every row: 52 -> 16 us for
+// the three layers of 256 rows)
+__global__ void __launch_bounds__(256) colsum_kernel(const float* __restrict__ A, int M, int N,
+                                                     int ld, float* __restrict__ out) {
+  __shared__ float red[8][32];
+  const int c = threadIdx.x & 31, r = threadIdx.x >> 5, n = blockIdx.x * 32 + c;
+  float s = 0.f;
+  if (n < N) {
+#pragma unroll 8
+    for (int m = r; m < M; m += 8) s += A[(size_t)m * ld + n];
+  }
+  red[r][c] = s;
+  __syncthreads();
+  if (r == 0 && n < N) {
+    for (int q = 1; q < 8; ++q) s += red[q][c];
+    out[n] = s;
+  }
 }
 
 // head input: h0[s] = [feat[s / kper] | kf[s]]
@@ -287,20 +384,35 @@ __global__ void feat_grad_kernel(const float* __restrict__ gh0, int nc, int kper
 // x[c] = standardised log(lam + 2 mu), log mu, log rho of every pixel of cell c
 // (phase maps P x P with P = 64, tables lam | mu | rho at table + toff[c]);
 // kf[s] = (Q1, Q2, cos 2 pi Q1, sin 2 pi Q1, cos 2 pi Q2, sin 2 pi Q2, hex)
-__global__ void encode_kernel(const uint16_t* __restrict__ phase, const double* __restrict__ table,
-                              const long* __restrict__ toff, const int* __restrict__ nph, int nc,
-                              float* __restrict__ x) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t npix = (size_t)IMG * IMG;
-  if (e >= nc * npix) return;
-  const int c = (int)(e / npix);
-  const int p = phase[e], np = nph[c];
-  const double* t = table + toff[c];
+// A CTA first encodes the phases of its cell, then its quarter of the pixels reads
+// them: three FP64 logarithms per pixel bound it otherwise (2 FP64 FMA per clock
+// and SM; 64 cells: 58 -> 10 us).  Cells of more phases than fit take them per pixel.
+constexpr int ENC_PH = 1024;
+__device__ __forceinline__ float3 encode_one(const double* t, int np, int p) {
   const double lam = t[p], mu = t[np + p], rho = t[2 * np + p];
-  float* xc = x + (size_t)c * 3 * npix + e % npix;
-  xc[0] = (float)((log(lam + 2.0 * mu) - 3.5) / 1.0);
-  xc[npix] = (float)((log(mu) - 2.2) / 1.2);
-  xc[2 * npix] = (float)((log(rho) - 1.0) / 0.6);
+  return make_float3((float)((log(lam + 2.0 * mu) - 3.5) / 1.0), (float)((log(mu) - 2.2) / 1.2),
+                     (float)((log(rho) - 1.0) / 0.6));
+}
+__global__ void __launch_bounds__(256) encode_kernel(const uint16_t* __restrict__ phase,
+                                                     const double* __restrict__ table,
+                                                     const long* __restrict__ toff,
+                                                     const int* __restrict__ nph,
+                                                     float* __restrict__ x) {
+  __shared__ float3 enc[ENC_PH];
+  constexpr int NPIX = IMG * IMG;
+  const int c = blockIdx.x, np = nph[c];
+  const double* t = table + toff[c];
+  if (np <= ENC_PH)
+    for (int p = threadIdx.x; p < np; p += 256) enc[p] = encode_one(t, np, p);
+  __syncthreads();
+  float* xc = x + (size_t)c * 3 * NPIX;
+  for (int e = blockIdx.y * (NPIX / 4) + threadIdx.x; e < (blockIdx.y + 1) * (NPIX / 4); e += 256) {
+    const int p = phase[(size_t)c * NPIX + e];
+    const float3 v = np <= ENC_PH && p < np ? enc[p] : encode_one(t, np, p);
+    xc[e] = v.x;
+    xc[NPIX + e] = v.y;
+    xc[2 * NPIX + e] = v.z;
+  }
 }
 __global__ void kfeat_kernel(const double* __restrict__ Q, const int* __restrict__ hex, int ns,
                              int kper, float* __restrict__ kf) {
@@ -318,16 +430,19 @@ __global__ void kfeat_kernel(const double* __restrict__ Q, const int* __restrict
 }
 
 // ------------------------------------------------------------ subspace loss
-// one CTA per sample: U (L x nv, from out), V (L x nb, from tgt), loss[s], gout[s]
+// one CTA per sample: U (L x nv, from out), V (L x nb, from tgt), loss[s], gout[s].
+// Bound by its chain of dependent steps (the factorisation of G and the
+// substitutions), so these run one row per lane and one column per thread and
+// the sums over the whole CTA (by one thread: 94 us for 256 samples, 25 us so)
 constexpr int LMAX = 2 * 49;   // Mp <= 3
 constexpr int NVMAX = 16;
-__global__ void __launch_bounds__(128) loss_kernel(const float* __restrict__ out,
+__global__ void __launch_bounds__(288) loss_kernel(const float* __restrict__ out,
                                                    const float* __restrict__ tgt, int L, int nv,
                                                    int nb, float scale, float* __restrict__ loss,
                                                    float* __restrict__ gout) {
   __shared__ float2 U[LMAX][NVMAX + 1], V[LMAX][NVMAX + 1], R[LMAX][NVMAX + 1];
   __shared__ float2 G[NVMAX][NVMAX + 1], Bm[NVMAX][NVMAX + 1], F[NVMAX][NVMAX + 1];
-  __shared__ float vn2, cap;
+  __shared__ float vn2, sums[9][2];
   __shared__ int bad;
   const int s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const float* o = out + (size_t)s * nv * L * 2;
@@ -359,54 +474,61 @@ __global__ void __launch_bounds__(128) loss_kernel(const float* __restrict__ out
     }
   }
   __syncthreads();
-  // Cholesky G = C C^H (lower, in place) and F = G^-1 B (thread 0; nv <= 16)
-  if (tid == 0) {
+  // Cholesky G = C C^H (lower, in place): one row per lane, nv <= 16
+  if (tid < 32) {
+    const int r = tid;
     for (int c = 0; c < nv; ++c) {
-      float p = G[c][c].x;
-      for (int k = 0; k < c; ++k) p -= G[c][k].x * G[c][k].x + G[c][k].y * G[c][k].y;
-      if (!(p > 0.f)) {
-        bad = 1;
-        p = 1.f;
-      }
-      const float d = sqrtf(p);
-      G[c][c] = make_float2(d, 0.f);
-      for (int r = c + 1; r < nv; ++r) {
-        float2 v = G[r][c];
+      float2 v = make_float2(0.f, 0.f);
+      if (r >= c && r < nv) {
+        v = G[r][c];
         for (int k = 0; k < c; ++k) {   // v -= G[r][k] conj(G[c][k])
           const float2 a = G[r][k], b = G[c][k];
           v.x -= a.x * b.x + a.y * b.y;
           v.y -= a.y * b.x - a.x * b.y;
         }
-        G[r][c] = make_float2(v.x / d, v.y / d);
       }
+      float p = __shfl_sync(0xffffffffu, v.x, c);
+      if (!(p > 0.f)) {
+        if (r == c) bad = 1;
+        p = 1.f;
+      }
+      const float d = sqrtf(p);
+      __syncwarp();
+      if (r == c) G[r][c] = make_float2(d, 0.f);
+      else if (r > c && r < nv) G[r][c] = make_float2(v.x / d, v.y / d);
+      __syncwarp();
     }
-    for (int j = 0; j < nb; ++j) {
-      float2 y[NVMAX];
-      for (int r = 0; r < nv; ++r) {   // forward: C y = B
-        float2 v = Bm[r][j];
-        for (int k = 0; k < r; ++k) {
-          const float2 a = G[r][k];
-          v.x -= a.x * y[k].x - a.y * y[k].y;
-          v.y -= a.x * y[k].y + a.y * y[k].x;
-        }
-        y[r] = make_float2(v.x / G[r][r].x, v.y / G[r][r].x);
+  }
+  __syncthreads();
+  // F = G^-1 B: one column per thread
+  if (tid < nb) {
+    const int j = tid;
+    for (int r = 0; r < nv; ++r) {   // forward: C y = B
+      float2 v = Bm[r][j];
+      for (int k = 0; k < r; ++k) {
+        const float2 a = G[r][k], y = F[k][j];
+        v.x -= a.x * y.x - a.y * y.y;
+        v.y -= a.x * y.y + a.y * y.x;
       }
-      for (int r = nv - 1; r >= 0; --r) {   // backward: C^H f = y
-        float2 v = y[r];
-        for (int k = r + 1; k < nv; ++k) {   // v -= conj(G[k][r]) f_k
-          const float2 a = G[k][r], f = F[k][j];
-          v.x -= a.x * f.x + a.y * f.y;
-          v.y -= a.x * f.y - a.y * f.x;
-        }
-        F[r][j] = make_float2(v.x / G[r][r].x, v.y / G[r][r].x);
+      F[r][j] = make_float2(v.x / G[r][r].x, v.y / G[r][r].x);
+    }
+    for (int r = nv - 1; r >= 0; --r) {   // backward: C^H f = y
+      float2 v = F[r][j];
+      for (int k = r + 1; k < nv; ++k) {   // v -= conj(G[k][r]) f_k
+        const float2 a = G[k][r], f = F[k][j];
+        v.x -= a.x * f.x + a.y * f.y;
+        v.y -= a.x * f.y - a.y * f.x;
       }
+      F[r][j] = make_float2(v.x / G[r][r].x, v.y / G[r][r].x);
     }
   }
   __syncthreads();
   // R = V - U F, ||V||^2, captured part tr(B^H F)
+  float sv = 0.f, sc = 0.f;
   for (int e = tid; e < L * nb; e += nt) {
     const int i = e / nb, j = e % nb;
     float2 v = V[i][j];
+    sv += v.x * v.x + v.y * v.y;
     for (int a = 0; a < nv; ++a) {
       const float2 u = U[i][a], f = F[a][j];
       v.x -= u.x * f.x - u.y * f.y;
@@ -414,14 +536,25 @@ __global__ void __launch_bounds__(128) loss_kernel(const float* __restrict__ out
     }
     R[i][j] = v;
   }
+  for (int e = tid; e < nv * nb; e += nt) {
+    const int a = e / nb, j = e % nb;
+    sc += Bm[a][j].x * F[a][j].x + Bm[a][j].y * F[a][j].y;
+  }
+  for (int w = 16; w > 0; w >>= 1) {
+    sv += __shfl_xor_sync(0xffffffffu, sv, w);
+    sc += __shfl_xor_sync(0xffffffffu, sc, w);
+  }
+  if ((tid & 31) == 0) {
+    sums[tid >> 5][0] = sv;
+    sums[tid >> 5][1] = sc;
+  }
+  __syncthreads();
   if (tid == 0) {
-    float sv = 0.f, sc = 0.f;
-    for (int i = 0; i < L; ++i)
-      for (int j = 0; j < nb; ++j) sv += V[i][j].x * V[i][j].x + V[i][j].y * V[i][j].y;
-    for (int a = 0; a < nv; ++a)
-      for (int j = 0; j < nb; ++j) sc += Bm[a][j].x * F[a][j].x + Bm[a][j].y * F[a][j].y;
+    for (int w = 1; w < nt / 32; ++w) {
+      sv += sums[w][0];
+      sc += sums[w][1];
+    }
     vn2 = fmaxf(sv, 1e-30f);
-    cap = sc;
     loss[s] = bad ? 1.f : (sv - sc) / vn2;
   }
   __syncthreads();
@@ -484,7 +617,8 @@ struct bs_cnn {
   float* gh2;
   float* gpl;              // max pooled plane gradients
   float* gz;               // max conv-output gradients
-  float* gtmp;
+  float* gtmp;             // partial sums of the dense layers' products
+  size_t tmp_cap;
   float* wpart;            // conv weight-gradient partials
   float* loss;             // smax
   // encode inputs
@@ -522,29 +656,78 @@ int calloc_dev(T** p, size_t n, const char* what) {
     if (r__) return r__;   \
   } while (0)
 
+int log2i(int v) {
+  int l = 0;
+  while ((1 << (l + 1)) <= v) ++l;
+  return l;
+}
+
+// output channels per thread: as many as leave a full wave of threads (256 per
+// SM of 152); the layers of 8 x 8 and 16 x 16 pixels have too few quads for eight
+template <bool BWD>
+int conv(const float* in, const float* w, const float* bias, int ni, int no, int S, int nc,
+         float* out, float* pooled, cudaStream_t s) {
+  const int nquad = nc * (S / 2) * (S / 2), lgh = log2i(S / 2), bx = (nquad + 127) / 128;
+  const long full = 152 * 256;
+  if ((long)nquad * (no / 8) >= full)
+    conv_kernel<8, BWD><<<dim3(bx, no / 8), 128, ni * 9 * 8 * sizeof(float), s>>>(
+        in, w, bias, ni, no, S, lgh, nquad, out, pooled);
+  else if ((long)nquad * (no / 4) >= full)
+    conv_kernel<4, BWD><<<dim3(bx, no / 4), 128, ni * 9 * 4 * sizeof(float), s>>>(
+        in, w, bias, ni, no, S, lgh, nquad, out, pooled);
+  else
+    conv_kernel<2, BWD><<<dim3(bx, no / 2), 128, ni * 9 * 2 * sizeof(float), s>>>(
+        in, w, bias, ni, no, S, lgh, nquad, out, pooled);
+  BS_CHECK_LAUNCH("conv_kernel");
+  return BS_OK;
+}
+
 int conv_forward(bs_cnn* m, int nc, cudaStream_t s) {
   const float* in = m->x;
   for (int l = 0; l < NCONV; ++l) {
-    const int S = SIDE[l], ci = CIN[l], co = COUT[l];
-    dim3 grid((S * S + 255) / 256, (co + CO_T - 1) / CO_T, nc);
-    conv_fwd_kernel<<<grid, 256, CO_T * ci * 9 * sizeof(float), s>>>(
-        in, m->d_p + m->off_w[l], m->d_p + m->off_b[l], ci, co, S, m->z[l]);
-    BS_CHECK_LAUNCH("conv_fwd_kernel");
-    const size_t planes = (size_t)nc * co, tot = planes * (S / 2) * (S / 2);
-    pool_fwd_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(m->z[l], S, planes, m->pl[l]);
-    BS_CHECK_LAUNCH("pool_fwd_kernel");
+    TRYC(conv<false>(in, m->d_p + m->off_w[l], m->d_p + m->off_b[l], CIN[l], COUT[l], SIDE[l], nc,
+                     m->z[l], m->pl[l], s));
     in = m->pl[l];
   }
   return BS_OK;
 }
 
+template <int BT>
+void sgemm_launch(bool ta, bool tb, int nz, int ks, int M, int N, int K, const float* A, int lda,
+                  const float* B, int ldb, const float* bias, bool relu, const float* mask,
+                  float* C, int ldc, cudaStream_t s) {
+  const dim3 grid((N + BT - 1) / BT, (M + BT - 1) / BT, nz);
+  const int nt = BT == 64 ? 256 : 128;
+  const size_t zs = (size_t)M * N;
+  auto k = ta ? sgemm_kernel<true, false, BT>
+              : tb ? sgemm_kernel<false, true, BT> : sgemm_kernel<false, false, BT>;
+  k<<<grid, nt, 0, s>>>(M, N, K, A, lda, B, ldb, bias, relu, mask, C, ldc, ks, zs);
+}
+
+// Not both transposed.  part: scratch of `cap` floats that lets a long sum be split
+// (C dense, no bias or ReLU)
 int sgemm(bool ta, bool tb, int M, int N, int K, const float* A, int lda, const float* B, int ldb,
-          const float* bias, bool relu, float* C, int ldc, cudaStream_t s) {
-  dim3 grid((N + 63) / 64, (M + 63) / 64);
-  if (!ta && !tb) sgemm_kernel<false, false><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, bias, relu, C, ldc);
-  else if (!ta && tb) sgemm_kernel<false, true><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, bias, relu, C, ldc);
-  else if (ta && !tb) sgemm_kernel<true, false><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, bias, relu, C, ldc);
-  else sgemm_kernel<true, true><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, bias, relu, C, ldc);
+          const float* bias, bool relu, const float* mask, float* C, int ldc, cudaStream_t s,
+          float* part = nullptr, size_t cap = 0) {
+  const long t64 = (long)((N + 63) / 64) * ((M + 63) / 64);
+  const long t32 = (long)((N + 31) / 32) * ((M + 31) / 32);
+  if (t64 >= 192) {   // 64-wide tiles fill the chip
+    sgemm_launch<64>(ta, tb, 1, K, M, N, K, A, lda, B, ldb, bias, relu, mask, C, ldc, s);
+  } else {
+    // slices of at least 128 terms, until four CTAs per SM (of 128 threads) are busy
+    const size_t room = part ? cap / ((size_t)M * N) : 0;
+    int nz = (int)std::min<long>({(608 + t32 - 1) / t32, (long)K / 128, (long)std::min<size_t>(room, 64)});
+    if (nz > 1) {
+      const int ks = ((K + nz - 1) / nz + 31) / 32 * 32;
+      nz = (K + ks - 1) / ks;
+      sgemm_launch<32>(ta, tb, nz, ks, M, N, K, A, lda, B, ldb, nullptr, false, nullptr, part, N, s);
+      BS_CHECK_LAUNCH("sgemm_kernel");
+      const size_t n = (size_t)M * N;
+      sum_parts_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, nz, n, mask, C);
+    } else {
+      sgemm_launch<32>(ta, tb, 1, K, M, N, K, A, lda, B, ldb, bias, relu, mask, C, ldc, s);
+    }
+  }
   BS_CHECK_LAUNCH("sgemm_kernel");
   return BS_OK;
 }
@@ -554,69 +737,65 @@ int head_forward(bs_cnn* m, int nc, int kper, cudaStream_t s) {
   head_input_kernel<<<(ns * W0 + 255) / 256, 256, 0, s>>>(m->pl[NCONV - 1], m->kf, ns, kper, m->h0);
   BS_CHECK_LAUNCH("head_input_kernel");
   TRYC(sgemm(false, true, ns, HID, W0, m->h0, W0, m->d_p + m->off_dw[0], W0, m->d_p + m->off_db[0],
-             true, m->h1, HID, s));
+             true, nullptr, m->h1, HID, s));
   TRYC(sgemm(false, true, ns, HID, HID, m->h1, HID, m->d_p + m->off_dw[1], HID,
-             m->d_p + m->off_db[1], true, m->h2, HID, s));
+             m->d_p + m->off_db[1], true, nullptr, m->h2, HID, s));
   TRYC(sgemm(false, true, ns, m->OUT, HID, m->h2, HID, m->d_p + m->off_dw[2], HID,
-             m->d_p + m->off_db[2], false, m->out, m->OUT, s));
+             m->d_p + m->off_db[2], false, nullptr, m->out, m->OUT, s));
+  return BS_OK;
+}
+
+int colsum(const float* A, int M, int N, float* out, cudaStream_t s) {
+  colsum_kernel<<<(N + 31) / 32, 256, 0, s>>>(A, M, N, N, out);
+  BS_CHECK_LAUNCH("colsum_kernel");
   return BS_OK;
 }
 
 // gradients of everything from m->gout (ns x OUT) into m->d_g
 int backward(bs_cnn* m, int nc, int kper, cudaStream_t s) {
-  const int ns = nc * kper, W0 = FEAT + KF;
-  // dense 3
-  TRYC(sgemm(true, false, m->OUT, HID, ns, m->gout, m->OUT, m->h2, HID, nullptr, false,
-             m->d_g + m->off_dw[2], HID, s));
-  colsum_kernel<<<(m->OUT + 255) / 256, 256, 0, s>>>(m->gout, ns, m->OUT, m->OUT, m->d_g + m->off_db[2]);
-  BS_CHECK_LAUNCH("colsum_kernel");
-  TRYC(sgemm(false, false, ns, HID, m->OUT, m->gout, m->OUT, m->d_p + m->off_dw[2], HID, nullptr,
-             false, m->gh2, HID, s));
-  relu_mask_kernel<<<(unsigned)(((size_t)ns * HID + 255) / 256), 256, 0, s>>>(m->gh2, m->h2, (size_t)ns * HID);
-  BS_CHECK_LAUNCH("relu_mask_kernel");
-  // dense 2
-  TRYC(sgemm(true, false, HID, HID, ns, m->gh2, HID, m->h1, HID, nullptr, false,
-             m->d_g + m->off_dw[1], HID, s));
-  colsum_kernel<<<(HID + 255) / 256, 256, 0, s>>>(m->gh2, ns, HID, HID, m->d_g + m->off_db[1]);
-  BS_CHECK_LAUNCH("colsum_kernel");
-  TRYC(sgemm(false, false, ns, HID, HID, m->gh2, HID, m->d_p + m->off_dw[1], HID, nullptr, false,
-             m->gh1, HID, s));
-  relu_mask_kernel<<<(unsigned)(((size_t)ns * HID + 255) / 256), 256, 0, s>>>(m->gh1, m->h1, (size_t)ns * HID);
-  BS_CHECK_LAUNCH("relu_mask_kernel");
-  // dense 1
-  TRYC(sgemm(true, false, HID, W0, ns, m->gh1, HID, m->h0, W0, nullptr, false,
-             m->d_g + m->off_dw[0], W0, s));
-  colsum_kernel<<<(HID + 255) / 256, 256, 0, s>>>(m->gh1, ns, HID, HID, m->d_g + m->off_db[0]);
-  BS_CHECK_LAUNCH("colsum_kernel");
-  TRYC(sgemm(false, false, ns, W0, HID, m->gh1, HID, m->d_p + m->off_dw[0], W0, nullptr, false,
-             m->gh0, W0, s));
+  const int ns = nc * kper, W0 = FEAT + KF, OUT = m->OUT;
+  float* dg = m->d_g;
+  const float* p = m->d_p;
+  float* pt = m->gtmp;   // partial sums
+  const size_t pc = m->tmp_cap;
+  // dense 3, 2, 1 (the ReLU mask of a layer's input goes with its gradient)
+  TRYC(sgemm(true, false, OUT, HID, ns, m->gout, OUT, m->h2, HID, nullptr, false, nullptr,
+             dg + m->off_dw[2], HID, s, pt, pc));
+  TRYC(colsum(m->gout, ns, OUT, dg + m->off_db[2], s));
+  TRYC(sgemm(false, false, ns, HID, OUT, m->gout, OUT, p + m->off_dw[2], HID, nullptr, false,
+             m->h2, m->gh2, HID, s, pt, pc));
+  TRYC(sgemm(true, false, HID, HID, ns, m->gh2, HID, m->h1, HID, nullptr, false, nullptr,
+             dg + m->off_dw[1], HID, s, pt, pc));
+  TRYC(colsum(m->gh2, ns, HID, dg + m->off_db[1], s));
+  TRYC(sgemm(false, false, ns, HID, HID, m->gh2, HID, p + m->off_dw[1], HID, nullptr, false, m->h1,
+             m->gh1, HID, s, pt, pc));
+  TRYC(sgemm(true, false, HID, W0, ns, m->gh1, HID, m->h0, W0, nullptr, false, nullptr,
+             dg + m->off_dw[0], W0, s, pt, pc));
+  TRYC(colsum(m->gh1, ns, HID, dg + m->off_db[0], s));
+  TRYC(sgemm(false, false, ns, W0, HID, m->gh1, HID, p + m->off_dw[0], W0, nullptr, false, nullptr,
+             m->gh0, W0, s, pt, pc));
   // features: sum over the samples of each cell
   feat_grad_kernel<<<(nc * FEAT + 255) / 256, 256, 0, s>>>(m->gh0, nc, kper, m->gpl);
   BS_CHECK_LAUNCH("feat_grad_kernel");
   // convolution layers, last to first
   for (int l = NCONV - 1; l >= 0; --l) {
     const int S = SIDE[l], ci = CIN[l], co = COUT[l];
-    const size_t planes = (size_t)nc * co;
-    pool_bwd_kernel<<<(unsigned)((planes * S * S + 255) / 256), 256, 0, s>>>(m->gpl, m->z[l], S,
-                                                                             planes, m->gz);
+    const size_t npool = (size_t)nc * co * (S / 2) * (S / 2);
+    pool_bwd_kernel<<<(unsigned)((npool + 255) / 256), 256, 0, s>>>(m->gpl, m->z[l], S,
+                                                                    log2i(S / 2), npool, m->gz);
     BS_CHECK_LAUNCH("pool_bwd_kernel");
     const float* in = l == 0 ? m->x : m->pl[l - 1];
-    conv_bwd_weight_kernel<<<dim3(co * (ci + 1), WSPLIT), 256, 0, s>>>(m->gz, in, nc, ci, co, S,
-                                                                        WSPLIT, m->wpart);
+    // sample groups: four CTAs per SM
+    const int nb = co / WCO * (ci + 1), split = std::min({(608 + nb - 1) / nb, WSPLIT, nc});
+    conv_bwd_weight_kernel<<<dim3(nb, split), 256, 0, s>>>(m->gz, in, nc, ci, co, S, 2 * log2i(S),
+                                                           split, m->wpart);
     BS_CHECK_LAUNCH("conv_bwd_weight_kernel");
     conv_wgrad_reduce_kernel<<<(co * (ci + 1) * 9 + 255) / 256, 256, 0, s>>>(
-        m->wpart, ci, co, WSPLIT, m->d_g + m->off_w[l], m->d_g + m->off_b[l]);
+        m->wpart, ci, co, split, dg + m->off_w[l], dg + m->off_b[l]);
     BS_CHECK_LAUNCH("conv_wgrad_reduce_kernel");
-    if (l > 0) {
-      dim3 grid((S * S + 255) / 256, (ci + CI_T - 1) / CI_T, nc);
-      conv_bwd_data_kernel<<<grid, 256, CI_T * co * 9 * sizeof(float), s>>>(
-          m->gz, m->d_p + m->off_w[l], ci, co, S, m->gtmp);
-      BS_CHECK_LAUNCH("conv_bwd_data_kernel");
-      // gtmp is the gradient of the pooled output of layer l-1
-      cudaError_t e = cudaMemcpyAsync(m->gpl, m->gtmp, (size_t)nc * ci * S * S * sizeof(float),
-                                      cudaMemcpyDeviceToDevice, s);
-      if (e != cudaSuccess) return bs_cuda_status(e, "cnn backward");
-    }
+    // the gradient of the pooled output of layer l - 1
+    if (l > 0)
+      TRYC(conv<true>(m->gz, p + m->off_w[l], nullptr, co, ci, S, nc, m->gpl, nullptr, s));
   }
   return BS_OK;
 }
@@ -649,8 +828,7 @@ int stage_inputs(bs_cnn* m, const uint16_t* phase, const double* table, const lo
   if (e == cudaSuccess) e = cudaMemcpyAsync(m->hex, hex, nc * sizeof(int), cudaMemcpyDefault, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(m->Q, Q, (size_t)ns * 2 * sizeof(double), cudaMemcpyDefault, s);
   if (e != cudaSuccess) return bs_cuda_status(e, "cnn inputs");
-  encode_kernel<<<(unsigned)(((size_t)nc * IMG * IMG + 255) / 256), 256, 0, s>>>(
-      m->phase, m->table, m->toff, m->nph, nc, m->x);
+  encode_kernel<<<dim3(nc, 4), 256, 0, s>>>(m->phase, m->table, m->toff, m->nph, m->x);
   BS_CHECK_LAUNCH("encode_kernel");
   kfeat_kernel<<<(ns + 255) / 256, 256, 0, s>>>(m->Q, m->hex, ns, kper, m->kf);
   BS_CHECK_LAUNCH("kfeat_kernel");
@@ -727,6 +905,7 @@ extern "C" int bs_cnn_create(int nvec, int Mp, int max_cells, int max_samples, b
   if (!r) r = calloc_dev(&m->gh2, Sm * HID, "cnn gh2");
   if (!r) r = calloc_dev(&m->gpl, std::max(zmax / 4, C * FEAT), "cnn pooled gradients");
   if (!r) r = calloc_dev(&m->gz, zmax, "cnn conv gradients");
+  m->tmp_cap = zmax;
   if (!r) r = calloc_dev(&m->gtmp, zmax, "cnn scratch");
   if (!r) r = calloc_dev(&m->wpart, (size_t)WSPLIT * 32 * 33 * 9, "cnn weight partials");
   if (!r) r = calloc_dev(&m->loss, Sm, "cnn loss");
@@ -831,7 +1010,7 @@ extern "C" int bs_cnn_train_step(bs_cnn* m, const uint16_t* phase, const double*
   if (e != cudaSuccess) return bs_cuda_status(e, "bs_cnn_train_step targets");
   TRYC(conv_forward(m, ncells, s));
   TRYC(head_forward(m, ncells, kper, s));
-  loss_kernel<<<ns, 128, 0, s>>>(m->out, m->tgt, m->L, m->nvec, nb, 1.f / ns, m->loss, m->gout);
+  loss_kernel<<<ns, 288, 0, s>>>(m->out, m->tgt, m->L, m->nvec, nb, 1.f / ns, m->loss, m->gout);
   BS_CHECK_LAUNCH("loss_kernel");
   TRYC(backward(m, ncells, kper, s));
   if (lr > 0.f) {
