@@ -271,6 +271,7 @@ static int ensure_workspace(bs_cell* c, int kb, int nb) {
   TRY(dalloc(&c->d_stat, (size_t)kb, "status"));
   if (c->precision == BS_PREC_MIXED) {
     const int b = bs_mixed_guard(nb, n);
+    TRY(bs_side_create(&c->side));
     TRY(dalloc(&c->d_C32, (size_t)kb * n * n, "C32"));
     TRY(dalloc(&c->d_vec32, (size_t)kb * bs_tridiag_vec_elems(n), "vec32"));
     TRY(dalloc(&c->d_part32, (size_t)kb * bs_tridiag_part_elems(n), "part32"));
@@ -638,6 +639,7 @@ extern "C" int bs_destroy_cell(bs_cell* c) {
   free_workspace(c);
   bs_free_mode_workspace(c);
   free_lob_workspace(c);
+  bs_side_free(c->side);
   cudaFree(c->d_phase);
   cudaFree(c->d_table);
   cudaFree(c->d_E);
@@ -767,7 +769,7 @@ static int solve_chunk_mixed(bs_cell* c, int kb, int nbands, cudaStream_t s) {
   bs_phase_end(c, PH_BUILD, s);
   bs_phase_begin(c, PH_TRID, s);
   TRY(bs_launch_tridiag<float>(c->d_C32, n, kb, c->d_vec32, c->d_part32, c->d_de, c->d_tau,
-                               c->d_beta, c->d_count, s));
+                               c->d_beta, c->d_count, s, 64, c->side));
   bs_phase_end(c, PH_TRID, s);
   bs_phase_begin(c, PH_BISECT, s);
   TRY(bs_launch_bisect(c->d_de, n, kb, std::min(b + 1, n), c->d_lamT, nullptr, s, false, 1e-9));

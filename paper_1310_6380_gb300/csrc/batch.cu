@@ -162,6 +162,7 @@ struct BatchGroup {
   zd* part64;
   BandWs* band;               // FP64 solver: two-stage reduction workspace (large n)
   FilterWs* filt;             // filtered iteration workspace (FP64 and dense solvers)
+  SideStreams* side;
   // [0] tensor-core pipeline timeout of a main-stream product, [1] a Gram
   // Cholesky failed, [2] a tensor-core timeout during a cell's assembly
   // (the workers' own flags are reset by every assembly, so each assembly's
@@ -225,6 +226,8 @@ static bool group_filter(const bs_batch* B, const BatchGroup& g) {
 }
 
 static void free_group(BatchGroup& g) {
+  bs_side_free(g.side);
+  g.side = nullptr;
   if (g.band) {
     bs_band_ws_free(g.band);
     delete g.band;
@@ -607,7 +610,7 @@ static int reduce_chunk_body(bs_batch* B, BatchGroup& g, int c0, int cn, int p, 
     return BS_OK;
   } else {
   TRY_LAUNCH(bs_launch_tridiag<float>(g.C32, n, K, g.vec32, g.part32, g.de, g.tau, g.beta, g.count,
-                                      s, tile));
+                                      s, tile, g.side));
   prof_mark(B, s);
   TRY_LAUNCH(bs_launch_bisect(g.de, n, K, b + 1, g.lamT, nullptr, s, false, 1e-9));
   prof_mark(B, s);
@@ -788,6 +791,7 @@ extern "C" int bs_batch_create(const bs_cell_desc* descs, int ncells, int nk, in
           e = cudaEventCreateWithFlags(&g.adone[p][w], cudaEventDisableTiming);
       }
       if (e != cudaSuccess) r = bs_cuda_status(e, "bs_batch_create events");
+      if (!r) r = bs_side_create(&g.side);
     }
     if (r) {
       B->groups.push_back(g);
@@ -1143,7 +1147,7 @@ static int mixed_rescue(bs_batch* B, BatchGroup& g, int c0, const std::vector<in
      "batch rescue rows");
   TRY_LAUNCH(bs_launch_c64_to_c32(g.C64, g.C32, n, nf, s));
   TRY_LAUNCH(bs_launch_tridiag<float>(g.C32, n, nf, g.vec32, g.part32, g.de, g.tau, g.beta,
-                                      g.count, s, g.tile));
+                                      g.count, s, g.tile, g.side));
   TRY_LAUNCH(bs_launch_bisect(g.de, n, nf, g.b + 1, g.lamT, nullptr, s, false, 1e-9));
   MixedWs w;
   w.C64 = g.C64; w.C32 = g.C32; w.de = g.de; w.tau = g.tau; w.beta = g.beta; w.lamT = g.lamT;

@@ -228,6 +228,7 @@ struct bs_cell {
   struct BandWs* band;  // two-stage reduction workspace (allocated on first use)
   bool band_used;       // the last FP64 solve took the two-stage reduction
   struct FilterWs* filt;  // filtered iteration workspace (allocated on first use)
+  struct SideStreams* side;  // with the mixed workspace
 
   bool prof;
   bool prof_ready[PH_COUNT];
@@ -495,6 +496,19 @@ int bs_launch_builder(const zd* Cm, int n, const double* Q, int nk, double q1x, 
 // return column j of A below row j+1 holds v_j (v_j[j+1] = 1 implied),
 // de = [d | |beta|], tau[b*n + j] = tau_j and beta[b*n + j] = beta_j, the
 // (j+1, j) entry of the unitarily reduced (complex) tridiagonal.
+// Streams beside the caller's for parts of a batch that run at the same time
+// (fork on the caller's stream, join before the call returns; safe in a
+// capture).  Owned by the cell or group whose workspace the parts use.
+#define BS_SIDE 1
+struct SideStreams {
+  cudaStream_t s[BS_SIDE] = {};
+  cudaEvent_t fork = nullptr, join[BS_SIDE] = {};
+};
+int bs_side_create(SideStreams** out);
+void bs_side_free(SideStreams* w);
+int bs_side_fork(const SideStreams* w, int parts, cudaStream_t s);
+int bs_side_join(const SideStreams* w, int parts, cudaStream_t s);
+
 size_t bs_tridiag_vec_elems(int n);
 size_t bs_tridiag_part_elems(int n);
 // tile: 64 (default) or 32 (tile edge of the fused update + matrix-vector
@@ -502,7 +516,8 @@ size_t bs_tridiag_part_elems(int n);
 template <typename R>
 int bs_launch_tridiag(typename Cplx<R>::T* A, int n, int batch, typename Cplx<R>::T* vec,
                       typename Cplx<R>::T* part, double* de, double* tau, zd* beta,
-                      unsigned* count, cudaStream_t s, int tile = 64);
+                      unsigned* count, cudaStream_t s, int tile = 64,
+                      const SideStreams* side = nullptr);
 
 // mixed.cu: FP32 reduction + FP64 Rayleigh-Ritz refinement
 struct MixedWs {

@@ -50,6 +50,18 @@ __device__ double block_sum(double v, double* sh) {
 template <typename C>
 __device__ __forceinline__ C ldg_cg(const C* p) { return __ldcg(p); }
 
+// tau, 1 / (x0 - beta) and beta of the reflector of (alpha = x0, ...), aa = |x0|, nu = ||x||
+__device__ __forceinline__ void reflector(zd alpha, double aa, double nu, double& tau, zd& scale,
+                                          zd& beta) {
+  if (nu > 0.0) {
+    beta = aa > 0.0 ? zscale(alpha, -nu / aa) : zmake(-nu, 0.0);
+    tau = (aa + nu) / nu;
+    const zd den = zsub(alpha, beta);
+    const double d2 = den.x * den.x + den.y * den.y;
+    scale = zmake(den.x / d2, -den.y / d2);
+  }
+}
+
 // Reflector of column c below the diagonal, x = A[c+1:n, c]: H x = beta e1
 // with beta = -(x0/|x0|) ||x||, tau = (|x0| + ||x||)/||x||, v = x / (x0 - beta).
 // The scalars are formed in FP64 for both precisions.  Writes v to the
@@ -71,13 +83,7 @@ __device__ void householder(typename Cplx<R>::T* a, int n, int c, typename Cplx<
   const double nu = sqrt(fma(aa, aa, s));
   double tau = 0.0;
   zd scale = zmake(0.0, 0.0), beta = zmake(0.0, 0.0);
-  if (nu > 0.0) {
-    beta = aa > 0.0 ? zscale(alpha, -nu / aa) : zmake(-nu, 0.0);
-    tau = (aa + nu) / nu;
-    const zd den = zsub(alpha, beta);
-    const double d2 = den.x * den.x + den.y * den.y;
-    scale = zmake(den.x / d2, -den.y / d2);
-  }
+  reflector(alpha, aa, nu, tau, scale, beta);
   for (int r = r0 + 1 + tid; r < n; r += NT) {
     C* ap = a + r + (size_t)c * n;
     const C x = ldg_cg(ap);
@@ -137,6 +143,113 @@ __device__ __forceinline__ void tri_index(int l, int& bi, int& bk) {
   bk = l - r * (r + 1) / 2;
 }
 
+// What the last CTA of a matrix does after step j - 1's tiles, r0 = j + 1 and
+// n - r0 <= EPR NT rows: w from the tile partials, the update of column r0 and
+// its reflector.  A chain that nothing overlaps within a matrix, so the rows stay
+// in registers, the column in shared memory (col, n - r0 entries), and the
+// partials of four tiles are loaded together (instead of through global memory
+// at every stage: 1.2 us less per step at n = 882, mixed solve of 8 wavevectors
+// 44.6 -> 43.6 ms, of 90 77.0 -> 75.3 ms).  The sums take the same terms in the
+// same order as the general form in tridiag_tile.
+constexpr int EPR = 4;
+template <typename R>
+__device__ __forceinline__ void column_step(typename Cplx<R>::T* a, int n, int r0,
+                                            const typename Cplx<R>::T* vcur,
+                                            typename Cplx<R>::T* w, typename Cplx<R>::T* vnext,
+                                            const typename Cplx<R>::T* pt, int t0, int nt,
+                                            double* d, const double* tau, double* tau_out,
+                                            zd* beta_out, typename Cplx<R>::T* col, double* sh) {
+  typedef typename Cplx<R>::T C;
+  __shared__ C first[2];
+  const int tid = threadIdx.x;
+  const C zero = Cplx<R>::make((R)0, (R)0);
+  C p[EPR], v[EPR], x[EPR];
+#pragma unroll
+  for (int i = 0; i < EPR; ++i) {
+    const int rr = r0 + tid + i * NT;
+    p[i] = zero;
+    v[i] = rr < n ? vcur[rr] : zero;
+    x[i] = rr < n ? ldg_cg(a + rr + (size_t)r0 * n) : zero;
+  }
+  const R tj = (R)*tau;
+  for (int t = t0; t < nt; t += 4) {
+    C q[EPR][4];
+#pragma unroll
+    for (int i = 0; i < EPR; ++i)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int rr = r0 + tid + i * NT;
+        q[i][u] = rr < n && t + u < nt ? ldg_cg(pt + (size_t)(t + u) * n + rr) : zero;
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (t + u < nt) {
+#pragma unroll
+        for (int i = 0; i < EPR; ++i) p[i] = zadd(p[i], q[i][u]);
+      }
+  }
+  double kp = 0.0;
+#pragma unroll
+  for (int i = 0; i < EPR; ++i) {
+    // (not contracted with the subtraction of K v below)
+    if constexpr (sizeof(R) == 4) p[i] = make_float2(__fmul_rn(p[i].x, tj), __fmul_rn(p[i].y, tj));
+    else p[i] = zmake(__dmul_rn(p[i].x, tj), __dmul_rn(p[i].y, tj));
+    if (r0 + tid + i * NT < n)
+      kp = fma((double)v[i].x, (double)p[i].x, fma((double)v[i].y, (double)p[i].y, kp));
+  }
+  const R K = (R)(0.5 * (double)tj * block_sum(kp, sh));
+#pragma unroll
+  for (int i = 0; i < EPR; ++i) {
+    const int rr = r0 + tid + i * NT;
+    p[i] = zsub(p[i], zscale(v[i], K));   // w
+    if (rr < n) w[rr] = p[i];
+  }
+  if (tid == 0) {
+    first[0] = p[0];
+    first[1] = v[0];
+  }
+  __syncthreads();
+  const C wj = first[0], vj = first[1];
+#pragma unroll
+  for (int i = 0; i < EPR; ++i) {
+    const int rr = r0 + tid + i * NT;
+    if (rr >= n) continue;
+    x[i] = zfnmac(v[i], wj, x[i]);
+    x[i] = zfnmac(p[i], vj, x[i]);
+    if (rr == r0) x[i].y = (R)0;
+    col[rr - r0] = x[i];
+    if (rr <= r0 + 1) a[rr + (size_t)r0 * n] = x[i];   // the rows below become the reflector
+  }
+  if (tid == 0) d[r0] = (double)x[0].x;
+  if (r0 + 1 >= n) return;
+  __syncthreads();
+  double s = 0.0;
+  for (int r = 2 + tid; r < n - r0; r += NT) {
+    const C y = col[r];
+    s = fma((double)y.x, (double)y.x, fma((double)y.y, (double)y.y, s));
+  }
+  s = block_sum(s, sh);
+  const zd alpha = zmake(col[1].x, col[1].y);
+  const double aa = hypot(alpha.x, alpha.y);
+  const double nu = sqrt(fma(aa, aa, s));
+  double tn = 0.0;
+  zd scale = zmake(0.0, 0.0), beta = zmake(0.0, 0.0);
+  reflector(alpha, aa, nu, tn, scale, beta);
+  for (int r = 2 + tid; r < n - r0; r += NT) {
+    const C z = col[r];
+    const zd y = zmul(zmake(z.x, z.y), scale);
+    const C vr = Cplx<R>::make((R)y.x, (R)y.y);
+    vnext[r0 + r] = vr;
+    a[r0 + r + (size_t)r0 * n] = vr;
+  }
+  if (tid == 0) {
+    vnext[r0 + 1] = Cplx<R>::make((R)1, (R)0);
+    *tau_out = tn;
+    *beta_out = beta;
+    d[n + r0] = nu;
+  }
+}
+
 // One tile of step j of matrix b (tile: its index among the ntl lower tiles).
 template <typename R, int TS>
 __device__ __forceinline__ void tridiag_tile(typename Cplx<R>::T* __restrict__ A, int n, int j,
@@ -151,8 +264,9 @@ __device__ __forceinline__ void tridiag_tile(typename Cplx<R>::T* __restrict__ A
   // reduced once per tile through shared memory.
   constexpr int EPT = TS / 16;
   __shared__ C vpS[TS], wpS[TS], vcS[TS];
-  __shared__ C rowred[16][TS];   // [ty][row]
-  __shared__ C colred[16][TS];   // [tx][col]
+  __shared__ C red[2][16][TS];
+  C(*rowred)[TS] = red[0];       // [ty][row]
+  C(*colred)[TS] = red[1];       // [tx][col]
   __shared__ double sh[NT / 32 + 1];
   __shared__ int is_last;
 
@@ -263,6 +377,14 @@ __device__ __forceinline__ void tridiag_tile(typename Cplx<R>::T* __restrict__ A
   __threadfence();
 
   // ---- epilogue: one CTA per matrix
+  if (n - r0 <= EPR * NT) {
+    static_assert(2 * 16 * TS >= EPR * NT, "the column fits the reduction buffers");
+    column_step<R>(a, n, r0, vcur, w, vprev, pt, t0, nt, de + (size_t)b * 2 * n,
+                   tau + (size_t)b * n + j, tau + (size_t)b * n + r0, beta + (size_t)b * n + r0,
+                   &red[0][0][0], sh);
+    if (tid == 0) count[b] = 0u;
+    return;
+  }
   const R tj = (R)tau[(size_t)b * n + j];
   double kp = 0.0;
   for (int rr = r0 + tid; rr < n; rr += NT) {
@@ -361,21 +483,72 @@ int bs_launch_tridiag_list(zd* A, int n, zd* vec, zd* part, double* de, double* 
 size_t bs_tridiag_vec_elems(int n) { return 3 * (size_t)n; }
 size_t bs_tridiag_part_elems(int n) { return (size_t)((n + TSMIN - 1) / TSMIN) * n; }
 
+int bs_side_create(SideStreams** out) {
+  if (*out) return BS_OK;
+  SideStreams* w = new SideStreams();
+  cudaError_t e = cudaEventCreateWithFlags(&w->fork, cudaEventDisableTiming);
+  for (int h = 0; e == cudaSuccess && h < BS_SIDE; ++h) {
+    e = cudaStreamCreateWithFlags(&w->s[h], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&w->join[h], cudaEventDisableTiming);
+  }
+  if (e != cudaSuccess) {
+    bs_side_free(w);
+    return bs_cuda_status(e, "side stream");
+  }
+  *out = w;
+  return BS_OK;
+}
+void bs_side_free(SideStreams* w) {
+  if (!w) return;
+  for (int h = 0; h < BS_SIDE; ++h) {
+    if (w->s[h]) cudaStreamDestroy(w->s[h]);
+    if (w->join[h]) cudaEventDestroy(w->join[h]);
+  }
+  if (w->fork) cudaEventDestroy(w->fork);
+  delete w;
+}
+int bs_side_fork(const SideStreams* w, int parts, cudaStream_t s) {
+  cudaError_t e = parts > 1 ? cudaEventRecord(w->fork, s) : cudaSuccess;
+  for (int h = 0; e == cudaSuccess && h + 1 < parts; ++h) e = cudaStreamWaitEvent(w->s[h], w->fork, 0);
+  return e == cudaSuccess ? BS_OK : bs_cuda_status(e, "side stream fork");
+}
+int bs_side_join(const SideStreams* w, int parts, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  for (int h = 0; e == cudaSuccess && h + 1 < parts; ++h) {
+    e = cudaEventRecord(w->join[h], w->s[h]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, w->join[h], 0);
+  }
+  return e == cudaSuccess ? BS_OK : bs_cuda_status(e, "side stream join");
+}
+
+// With side streams the batch is cut into parts whose steps run at the same
+// time: the last CTA of a matrix goes on alone (partial sums, w, the next
+// reflector), and the tiles of the other part fill the SMs meanwhile (90
+// matrices of n = 882, FP32: 64 -> 50 ms for the reduction; a third part gains
+// 0.5 ms more at 90 and loses 2.6 ms at 16; below 16 matrices the tiles of one
+// part do not fill the chip and there is nothing to overlap).  Each matrix sees
+// the same operations in the same order.
 template <typename R, int TS>
 static int launch_steps(typename Cplx<R>::T* A, int n, int batch, typename Cplx<R>::T* vec,
                         typename Cplx<R>::T* part, double* de, double* tau, zd* beta,
-                        unsigned* count, cudaStream_t s) {
+                        unsigned* count, cudaStream_t s, const SideStreams* side = nullptr) {
   tridiag_init_kernel<R><<<batch, NT, 0, s>>>(A, n, vec, de, tau, beta, count);
   BS_CHECK_LAUNCH("tridiag_init_kernel");
   const int nt = (n + TS - 1) / TS;
+  const int parts = side && batch >= 8 * (BS_SIDE + 1) ? BS_SIDE + 1 : 1;
+  TRY_LAUNCH(bs_side_fork(side, parts, s));
   for (int j = 0; j + 1 < n; ++j) {
     const int m = nt - (j + 1) / TS;
     const int ntl = m * (m + 1) / 2;
-    tridiag_step_kernel<R, TS><<<dim3(ntl, batch), NT, 0, s>>>(A, n, j, vec, part, de, tau, beta,
-                                                               count, ntl);
-    BS_CHECK_LAUNCH("tridiag_step_kernel");
+    for (int h = 0; h < parts; ++h) {
+      const size_t b0 = (size_t)batch * h / parts, b1 = (size_t)batch * (h + 1) / parts;
+      tridiag_step_kernel<R, TS><<<dim3(ntl, (unsigned)(b1 - b0)), NT, 0, h ? side->s[h - 1] : s>>>(
+          A + b0 * n * n, n, j, vec + b0 * 3 * n, part + b0 * nt * n, de + b0 * 2 * n, tau + b0 * n,
+          beta + b0 * n, count + b0, ntl);
+      BS_CHECK_LAUNCH("tridiag_step_kernel");
+    }
   }
-  return BS_OK;
+  return bs_side_join(side, parts, s);
 }
 
 // FP64, n <= 600: 64-tiles while a step has enough of them to fill the GPU,
@@ -410,19 +583,19 @@ static int launch_steps_fp64(zd* A, int n, int batch, zd* vec, zd* part, double*
 template <typename R>
 int bs_launch_tridiag(typename Cplx<R>::T* A, int n, int batch, typename Cplx<R>::T* vec,
                       typename Cplx<R>::T* part, double* de, double* tau, zd* beta,
-                      unsigned* count, cudaStream_t s, int tile) {
+                      unsigned* count, cudaStream_t s, int tile, const SideStreams* side) {
   if (tile == 0) tile = 64;
   // The whole batch runs in every step launch.  (Reducing it in L2-sized
   // groups one after another was measured slower for FP32: the per-step
   // launch and epilogue latency then repeats once per group.)
   if (tile == 32)
-    return launch_steps<R, 32>(A, n, batch, vec, part, de, tau, beta, count, s);
+    return launch_steps<R, 32>(A, n, batch, vec, part, de, tau, beta, count, s, side);
   if constexpr (sizeof(R) == 8)
     return launch_steps_fp64(A, n, batch, vec, part, de, tau, beta, count, s);
-  return launch_steps<R, 64>(A, n, batch, vec, part, de, tau, beta, count, s);
+  return launch_steps<R, 64>(A, n, batch, vec, part, de, tau, beta, count, s, side);
 }
 
 template int bs_launch_tridiag<double>(zd*, int, int, zd*, zd*, double*, double*, zd*, unsigned*,
-                                       cudaStream_t, int);
+                                       cudaStream_t, int, const SideStreams*);
 template int bs_launch_tridiag<float>(zf*, int, int, zf*, zf*, double*, double*, zd*, unsigned*,
-                                      cudaStream_t, int);
+                                      cudaStream_t, int, const SideStreams*);
