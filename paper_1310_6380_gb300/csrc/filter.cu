@@ -984,12 +984,15 @@ __device__ __forceinline__ int jacobi32(JacobiSmem& sm, float offtol, int maxswe
 // H w = theta G w per matrix from the Gram partials: Cholesky of the
 // unit-diagonal G and its inverse factor (one barrier per column, as
 // ldl64_block), A = L^-1 H L^-dagger, Jacobi, W = S L^-dagger V, all but the
-// Jacobi in R (FP64 throughout but in the steps that only steer).  In FP64 a
-// Newton-Schulz step makes the FP32 vectors orthonormal to 1e-12 and their
-// norms are divided out.  fail: G not positive definite.
+// Jacobi in R (FP64 but in the steps that only steer).  In the FP64 steps a
+// Newton-Schulz step makes the FP32 vectors orthonormal to 1e-12, their norms
+// are divided out and W is formed in two FP32 terms: one SM's FP64 pipe, two
+// multiply-adds a clock, bounds a matrix otherwise (with the products in FP64
+// 210 us per step of one matrix, 155 us so).  fail: G not
+// positive definite.
 template <typename R>
 struct EigSmem {
-  typename Cplx<R>::T G[FB][FB + 1], H[FB][FB + 1], Li[FB][FB + 1], V[FB][FB + 1];
+  typename Cplx<R>::T G[FB][FB + 1], H[FB][FB + 1], Li[FB][FB + 1];
   JacobiSmem J;
 };
 
@@ -1106,39 +1109,60 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
   __syncthreads();
   // off-diagonal norm below 3e-10 of the whole (3e-7 in the steps that steer)
   const int cur = jacobi32(sm.J, sizeof(R) == 8 ? 1e-19f : 1e-13f, 10);
-  for (int e = tid; e < FB * FB; e += 256) {
-    const zf v = sm.J.V[e / FB][e % FB];
-    sm.V[e / FB][e % FB] = Cplx<R>::make((R)v.x, (R)v.y);
-  }
   if (tid < FB) ev[tid] = (double)sm.J.D[cur][tid].x + (double)sm.J.D[cur][tid].y;
   __syncthreads();
-  if (sizeof(R) == 8) {
-    // G <- (3 I - V^dagger V) / 2, H <- V G, columns to unit length
+  float4(*V4)[FB + 1] = reinterpret_cast<float4(*)[FB + 1]>(&sm.G[0][0]);   // vectors, two terms
+  float4(*L4)[FB + 1] = reinterpret_cast<float4(*)[FB + 1]>(&sm.H[0][0]);   // Li, two terms
+  if constexpr (sizeof(R) == 8) {
+    // V <- V + V F, F = (I - V^dagger V) / 2, columns to unit length.  F is 1e-6
+    // and needs no more than FP32; V^dagger V is summed in two FP32 terms
+    zf(*F)[FB + 1] = sm.J.A[0];
     for (int e = tid; e < NT2; e += 256) {
       int r, c;
       tile_of(e, r, c);
-      T s = zero;
-#pragma unroll 8
-      for (int t = 0; t < FB; ++t) s = zfmac(sm.V[t][c], sm.V[t][r], s);   // conj(V_tr) V_tc
-      s = Cplx<R>::make((r == c ? (R)1.5 : (R)0) - (R)0.5 * s.x, r == c ? (R)0 : (R)-0.5 * s.y);
-      sm.G[r][c] = s;
-      sm.G[c][r] = zconj(s);
+      df re = {0.f, 0.f}, im = {0.f, 0.f};
+#pragma unroll 4
+      for (int t = 0; t < FB; ++t) {   // conj(V_tr) V_tc
+        const zf a = sm.J.V[t][r], b = sm.J.V[t][c];
+        df_fma({a.x, 0.f}, {b.x, 0.f}, re);
+        df_fma({a.y, 0.f}, {b.y, 0.f}, re);
+        df_fma({a.x, 0.f}, {b.y, 0.f}, im);
+        df_fma({-a.y, 0.f}, {b.x, 0.f}, im);
+      }
+      const zf f = make_float2(-0.5f * ((re.h - (r == c ? 1.f : 0.f)) + re.l),
+                               r == c ? 0.f : -0.5f * (im.h + im.l));
+      F[r][c] = f;
+      F[c][r] = zconj(f);
+    }
+    for (int e = tid; e < FB * FB; e += 256) {
+      const int r = e / FB, c = e % FB;
+      zd l = r >= c ? sm.Li[r][c] : zmake(0.0, 0.0);
+      const df x = df_of(l.x), y = df_of(l.y);
+      L4[r][c] = make_float4(x.h, y.h, x.l, y.l);
     }
     __syncthreads();
     for (int e = tid; e < FB * FB; e += 256) {
       const int r = e / FB, c = e % FB;
-      T s = zero;
+      zf d = make_float2(0.f, 0.f);
 #pragma unroll 8
-      for (int t = 0; t < FB; ++t) s = zfma(sm.V[r][t], sm.G[t][c], s);
-      sm.H[r][c] = s;
+      for (int t = 0; t < FB; ++t) d = zfma(sm.J.V[r][t], F[t][c], d);
+      const zf v = sm.J.V[r][c];
+      V4[r][c] = make_float4(v.x, v.y, d.x, d.y);
     }
     __syncthreads();
     const int c = tid >> 3, q = tid & 7;
     R v2 = (R)0;
-    for (int r = q; r < FB; r += 8) v2 += sm.H[r][c].x * sm.H[r][c].x + sm.H[r][c].y * sm.H[r][c].y;
+    for (int r = q; r < FB; r += 8) {
+      const float4 f = V4[r][c];
+      const R x = (R)f.x + (R)f.z, y = (R)f.y + (R)f.w;
+      v2 += x * x + y * y;
+    }
     for (int o = 4; o > 0; o >>= 1) v2 += __shfl_xor_sync(0xffffffffu, v2, o);
-    const R iv = rsqrt(v2);
-    for (int r = q; r < FB; r += 8) sm.V[r][c] = zscale(sm.H[r][c], iv);
+    const float iv = (float)(rsqrt(v2) - 1.0);
+    for (int r = q; r < FB; r += 8) {
+      V4[r][c].z = fmaf(iv, V4[r][c].x, V4[r][c].z);
+      V4[r][c].w = fmaf(iv, V4[r][c].y, V4[r][c].w);
+    }
     __syncthreads();
   }
   if (tid < FB) {
@@ -1151,10 +1175,25 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
   __syncthreads();
   for (int e = tid; e < FB * FB; e += 256) {
     const int r = e / FB, c = e % FB;   // W[r][rank(c)] = sc_r sum_t conj(Li[t][r]) V[t][c]
-    T s = zero;
-    for (int t = r; t < FB; ++t) s = zfmac(sm.V[t][c], sm.Li[t][r], s);
-    s = zscale(s, sc[r]);
-    W[(size_t)k * FB * FB + r + (size_t)rank[c] * FB] = zmake((double)s.x, (double)s.y);
+    zd o;
+    if constexpr (sizeof(R) == 8) {
+      // 48 bits, as the rotation of the block takes them
+      df re = {0.f, 0.f}, im = {0.f, 0.f};
+      for (int t = r; t < FB; ++t) {
+        const float4 l = L4[t][r], v = V4[t][c];
+        df_fma({l.x, l.z}, {v.x, v.z}, re);
+        df_fma({l.y, l.w}, {v.y, v.w}, re);
+        df_fma({l.x, l.z}, {v.y, v.w}, im);
+        df_fma({-l.y, -l.w}, {v.x, v.z}, im);
+      }
+      o = zmake(((double)re.h + (double)re.l) * sc[r], ((double)im.h + (double)im.l) * sc[r]);
+    } else {
+      zf x = make_float2(0.f, 0.f);
+      for (int t = r; t < FB; ++t) x = zfmac(sm.J.V[t][c], sm.Li[t][r], x);
+      x = zscale(x, sc[r]);
+      o = zmake((double)x.x, (double)x.y);
+    }
+    W[(size_t)k * FB * FB + r + (size_t)rank[c] * FB] = o;
     if (r == 0) theta[(size_t)k * FB + rank[c]] = ev[c];
   }
 }
