@@ -460,10 +460,10 @@ struct FilterWs {
   float* coef = nullptr;    // kf x BS_FILT_MAXDEG x 4 x 32
   double* shift = nullptr;  // kf
   double* cmax = nullptr;   // kf
-  double* sigma = nullptr;  // kf
+  double* sigma = nullptr;  // 2 kf: the shift of the count and a second one
   int* ord = nullptr;       // kf x 32
   float* w = nullptr;       // kf x np row scales
-  int* iw = nullptr;        // neg, flag, expected count, list (kf each), list length, fail, done (kf)
+  int* iw = nullptr;        // neg, flag, expected count, list (kf each), list length, fail, done, again (kf)
 };
 // the buffers of the Householder reduction that takes what is not certified
 struct FilterFallback {

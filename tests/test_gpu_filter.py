@@ -128,3 +128,13 @@ def test_smallest_matrices(M, nb, nk):
         Q = cells.ibz_path(cell.lattice, max(nk, 2), cell.h1, cell.h2)[:nk].copy()
         a, b, n, cmax = solve2(cell, M, Q, nb)
         assert np.abs(a ** 2 - b ** 2).max() <= (n + 128) * EPS * cmax
+
+
+def test_many_matrices():
+    """2160 matrices of 24 cells: among so many the FP32 count of one or two is
+    spoilt by a pivot near zero and taken again at the second shift."""
+    for seed in range(24):
+        cell = cells.voronoi_cell(32, 12, seed=seed, lattice="hex" if seed % 2 else "square")
+        Q = cells.ibz_path(cell.lattice, 90, cell.h1, cell.h2)[:90].copy()
+        a, b, n, cmax = solve2(cell, 5, Q, 18)
+        assert np.abs(a ** 2 - b ** 2).max() <= (n + 128) * EPS * cmax, seed
