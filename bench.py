@@ -3,8 +3,8 @@
 
 One step = the whole hot path over one cell: bs_assemble (material fields,
 form factors, Gram Cholesky factors, k-monomials) and bs_solve_k over the
-workload's wavevectors (per-k builder, reduction to tridiagonal form,
-bisection).  Inputs are resident in HBM when the timed region starts; L2
+workload's wavevectors (per-k builder, filtered iteration or reduction to
+tridiagonal form and bisection).  Inputs are resident in HBM when the timed region starts; L2
 is flushed (a 256 MiB write) between timed steps, outside the timed
 events.  Each step is timed with CUDA events on the launching stream.
 
@@ -488,22 +488,14 @@ def measure_c3(bs, torch, rep, args, ncell, steps, warmup, graph=True, oracle_ce
            "d2h_bytes_per_step": hw.numel() * 8 + hs.numel() * 4,
            "api": "bs_batch_create (host arrays) + bs_batch_solve (host Q, outputs; first call "
                   "includes tile autotuning) + bs_batch_destroy"}
-    # dominant kernel: the FP32 Householder reduction, bound by HBM on the
-    # read + write of every trailing triangle
-    hbm_peak, _, note = measured_peaks()
-    tri_bytes = sum(nk * sum(m * (m + 1) // 2 for m in range(1, int(n))) * 16.0 for n in ns)
-    achieved = tri_bytes / (ph["reduction"] / 1e3) / 1e9
-    roofline = {"bound": "hbm", "kernel": "tridiag_step_kernel<float> (all launches of one step)",
-                "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
-                "traffic": None, "peak_source": "copy bandwidth, " + note,
-                "algorithmic": "read + write (8 B each) of every trailing lower triangle of "
-                               f"{ncell * nk} matrices (n = 242..578)"}
+    roofline = filter_roofline(np.repeat(ns, nk), ph["reduction"], device_peaks(torch),
+                               "one step's groups")
     value = world * ncell * nk / (ms / 1e3)
     out = {
         "metric": METRIC, "value": value, "unit": "k-solves/s", "n_gpus": world,
         "steps": steps, "warmup": warmup, "ms_per_step": ms, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None,
-        "dtype": "f32 reduction, bf16 exact-slice tensor products, f64 refinement",
+        "dtype": "f64 Rayleigh-Ritz and certificate, f32 factorisations, bf16 split tensor products",
         "data": "synthetic",
         "config": {"workload": f"c3: {ncell} cells (seeds 6380+i), 64x64 pixels, square/hex, "
                                "ellipse/Voronoi maps with 2-16 phases, M = 5..8 (n = 242..578), "
@@ -638,6 +630,29 @@ def run_reference_batch(args):
 
 
 BAND_NB = 8
+
+
+def filter_taken(n, nb):
+    """The solves that the library routes to the filtered iteration by default."""
+    return 96 <= n <= 2048 and nb <= 22
+
+
+def filter_roofline(ns, ms, peaks, what):
+    """Roofline of the filtered iteration on matrices of orders ns: its FP32
+    factorisation, triangular inverse, operator and inertia check (4/3 n^3 real
+    flops each) against the FP32 pipe, which its largest kernels run on; the
+    time also holds the tensor-core products and the Rayleigh-Ritz steps."""
+    flops = 16.0 / 3.0 * float(np.sum(np.asarray(ns, float) ** 3))
+    peak = peaks["fp32_nominal_tflops"]
+    achieved = flops / (ms / 1e3) / 1e12
+    return {"bound": "alu", "kernel": "filtered iteration (ldl64_*, trinv64, filt_operator in "
+                                      f"FP32; {what})",
+            "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+            "traffic": None,
+            "peak_source": "nominal FP32 CUDA-core rate: SMs x 128 FMA/clk x 2 x max SM clock "
+                           "(queried)",
+            "algorithmic": f"(16/3) n^3 real FP32 flops per matrix, {len(ns)} matrices, "
+                           f"n = {int(min(ns))}..{int(max(ns))}"}
 
 
 def band_roofline(red, n, nk_all, ph, peaks):
@@ -818,13 +833,16 @@ def run_ours(args):
     value = world * nk / (ms / 1e3)
     omega = w.cpu().numpy()
 
-    # dominant kernel: the reduction to tridiagonal form (its largest kernel
-    # group when the reduction is two-stage)
+    # dominant kernels: the filtered iteration, or the reduction to tridiagonal
+    # form (its largest kernel group when that is two-stage)
     ph = {k: statistics.mean(p[k] for p in phases) for k in phases[0]}
     peaks = device_peaks(torch, bs)
     red = {k: statistics.mean(r[k] for r in reds) for k in reds[0]}
     if prec == 0 and red["matrices"] > 0:
         roofline, reduction = band_roofline(red, n, nk, ph, peaks)
+    elif prec == 0 and filter_taken(n, nb):
+        reduction = None
+        roofline = filter_roofline([n] * nk, ph["tridiag"], peaks, "all launches of one step")
     elif prec == 0:
         reduction = None
         trid_flops = nk * 16.0 / 3.0 * n ** 3
@@ -1041,8 +1059,7 @@ def measure_c4(bs, torch, rep, args, ncell, steps, warmup, oracle_cells=6, fp64_
     ms = rep.max(ms)
     value = world * ncell * nk / (ms / 1e3)
 
-    # the plain FP64 dense GPU path (FP64 C(k), reduction to tridiagonal form,
-    # Sturm multisection), batched over the cells like the other solvers, on a
+    # the FP64 solver (FP64 C(k), filtered iteration), batched over the cells like the other solvers, on a
     # sample of the cells
     samp = list(range(0, ncell, max(1, ncell // fp64_cells)))[:fp64_cells]
     bf = bs.bs_batch_create([cargs[i] for i in samp], nk, nb)
@@ -1124,9 +1141,8 @@ def measure_c4(bs, torch, rep, args, ncell, steps, warmup, oracle_cells=6, fp64_
                        "speedup_vs_cold": ms_cold / ms_warm},
         "fp64_dense_gpu": {"value": fp64_rate, "unit": "k-solves/s",
                            "sample": f"{len(samp)} of the cells x {nk} k, one ragged batch "
-                                     "on BS_SOLVER_FP64 (assembly, FP64 C(k), FP64 reduction "
-                                     "to tridiagonal form, two-stage for n >= 400, Sturm "
-                                     "multisection)",
+                                     "on BS_SOLVER_FP64 (assembly, FP64 C(k), filtered "
+                                     "iteration with its FP64 certificate)",
                            "speedup_of_value": value / fp64_rate},
         "speedup_vs_fp64_batched": value / fp64_rate,
         "speedup_target": 10.0,
@@ -1290,26 +1306,28 @@ def run_modes(args):
     W = 2 * M + 1
     stress_flops = units * 3 * 8.0 * N * N          # three Gram solves, two triangular products
     fld = nk * 5 * nvec
-    field_flops = fld * (8.0 * W * G * G + 8.0 * W * W * G)
+    field_flops = fld * (4.0 * W * G * G + 8.0 * W * W * G)   # rows p, G - 1 - p share sums
     field_bytes = fld * G * G * 8.0 + fld * N * 16.0
     dpk = device_peaks(torch)
     fp32_peak = dpk["fp32_nominal_tflops"]
     hbm_peak, _, note = measured_peaks()
     t_field = (pm["field_u"] + pm["field_sigma"]) / 1e3
     rl_stress = {"bound": "alu", "kernel": "bs_stress_coefficients (stress_rhs_kernel, "
-                                           "zgemm_kernel x4, stress_combine_kernel)",
+                                           "digit products of the Gram solves, "
+                                           "stress_combine_kernel)",
                  "achieved": stress_flops / (pm["stress"] / 1e3) / 1e12,
                  "peak": dpk["fp64_nominal_tflops"], "unit": "TFLOP/s", "traffic": None,
                  "peak_source": "nominal FP64: SMs (queried) x 2 FMA/clk x 2 flop x max SM clock",
                  "algorithmic": "3 Gram solves per mode, each two triangular products: 24 N^2 "
-                                "real flops per mode"}
+                                "FP64-equivalent real flops per mode (on the tensor cores, so "
+                                "above 1.0 of the FP64 peak)"}
     rl_stress["frac"] = rl_stress["achieved"] / rl_stress["peak"]
-    rl_field = {"bound": "alu", "kernel": "field_kernel<24> (+ field_table_kernel)",
+    rl_field = {"bound": "alu", "kernel": "field_kernel<24> (+ field_roots_kernel)",
                 "achieved": field_flops / t_field / 1e12, "peak": fp32_peak, "unit": "TFLOP/s",
                 "traffic": None,
                 "peak_source": "nominal FP32 CUDA-core rate: SMs (queried) x 128 FMA/clk x 2 x max "
                                "SM clock",
-                "algorithmic": "8 W G^2 + 8 W^2 G real flops per field (W = 2M+1 = 21, G = 256); "
+                "algorithmic": "4 W G^2 + 8 W^2 G real flops per field (W = 2M+1 = 21, G = 256); "
                                f"stores {field_bytes / 1e9:.2f} GB per step",
                 "hbm_gbs": field_bytes / t_field / 1e9, "hbm_frac": field_bytes / t_field / 1e9
                 / hbm_peak, "hbm_peak_source": "copy bandwidth, " + note}
@@ -1485,21 +1503,8 @@ def run_3d(args):
     value = rep.value(nk, ms)
     omega = w.cpu().numpy()
     t_sol = statistics.mean(sol_ms)
-    flops = nk * 16.0 / 3.0 * n ** 3
-    achieved = flops / (t_sol / 1e3) / 1e12
-    two_stage = n >= 400   # BS_REDUCE_AUTO: the two-stage reduction from n = 400 on
-    kern = ("bs_solve_k3 of one step: two-stage reduction (tcgen05 dense -> band, FP64 bulge "
-            "chase), per-k builder, bisection" if two_stage else
-            "tridiag_step_kernel<double> (with the per-k builder and bisection: bs_solve_k3 of "
-            "one step)")
-    roofline = {"bound": "alu", "kernel": kern,
-                "achieved": achieved, "peak": device_peaks(torch)["fp64_nominal_tflops"],
-                "unit": "TFLOP/s", "traffic": None,
-                "peak_source": "nominal FP64: SMs (queried) x 2 FMA/clk x 2 flop x max SM clock",
-                "algorithmic": f"(16/3) n^3 real flops per k x {nk} k, n={n}" +
-                               ("; the one-stage reduction's flop count, so above 1.0 of the "
-                                "FP64 peak means the work left the FP64 pipe" if two_stage else "")}
-    roofline["frac"] = roofline["achieved"] / roofline["peak"]
+    roofline = filter_roofline([n] * nk, t_sol, device_peaks(torch),
+                               "bs_solve_k3 of one step, with the per-k builder")
     pin = lambda a: torch.from_numpy(np.ascontiguousarray(a)).pin_memory()
     hp, hl, hm, hr, hQ = (pin(cell.phase.astype(np.uint16)), pin(cell.lam), pin(cell.mu),
                           pin(cell.rho), pin(Q))

@@ -266,7 +266,7 @@ int bs_set_iteration_limits(int lobpcg_maxit, int bisect_sweeps);
  *     QR, the trailing two-sided updates as FP64-exact digit-plane products
  *     on the tensor cores (8 digits of 7 bits per operand), then band ->
  *     tridiagonal by bulge chasing in FP64 (O(n^2) work per k);
- *   BS_REDUCE_AUTO (default): solves of at most 22 branches with n >= 200
+ *   BS_REDUCE_AUTO (default): solves of at most 22 branches with n >= 96
  *     take a filtered subspace iteration without a reduction: Chebyshev
  *     filters of the shifted inverse (FP32) on 32 vectors between float64
  *     Rayleigh-Ritz steps, until the sum of the squared float64 residuals over

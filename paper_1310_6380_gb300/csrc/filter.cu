@@ -29,7 +29,8 @@
 //     the eigenvalues outside the block),
 //     and when the inertia of C - sigma I (FP32 LDL^dagger of the scaled
 //     matrix, sigma in a gap above theta_m) counts exactly m eigenvalues
-//     below sigma, so that none was skipped.
+//     below sigma, so that none was skipped (a count that a pivot near zero
+//     spoils is taken again at a second shift).
 //  4. Matrices that do not pass are reduced by the FP64 Householder reduction
 //     and bisected (tridiag.cu, bisect.cu) in one launch each that returns at
 //     once when there are none; nothing waits for the host.

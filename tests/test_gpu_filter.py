@@ -138,3 +138,21 @@ def test_many_matrices():
         Q = cells.ibz_path(cell.lattice, 90, cell.h1, cell.h2)[:90].copy()
         a, b, n, cmax = solve2(cell, 5, Q, 18)
         assert np.abs(a ** 2 - b ** 2).max() <= (n + 128) * EPS * cmax, seed
+
+
+def test_batch_dense_solver():
+    """The dense batch solver's groups take the iteration on their FP64 C(k)."""
+    cl = [cells.config3_cell(i) for i in (0, 3, 5, 8)]
+    args = [(c["cell"].h1, c["cell"].h2, np.ascontiguousarray(c["cell"].phase, np.uint16),
+             c["cell"].lam, c["cell"].mu, c["cell"].rho, c["M"], bs.BS_PREC_MIXED) for c in cl]
+    Q = np.stack([c["Q"][:6] for c in cl])
+    b = bs.bs_batch_create(args, 6, 10)
+    try:
+        w, st = np.empty((4, 6, 10)), np.full((4, 6), 7, np.int32)
+        bs.bs_batch_solve(b, Q, w, st)
+    finally:
+        bs.bs_batch_destroy(b)
+    assert not st.any()
+    for i, c in enumerate(cl):
+        _, ref, n, cmax = solve2(c["cell"], c["M"], np.ascontiguousarray(Q[i]), 10)
+        assert np.abs(w[i] ** 2 - ref ** 2).max() <= (n + 128) * EPS * cmax
