@@ -888,16 +888,18 @@ __device__ __forceinline__ void rotation(zf c, float diff, float skip, float& cs
   sn = shift = 0.f;
   ph = make_float2(1.f, 0.f);
   const float ica = frsqrt(c2), ca = c2 * ica;
-  const float zeta = 0.5f * diff * ica, az = fabsf(zeta);
-  // t = 1 / (|zeta| + sqrt(1 + zeta^2)); for large zeta 1 / (2 |zeta|)
-  const float z2 = 1.f + az * az;
-  float t = frcp(az > 1e4f ? 2.f * az : az + z2 * frsqrt(z2));
-  t = copysignf(t, zeta);
+  // t = 1 / (|zeta| + sqrt(1 + zeta^2)) is the tangent: cs^2 = (1 + |zeta| r) / 2
+  // and sn = r / (2 cs) with r = 1 / sqrt(1 + zeta^2), three dependent
+  // approximations instead of four
+  const float zeta = 0.5f * diff * ica, az = fminf(fabsf(zeta), 1e18f);
+  const float r = frsqrt(fmaf(az, az, 1.f));
+  const float cs2 = fmaf(0.5f * az, r, 0.5f), ic = frsqrt(cs2);
+  const float s1 = copysignf(0.5f * r * ic, zeta);
   if (c2 > skip) {
     ph = make_float2(c.x * ica, c.y * ica);
-    cs = frsqrt(1.f + t * t);
-    sn = t * cs;
-    shift = t * ca;
+    cs = cs2 * ic;
+    sn = s1;
+    shift = s1 * ic * ca;
   }
 }
 
