@@ -832,9 +832,8 @@ int stage_inputs(bs_cnn* m, const uint16_t* phase, const double* table, const lo
   BS_CHECK_LAUNCH("encode_kernel");
   kfeat_kernel<<<(ns + 255) / 256, 256, 0, s>>>(m->Q, m->hex, ns, kper, m->kf);
   BS_CHECK_LAUNCH("kfeat_kernel");
-  // the stack copies above must complete before the vectors go out of scope
-  e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return bs_cuda_status(e, "cnn inputs");
+  // (the copies read the caller's arrays; both entry points end with a
+  // synchronisation, so none is needed here and the layers queue up behind)
   return BS_OK;
 }
 
