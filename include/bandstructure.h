@@ -271,10 +271,14 @@ int bs_set_iteration_limits(int lobpcg_maxit, int bisect_sweeps);
  *     filters of the shifted inverse (FP32) on 32 vectors between float64
  *     Rayleigh-Ritz steps, until the sum of the squared float64 residuals over
  *     their distances to the rest of the spectrum bounds the error of every
- *     eigenvalue by 64 eps64 ||C|| and an inertia count shows that none was
- *     skipped.  Matrices it does not certify so are reduced (one-stage) in
- *     the same call, without a wait for the host.  Other solves: two-stage
- *     for n >= 400, one-stage below.
+ *     eigenvalue by 64 eps64 ||C||.  That the rest begins where the sum takes
+ *     it to, so that none was skipped, is shown by an FP32 Cholesky
+ *     factorisation of C + tau X X^dagger - sigma (X: the vectors below the cut),
+ *     with room for its rounding errors (their norm taken as 16 sqrt(n) 2^-24
+ *     of the matrix scaled to a unit diagonal; 28 2^-24 was the most seen).
+ *     Matrices it does not certify so are reduced (one-stage) in the same
+ *     call, without a wait for the host.  Other solves: two-stage for
+ *     n >= 400, one-stage below.
  * Process-wide; takes effect at the next solve.  The two-stage reduction
  * needs an n x 8 complex panel in shared memory (n up to about 1800 on
  * GB300); larger n use the one-stage reduction in every mode.
@@ -336,6 +340,22 @@ int bs_reduced_matrix(bs_cell* cell, const double* Q, double* out, void* stream)
  */
 int bs_tridiag_eigenvalues(const double* d, const double* e, int n, int batch, int nbands,
                            double* lam_out, void* stream);
+
+/*
+ * bs_lowest_eigenvalues - the filtered subspace iteration of
+ * bs_set_reduction's BS_REDUCE_AUTO on its own: omega = sqrt(max(lambda, 0)) of
+ * the lowest `nbands` eigenvalues (ascending) of `batch` Hermitian matrices
+ * with a diagonal that is not negative.
+ *   C           : batch x n x n complex128 (interleaved re, im), full Hermitian
+ *                 storage, column-major, host or device; 96 <= n <= 2048.
+ *   omega_out   : batch x nbands doubles, host or device; 1 <= nbands <= 22.
+ *   reduced_out : batch ints, host or device, or NULL: 1 where the iteration
+ *                 was not certified and the matrix was reduced to tridiagonal
+ *                 form instead.
+ * Allocates and frees its own device scratch; synchronises `stream`.
+ */
+int bs_lowest_eigenvalues(const double* C, int n, int batch, int nbands, double* omega_out,
+                          int* reduced_out, void* stream);
 
 /*
  * bs_gemm_bf16 - the tensor-core contraction primitive on its own:

@@ -81,6 +81,7 @@ def _load():
         "bs_phase_times": [vp, dp],
         "bs_launch_count": [ctypes.POINTER(ctypes.c_longlong)],
         "bs_tridiag_eigenvalues": [dp, dp, i32, i32, i32, dp, vp],
+        "bs_lowest_eigenvalues": [dp, i32, i32, i32, dp, dp, vp],
         "bs_gemm_bf16": [dp, dp, dp, i32, i32, i32, i32, vp],
         "bs_tridiag_eigenvalues_static": [dp, dp, i32, i32, i32, dp, vp],
         "bs_batch_create": [ctypes.POINTER(bs_cell_desc), i32, i32, i32, ctypes.POINTER(vp)],
@@ -136,7 +137,7 @@ EXPORTED = ["bs_create_cell", "bs_assemble", "bs_solve_k", "bs_bands", "bs_form_
             "bs_mode_field", "bs_create_cell_mesh", "bs_set_stiffness", "bs_create_cell3",
             "bs_assemble3", "bs_solve_k3", "bs_form_factors3", "bs_reduced_matrix3",
             "bs_cell3_dims", "bs_destroy_cell3", "bs_set_iteration_limits", "bs_probe_fp64",
-            "bs_set_reduction", "bs_reduction_times"]
+            "bs_set_reduction", "bs_reduction_times", "bs_lowest_eigenvalues"]
 BS_SOLVER_DENSE, BS_SOLVER_LOBPCG, BS_SOLVER_FP64 = 0, 1, 2
 BS_LOB_MAX_BANDS, BS_LOB_MAXIT = 12, 80
 BS_REDUCE_AUTO, BS_REDUCE_ONESTAGE, BS_REDUCE_TWOSTAGE = 0, 1, 2
@@ -328,6 +329,16 @@ def bs_tridiag_eigenvalues(d, e, nbands: int, lam_out, stream=None):
     _check(_lib.bs_tridiag_eigenvalues(_ptr(d, np.float64), _ptr(e, np.float64), n, batch,
                                        int(nbands), _ptr(lam_out, np.float64), _stream(stream)))
     return lam_out
+
+
+def bs_lowest_eigenvalues(C, nbands: int, omega_out, reduced_out=None, stream=None):
+    """C: (batch, n, n) complex128 Hermitian (row-major: its conjugate is solved,
+    which has the same eigenvalues); omega_out: (batch, nbands)."""
+    batch, n = int(C.shape[0]), int(C.shape[1])
+    _check(_lib.bs_lowest_eigenvalues(_ptr(C, np.complex128), n, batch, int(nbands),
+                                      _ptr(omega_out, np.float64), _ptr(reduced_out, np.int32),
+                                      _stream(stream)))
+    return omega_out
 
 
 def _desc(cell_args):

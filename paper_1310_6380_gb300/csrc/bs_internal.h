@@ -460,10 +460,12 @@ struct FilterWs {
   float* coef = nullptr;    // kf x BS_FILT_MAXDEG x 4 x 32
   double* shift = nullptr;  // kf
   double* cmax = nullptr;   // kf
-  double* sigma = nullptr;  // 2 kf: the shift of the count and a second one
+  double* sigma = nullptr;  // 2 kf: sigma and tau of the certificate
+  double* kappa = nullptr;  // kf: bound of ||A^-1||
+  float* rsum = nullptr;    // kf x np / 64 x np: row sums of |A^-1| by block column
   int* ord = nullptr;       // kf x 32
   float* w = nullptr;       // kf x np row scales
-  int* iw = nullptr;        // neg, flag, expected count, list (kf each), list length, fail, done, again (kf)
+  int* iw = nullptr;        // neg, flag, certified count, list (kf each), list length, fail, done, skip (kf)
 };
 // the buffers of the Householder reduction that takes what is not certified
 struct FilterFallback {
@@ -479,9 +481,11 @@ bool bs_filter_fits(int n, int nbands);
 bool bs_use_filter(int n, int nbands);
 int bs_filter_ws_alloc(FilterWs* w, int n, int kb);
 void bs_filter_ws_free(FilterWs* w);
-// C: kb full Hermitian matrices (kept, but for those that take the fallback)
+// C: kb full Hermitian matrices (kept, but for those that take the fallback);
+// reduced (optional, kb): 1 where the fallback ran
 int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const FilterFallback& fb,
-                         double* omega, int* stat, int* err, cudaStream_t s);
+                         double* omega, int* stat, int* err, cudaStream_t s,
+                         int* reduced = nullptr);
 // tridiag.cu, bisect.cu: the matrices list[0 .. *nlist) of a batch (device list)
 int bs_launch_tridiag_list(zd* A, int n, zd* vec, zd* part, double* de, double* tau, zd* beta,
                            unsigned* count, const int* list, const int* nlist, cudaStream_t s);

@@ -26,11 +26,11 @@
 //     A matrix passes when that sum is at most 64 eps64 max_r C_rr (the
 //     backward error of a reduction to tridiagonal form and its bisection is
 //     of that size; the sum overestimates the error, whose own gap is that to
-//     the eigenvalues outside the block),
-//     and when the inertia of C - sigma I (FP32 LDL^dagger of the scaled
-//     matrix, sigma in a gap above theta_m) counts exactly m eigenvalues
-//     below sigma, so that none was skipped (a count that a pivot near zero
-//     spoils is taken again at a second shift).
+//     the eigenvalues outside the block).  That rho is such a bound, so that
+//     no eigenvalue was skipped, is shown by an FP32 Cholesky factorisation:
+//     C + tau X_m X_m^dagger has rank m more than C, so if it is above sigma
+//     then lambda_{m+1} is, whatever X_m is; see filt_cert_kernel for what the
+//     rounding errors of the factorisation take from sigma.
 //  4. Matrices that do not pass are reduced by the FP64 Householder reduction
 //     and bisected (tridiag.cu, bisect.cu) in one launch each that returns at
 //     once when there are none; nothing waits for the host.
@@ -138,23 +138,19 @@ __device__ __forceinline__ float to_float(double x) {
   return __uint_as_float((m & 0x7fffffffu) | ((unsigned)(b >> 32) & 0x80000000u));
 }
 
-// A <- W (C / s - beta I) W, lower 64-tiles, FP32, identity in the padding.
-// beta = -1 (the operator) or sigma / s (the inertia check).
+// A <- W (C / s + I) W, lower 64-tiles, FP32, identity in the padding
 __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ C, int n, int np,
                                                          const double* __restrict__ shift,
-                                                         const double* __restrict__ sigma,
                                                          const float* __restrict__ w,
                                                          zf* __restrict__ A, int* __restrict__ neg,
-                                                         int* __restrict__ flag,
-                                                         const int* __restrict__ skip) {
+                                                         int* __restrict__ flag) {
   int bi, bk;
   tile_of(blockIdx.x, bi, bk);
   const int k = blockIdx.y, tid = threadIdx.x;
-  if (skip && skip[k]) return;
   const zd* ck = C + (size_t)k * n * n;
   const float* wk = w + (size_t)k * np;
   zf* ak = A + (size_t)k * np * np;
-  const double is = 1.0 / shift[k], beta = sigma ? sigma[k] * is : -1.0;
+  const double is = 1.0 / shift[k];
   const float fs = (float)is;
   if (blockIdx.x == 0 && tid == 0) {
     neg[k] = 0;
@@ -170,7 +166,7 @@ __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ 
       const zd z = ck[(size_t)c * n + r];
       const float f = wr * wk[c];
       if (r == c) {
-        v = make_float2((float)(z.x * is - beta) * f, 0.f);
+        v = make_float2((float)(z.x * is + 1.0) * f, 0.f);
       } else {
         v = make_float2(to_float(z.x) * fs * f, to_float(z.y) * fs * f);
       }
@@ -371,21 +367,21 @@ __global__ void __launch_bounds__(256) ldl64_diag_kernel(zf* __restrict__ A, zf*
   ldl64_diag(a, X + (size_t)k * np * np, dv + (size_t)k * np, np, 0, k, S, Xs, d, &bad, neg, flag);
 }
 
-// 64 x 64 x 64 product on 256 threads, 4 x 4 complex per thread:
+// 64 x 64 x K product on 256 threads, 4 x 4 complex per thread:
 // acc[i][j] += sum_t As[t][row(i)] op(Bs[t][col(j)]), rows 2 tx + {0, 1, 32, 33} and
 // columns 2 ty + {0, 1, 32, 33}, so that two 16-byte loads fetch each operand
 // (eight 8-byte ones kept the shared-memory pipe half busy: 205 -> 183 us per
 // update launch of 90 x 896^2).  Rows t of the tiles are LA, LB apart.
 __device__ __forceinline__ int own(int x, int i) { return 2 * x + (i & 1) + 32 * (i >> 1); }
 
-template <bool CONJB, int LA = TB, int LB = TB>
+template <bool CONJB, int LA = TB, int LB = TB, int K = TB>
 __device__ __forceinline__ void mm64(const zf* __restrict__ As, const zf* __restrict__ Bs,
                                      zf (&acc)[4][4]) {
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const float4* A4 = reinterpret_cast<const float4*>(As) + tx;
   const float4* B4 = reinterpret_cast<const float4*>(Bs) + ty;
 #pragma unroll 8
-  for (int t = 0; t < TB; ++t) {
+  for (int t = 0; t < K; ++t) {
     const float4 a0 = A4[t * (LA / 2)], a1 = A4[t * (LA / 2) + 16];
     const float4 b0 = B4[t * (LB / 2)], b1 = B4[t * (LB / 2) + 16];
     const zf a[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
@@ -562,11 +558,14 @@ __global__ void __launch_bounds__(256) trinv64_kernel(const zf* __restrict__ A, 
 
 // B = W X^dagger D^-1 X W (X = L^-1), 64-tiles (bi, bk) and their mirrors,
 // straight to the BF16 split [Re | Im] hi, [Re | Im] lo of rows of 4 np.  The
-// tile sums over the block rows t >= bi; the longest sums come first.
+// tile sums over the block rows t >= bi; the longest sums come first.  rsum (block
+// column, row): the tile's part of the row sums of |X^dagger D^-1 X|, for
+// filt_kappa_kernel.
 __global__ void __launch_bounds__(256) filt_operator_kernel(const zf* __restrict__ X,
                                                             const float* __restrict__ d, int np,
                                                             const float* __restrict__ w,
-                                                            uint16_t* __restrict__ Bp) {
+                                                            uint16_t* __restrict__ Bp,
+                                                            float* __restrict__ rsum) {
   extern __shared__ __align__(16) unsigned char dsm[];
   zf* As = reinterpret_cast<zf*>(dsm);   // [t][column], stride LDT
   zf* Bs = As + TB * LDT;
@@ -596,7 +595,35 @@ __global__ void __launch_bounds__(256) filt_operator_kernel(const zf* __restrict
       As[own(tx, i) * LDS + own(ty, j)] =
           zscale(zconj(acc[i][j]), wk[bi * TB + own(tx, i)] * wc);
   }
+  // row sums of |tile| and of its mirror (the padding, whose w is zero, adds nothing)
+  float rp[4] = {}, cp[4] = {};
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float a = wk[bi * TB + own(tx, i)] > 0.f && wk[bk * TB + own(ty, j)] > 0.f
+                          ? sqrtf(acc[i][j].x * acc[i][j].x + acc[i][j].y * acc[i][j].y)
+                          : 0.f;
+      rp[i] += a;
+      cp[j] += a;
+    }
+  float(*red)[TB] = reinterpret_cast<float(*)[TB]>(Bs);   // [ty][row]
+  float* rs = rsum + (size_t)k * (np / TB) * np;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) red[ty][own(tx, i)] = rp[i];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) cp[j] += __shfl_xor_sync(0xffffffffu, cp[j], o);
+    if (tx == 0 && bi != bk) rs[(size_t)bi * np + bk * TB + own(ty, j)] = cp[j];
+  }
   __syncthreads();
+  if (tid < TB) {
+    float v = 0.f;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v += red[q][tid];
+    rs[(size_t)bk * np + bi * TB + tid] = v;
+  }
   uint16_t* b = Bp + (size_t)k * np * 4 * np;
   for (int h = 0; h < (bi == bk ? 1 : 2); ++h) {
     // h = 0: rows of bi, columns of bk; h = 1: the conjugate mirror
@@ -616,6 +643,99 @@ __global__ void __launch_bounds__(256) filt_operator_kernel(const zf* __restrict
       uint16_t* o = b + (size_t)(r0 + r) * 4 * np + c0 + c;
 #pragma unroll
       for (int m = 0; m < 4; ++m) *reinterpret_cast<uint32_t*>(o + (size_t)m * np) = v[m];
+    }
+  }
+}
+
+// kappa = the largest row sum of |A^-1|, A = W (C / s + I) W: an upper bound of
+// its norm, so that s / w^2 = diag(C) + s <= kappa (C + s) as quadratic forms.
+// Infinite where the factorisation met a pivot that is not positive.
+__global__ void __launch_bounds__(256) filt_kappa_kernel(const float* __restrict__ rsum, int np,
+                                                         const int* __restrict__ neg,
+                                                         const int* __restrict__ flag,
+                                                         double* __restrict__ kappa) {
+  __shared__ float red[8];
+  const int k = blockIdx.x, tid = threadIdx.x, nt = np / TB;
+  const float* rs = rsum + (size_t)k * nt * np;
+  float m = 0.f;
+  for (int r = tid; r < np; r += 256) {
+    float v = 0.f;
+#pragma unroll 4
+    for (int q = 0; q < nt; ++q) v += rs[(size_t)q * np + r];
+    if (!(v <= m)) m = v == v ? v : INFINITY;
+  }
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((tid & 31) == 0) red[tid >> 5] = m;
+  __syncthreads();
+  if (tid == 0) {
+    for (int q = 0; q < 8; ++q) m = fmaxf(m, red[q]);
+    kappa[k] = neg[k] || flag[k] ? INFINITY : (double)m;
+  }
+}
+
+// A <- W (C / s - sigma / s I) W + Z Z^dagger, Z = (tau / s)^1/2 W X_m for the first m =
+// expect[k] Ritz vectors, lower 64-tiles, FP32, identity in the padding: the
+// matrix whose factorisation shows that nothing was skipped.  A zero in
+// expect or below: the matrix is not certified and is left out.
+__global__ void __launch_bounds__(256) filt_lift_kernel(const zd* __restrict__ C, int n, int np,
+                                                        const double* __restrict__ shift,
+                                                        const double* __restrict__ sigma,
+                                                        const double* __restrict__ tau,
+                                                        const zd* __restrict__ X,
+                                                        const int* __restrict__ expect,
+                                                        const float* __restrict__ w,
+                                                        zf* __restrict__ A, int* __restrict__ neg,
+                                                        int* __restrict__ flag) {
+  __shared__ __align__(16) zf Zr[FB * TB], Zc[FB * TB];   // [vector][row]
+  const int k = blockIdx.y, m = expect[k], tid = threadIdx.x;
+  if (m <= 0) return;
+  int bi, bk;
+  tile_of(blockIdx.x, bi, bk);
+  const zd* ck = C + (size_t)k * n * n;
+  const zd* xk = X + (size_t)k * FB * n;
+  const float* wk = w + (size_t)k * np;
+  zf* ak = A + (size_t)k * np * np;
+  const double is = 1.0 / shift[k], beta = sigma[k] * is;
+  const float fs = (float)is, q = sqrtf((float)(tau[k] * is));
+  if (blockIdx.x == 0 && tid == 0) {
+    neg[k] = 0;
+    flag[k] = 0;
+  }
+  for (int h = 0; h < 2; ++h)
+    for (int e = tid; e < FB * TB; e += 256) {
+      const int t = e / TB, r = (h ? bk : bi) * TB + e % TB;
+      zf z = make_float2(0.f, 0.f);
+      if (t < m && r < n) {
+        const zd x = xk[(size_t)t * n + r];
+        const float f = wk[r] * q;
+        z = make_float2(to_float(x.x) * f, to_float(x.y) * f);
+      }
+      (h ? Zc : Zr)[e] = z;
+    }
+  __syncthreads();
+  const int tx = tid & 15, ty = tid >> 4;
+  zf acc[4][4] = {};
+  mm64<true, TB, TB, FB>(Zr, Zc, acc);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = bk * TB + own(ty, j);
+#pragma unroll
+    for (int i = 0; i < 4; i += 2) {
+      const int r = bi * TB + own(tx, i);
+      zf v[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        v[u] = make_float2(r + u == c ? 1.f : 0.f, 0.f);
+        if (r + u < n && c < n) {
+          const zd z = ck[(size_t)c * n + r + u];
+          const float f = wk[r + u] * wk[c];
+          if (r + u == c) v[u] = make_float2((float)(z.x * is - beta) * f, 0.f);
+          else v[u] = make_float2(to_float(z.x) * fs * f, to_float(z.y) * fs * f);
+          v[u] = zadd(v[u], acc[i + u][j]);
+        }
+      }
+      *reinterpret_cast<float4*>(ak + (size_t)c * np + r) =
+          make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
     }
   }
 }
@@ -1257,88 +1377,88 @@ __global__ void __launch_bounds__(128) filt_coef_kernel(const double* __restrict
   }
 }
 
-// Certificate of a Rayleigh-Ritz step, one warp per matrix: a cut (a gap of at
-// least 2e-3 above a Ritz value i >= nb - 1, sigma in it) whose error sum is small; omega; sigma and the count it has to have (-1: the
-// sum is too large or there is no gap).  The inertia of the scaled matrix in
-// FP32 is exact for a matrix within a relative 1e-4 of C in the form sense
-// (n 2^-24 of the scaled diagonal, doubled), so rho is sigma less that.
+// Certificate of a Rayleigh-Ritz step, one warp per matrix: omega, and a cut
+// above a Ritz value i >= nb - 1 whose error sum is small: m = i + 1 in expect
+// (0: there is none) with sigma and tau for filt_lift_kernel.
+//
+// sigma lies halfway between theta_i and the next eigenvalue as far as the block
+// knows it (theta_{i+1} less its residual norm).  If the factorisation of
+// A + E, A = W (C - sigma + tau X X^dagger) W / s and E its rounding errors, has
+// positive pivots only, then for some x in the span of the lowest m + 1
+// eigenvectors with X^dagger x = 0
+//   0 < x^dagger (C - sigma) x + s ||E|| x^dagger W^-2 x
+//    <= lambda_{m+1} - sigma + ||E|| kappa (lambda_{m+1} + s),
+// so lambda_{m+1} > rho = (sigma - e kappa s) / (1 + e kappa) for any e >= ||E||.
+// No pivot grows in a definite matrix (|L| |D| |L^dagger| has A's diagonal), so E is
+// what roundings of either sign add up to: at most 28 u in the spectral norm
+// and 6.7 u sqrt(n) in Frobenius', u = 2^-24, over cells of n = 98 .. 1029 whose
+// stiffnesses differ by up to 1e5 (numpy model); e = 16 u sqrt(n) is taken.  (The inertia of the
+// indefinite C - sigma has no such bound: its pivots grow by 10 to 2000 there,
+// and E with them.)
 __global__ void __launch_bounds__(128) filt_cert_kernel(
     const double* __restrict__ theta, const float* __restrict__ rpart, int nch,
-    const double* __restrict__ shift, const double* __restrict__ cmax, int kb, int nb,
-    const int* __restrict__ fail, double* __restrict__ omega, double* __restrict__ sigma,
-    int kf, int* __restrict__ expect, int* __restrict__ done) {
+    const double* __restrict__ shift, const double* __restrict__ cmax,
+    const double* __restrict__ kappa, int n, int kb, int nb, const int* __restrict__ fail,
+    double* __restrict__ omega, double* __restrict__ sigma, double* __restrict__ tau,
+    int* __restrict__ expect, int* __restrict__ skip, int* __restrict__ done) {
   const int k = blockIdx.x * 4 + (threadIdx.x >> 5), c = threadIdx.x & 31;
   if (k >= kb || done[k]) return;
-  const double s = shift[k];
+  const double s = shift[k], ek = 16.0 / 16777216.0 * sqrt((double)n) * kappa[k];
   float q32 = 0.f;
   for (int q = 0; q < 2 * nch; ++q) q32 += rpart[((size_t)k * 2 * nch + q) * FB + c];
   const double t = theta[(size_t)k * FB + c];
   const double r2 = 1.001 * (double)q32 * s * s;   // 0.1 % for the FP32 sum
   const double tn = __shfl_down_sync(0xffffffffu, t, 1);
+  const double rn = sqrt(__shfl_down_sync(0xffffffffu, r2, 1));
   // lane i: the cut above Ritz value i
   const double gap = tn - t, at = fmax(t, 1e-3 * s);
-  const double sig = t + 0.5 * fmin(gap, 0.02 * at);
-  const double rho = sig - 1e-4 * at;
+  const double sig = t + 0.5 * fmax(gap - rn, fmin(gap, 0.02 * at));
+  const double rho = (sig - ek * s) / (1.0 + ek);
   double err = 0.0;
   for (int i = 0; i < FB; ++i) {
     const double ti = __shfl_sync(0xffffffffu, t, i), ri = __shfl_sync(0xffffffffu, r2, i);
     if (i <= c) err += ri / (rho - ti);
   }
-  const bool usable = c >= nb - 1 && c < FB - 1 && gap >= 2e-3 * fmax(tn, 1e-3 * s) && rho > t &&
-                      err >= 0.0;
-  // of the cuts whose sum is small enough the one with the widest gap (where
-  // the FP32 count is safest), else the one with the smallest sum
-  const double tol = 64.0 * DBL_EPSILON * cmax[k];
-  double best = !usable ? INFINITY : err <= tol ? -gap / at : err;
+  // of the cuts whose sum is small enough the one with the most room below rho
+  const bool usable = c >= nb - 1 && c < FB - 1 && rho > t && err >= 0.0 &&
+                      err <= 64.0 * DBL_EPSILON * cmax[k];
+  double best = usable ? (rho - t) / at : -1.0;
   int at_i = c;
   for (int o = 16; o > 0; o >>= 1) {
-    const double e2 = __shfl_xor_sync(0xffffffffu, best, o);
+    const double b2 = __shfl_xor_sync(0xffffffffu, best, o);
     const int i2 = __shfl_xor_sync(0xffffffffu, at_i, o);
-    if (e2 < best || (e2 == best && i2 < at_i)) {
-      best = e2;
+    if (b2 > best || (b2 == best && i2 < at_i)) {
+      best = b2;
       at_i = i2;
     }
   }
-  const double sg = __shfl_sync(0xffffffffu, sig, at_i);
-  const double sg2 = __shfl_sync(0xffffffffu, t + 0.75 * fmin(gap, 0.02 * at), at_i);
-  const bool ok = best <= tol && !fail[k];
+  const double sg = __shfl_sync(0xffffffffu, sig, at_i), tg = __shfl_sync(0xffffffffu, tn, at_i);
+  const bool ok = best > 0.0 && !fail[k];
   if (c < nb) omega[(size_t)k * nb + c] = sqrt(fmax(t, 0.0));
   if (c == 0) {
     done[k] = ok;
-    sigma[k] = ok ? sg : 0.0;
-    sigma[kf + k] = ok ? sg2 : 0.0;
-    expect[k] = ok ? at_i + 1 : -1;
+    skip[k] = !ok;
+    sigma[k] = sg;
+    tau[k] = 2.0 * tg;
+    expect[k] = ok ? at_i + 1 : 0;
   }
 }
 
-// A pivot that is zero to 1e-6 by chance (one matrix of some 2000), or a cut too
-// close to an eigenvalue, spoils the FP32 count of a matrix whose error sum is
-// small: it is counted once more at a shift nearer the next Ritz value, which
-// serves the same certificate (sigma only has to lie above rho).  The launches
-// take 0.1 ms when there is none; reducing one matrix of n = 1029 takes 13 ms.
-__global__ void filt_again_kernel(const int* __restrict__ neg, const int* __restrict__ flag,
-                                  const int* __restrict__ expect, int kf,
-                                  double* __restrict__ sigma, int kcap, int* __restrict__ skip) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= kf) return;
-  const bool again = expect[k] >= 0 && (flag[k] || neg[k] != expect[k]);
-  skip[k] = !again;
-  if (again) sigma[k] = sigma[kcap + k];
-}
-
-// the matrices that did not pass, in order; one CTA
+// the matrices that did not pass (no cut, or a pivot that is not positive), in
+// order; one CTA
 __global__ void __launch_bounds__(1024) filt_decide_kernel(const int* __restrict__ neg,
                                                            const int* __restrict__ flag,
                                                            const int* __restrict__ expect, int kb,
                                                            int* __restrict__ stat,
                                                            int* __restrict__ list,
-                                                           int* __restrict__ nlist) {
+                                                           int* __restrict__ nlist,
+                                                           int* __restrict__ reduced) {
   __shared__ int cnt[32], base;
   const int tid = threadIdx.x;
   if (tid == 0) base = 0;
   for (int k0 = 0; k0 < kb; k0 += 1024) {
     const int k = k0 + tid;
-    const bool bad = k < kb && (expect[k] < 0 || flag[k] || neg[k] != expect[k]);
+    const bool bad = k < kb && (expect[k] <= 0 || flag[k] || neg[k] > 0);
     const unsigned m = __ballot_sync(0xffffffffu, bad);
     if ((tid & 31) == 0) cnt[tid >> 5] = __popc(m);
     __syncthreads();
@@ -1346,6 +1466,7 @@ __global__ void __launch_bounds__(1024) filt_decide_kernel(const int* __restrict
     for (int w = 0; w < (tid >> 5); ++w) off += cnt[w];
     if (bad) list[off + __popc(m & ((1u << (tid & 31)) - 1u))] = k;
     if (k < kb) stat[k] = 0;
+    if (k < kb && reduced) reduced[k] = bad;
     __syncthreads();
     if (tid == 0)
       for (int w = 0; w < 32; ++w) base += cnt[w];
@@ -1370,7 +1491,8 @@ bool bs_filter_fits(int n, int nbands) {
 
 void bs_filter_ws_free(FilterWs* w) {
   void* p[] = {w->A, w->X, w->pA, w->pB, w->pD, w->eA, w->eB, w->Xb, w->CX, w->vec, w->vs, w->d, w->part,
-               w->rpart, w->theta, w->W, w->coef, w->shift, w->cmax, w->sigma, w->ord, w->w, w->iw};
+               w->rpart, w->theta, w->W, w->coef, w->shift, w->cmax, w->sigma, w->kappa, w->rsum, w->ord, w->w,
+               w->iw};
   for (void* q : p) cudaFree(q);
   *w = FilterWs();
 }
@@ -1381,7 +1503,7 @@ static size_t filter_bytes(int n) {
   const size_t np = (n + TB - 1) / TB * TB, Kp = (2 * (size_t)n + 63) / 64 * 64;
   return 2 * np * np * sizeof(zf) + (size_t)n * 8 * Kp * 2 + 2 * FB * 8 * Kp * 2 +
          (size_t)24 * 2 * FB * n * 4 + 2 * (size_t)FB * n * sizeof(zd) +
-         7 * FB * np * sizeof(zf) + 65536;
+         7 * FB * np * sizeof(zf) + np / TB * np * sizeof(float) + 65536;
 }
 
 int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
@@ -1418,6 +1540,8 @@ int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
       {(void**)&w->shift, k * sizeof(double)},
       {(void**)&w->cmax, k * sizeof(double)},
       {(void**)&w->sigma, 2 * k * sizeof(double)},
+      {(void**)&w->kappa, k * sizeof(double)},
+      {(void**)&w->rsum, k * (np / TB) * np * sizeof(float)},
       {(void**)&w->ord, k * FB * sizeof(int)},
       {(void**)&w->w, k * np * sizeof(float)},
       {(void**)&w->iw, (7 * k + 1) * sizeof(int)},
@@ -1487,8 +1611,10 @@ static int filter_factor(FilterWs& w, int np, int kf, bool inverse, cudaStream_t
     BS_CHECK_LAUNCH("trinv64_kernel");
   }
   filt_operator_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 2 * TB * LDT * sizeof(zf), s>>>(
-      w.X, w.d, np, w.w, reinterpret_cast<uint16_t*>(w.A));
+      w.X, w.d, np, w.w, reinterpret_cast<uint16_t*>(w.A), w.rsum);
   BS_CHECK_LAUNCH("filt_operator_kernel");
+  filt_kappa_kernel<<<kf, 256, 0, s>>>(w.rsum, np, neg, flag, w.kappa);
+  BS_CHECK_LAUNCH("filt_kappa_kernel");
   return BS_OK;
 }
 
@@ -1509,7 +1635,7 @@ static int filter_ritz(FilterWs& w, int n, int np, int kf, cudaStream_t s) {
 }
 
 int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const FilterFallback& fb,
-                         double* omega, int* stat, int* err, cudaStream_t s) {
+                         double* omega, int* stat, int* err, cudaStream_t s, int* reduced) {
   static_assert(TB == GR, "padded rows are covered by the row chunks");
   // filter degrees of the rounds: the first Ritz values come from plane
   // waves and misplace the cut, so the first filters are short; the later ones
@@ -1527,12 +1653,13 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
     const int kf = std::min(w.kf, kb - k0);
     zd* Ck = C + (size_t)k0 * n * n;
     int *neg = w.iw, *flag = w.iw + w.kf, *expect = w.iw + 2 * w.kf, *list = w.iw + 3 * w.kf,
-        *nlist = w.iw + 4 * w.kf, *fail = nlist + 1, *done = fail + w.kf, *again = done + w.kf;
+        *nlist = w.iw + 4 * w.kf, *fail = nlist + 1, *done = fail + w.kf, *skip = done + w.kf;
+    double *sigma = w.sigma, *tau = w.sigma + w.kf;
     filt_prep_kernel<<<kf, 256, n * sizeof(double), s>>>(Ck, n, np, nbands, 0.2, w.shift, w.cmax,
                                                          w.ord, w.w, fail, done);
     BS_CHECK_LAUNCH("filt_prep_kernel");
-    filt_scale_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(Ck, n, np, w.shift, nullptr, w.w,
-                                                                  w.A, neg, flag, nullptr);
+    filt_scale_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(Ck, n, np, w.shift, w.w, w.A, neg,
+                                                                  flag);
     BS_CHECK_LAUNCH("filt_scale_kernel");
     TRY_LAUNCH(filter_factor(w, np, kf, true, s));
     TRY_LAUNCH(bs_launch_band_pack_trail(Ck, n, 0, n, kf, w.pA, w.eA, s));
@@ -1550,9 +1677,10 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
       if (rd < 3) TRY_LAUNCH(filter_ritz<float>(w, n, np, kf, s));
       else TRY_LAUNCH(filter_ritz<double>(w, n, np, kf, s));
       if (rd >= base) {
-        filt_cert_kernel<<<(kf + 3) / 4, 128, 0, s>>>(w.theta, w.rpart, nch, w.shift, w.cmax, kf,
-                                                      nbands, fail, omega + (size_t)k0 * nbands,
-                                                      w.sigma, w.kf, expect, done);
+        filt_cert_kernel<<<(kf + 3) / 4, 128, 0, s>>>(w.theta, w.rpart, nch, w.shift, w.cmax,
+                                                      w.kappa, n, kf, nbands, fail,
+                                                      omega + (size_t)k0 * nbands, sigma, tau,
+                                                      expect, skip, done);
         BS_CHECK_LAUNCH("filt_cert_kernel");
       }
       if (rd == rounds) break;
@@ -1572,18 +1700,12 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
                                    w.pA, w.pB, w.pD, w.eA,
                                    w.eB, w.CX, n, (long)FB * n, err, s, done));
     }
-    filt_scale_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(Ck, n, np, w.shift, w.sigma, w.w,
-                                                                  w.A, neg, flag, nullptr);
-    BS_CHECK_LAUNCH("filt_scale_kernel");
-    TRY_LAUNCH(filter_factor(w, np, kf, false, s));
-    // once more for certified matrices whose count failed, at another shift
-    filt_again_kernel<<<(kf + 127) / 128, 128, 0, s>>>(neg, flag, expect, kf, w.sigma, w.kf, again);
-    BS_CHECK_LAUNCH("filt_again_kernel");
-    filt_scale_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(Ck, n, np, w.shift, w.sigma, w.w,
-                                                                  w.A, neg, flag, again);
-    BS_CHECK_LAUNCH("filt_scale_kernel");
-    TRY_LAUNCH(filter_factor(w, np, kf, false, s, again));
-    filt_decide_kernel<<<1, 1024, 0, s>>>(neg, flag, expect, kf, stat + k0, list, nlist);
+    filt_lift_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(
+        Ck, n, np, w.shift, sigma, tau, w.Xb, expect, w.w, w.A, neg, flag);
+    BS_CHECK_LAUNCH("filt_lift_kernel");
+    TRY_LAUNCH(filter_factor(w, np, kf, false, s, skip));
+    filt_decide_kernel<<<1, 1024, 0, s>>>(neg, flag, expect, kf, stat + k0, list, nlist,
+                                          reduced ? reduced + k0 : nullptr);
     BS_CHECK_LAUNCH("filt_decide_kernel");
     TRY_LAUNCH(bs_launch_tridiag_list(Ck, n, fb.vec + (size_t)k0 * bs_tridiag_vec_elems(n),
                                       fb.part + (size_t)k0 * bs_tridiag_part_elems(n),
@@ -1593,4 +1715,54 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
                                      omega + (size_t)k0 * nbands, stat + k0, list, nlist, s));
   }
   return BS_OK;
+}
+
+extern "C" int bs_lowest_eigenvalues(const double* C, int n, int batch, int nbands,
+                                     double* omega_out, int* reduced_out, void* stream) {
+  if (!C || !omega_out || batch < 1 || !bs_filter_fits(n, nbands)) {
+    bs_set_error("bs_lowest_eigenvalues: need non-NULL arrays, batch >= 1, %d <= n <= 2048 and "
+                 "1 <= nbands <= %d", BS_FILT_MIN_N, BS_FILT_MAX_BANDS);
+    return BS_EINVAL;
+  }
+  cudaStream_t s = (cudaStream_t)stream;
+  const size_t K = batch, mat = K * n * n * sizeof(zd);
+  void* p[11] = {};
+  const size_t bytes[11] = {mat, K * bs_tridiag_vec_elems(n) * sizeof(zd),
+                            K * bs_tridiag_part_elems(n) * sizeof(zd), K * 2 * n * sizeof(double),
+                            K * n * sizeof(double), K * n * sizeof(zd), K * sizeof(unsigned),
+                            K * nbands * sizeof(double), K * sizeof(int), K * sizeof(int),
+                            sizeof(int)};
+  FilterWs w;
+  int r = BS_OK, late = 0;
+  for (int i = 0; !r && i < 11; ++i)
+    if (cudaMalloc(&p[i], bytes[i]) != cudaSuccess) {
+      cudaGetLastError();
+      bs_set_error("bs_lowest_eigenvalues: out of device memory (%zu bytes)", bytes[i]);
+      r = BS_ENOMEM;
+    }
+  if (!r) r = bs_filter_ws_alloc(&w, n, batch);
+  if (!r) {
+    int* err = (int*)p[10];
+    const FilterFallback fb{(zd*)p[1], (zd*)p[2], (double*)p[3], (double*)p[4], (zd*)p[5],
+                            (unsigned*)p[6]};
+    cudaError_t e = cudaMemcpyAsync(p[0], C, mat, cudaMemcpyDefault, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
+    if (e == cudaSuccess)
+      r = bs_launch_eig_filter((zd*)p[0], n, batch, nbands, w, fb, (double*)p[7], (int*)p[8], err,
+                               s, (int*)p[9]);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(omega_out, p[7], bytes[7], cudaMemcpyDefault, s);
+    if (e == cudaSuccess && reduced_out)
+      e = cudaMemcpyAsync(reduced_out, p[9], bytes[9], cudaMemcpyDefault, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&late, err, sizeof(int), cudaMemcpyDeviceToHost, s);
+    const cudaError_t es = cudaStreamSynchronize(s);   // the scratch is freed below
+    if (!r && (e != cudaSuccess || es != cudaSuccess))
+      r = bs_cuda_status(e != cudaSuccess ? e : es, "bs_lowest_eigenvalues");
+    if (!r && late) {
+      bs_set_error("a tensor-core pipeline wait reached its limit");
+      r = BS_ECUDA;
+    }
+  }
+  bs_filter_ws_free(&w);
+  for (void* q : p) cudaFree(q);
+  return r;
 }

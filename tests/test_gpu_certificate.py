@@ -1,0 +1,71 @@
+"""The certificate of the filtered iteration on matrices it has to refuse.
+
+Each matrix is block diagonal: 64 rows with the eigenvalues 1, 2, 3, ... (rotated
+a little, so that there is something to iterate on) and a dense block of
+large diagonal D whose eigenvalues are D and above, but for one that may lie
+among the wanted ones.  The starting vectors, unit vectors of the smallest
+diagonal entries, have no part in the dense block and the products keep
+exact zeros there, so an eigenvalue in it is always skipped by the iteration;
+only the factorisation can show it.  From D = 1e7 on its mark in the scaled
+matrix is below the rounding errors of an FP32 factorisation.
+
+Tolerance on lambda: a Householder reduction and its bisection err by less
+than (n + 4) eps64 ||C||, the certificate allows 64 eps64 max C_rr; ||C|| <= 2 D
+here and max C_rr >= D, so 2 (n + 128) eps64 max C_rr.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+from paper_1310_6380_gb300 import binding as bs  # noqa: E402
+
+EPS = np.finfo(float).eps
+NV = 64
+
+
+def matrices(n, D, hidden, count, seed):
+    """(count, n, n) and their eigenvalues; hidden: the dense block's low eigenvalue or None."""
+    rng = np.random.default_rng(seed)
+    C, lam = np.zeros((count, n, n), complex), np.empty((count, n))
+    for i in range(count):
+        q = n - NV
+        low = np.arange(1.0, NV + 1) + 0.1 * rng.random(NV)
+        K = rng.standard_normal((NV, NV)) + 1j * rng.standard_normal((NV, NV))
+        V = np.linalg.qr(np.eye(NV) + 0.02 * (K - K.conj().T))[0]
+        C[i, :NV, :NV] = (V * low) @ V.conj().T
+        high = D * (1.0 + rng.random(q))
+        if hidden is not None:
+            high[0] = hidden
+        V = np.linalg.qr(rng.standard_normal((q, q)) + 1j * rng.standard_normal((q, q)))[0]
+        C[i, NV:, NV:] = (V * high) @ V.conj().T
+        C[i] = 0.5 * (C[i] + C[i].conj().T)
+        lam[i] = np.sort(np.concatenate([low, high]))
+    return C, lam
+
+
+def solve(C, nb):
+    w, red = np.empty((len(C), nb)), np.full(len(C), 7, np.int32)
+    bs.bs_lowest_eigenvalues(np.ascontiguousarray(C), nb, w, red)
+    return w ** 2, red
+
+
+@pytest.mark.parametrize("n, D", [(192, 1e2), (192, 1e4), (200, 1e6), (200, 1e7), (256, 1e8),
+                                  (256, 1e9)])
+def test_a_skipped_eigenvalue_is_found(n, D):
+    nb = 6
+    C, lam = matrices(n, D, 2.5, 24, int(np.log10(D)))
+    got, red = solve(C, nb)
+    assert np.abs(got - lam[:, :nb]).max() <= 2 * (n + 128) * EPS * np.abs(C).max()
+    assert red.all()
+
+
+@pytest.mark.parametrize("n, D, nb", [(128, 1e2, 1), (192, 1e2, 6), (200, 1e3, 22)])
+def test_nothing_skipped_is_certified(n, D, nb):
+    C, lam = matrices(n, D, None, 24, n)
+    got, red = solve(C, nb)
+    assert np.abs(got - lam[:, :nb]).max() <= 2 * (n + 128) * EPS * np.abs(C).max()
+    assert not red.any()
