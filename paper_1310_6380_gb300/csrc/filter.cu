@@ -556,6 +556,12 @@ __global__ void __launch_bounds__(256) trinv64_kernel(const zf* __restrict__ A, 
           make_float4(-acc[i][j].x, -acc[i][j].y, -acc[i + 1][j].x, -acc[i + 1][j].y);
 }
 
+__device__ __forceinline__ float fsqrt(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // B = W X^dagger D^-1 X W (X = L^-1), 64-tiles (bi, bk) and their mirrors,
 // straight to the BF16 split [Re | Im] hi, [Re | Im] lo of rows of 4 np.  The
 // tile sums over the block rows t >= bi; the longest sums come first.  rsum (block
@@ -595,15 +601,13 @@ __global__ void __launch_bounds__(256) filt_operator_kernel(const zf* __restrict
       As[own(tx, i) * LDS + own(ty, j)] =
           zscale(zconj(acc[i][j]), wk[bi * TB + own(tx, i)] * wc);
   }
-  // row sums of |tile| and of its mirror (the padding, whose w is zero, adds nothing)
+  // row sums of |tile| and of its mirror (the padding, an identity, adds rows of sum 1)
   float rp[4] = {}, cp[4] = {};
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const float a = wk[bi * TB + own(tx, i)] > 0.f && wk[bk * TB + own(ty, j)] > 0.f
-                          ? sqrtf(acc[i][j].x * acc[i][j].x + acc[i][j].y * acc[i][j].y)
-                          : 0.f;
+      const float a = fsqrt(fmaf(acc[i][j].x, acc[i][j].x, acc[i][j].y * acc[i][j].y));
       rp[i] += a;
       cp[j] += a;
     }
@@ -701,8 +705,9 @@ __global__ void __launch_bounds__(256) filt_lift_kernel(const zd* __restrict__ C
     neg[k] = 0;
     flag[k] = 0;
   }
+  const int m8 = (m + 7) / 8 * 8;   // at most FB
   for (int h = 0; h < 2; ++h)
-    for (int e = tid; e < FB * TB; e += 256) {
+    for (int e = tid; e < m8 * TB; e += 256) {
       const int t = e / TB, r = (h ? bk : bi) * TB + e % TB;
       zf z = make_float2(0.f, 0.f);
       if (t < m && r < n) {
@@ -715,7 +720,7 @@ __global__ void __launch_bounds__(256) filt_lift_kernel(const zd* __restrict__ C
   __syncthreads();
   const int tx = tid & 15, ty = tid >> 4;
   zf acc[4][4] = {};
-  mm64<true, TB, TB, FB>(Zr, Zc, acc);
+  for (int t = 0; t < m8; t += 8) mm64<true, TB, TB, 8>(Zr + t * TB, Zc + t * TB, acc);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int c = bk * TB + own(ty, j);
