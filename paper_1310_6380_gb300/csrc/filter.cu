@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(256) filt_prep_kernel(const zd* __restrict__ C
   __syncthreads();
   double s = sfac * dg[so[nb - 1]];
   // a zero or non-finite diagonal: any scale will do, the certificate decides
-  if (!(s > 0.0) || !(s < 1e300)) s = 1.0;
+  if (!(s > 1e-250) || !(s < 1e250)) s = 1.0;   // (to_float takes |es| < 897)
   if (tid < FB) ord[(size_t)k * FB + tid] = so[tid];
   if (tid == 0) {
     double v = 0.0;
@@ -128,15 +128,24 @@ __device__ __forceinline__ void tile_of(int l, int& bi, int& bk) {
 // (float)x by integer arithmetic (round half up; below the FP32 normal range
 // 0): the FP64 to FP32 conversion runs on the FP64 pipe, 2 per clock and SM
 // (the scaling of 90 matrices of n = 882: 456 us with it, 158 us without).
-// |x| of 2^127 and more is left to it.
-__device__ __forceinline__ float to_float(double x) {
+// es: (float)(x 2^-es).  Everything in FP32 is held in units of 2^es, es the
+// exponent of the matrix's shift, so that no unit of length or mass takes the
+// entries, or the squares of Ritz values that the Jacobi sums, out of its range.
+__device__ __forceinline__ float to_float(double x, int es = 0) {
   const long long b = __double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7ff);
-  if (e >= 1023 + 127) return (float)x;
-  if (e < 1023 - 126) return 0.f;
-  const unsigned m = (unsigned)((b - ((long long)(1023 - 127) << 52) + (1LL << 28)) >> 29);
+  const int e = ((int)(b >> 52) & 0x7ff) - es;
+  if ((unsigned)(e - (1023 - 126)) > 252u) {
+    if (e - 1023 < 127 && e + es < 0x7ff) return 0.f;
+    return e + es == 0x7ff ? (float)x : x < 0.0 ? -INFINITY : INFINITY;
+  }
+  const unsigned m = (unsigned)((b + (1LL << 28)) >> 29) - ((unsigned)(1023 - 127 + es) << 23);
   return __uint_as_float((m & 0x7fffffffu) | ((unsigned)(b >> 32) & 0x80000000u));
 }
+// exponent of a positive normal number, and 2^e
+__device__ __forceinline__ int exponent(double s) {
+  return ((__double2hiint(s) >> 20) & 0x7ff) - 1023;
+}
+__device__ __forceinline__ double exp2i(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
 // A <- W (C / s + I) W, lower 64-tiles, FP32, identity in the padding
 __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ C, int n, int np,
@@ -151,7 +160,8 @@ __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ 
   const float* wk = w + (size_t)k * np;
   zf* ak = A + (size_t)k * np * np;
   const double is = 1.0 / shift[k];
-  const float fs = (float)is;
+  const int es = exponent(shift[k]);
+  const float fs = (float)(is * exp2i(es));
   if (blockIdx.x == 0 && tid == 0) {
     neg[k] = 0;
     flag[k] = 0;
@@ -168,7 +178,7 @@ __global__ void __launch_bounds__(256) filt_scale_kernel(const zd* __restrict__ 
       if (r == c) {
         v = make_float2((float)(z.x * is + 1.0) * f, 0.f);
       } else {
-        v = make_float2(to_float(z.x) * fs * f, to_float(z.y) * fs * f);
+        v = make_float2(to_float(z.x, es) * fs * f, to_float(z.y, es) * fs * f);
       }
     }
     ak[(size_t)c * np + r] = v;
@@ -700,7 +710,8 @@ __global__ void __launch_bounds__(256) filt_lift_kernel(const zd* __restrict__ C
   const float* wk = w + (size_t)k * np;
   zf* ak = A + (size_t)k * np * np;
   const double is = 1.0 / shift[k], beta = sigma[k] * is;
-  const float fs = (float)is, q = sqrtf((float)(tau[k] * is));
+  const int es = exponent(shift[k]);
+  const float fs = (float)(is * exp2i(es)), q = sqrtf((float)(tau[k] * is));
   if (blockIdx.x == 0 && tid == 0) {
     neg[k] = 0;
     flag[k] = 0;
@@ -735,7 +746,7 @@ __global__ void __launch_bounds__(256) filt_lift_kernel(const zd* __restrict__ C
           const zd z = ck[(size_t)c * n + r + u];
           const float f = wk[r + u] * wk[c];
           if (r + u == c) v[u] = make_float2((float)(z.x * is - beta) * f, 0.f);
-          else v[u] = make_float2(to_float(z.x) * fs * f, to_float(z.y) * fs * f);
+          else v[u] = make_float2(to_float(z.x, es) * fs * f, to_float(z.y, es) * fs * f);
           v[u] = zadd(v[u], acc[i + u][j]);
         }
       }
@@ -768,13 +779,13 @@ __global__ void filt_add_kernel(zd* __restrict__ X, const zf* __restrict__ E, in
 }
 
 template <typename R>
-struct RrSmem {   // rows of X and C X in the arithmetic of the step
+struct RrSmem {   // rows of X and C X (FP32: in units of 2^es) in the arithmetic of the step
   typename Cplx<R>::T X[GR][FB + 1], Y[GR][FB + 1];
 };
 
 template <typename R>
 __device__ __forceinline__ void rr_load(RrSmem<R>& sm, const zd* X, const zd* CX, int n, int r0,
-                                        int nthreads) {
+                                        int nthreads, int es) {
   typedef typename Cplx<R>::T T;
   for (int e = threadIdx.x; e < GR * FB; e += nthreads) {
     const int c = e / GR, r = e % GR;
@@ -786,7 +797,7 @@ __device__ __forceinline__ void rr_load(RrSmem<R>& sm, const zd* X, const zd* CX
         y = b;
       } else {
         x = make_float2(to_float(a.x), to_float(a.y));
-        y = make_float2(to_float(b.x), to_float(b.y));
+        y = make_float2(to_float(b.x, es), to_float(b.y, es));
       }
     }
     sm.X[r][c] = x;
@@ -800,8 +811,10 @@ constexpr int GT = 288;
 template <typename R>
 __global__ void __launch_bounds__(GT) filt_gram_kernel(const zd* __restrict__ X,
                                                        const zd* __restrict__ CX, int n,
+                                                       const double* __restrict__ shift,
                                                        zd* __restrict__ part,
                                                        const int* __restrict__ done) {
+  const int es = sizeof(R) == 4 ? exponent(shift[blockIdx.y]) : 0;
   if (done[blockIdx.y]) return;
   extern __shared__ __align__(16) unsigned char dsm[];
   typedef typename Cplx<R>::T T;
@@ -816,7 +829,7 @@ __global__ void __launch_bounds__(GT) filt_gram_kernel(const zd* __restrict__ X,
 #pragma unroll
     for (int j = 0; j < 2; ++j) acc[i][j] = Cplx<R>::make((R)0, (R)0);
   const int r0 = ch * GR, rows = min(GR, n - r0);
-  rr_load(sm, X + (size_t)k * FB * n, CX + (size_t)k * FB * n, n, r0, GT);
+  rr_load(sm, X + (size_t)k * FB * n, CX + (size_t)k * FB * n, n, r0, GT, es);
   __syncthreads();
   if (tid >= 272) return;
 #pragma unroll 4
@@ -830,11 +843,13 @@ __global__ void __launch_bounds__(GT) filt_gram_kernel(const zd* __restrict__ X,
     acc[1][1] = zfmac(b1, a1, acc[1][1]);
   }
   zd* p = part + (((size_t)k * gridDim.x + ch) * 2 + mat) * FB * FB;
+  const double unit = mat ? exp2i(es) : 1.0;
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j)
-      p[(2 * bi + i) * FB + 2 * bj + j] = zmake((double)acc[i][j].x, (double)acc[i][j].y);
+      p[(2 * bi + i) * FB + 2 * bj + j] =
+          zmake((double)acc[i][j].x * unit, (double)acc[i][j].y * unit);
 }
 
 // A real number as two FP32 terms, and acc += a b with it: the product's high
@@ -845,9 +860,9 @@ struct df {
 };
 // the upper 24 bits of the mantissa are an FP32 number as they stand, so one
 // FP64 subtraction is all that the split takes from the FP64 pipe
-__device__ __forceinline__ df df_of(double x) {
+__device__ __forceinline__ df df_of(double x, int es = 0) {
   const double xh = __longlong_as_double(__double_as_longlong(x) & ~0x1FFFFFFFLL);
-  return {to_float(xh), to_float(x - xh)};
+  return {to_float(xh, es), to_float(x - xh, es)};
 }
 __device__ __forceinline__ void df_fma(df a, df b, df& acc) {
   const float p = a.h * b.h;
@@ -863,14 +878,14 @@ __device__ __forceinline__ df df_neg(df a) { return {-a.h, -a.l}; }
 template <typename R> struct RotSmem;
 template <> struct RotSmem<float> {
   zf W[FB][FB], X[FB][GR], Y[FB][GR];
-  static __device__ __forceinline__ void put(zf& o, zd v) {
-    o = make_float2(to_float(v.x), to_float(v.y));
+  static __device__ __forceinline__ void put(zf& o, zd v, int es = 0) {
+    o = make_float2(to_float(v.x, es), to_float(v.y, es));
   }
 };
 template <> struct RotSmem<double> {
   float4 W[FB][FB], X[FB][GR], Y[FB][GR];
-  static __device__ __forceinline__ void put(float4& o, zd v) {
-    const df a = df_of(v.x), b = df_of(v.y);
+  static __device__ __forceinline__ void put(float4& o, zd v, int es = 0) {
+    const df a = df_of(v.x, es), b = df_of(v.y, es);
     o = make_float4(a.h, b.h, a.l, b.l);
   }
 };
@@ -890,6 +905,8 @@ __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
                                                           uint16_t* __restrict__ Rs,
                                                           float* __restrict__ rpart,
                                                           const int* __restrict__ done) {
+  const double sh = shift[blockIdx.y];   // (beside the load of done)
+  const int es = exponent(sh);
   if (done[blockIdx.y]) return;
   constexpr bool D = sizeof(R) == 8;
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -903,7 +920,7 @@ __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
     const int l = e / GR, r = e % GR, row = ch * GR + r;
     const bool ok = row < n;
     RotSmem<R>::put(sm.X[l][r], ok ? xk[(size_t)l * n + row] : zmake(0.0, 0.0));
-    RotSmem<R>::put(sm.Y[l][r], ok ? yk[(size_t)l * n + row] : zmake(0.0, 0.0));
+    RotSmem<R>::put(sm.Y[l][r], ok ? yk[(size_t)l * n + row] : zmake(0.0, 0.0), es);
   }
   __syncthreads();
   const int r = tid & 63, c0 = (tid >> 6) * 8;
@@ -942,11 +959,11 @@ __global__ void __launch_bounds__(256) filt_rotate_kernel(zd* __restrict__ X,
       }
     }
   }
-  const double is = 1.0 / shift[k];
+  const double is = exp2i(es) / sh, unit = exp2i(-es);
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int c = c0 + j;
-    const double t = theta[(size_t)k * FB + c];
+    const double t = theta[(size_t)k * FB + c] * unit;
     zf rv = make_float2(0.f, 0.f);
     if (live) {
       const zd x = zmake((double)xr[j].h + (double)xr[j].l, (double)xi[j].h + (double)xi[j].l);
@@ -1133,10 +1150,13 @@ struct EigSmem {
 
 template <typename R>
 __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ part, int nch,
+                                                       const double* __restrict__ shift,
                                                        double* __restrict__ theta,
                                                        zd* __restrict__ W,
                                                        int* __restrict__ fail,
                                                        const int* __restrict__ done) {
+  const int es = exponent(shift[blockIdx.x]);
+  const double unit = exp2i(-es);   // H and the Ritz values in units of 2^es
   if (done[blockIdx.x]) return;
   extern __shared__ __align__(16) unsigned char dsm[];
   typedef typename Cplx<R>::T T;
@@ -1162,7 +1182,7 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
     }
     if (r == c) g.y = h.y = 0.0;
     sm.G[r][c] = Cplx<R>::make((R)g.x, (R)g.y);
-    sm.H[r][c] = Cplx<R>::make((R)h.x, (R)h.y);
+    sm.H[r][c] = Cplx<R>::make((R)(h.x * unit), (R)(h.y * unit));
     if (r == c) {
       sc[r] = g.x > 0.0 ? (R)rsqrt((R)g.x) : (R)0;
       out[r] = 0;
@@ -1329,7 +1349,7 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
       o = zmake((double)x.x, (double)x.y);
     }
     W[(size_t)k * FB * FB + r + (size_t)rank[c] * FB] = o;
-    if (r == 0) theta[(size_t)k * FB + rank[c]] = ev[c];
+    if (r == 0) theta[(size_t)k * FB + rank[c]] = ev[c] * exp2i(es);
   }
 }
 
@@ -1627,10 +1647,11 @@ template <typename R>
 static int filter_ritz(FilterWs& w, int n, int np, int kf, cudaStream_t s) {
   const int nch = (n + GR - 1) / GR;
   int *fail = w.iw + 4 * w.kf + 1, *done = fail + w.kf;
-  filt_gram_kernel<R><<<dim3(nch, kf), GT, sizeof(RrSmem<R>), s>>>(w.Xb, w.CX, n, w.part, done);
+  filt_gram_kernel<R><<<dim3(nch, kf), GT, sizeof(RrSmem<R>), s>>>(w.Xb, w.CX, n, w.shift, w.part,
+                                                                  done);
   BS_CHECK_LAUNCH("filt_gram_kernel");
-  filt_eig_kernel<R><<<kf, 256, sizeof(EigSmem<R>), s>>>(w.part, nch, w.theta, w.W,
-                                                         fail, done);
+  filt_eig_kernel<R><<<kf, 256, sizeof(EigSmem<R>), s>>>(w.part, nch, w.shift, w.theta, w.W, fail,
+                                                         done);
   BS_CHECK_LAUNCH("filt_eig_kernel");
   // the rotation covers the padded rows as well (np <= nch GR)
   filt_rotate_kernel<R><<<dim3(nch, kf), 256, sizeof(RotSmem<R>), s>>>(w.Xb, w.CX, n, np, w.W, w.theta, w.shift,

@@ -22,6 +22,7 @@ if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
 from paper_1310_6380_gb300 import binding as bs  # noqa: E402
+from paper_1310_6380_gb300 import cells  # noqa: E402
 
 EPS = np.finfo(float).eps
 NV = 64
@@ -69,3 +70,54 @@ def test_nothing_skipped_is_certified(n, D, nb):
     got, red = solve(C, nb)
     assert np.abs(got - lam[:, :nb]).max() <= 2 * (n + 128) * EPS * np.abs(C).max()
     assert not red.any()
+
+
+@pytest.mark.parametrize("e", [-400, -120, -40, 40, 62, 124, 400])
+def test_any_unit(e):
+    """A power of two as the unit changes no bit of any step: the same matrices
+    are certified and omega is 2^(e/2) times as large.  (The Ritz values of an
+    epoxy/steel cell of 10 um in SI units, near 2^62, have squares beyond FP32.)"""
+    C, _ = matrices(150, 1e2, None, 4, 3)
+    C = np.ascontiguousarray(C)
+    w, red = np.empty((4, 8)), np.full(4, 7, np.int32)
+    bs.bs_lowest_eigenvalues(C, 8, w, red)
+    we, rede = np.empty((4, 8)), np.full(4, 7, np.int32)
+    bs.bs_lowest_eigenvalues(C * 2.0 ** e, 8, we, rede)
+    assert not red.any() and not rede.any()
+    assert np.array_equal(we, w * 2.0 ** (e // 2))
+
+
+@pytest.mark.parametrize("a", [1e-6, 1e-5, 6.023e-3, 1e3])
+def test_cells_of_any_size_are_certified(a):
+    """The steel/epoxy cell in SI units at lattice constants from 1 um to 1 km:
+    omega a does not depend on a."""
+    cell = cells.steel_epoxy_hex_cell(48)
+    scale = a / np.linalg.norm(cell.h1)
+    Q = np.array([[0.13, 0.21], [0.5, 0.0], [0.3, 0.3]])
+    ref = None
+    for f in (1.0, scale):
+        h = bs.bs_create_cell(np.asarray(cell.h1) * f, np.asarray(cell.h2) * f,
+                              np.ascontiguousarray(cell.phase, np.uint16), cell.lam.copy(),
+                              cell.mu.copy(), cell.rho.copy(), 4, bs.BS_PREC_FP64)
+        try:
+            bs.bs_assemble(h)
+            n = bs.bs_cell_dims(h)[1]
+            C = np.empty((3, n, n), np.complex128)
+            for k in range(3):
+                bs.bs_reduced_matrix(h, Q[k].copy(), C[k].view(np.float64))
+            st = np.full(3, 7, np.int32)
+            ws = np.empty((3, 12))
+            bs.bs_solve_k(h, Q, 12, ws, st)
+        finally:
+            bs.bs_destroy_cell(h)
+        low = np.tril(C.transpose(0, 2, 1), -1)
+        C = low + low.conj().transpose(0, 2, 1) + np.einsum("kii->ki", C).real[:, :, None] * np.eye(n)
+        w, red = np.empty((3, 12)), np.full(3, 7, np.int32)
+        bs.bs_lowest_eigenvalues(np.ascontiguousarray(C), 12, w, red)
+        assert not red.any() and not st.any()
+        tol = 2 * (n + 128) * EPS * np.abs(C).max()
+        assert np.abs(w ** 2 - ws ** 2).max() <= tol
+        if ref is None:
+            ref = w
+        else:
+            assert np.abs((w * f) ** 2 - ref ** 2).max() <= 2 * tol * f * f
