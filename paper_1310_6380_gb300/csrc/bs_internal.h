@@ -456,6 +456,7 @@ struct FilterWs {
   zd* part = nullptr;       // kf x chunks x 2 x 32 x 32 partial Gram matrices
   float* rpart = nullptr;   // kf x chunks x 2 x 32 partial residual sums
   double* theta = nullptr;  // kf x 32
+  double* rerr = nullptr;   // kf x 32: what the Ritz values may be off by
   zd* W = nullptr;          // kf x 32 x 32
   float* coef = nullptr;    // kf x BS_FILT_MAXDEG x 4 x 32
   double* shift = nullptr;  // kf

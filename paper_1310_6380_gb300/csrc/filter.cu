@@ -23,7 +23,8 @@
 //     bound of lambda_{m+1}, Lehmann's bound in its trace form (the residual
 //     Gram matrix replaced by its trace) gives
 //       lambda_i >= theta_i - sum_{c <= m} ||r_c||^2 / (rho - theta_c),  i <= m.
-//     A matrix passes when that sum is at most 64 eps64 max_r C_rr (the
+//     A matrix passes when that sum, and what the small eigenproblem may have
+//     left of the Ritz values, are at most 64 eps64 max_r C_rr (the
 //     backward error of a reduction to tridiagonal form and its bisection is
 //     of that size; the sum overestimates the error, whose own gap is that to
 //     the eigenvalues outside the block).  That rho is such a bound, so that
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(GT) filt_gram_kernel(const zd* __restrict__ X,
                                                        const double* __restrict__ shift,
                                                        zd* __restrict__ part,
                                                        const int* __restrict__ done) {
-  const int es = sizeof(R) == 4 ? exponent(shift[blockIdx.y]) : 0;
+  const int es = exponent(shift[blockIdx.y]);
   if (done[blockIdx.y]) return;
   extern __shared__ __align__(16) unsigned char dsm[];
   typedef typename Cplx<R>::T T;
@@ -843,7 +844,8 @@ __global__ void __launch_bounds__(GT) filt_gram_kernel(const zd* __restrict__ X,
     acc[1][1] = zfmac(b1, a1, acc[1][1]);
   }
   zd* p = part + (((size_t)k * gridDim.x + ch) * 2 + mat) * FB * FB;
-  const double unit = mat ? exp2i(es) : 1.0;
+  // H in units of 2^es (FP32: its operand is)
+  const double unit = sizeof(R) == 8 && mat ? exp2i(-es) : 1.0;
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -1142,26 +1144,38 @@ __device__ __forceinline__ int jacobi32(JacobiSmem& sm, float offtol, int maxswe
 // multiply-adds a clock, bounds a matrix otherwise (with the products in FP64
 // 210 us per step of one matrix, 155 us so).  fail: G not
 // positive definite.
+//
+// CHECK (the steps that can certify): the Ritz values are replaced by v^dagger A v of
+// the corrected vectors, and rerr gets what they may still be off by.  Jacobi's
+// FP32 entries leave errors of 6e-8 of what they begin with, which in a step
+// whose block was far from diagonal (an ill-conditioned Gram matrix before it)
+// made Ritz values wrong by 1e4 eps64 ||C|| that no residual shows.  With
+// S = V^dagger A V, a Ritz value is within sum_j min(|S_ij|, 2 |S_ij|^2 / |S_ii - S_jj|) of
+// S_ii, and A itself within eps64 ||A|| / (smallest pivot of G).  The products
+// take 48 bits, the off-diagonal part from U = A V - V diag(S) in FP32: 7 us.
 template <typename R>
 struct EigSmem {
   typename Cplx<R>::T G[FB][FB + 1], H[FB][FB + 1], Li[FB][FB + 1];
   JacobiSmem J;
 };
+struct EigCheckSmem : EigSmem<double> {
+  float4 A[FB][FB + 1];   // two terms
+};
 
-template <typename R>
+template <typename R, bool CHECK>
 __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ part, int nch,
                                                        const double* __restrict__ shift,
                                                        double* __restrict__ theta,
                                                        zd* __restrict__ W,
                                                        int* __restrict__ fail,
+                                                       double* __restrict__ rerr,
                                                        const int* __restrict__ done) {
-  const int es = exponent(shift[blockIdx.x]);
-  const double unit = exp2i(-es);   // H and the Ritz values in units of 2^es
   if (done[blockIdx.x]) return;
   extern __shared__ __align__(16) unsigned char dsm[];
   typedef typename Cplx<R>::T T;
   EigSmem<R>& sm = *reinterpret_cast<EigSmem<R>*>(dsm);
   __shared__ double ev[FB];
+  __shared__ float re_max[FB];
   __shared__ R sc[FB], pinv[FB], sc_top;
   __shared__ int rank[FB], bad, out[FB];
   // a pivot of the unit-diagonal G below the rounding of its entries
@@ -1182,7 +1196,7 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
     }
     if (r == c) g.y = h.y = 0.0;
     sm.G[r][c] = Cplx<R>::make((R)g.x, (R)g.y);
-    sm.H[r][c] = Cplx<R>::make((R)(h.x * unit), (R)(h.y * unit));
+    sm.H[r][c] = Cplx<R>::make((R)h.x, (R)h.y);
     if (r == c) {
       sc[r] = g.x > 0.0 ? (R)rsqrt((R)g.x) : (R)0;
       out[r] = 0;
@@ -1251,6 +1265,12 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
     if (r < c) continue;
     T s = sm.H[r][c];
     if (bad && (out[r] || out[c])) s = Cplx<R>::make(r == c ? sc_top : (R)0, (R)0);
+    if constexpr (CHECK) {
+        float4(*A4)[FB + 1] = reinterpret_cast<EigCheckSmem&>(sm).A;
+        const df x = df_of(s.x), y = df_of(s.y);
+        A4[r][c] = make_float4(x.h, y.h, x.l, y.l);
+        if (r != c) A4[c][r] = make_float4(x.h, -y.h, x.l, -y.l);
+      }
     if (r == c) {
       const float h = (float)s.x;
       sm.J.D[0][r] = make_float2(h, (float)(s.x - (R)h));
@@ -1319,13 +1339,94 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
       V4[r][c].w = fmaf(iv, V4[r][c].y, V4[r][c].w);
     }
     __syncthreads();
+    if constexpr (CHECK) {
+      float4(*A4)[FB + 1] = reinterpret_cast<EigCheckSmem&>(sm).A;
+      zf(*U)[FB + 1] = sm.J.A[0];
+      float(*S)[FB + 1] = reinterpret_cast<float(*)[FB + 1]>(&sm.J.A[1][0][0]);
+      // (A V)_rc, thread: column c = tid % 32, rows tid / 32 + 8 j
+      const int col = tid & 31, row = tid >> 5;
+      df re[4], im[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) re[j] = im[j] = {0.f, 0.f};
+#pragma unroll 2
+      for (int t = 0; t < FB; ++t) {
+        const float4 v = V4[t][col];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 a = A4[row + 8 * j][t];
+          df_fma({a.x, a.z}, {v.x, v.z}, re[j]);
+          df_fma({a.x, a.z}, {v.y, v.w}, im[j]);
+          df_fma({-a.y, -a.w}, {v.y, v.w}, re[j]);
+          df_fma({a.y, a.w}, {v.x, v.z}, im[j]);
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        A4[row + 8 * j][col] = make_float4(re[j].h, im[j].h, re[j].l, im[j].l);
+      __syncthreads();
+      {   // S_cc = Re v_c^dagger (A v_c), eight lanes per column
+        df d = {0.f, 0.f};
+        for (int r = q; r < FB; r += 8) {
+          const float4 v = V4[r][c], a = A4[r][c];
+          df_fma({v.x, v.z}, {a.x, a.z}, d);
+          df_fma({v.y, v.w}, {a.y, a.w}, d);
+        }
+        double x = (double)d.h + (double)d.l;
+        for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (q == 0) ev[c] = x;
+      }
+      __syncthreads();
+      const df sc2 = df_of(-ev[col]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 v = V4[row + 8 * j][col];
+        df_fma(sc2, {v.x, v.z}, re[j]);
+        df_fma(sc2, {v.y, v.w}, im[j]);
+        U[row + 8 * j][col] = make_float2(re[j].h + re[j].l, im[j].h + im[j].l);
+      }
+      __syncthreads();
+      zf d[4] = {};
+#pragma unroll 4
+      for (int t = 0; t < FB; ++t) {
+        const zf u = U[t][col];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 v = V4[t][row + 8 * j];
+          d[j] = zfmac(u, make_float2(v.x, v.y), d[j]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)   // |S_rc|, r != c
+        S[row + 8 * j][col] = fsqrt(fmaf(d[j].x, d[j].x, d[j].y * d[j].y));
+      __syncthreads();
+      {   // the bound of Ritz value c from its row of S, eight lanes per value
+        float e = 0.f, top = 0.f, ip = 0.f;
+        for (int r = q; r < FB; r += 8) {
+          top = fmaxf(top, fabsf((float)ev[r]));
+          ip = fmaxf(ip, (float)pinv[r]);
+          const float a = fmaxf(S[r][c], S[c][r]), g = fabsf((float)(ev[r] - ev[c]));
+          if (r != c) e += 2.f * a < g ? 2.f * a * __fdividef(a, g) : a;
+        }
+        for (int o = 4; o > 0; o >>= 1) {
+          e += __shfl_xor_sync(0xffffffffu, e, o);
+          top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+          ip = fmaxf(ip, __shfl_xor_sync(0xffffffffu, ip, o));
+        }
+        e += (float)DBL_EPSILON * top * ip * ip;
+        if (q == 0) re_max[c] = e == e ? e : INFINITY;
+      }
+      __syncthreads();
+    }
   }
+  const double unit = exp2i(exponent(shift[k]));   // of H and the Ritz values
   if (tid < FB) {
     const double x = ev[tid];
     int rk = 0;
     for (int c = 0; c < FB; ++c) rk += ev[c] < x || (ev[c] == x && c < tid);
     if (!(x == x)) rk = tid;
     rank[tid] = rk;
+    if constexpr (CHECK) rerr[(size_t)k * FB + rk] = (double)re_max[tid] * unit;
   }
   __syncthreads();
   for (int e = tid; e < FB * FB; e += 256) {
@@ -1349,7 +1450,7 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
       o = zmake((double)x.x, (double)x.y);
     }
     W[(size_t)k * FB * FB + r + (size_t)rank[c] * FB] = o;
-    if (r == 0) theta[(size_t)k * FB + rank[c]] = ev[c] * exp2i(es);
+    if (r == 0) theta[(size_t)k * FB + rank[c]] = ev[c] * unit;
   }
 }
 
@@ -1421,9 +1522,9 @@ __global__ void __launch_bounds__(128) filt_coef_kernel(const double* __restrict
 // indefinite C - sigma has no such bound: its pivots grow by 10 to 2000 there,
 // and E with them.)
 __global__ void __launch_bounds__(128) filt_cert_kernel(
-    const double* __restrict__ theta, const float* __restrict__ rpart, int nch,
-    const double* __restrict__ shift, const double* __restrict__ cmax,
-    const double* __restrict__ kappa, int n, int kb, int nb, const int* __restrict__ fail,
+    const double* __restrict__ theta, const double* __restrict__ rerr,
+    const float* __restrict__ rpart, int nch, const double* __restrict__ shift,
+    const double* __restrict__ cmax, const double* __restrict__ kappa, int n, int kb, int nb, const int* __restrict__ fail,
     double* __restrict__ omega, double* __restrict__ sigma, double* __restrict__ tau,
     int* __restrict__ expect, int* __restrict__ skip, int* __restrict__ done) {
   const int k = blockIdx.x * 4 + (threadIdx.x >> 5), c = threadIdx.x & 31;
@@ -1432,21 +1533,29 @@ __global__ void __launch_bounds__(128) filt_cert_kernel(
   float q32 = 0.f;
   for (int q = 0; q < 2 * nch; ++q) q32 += rpart[((size_t)k * 2 * nch + q) * FB + c];
   const double t = theta[(size_t)k * FB + c];
-  const double r2 = 1.001 * (double)q32 * s * s;   // 0.1 % for the FP32 sum
+  q32 *= 1.001f;   // (residual / s)^2; 0.1 % for the FP32 sums
   const double tn = __shfl_down_sync(0xffffffffu, t, 1);
-  const double rn = sqrt(__shfl_down_sync(0xffffffffu, r2, 1));
+  const double rn = s * (double)sqrtf(__shfl_down_sync(0xffffffffu, q32, 1));
   // lane i: the cut above Ritz value i
   const double gap = tn - t, at = fmax(t, 1e-3 * s);
   const double sig = t + 0.5 * fmax(gap - rn, fmin(gap, 0.02 * at));
   const double rho = (sig - ek * s) / (1.0 + ek);
-  double err = 0.0;
+  // the error sum over s, in FP32 but for the differences
+  const double is = 1.0 / s;
+  float err = 0.f;
   for (int i = 0; i < FB; ++i) {
-    const double ti = __shfl_sync(0xffffffffu, t, i), ri = __shfl_sync(0xffffffffu, r2, i);
-    if (i <= c) err += ri / (rho - ti);
+    const double ti = __shfl_sync(0xffffffffu, t, i);
+    const float qi = __shfl_sync(0xffffffffu, q32, i);
+    if (i <= c) err += __fdividef(qi, (float)((rho - ti) * is));
+  }
+  double re = rerr[(size_t)k * FB + c];   // the most of Ritz values 0 .. c
+  for (int o = 1; o < FB; o <<= 1) {
+    const double x = __shfl_up_sync(0xffffffffu, re, o);
+    if (c >= o) re = fmax(re, x);
   }
   // of the cuts whose sum is small enough the one with the most room below rho
-  const bool usable = c >= nb - 1 && c < FB - 1 && rho > t && err >= 0.0 &&
-                      err <= 64.0 * DBL_EPSILON * cmax[k];
+  const bool usable = c >= nb - 1 && c < FB - 1 && rho > t && err >= 0.f &&
+                      (double)err * s + re <= 64.0 * DBL_EPSILON * cmax[k];
   double best = usable ? (rho - t) / at : -1.0;
   int at_i = c;
   for (int o = 16; o > 0; o >>= 1) {
@@ -1516,7 +1625,7 @@ bool bs_filter_fits(int n, int nbands) {
 
 void bs_filter_ws_free(FilterWs* w) {
   void* p[] = {w->A, w->X, w->pA, w->pB, w->pD, w->eA, w->eB, w->Xb, w->CX, w->vec, w->vs, w->d, w->part,
-               w->rpart, w->theta, w->W, w->coef, w->shift, w->cmax, w->sigma, w->kappa, w->rsum, w->ord, w->w,
+               w->rpart, w->theta, w->rerr, w->W, w->coef, w->shift, w->cmax, w->sigma, w->kappa, w->rsum, w->ord, w->w,
                w->iw};
   for (void* q : p) cudaFree(q);
   *w = FilterWs();
@@ -1560,6 +1669,7 @@ int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
       {(void**)&w->part, k * nch * 2 * FB * FB * sizeof(zd)},
       {(void**)&w->rpart, k * nch * 2 * FB * sizeof(float)},
       {(void**)&w->theta, k * FB * sizeof(double)},
+      {(void**)&w->rerr, k * FB * sizeof(double)},
       {(void**)&w->W, k * FB * FB * sizeof(zd)},
       {(void**)&w->coef, k * BS_FILT_MAXDEG * 4 * FB * sizeof(float)},
       {(void**)&w->shift, k * sizeof(double)},
@@ -1600,8 +1710,9 @@ static int filter_attrs() {
       {(const void*)filt_gram_kernel<float>, (int)sizeof(RrSmem<float>)},
       {(const void*)filt_rotate_kernel<double>, (int)sizeof(RotSmem<double>)},
       {(const void*)filt_rotate_kernel<float>, (int)sizeof(RotSmem<float>)},
-      {(const void*)filt_eig_kernel<double>, (int)sizeof(EigSmem<double>)},
-      {(const void*)filt_eig_kernel<float>, (int)sizeof(EigSmem<float>)},
+      {(const void*)filt_eig_kernel<double, true>, (int)sizeof(EigCheckSmem)},
+      {(const void*)filt_eig_kernel<double, false>, (int)sizeof(EigSmem<double>)},
+      {(const void*)filt_eig_kernel<float, false>, (int)sizeof(EigSmem<float>)},
   };
   for (auto& f : fs) {
     const cudaError_t e =
@@ -1643,15 +1754,16 @@ static int filter_factor(FilterWs& w, int np, int kf, bool inverse, cudaStream_t
   return BS_OK;
 }
 
-template <typename R>
+// CHECK: a step that can certify, whose Ritz values come with their error bound
+template <typename R, bool CHECK>
 static int filter_ritz(FilterWs& w, int n, int np, int kf, cudaStream_t s) {
   const int nch = (n + GR - 1) / GR;
   int *fail = w.iw + 4 * w.kf + 1, *done = fail + w.kf;
   filt_gram_kernel<R><<<dim3(nch, kf), GT, sizeof(RrSmem<R>), s>>>(w.Xb, w.CX, n, w.shift, w.part,
                                                                   done);
   BS_CHECK_LAUNCH("filt_gram_kernel");
-  filt_eig_kernel<R><<<kf, 256, sizeof(EigSmem<R>), s>>>(w.part, nch, w.shift, w.theta, w.W, fail,
-                                                         done);
+  filt_eig_kernel<R, CHECK><<<kf, 256, CHECK ? sizeof(EigCheckSmem) : sizeof(EigSmem<R>), s>>>(
+      w.part, nch, w.shift, w.theta, w.W, fail, w.rerr, done);
   BS_CHECK_LAUNCH("filt_eig_kernel");
   // the rotation covers the padded rows as well (np <= nch GR)
   filt_rotate_kernel<R><<<dim3(nch, kf), 256, sizeof(RotSmem<R>), s>>>(w.Xb, w.CX, n, np, w.W, w.theta, w.shift,
@@ -1700,11 +1812,12 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
     const int cstride = BS_FILT_MAXDEG * 4 * FB;
     for (int rd = 0; rd <= rounds; ++rd) {
       // the first three steps only steer the iteration: FP32 products of the block
-      if (rd < 3) TRY_LAUNCH(filter_ritz<float>(w, n, np, kf, s));
-      else TRY_LAUNCH(filter_ritz<double>(w, n, np, kf, s));
+      if (rd < 3) TRY_LAUNCH((filter_ritz<float, false>(w, n, np, kf, s)));
+      else if (rd < base) TRY_LAUNCH((filter_ritz<double, false>(w, n, np, kf, s)));
+      else TRY_LAUNCH((filter_ritz<double, true>(w, n, np, kf, s)));
       if (rd >= base) {
-        filt_cert_kernel<<<(kf + 3) / 4, 128, 0, s>>>(w.theta, w.rpart, nch, w.shift, w.cmax,
-                                                      w.kappa, n, kf, nbands, fail,
+        filt_cert_kernel<<<(kf + 3) / 4, 128, 0, s>>>(w.theta, w.rerr, w.rpart, nch, w.shift,
+                                                      w.cmax, w.kappa, n, kf, nbands, fail,
                                                       omega + (size_t)k0 * nbands, sigma, tau,
                                                       expect, skip, done);
         BS_CHECK_LAUNCH("filt_cert_kernel");

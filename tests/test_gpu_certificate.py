@@ -72,6 +72,34 @@ def test_nothing_skipped_is_certified(n, D, nb):
     assert not red.any()
 
 
+def spectrum_matrices(n, low, high, angle, count, seed):
+    """Hermitian matrices with the given eigenvalues `low`, the others evenly in `high`,
+    whose eigenvectors are unit vectors turned into each other by about `angle`."""
+    rng = np.random.default_rng(seed)
+    C, lam = np.empty((count, n, n), complex), np.empty((count, n))
+    for i in range(count):
+        lam[i] = np.sort(np.concatenate([low, np.linspace(*high, n - len(low))]))
+        K = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+        V = np.linalg.qr(np.eye(n) + angle / np.sqrt(n) * (K - K.conj().T))[0]
+        C[i] = (V * lam[i]) @ V.conj().T
+        C[i] = 0.5 * (C[i] + C[i].conj().T)
+        # positive semidefinite to rounding, with a diagonal that is not negative
+    return C, lam
+
+
+@pytest.mark.parametrize("n", [98, 200])
+@pytest.mark.parametrize("low", [[1e-6], [1e-4, 1e-4], [0.01, 0.02, 20.0]], ids=["one", "two", "three"])
+@pytest.mark.parametrize("top", [1e3, 1e5])
+@pytest.mark.parametrize("angle", [0.1, 0.5])
+def test_lone_low_eigenvalues(n, low, top, angle):
+    """A few eigenvalues far below the others, as at wavevectors near Gamma: the
+    filters grow them in every column, the Gram matrices become
+    ill-conditioned, and the small eigenproblem begins far from diagonal."""
+    C, lam = spectrum_matrices(n, low, (50.0, top), angle, 16, n)
+    got, red = solve(C, len(low))
+    assert np.abs(got - lam[:, :len(low)]).max() <= (n + 128) * EPS * top
+
+
 @pytest.mark.parametrize("e", [-400, -120, -40, 40, 62, 124, 400])
 def test_any_unit(e):
     """A power of two as the unit changes no bit of any step: the same matrices
