@@ -435,6 +435,7 @@ int bs_launch_rank2_update(const uint16_t* dA, const uint16_t* dB, const int* ex
 // filter.cu: the lowest branches by filtered subspace iteration (FP32
 // shift-invert operator, FP64 Rayleigh-Ritz, residual and inertia certificate)
 #define BS_FILT_BLOCK 32       // columns of the block
+#define BS_FILT_START 128      // plane waves that enter its starting vectors
 #define BS_FILT_MAX_BANDS 22   // wanted branches: at least 10 guard vectors remain
 #define BS_FILT_MIN_N 96
 #define BS_FILT_MAXDEG 12      // degrees of one filter
@@ -464,7 +465,7 @@ struct FilterWs {
   double* sigma = nullptr;  // 2 kf: sigma and tau of the certificate
   double* kappa = nullptr;  // kf: bound of ||A^-1||
   float* rsum = nullptr;    // kf x np / 64 x np: row sums of |A^-1| by block column
-  int* ord = nullptr;       // kf x 32
+  int* ord = nullptr;       // kf x BS_FILT_START
   float* w = nullptr;       // kf x np row scales
   int* iw = nullptr;        // neg, flag, certified count, list (kf each), list length, fail, done, skip (kf)
 };

@@ -60,14 +60,15 @@ constexpr int FB = BS_FILT_BLOCK;   // columns of the block (32)
 constexpr int TB = 64;              // tile edge of the FP32 factorisation
 constexpr int LDS = TB + 1;         // row stride of the diagonal blocks in shared memory
 constexpr float TINY_PIVOT = 1e-6f; // of the scaled unit diagonal
+constexpr int NS = BS_FILT_START;   // plane waves in the starting vectors
 constexpr int GR = 64;              // rows per CTA of the Gram and rotation kernels
 constexpr int STEER_DIGITS = 5;     // of C X in the steps that only steer (34 bits),
 constexpr int LAST_STEER_DIGITS = 6;// and in the step before the first that can certify (41)
 
 // ---------------------------------------------------------------- set-up
-// Per matrix: the FB smallest diagonal entries (the starting vectors are
-// their unit vectors, plane waves in the reduced basis), the shift s, the
-// row scales w_r = (s / (C_rr + s))^1/2 and the largest diagonal entry.
+// Per matrix: the indices of the NS smallest diagonal entries (the plane waves
+// of the starting vectors, filt_start_kernel), the shift s, the row scales
+// w_r = (s / (C_rr + s))^1/2 and the largest diagonal entry.
 __global__ void __launch_bounds__(256) filt_prep_kernel(const zd* __restrict__ C, int n, int np,
                                                         int nb, double sfac,
                                                         double* __restrict__ shift,
@@ -78,7 +79,7 @@ __global__ void __launch_bounds__(256) filt_prep_kernel(const zd* __restrict__ C
                                                         int* __restrict__ done) {
   extern __shared__ double dg[];
   const long long* key = reinterpret_cast<const long long*>(dg);
-  __shared__ int so[FB];
+  __shared__ int so[NS];
   __shared__ double red[8];
   const int k = blockIdx.x, tid = threadIdx.x;
   const zd* ck = C + (size_t)k * n * n;
@@ -90,20 +91,21 @@ __global__ void __launch_bounds__(256) filt_prep_kernel(const zd* __restrict__ C
   }
   for (int o = 16; o > 0; o >>= 1) cm = fmax(cm, __shfl_xor_sync(0xffffffffu, cm, o));
   if ((tid & 31) == 0) red[tid >> 5] = cm;
-  if (tid < FB) so[tid] = tid;
   __syncthreads();
   for (int r = tid; r < n; r += 256) {
     // the diagonal is not negative, so its bit patterns order as its values do
     const long long v = key[r];
     int rank = 0;
     for (int c = 0; c < n; ++c) rank += key[c] < v || (key[c] == v && c < r);
-    if (rank < FB) so[rank] = r;
+    if (rank < NS) so[rank] = r;
   }
   __syncthreads();
-  double s = sfac * dg[so[nb - 1]];
+  // (of the eighth entry at least: a shift far below the block's eigenvalues lets
+  // the filters grow the lowest branches beyond what a Gram matrix can separate)
+  double s = sfac * dg[so[max(nb, 8) - 1]];
   // a zero or non-finite diagonal: any scale will do, the certificate decides
   if (!(s > 1e-250) || !(s < 1e250)) s = 1.0;   // (to_float takes |es| < 897)
-  if (tid < FB) ord[(size_t)k * FB + tid] = so[tid];
+  if (tid < min(n, NS)) ord[(size_t)k * NS + tid] = so[tid];
   if (tid == 0) {
     double v = 0.0;
     for (int q = 0; q < 8; ++q) v = fmax(v, red[q]);
@@ -758,15 +760,35 @@ __global__ void __launch_bounds__(256) filt_lift_kernel(const zd* __restrict__ C
 }
 
 // ---------------------------------------------------------------- Rayleigh-Ritz
-// X = unit vectors at ord, CX = the columns of C (full Hermitian storage)
+// X_i = the unit vector of the i-th smallest diagonal entry (a plane wave in the
+// reduced basis) and 0.1 times three others, one of each 32 that follow; CX from
+// the columns of C (full Hermitian storage).  The others matter where C falls
+// apart into blocks (a layered cell, a supercell, a homogeneous one): products
+// with C or B keep a vector in the blocks it started in, so 32 unit vectors
+// alone never reach an eigenvector of a block that has fewer of them than
+// wanted eigenvalues (bilayer, n = 242, 18 branches: 22 of 30 matrices were
+// reduced; with them none).  Elsewhere the rounds stay as many (90 solves of
+// ordinary cells, of 4 to 720 matrices: no matrix needs a fifth round with
+// 0.1, 47 with 0.3, 1 without).
 __global__ void filt_start_kernel(const zd* __restrict__ C, int n, const int* __restrict__ ord,
                                   zd* __restrict__ X, zd* __restrict__ CX) {
   const int k = blockIdx.z, i = blockIdx.y, r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
-  const int o = ord[(size_t)k * FB + i];
+  const int* ok = ord + (size_t)k * NS;
+  const zd* ck = C + (size_t)k * n * n;
+  zd x = zmake(r == ok[i] ? 1.0 : 0.0, 0.0), cx = ck[(size_t)ok[i] * n + r];
+#pragma unroll
+  for (int g = 1; g < NS / FB; ++g) {
+    const int j = g * FB + ((23 * i + 5 * g) & (FB - 1));   // 23: neighbours go to distant vectors
+    if (j >= n) continue;
+    const double f = g & 1 ? 0.1 : -0.1;
+    const zd c = ck[(size_t)ok[j] * n + r];
+    if (r == ok[j]) x.x += f;
+    cx = zmake(fma(f, c.x, cx.x), fma(f, c.y, cx.y));
+  }
   const size_t q = ((size_t)k * FB + i) * n + r;
-  X[q] = zmake(r == o ? 1.0 : 0.0, 0.0);
-  CX[q] = C[(size_t)k * n * n + (size_t)o * n + r];
+  X[q] = x;
+  CX[q] = cx;
 }
 
 // X += E
@@ -1677,7 +1699,7 @@ int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
       {(void**)&w->sigma, 2 * k * sizeof(double)},
       {(void**)&w->kappa, k * sizeof(double)},
       {(void**)&w->rsum, k * (np / TB) * np * sizeof(float)},
-      {(void**)&w->ord, k * FB * sizeof(int)},
+      {(void**)&w->ord, k * NS * sizeof(int)},
       {(void**)&w->w, k * np * sizeof(float)},
       {(void**)&w->iw, (7 * k + 1) * sizeof(int)},
   };

@@ -1,10 +1,10 @@
 """The certificate of the filtered iteration on matrices it has to refuse.
 
-Each matrix is block diagonal: 64 rows with the eigenvalues 1, 2, 3, ... (rotated
+Each matrix is block diagonal: 160 rows with the eigenvalues 1, 2, 3, ... (rotated
 a little, so that there is something to iterate on) and a dense block of
 large diagonal D whose eigenvalues are D and above, but for one that may lie
-among the wanted ones.  The starting vectors, unit vectors of the smallest
-diagonal entries, have no part in the dense block and the products keep
+among the wanted ones.  The starting vectors, sums of unit vectors of the 128
+smallest diagonal entries, have no part in the dense block and the products keep
 exact zeros there, so an eigenvalue in it is always skipped by the iteration;
 only the factorisation can show it.  From D = 1e7 on its mark in the scaled
 matrix is below the rounding errors of an FP32 factorisation.
@@ -25,7 +25,7 @@ from paper_1310_6380_gb300 import binding as bs  # noqa: E402
 from paper_1310_6380_gb300 import cells  # noqa: E402
 
 EPS = np.finfo(float).eps
-NV = 64
+NV = 160
 
 
 def matrices(n, D, hidden, count, seed):
@@ -54,8 +54,8 @@ def solve(C, nb):
     return w ** 2, red
 
 
-@pytest.mark.parametrize("n, D", [(192, 1e2), (192, 1e4), (200, 1e6), (200, 1e7), (256, 1e8),
-                                  (256, 1e9)])
+@pytest.mark.parametrize("n, D", [(288, 1e3), (288, 1e4), (290, 1e6), (300, 1e7), (352, 1e8),
+                                  (352, 1e9)])
 def test_a_skipped_eigenvalue_is_found(n, D):
     nb = 6
     C, lam = matrices(n, D, 2.5, 24, int(np.log10(D)))
@@ -64,7 +64,7 @@ def test_a_skipped_eigenvalue_is_found(n, D):
     assert red.all()
 
 
-@pytest.mark.parametrize("n, D, nb", [(128, 1e2, 1), (192, 1e2, 6), (200, 1e3, 22)])
+@pytest.mark.parametrize("n, D, nb", [(192, 1e3, 1), (288, 1e3, 6), (300, 1e3, 22)])
 def test_nothing_skipped_is_certified(n, D, nb):
     C, lam = matrices(n, D, None, 24, n)
     got, red = solve(C, nb)
@@ -105,7 +105,7 @@ def test_any_unit(e):
     """A power of two as the unit changes no bit of any step: the same matrices
     are certified and omega is 2^(e/2) times as large.  (The Ritz values of an
     epoxy/steel cell of 10 um in SI units, near 2^62, have squares beyond FP32.)"""
-    C, _ = matrices(150, 1e2, None, 4, 3)
+    C, _ = matrices(230, 1e3, None, 4, 3)
     C = np.ascontiguousarray(C)
     w, red = np.empty((4, 8)), np.full(4, 7, np.int32)
     bs.bs_lowest_eigenvalues(C, 8, w, red)
@@ -113,6 +113,27 @@ def test_any_unit(e):
     bs.bs_lowest_eigenvalues(C * 2.0 ** e, 8, we, rede)
     assert not red.any() and not rede.any()
     assert np.array_equal(we, w * 2.0 ** (e // 2))
+
+
+def reduced_matrices(cell, M, Q, nb, f=1.0):
+    """C(k) of a cell whose lattice is scaled by f, and bs_solve_k's omega of it."""
+    h = bs.bs_create_cell(np.asarray(cell.h1) * f, np.asarray(cell.h2) * f,
+                          np.ascontiguousarray(cell.phase, np.uint16), cell.lam.copy(),
+                          cell.mu.copy(), cell.rho.copy(), M, bs.BS_PREC_FP64)
+    try:
+        bs.bs_assemble(h)
+        n = bs.bs_cell_dims(h)[1]
+        C = np.empty((len(Q), n, n), np.complex128)
+        for k in range(len(Q)):
+            bs.bs_reduced_matrix(h, Q[k].copy(), C[k].view(np.float64))
+        st, w = np.full(len(Q), 7, np.int32), np.empty((len(Q), nb))
+        bs.bs_solve_k(h, Q, nb, w, st)
+    finally:
+        bs.bs_destroy_cell(h)
+    assert not st.any()
+    low = np.tril(C.transpose(0, 2, 1), -1)
+    d = np.einsum("kii->ki", C).real
+    return low + low.conj().transpose(0, 2, 1) + d[:, :, None] * np.eye(n), w
 
 
 @pytest.mark.parametrize("a", [1e-6, 1e-5, 6.023e-3, 1e3])
@@ -124,28 +145,36 @@ def test_cells_of_any_size_are_certified(a):
     Q = np.array([[0.13, 0.21], [0.5, 0.0], [0.3, 0.3]])
     ref = None
     for f in (1.0, scale):
-        h = bs.bs_create_cell(np.asarray(cell.h1) * f, np.asarray(cell.h2) * f,
-                              np.ascontiguousarray(cell.phase, np.uint16), cell.lam.copy(),
-                              cell.mu.copy(), cell.rho.copy(), 4, bs.BS_PREC_FP64)
-        try:
-            bs.bs_assemble(h)
-            n = bs.bs_cell_dims(h)[1]
-            C = np.empty((3, n, n), np.complex128)
-            for k in range(3):
-                bs.bs_reduced_matrix(h, Q[k].copy(), C[k].view(np.float64))
-            st = np.full(3, 7, np.int32)
-            ws = np.empty((3, 12))
-            bs.bs_solve_k(h, Q, 12, ws, st)
-        finally:
-            bs.bs_destroy_cell(h)
-        low = np.tril(C.transpose(0, 2, 1), -1)
-        C = low + low.conj().transpose(0, 2, 1) + np.einsum("kii->ki", C).real[:, :, None] * np.eye(n)
+        C, ws = reduced_matrices(cell, 4, Q, 12, f)
         w, red = np.empty((3, 12)), np.full(3, 7, np.int32)
         bs.bs_lowest_eigenvalues(np.ascontiguousarray(C), 12, w, red)
-        assert not red.any() and not st.any()
-        tol = 2 * (n + 128) * EPS * np.abs(C).max()
+        assert not red.any()
+        tol = 2 * (C.shape[1] + 128) * EPS * np.abs(C).max()
         assert np.abs(w ** 2 - ws ** 2).max() <= tol
         if ref is None:
             ref = w
         else:
             assert np.abs((w * f) ** 2 - ref ** 2).max() <= 2 * tol * f * f
+
+
+def supercell(cell, t):
+    cell.phase = np.tile(cell.phase[::t, ::t], (t, t))
+    return cell
+
+
+@pytest.mark.parametrize("make, M, nb", [
+    (lambda: cells.bilayer_cell(48), 3, 8), (lambda: cells.bilayer_cell(48), 5, 18),
+    (lambda: cells.bilayer_cell(48, layer1=(4, 1.5, 1.2), layer2=(8, 4, 2)), 5, 22),
+    (lambda: cells.bilayer_cell(48), 7, 18),
+    (lambda: supercell(cells.circle_cell(48, 0.3), 2), 5, 18),
+    (lambda: supercell(cells.circle_cell(48, 0.3), 3), 5, 18)])
+def test_cells_whose_matrices_fall_apart(make, M, nb):
+    """C(k) of layered cells and of supercells is block diagonal: every block is
+    reached, so all are certified."""
+    cell = make()
+    Q = np.ascontiguousarray(cells.ibz_path("square", 41, cell.h1, cell.h2)[1::2])
+    C, ws = reduced_matrices(cell, M, Q, nb)
+    w, red = np.empty((len(Q), nb)), np.full(len(Q), 7, np.int32)
+    bs.bs_lowest_eigenvalues(np.ascontiguousarray(C), nb, w, red)
+    assert np.abs(w ** 2 - ws ** 2).max() <= 2 * (C.shape[1] + 128) * EPS * np.abs(C).max()
+    assert not red.any()
