@@ -273,9 +273,9 @@ int bs_set_iteration_limits(int lobpcg_maxit, int bisect_sweeps);
  *     their distances to the rest of the spectrum bounds the error of every
  *     eigenvalue by 64 eps64 ||C||.  That the rest begins where the sum takes
  *     it to, so that none was skipped, is shown by an FP32 Cholesky
- *     factorisation of C + tau X X^dagger - sigma (X: the vectors below the cut),
- *     with room for its rounding errors (their norm taken as 16 sqrt(n) 2^-24
- *     of the matrix scaled to a unit diagonal; 28 2^-24 was the most seen).
+ *     factorisation of C + X T X^dagger - sigma (X: the vectors below the cut),
+ *     with room for its rounding errors (their norm taken as (128 + 4 sqrt(n))
+ *     2^-24 of the matrix scaled to a unit diagonal; 57 2^-24 was the most seen).
  *     Matrices it does not certify so are reduced (one-stage) in the same
  *     call, without a wait for the host.  Other solves: two-stage for
  *     n >= 400, one-stage below.

@@ -462,7 +462,7 @@ struct FilterWs {
   float* coef = nullptr;    // kf x BS_FILT_MAXDEG x 4 x 32
   double* shift = nullptr;  // kf
   double* cmax = nullptr;   // kf
-  double* sigma = nullptr;  // 2 kf: sigma and tau of the certificate
+  double* sigma = nullptr;  // 2 kf: sigma and level of the certificate
   double* kappa = nullptr;  // kf: bound of ||A^-1||
   float* rsum = nullptr;    // kf x np / 64 x np: row sums of |A^-1| by block column
   int* ord = nullptr;       // kf x BS_FILT_START

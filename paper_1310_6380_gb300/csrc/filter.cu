@@ -29,8 +29,8 @@
 //     of that size; the sum overestimates the error, whose own gap is that to
 //     the eigenvalues outside the block).  That rho is such a bound, so that
 //     no eigenvalue was skipped, is shown by an FP32 Cholesky factorisation:
-//     C + tau X_m X_m^dagger has rank m more than C, so if it is above sigma
-//     then lambda_{m+1} is, whatever X_m is; see filt_cert_kernel for what the
+//     C + X_m T X_m^dagger, T >= 0, has rank m more than C, so if it is above sigma
+//     then lambda_{m+1} is, whatever X_m and T are; see filt_cert_kernel for what the
 //     rounding errors of the factorisation take from sigma.
 //  4. Matrices that do not pass are reduced by the FP64 Householder reduction
 //     and bisected (tridiag.cu, bisect.cu) in one launch each that returns at
@@ -690,20 +690,23 @@ __global__ void __launch_bounds__(256) filt_kappa_kernel(const float* __restrict
   }
 }
 
-// A <- W (C / s - sigma / s I) W + Z Z^dagger, Z = (tau / s)^1/2 W X_m for the first m =
-// expect[k] Ritz vectors, lower 64-tiles, FP32, identity in the padding: the
-// matrix whose factorisation shows that nothing was skipped.  A zero in
-// expect or below: the matrix is not certified and is left out.
+// A <- W (C / s - sigma / s I) W + Z Z^dagger, z_i = ((level - theta_i) / s)^1/2 W x_i for the
+// first m = expect[k] Ritz vectors, which lifts each to the level of the next
+// Ritz value (no higher, so that the diagonal stays near 1), lower 64-tiles,
+// FP32, identity in the padding: the matrix whose factorisation shows that
+// nothing was skipped.  m = 0: the matrix is not certified and is left out.
 __global__ void __launch_bounds__(256) filt_lift_kernel(const zd* __restrict__ C, int n, int np,
                                                         const double* __restrict__ shift,
                                                         const double* __restrict__ sigma,
-                                                        const double* __restrict__ tau,
+                                                        const double* __restrict__ level,
+                                                        const double* __restrict__ theta,
                                                         const zd* __restrict__ X,
                                                         const int* __restrict__ expect,
                                                         const float* __restrict__ w,
                                                         zf* __restrict__ A, int* __restrict__ neg,
                                                         int* __restrict__ flag) {
   __shared__ __align__(16) zf Zr[FB * TB], Zc[FB * TB];   // [vector][row]
+  __shared__ float q[FB];
   const int k = blockIdx.y, m = expect[k], tid = threadIdx.x;
   if (m <= 0) return;
   int bi, bk;
@@ -714,7 +717,9 @@ __global__ void __launch_bounds__(256) filt_lift_kernel(const zd* __restrict__ C
   zf* ak = A + (size_t)k * np * np;
   const double is = 1.0 / shift[k], beta = sigma[k] * is;
   const int es = exponent(shift[k]);
-  const float fs = (float)(is * exp2i(es)), q = sqrtf((float)(tau[k] * is));
+  const float fs = (float)(is * exp2i(es));
+  if (tid < FB) q[tid] = sqrtf((float)((level[k] - theta[(size_t)k * FB + tid]) * is));
+  __syncthreads();
   if (blockIdx.x == 0 && tid == 0) {
     neg[k] = 0;
     flag[k] = 0;
@@ -726,7 +731,7 @@ __global__ void __launch_bounds__(256) filt_lift_kernel(const zd* __restrict__ C
       zf z = make_float2(0.f, 0.f);
       if (t < m && r < n) {
         const zd x = xk[(size_t)t * n + r];
-        const float f = wk[r] * q;
+        const float f = wk[r] * q[t];
         z = make_float2(to_float(x.x) * f, to_float(x.y) * f);
       }
       (h ? Zc : Zr)[e] = z;
@@ -1527,31 +1532,31 @@ __global__ void __launch_bounds__(128) filt_coef_kernel(const double* __restrict
 
 // Certificate of a Rayleigh-Ritz step, one warp per matrix: omega, and a cut
 // above a Ritz value i >= nb - 1 whose error sum is small: m = i + 1 in expect
-// (0: there is none) with sigma and tau for filt_lift_kernel.
+// (0: there is none) with sigma and the level for filt_lift_kernel.
 //
 // sigma lies halfway between theta_i and the next eigenvalue as far as the block
 // knows it (theta_{i+1} less its residual norm).  If the factorisation of
-// A + E, A = W (C - sigma + tau X X^dagger) W / s and E its rounding errors, has
+// A + E, A = W (C - sigma + X T X^dagger) W / s and E its rounding errors, has
 // positive pivots only, then for some x in the span of the lowest m + 1
 // eigenvectors with X^dagger x = 0
 //   0 < x^dagger (C - sigma) x + s ||E|| x^dagger W^-2 x
 //    <= lambda_{m+1} - sigma + ||E|| kappa (lambda_{m+1} + s),
 // so lambda_{m+1} > rho = (sigma - e kappa s) / (1 + e kappa) for any e >= ||E||.
 // No pivot grows in a definite matrix (|L| |D| |L^dagger| has A's diagonal), so E is
-// what roundings of either sign add up to: at most 28 u in the spectral norm
-// and 6.7 u sqrt(n) in Frobenius', u = 2^-24, over cells of n = 98 .. 1029 whose
-// stiffnesses differ by up to 1e5 (numpy model); e = 16 u sqrt(n) is taken.  (The inertia of the
-// indefinite C - sigma has no such bound: its pivots grow by 10 to 2000 there,
-// and E with them.)
+// what roundings of either sign add up to: a numpy model of the kernels over 1600
+// cells of n = 98 .. 882, with stiffnesses up to 1e3 and densities up to 1e2
+// apart, has at most 57 u in the spectral norm, u = 2^-24, 18 u in 95 of 100, and no
+// growth with n; e = (128 + 4 sqrt(n)) u is taken.  (The inertia of the indefinite
+// C - sigma has no such bound: its pivots grow by 10 to 2000 there, and E with them.)
 __global__ void __launch_bounds__(128) filt_cert_kernel(
     const double* __restrict__ theta, const double* __restrict__ rerr,
     const float* __restrict__ rpart, int nch, const double* __restrict__ shift,
     const double* __restrict__ cmax, const double* __restrict__ kappa, int n, int kb, int nb, const int* __restrict__ fail,
-    double* __restrict__ omega, double* __restrict__ sigma, double* __restrict__ tau,
+    double* __restrict__ omega, double* __restrict__ sigma, double* __restrict__ level,
     int* __restrict__ expect, int* __restrict__ skip, int* __restrict__ done) {
   const int k = blockIdx.x * 4 + (threadIdx.x >> 5), c = threadIdx.x & 31;
   if (k >= kb || done[k]) return;
-  const double s = shift[k], ek = 16.0 / 16777216.0 * sqrt((double)n) * kappa[k];
+  const double s = shift[k], ek = (128.0 + 4.0 * sqrt((double)n)) / 16777216.0 * kappa[k];
   float q32 = 0.f;
   for (int q = 0; q < 2 * nch; ++q) q32 += rpart[((size_t)k * 2 * nch + q) * FB + c];
   const double t = theta[(size_t)k * FB + c];
@@ -1595,7 +1600,7 @@ __global__ void __launch_bounds__(128) filt_cert_kernel(
     done[k] = ok;
     skip[k] = !ok;
     sigma[k] = sg;
-    tau[k] = 2.0 * tg;
+    level[k] = tg;
     expect[k] = ok ? at_i + 1 : 0;
   }
 }
@@ -1814,7 +1819,7 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
     zd* Ck = C + (size_t)k0 * n * n;
     int *neg = w.iw, *flag = w.iw + w.kf, *expect = w.iw + 2 * w.kf, *list = w.iw + 3 * w.kf,
         *nlist = w.iw + 4 * w.kf, *fail = nlist + 1, *done = fail + w.kf, *skip = done + w.kf;
-    double *sigma = w.sigma, *tau = w.sigma + w.kf;
+    double *sigma = w.sigma, *level = w.sigma + w.kf;
     filt_prep_kernel<<<kf, 256, n * sizeof(double), s>>>(Ck, n, np, nbands, 0.2, w.shift, w.cmax,
                                                          w.ord, w.w, fail, done);
     BS_CHECK_LAUNCH("filt_prep_kernel");
@@ -1840,7 +1845,7 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
       if (rd >= base) {
         filt_cert_kernel<<<(kf + 3) / 4, 128, 0, s>>>(w.theta, w.rerr, w.rpart, nch, w.shift,
                                                       w.cmax, w.kappa, n, kf, nbands, fail,
-                                                      omega + (size_t)k0 * nbands, sigma, tau,
+                                                      omega + (size_t)k0 * nbands, sigma, level,
                                                       expect, skip, done);
         BS_CHECK_LAUNCH("filt_cert_kernel");
       }
@@ -1862,7 +1867,7 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
                                    w.eB, w.CX, n, (long)FB * n, err, s, done));
     }
     filt_lift_kernel<<<dim3(nt * (nt + 1) / 2, kf), 256, 0, s>>>(
-        Ck, n, np, w.shift, sigma, tau, w.Xb, expect, w.w, w.A, neg, flag);
+        Ck, n, np, w.shift, sigma, level, w.theta, w.Xb, expect, w.w, w.A, neg, flag);
     BS_CHECK_LAUNCH("filt_lift_kernel");
     TRY_LAUNCH(filter_factor(w, np, kf, false, s, skip));
     filt_decide_kernel<<<1, 1024, 0, s>>>(neg, flag, expect, kf, stat + k0, list, nlist,
