@@ -266,7 +266,10 @@ int bs_set_iteration_limits(int lobpcg_maxit, int bisect_sweeps);
  *     QR, the trailing two-sided updates as FP64-exact digit-plane products
  *     on the tensor cores (8 digits of 7 bits per operand), then band ->
  *     tridiagonal by bulge chasing in FP64 (O(n^2) work per k);
- *   BS_REDUCE_AUTO (default): solves of at most 22 branches with n >= 96
+ *   BS_REDUCE_AUTO (default): solves of at most 22 branches with n >= 96, of a
+ *     cell whose phases' wave speeds do not lie too far apart (n <c_max^2>
+ *     <1 / c_min^2> <= 90000 over the cell's volume, c^2 the extreme eigenvalues of
+ *     the stiffness over the density; of a batch group all cells but an eighth),
  *     take a filtered subspace iteration without a reduction: Chebyshev
  *     filters of the shifted inverse (FP32) on 32 vectors between float64
  *     Rayleigh-Ritz steps, until the sum of the squared float64 residuals over
@@ -284,6 +287,14 @@ int bs_set_iteration_limits(int lobpcg_maxit, int bisect_sweeps);
  * GB300); larger n use the one-stage reduction in every mode.
  * Errors: BS_EINVAL for any other mode.
  */
+/*
+ * bs_filter_counts, bs_filter_counts3, bs_batch_filter_counts - how the last
+ * solve (bs_solve_k or bs_bands; bs_solve_k3; bs_batch_solve) was done:
+ * counts[0] matrices that the filtered iteration took (0: none, the reductions
+ * or another solver ran), counts[1] those of them that it did not certify and
+ * that were reduced behind it.  Waits for the device.
+ */
+int bs_filter_counts(const bs_cell* cell, int counts[2]);
 /*
  * bs_reduction_times - with profiling on (bs_set_profiling), the device time
  * in ms of each kernel group of the last two-stage reduction of this cell's
@@ -484,6 +495,7 @@ int bs_batch_destroy(bs_batch* batch);
 #define BS_SOLVER_FP64   2
 int bs_batch_set_solver(bs_batch* batch, int solver);
 int bs_batch_set_start(bs_batch* batch, const float* U, int Mp, int nvec);
+int bs_batch_filter_counts(const bs_batch* batch, int counts[2]);   /* bs_filter_counts */
 int bs_batch_stats(const bs_batch* batch, int* iters_out, int* fallback_out);
 int bs_batch_set_vectors(bs_batch* batch, int Mp);
 int bs_batch_vectors(const bs_batch* batch, float* U_out);
@@ -639,6 +651,7 @@ int bs_reduced_matrix3(bs_cell3* cell, const double* Q, double* out, void* strea
 
 /* bs_cell3_dims - N = (2M+1)^3 and n = 3N of a 3-D cell. */
 int bs_cell3_dims(const bs_cell3* cell, int* N, int* n);
+int bs_filter_counts3(const bs_cell3* cell, int counts[2]);   /* bs_filter_counts */
 
 /* bs_destroy_cell3 - free a 3-D cell. NULL is a no-op. */
 int bs_destroy_cell3(bs_cell3* cell);

@@ -81,6 +81,9 @@ def _load():
         "bs_phase_times": [vp, dp],
         "bs_launch_count": [ctypes.POINTER(ctypes.c_longlong)],
         "bs_tridiag_eigenvalues": [dp, dp, i32, i32, i32, dp, vp],
+        "bs_filter_counts": [vp, dp],
+        "bs_filter_counts3": [vp, dp],
+        "bs_batch_filter_counts": [vp, dp],
         "bs_lowest_eigenvalues": [dp, i32, i32, i32, dp, dp, vp],
         "bs_gemm_bf16": [dp, dp, dp, i32, i32, i32, i32, vp],
         "bs_tridiag_eigenvalues_static": [dp, dp, i32, i32, i32, dp, vp],
@@ -137,7 +140,8 @@ EXPORTED = ["bs_create_cell", "bs_assemble", "bs_solve_k", "bs_bands", "bs_form_
             "bs_mode_field", "bs_create_cell_mesh", "bs_set_stiffness", "bs_create_cell3",
             "bs_assemble3", "bs_solve_k3", "bs_form_factors3", "bs_reduced_matrix3",
             "bs_cell3_dims", "bs_destroy_cell3", "bs_set_iteration_limits", "bs_probe_fp64",
-            "bs_set_reduction", "bs_reduction_times", "bs_lowest_eigenvalues"]
+            "bs_set_reduction", "bs_reduction_times", "bs_lowest_eigenvalues",
+            "bs_filter_counts", "bs_filter_counts3", "bs_batch_filter_counts"]
 BS_SOLVER_DENSE, BS_SOLVER_LOBPCG, BS_SOLVER_FP64 = 0, 1, 2
 BS_LOB_MAX_BANDS, BS_LOB_MAXIT = 12, 80
 BS_REDUCE_AUTO, BS_REDUCE_ONESTAGE, BS_REDUCE_TWOSTAGE = 0, 1, 2
@@ -329,6 +333,25 @@ def bs_tridiag_eigenvalues(d, e, nbands: int, lam_out, stream=None):
     _check(_lib.bs_tridiag_eigenvalues(_ptr(d, np.float64), _ptr(e, np.float64), n, batch,
                                        int(nbands), _ptr(lam_out, np.float64), _stream(stream)))
     return lam_out
+
+
+def _counts(f, handle):
+    c = np.zeros(2, np.int32)
+    _check(f(handle, c.ctypes.data))
+    return int(c[0]), int(c[1])
+
+
+def bs_filter_counts(cell):
+    """(matrices the filtered iteration took, of these reduced behind it) in the last solve."""
+    return _counts(_lib.bs_filter_counts, cell)
+
+
+def bs_filter_counts3(cell):
+    return _counts(_lib.bs_filter_counts3, cell)
+
+
+def bs_batch_filter_counts(batch):
+    return _counts(_lib.bs_batch_filter_counts, batch)
 
 
 def bs_lowest_eigenvalues(C, nbands: int, omega_out, reduced_out=None, stream=None):

@@ -82,9 +82,27 @@ bool bs_use_band(int n) {
 // factorisation and some 60 block products where the reductions do n or n/8
 // dependent steps.  A lowered bisection cap (a diagnostic) is meant for the
 // tridiagonal path, so that one runs.
-bool bs_use_filter(int n, int nbands) {
+//
+// The spread of the wave speeds (SpeedSpread) says what the iteration meets: the
+// further the wanted eigenvalues lie below the diagonal, the more rounds it
+// takes, and the more of the gap above them the rounding errors of its
+// certificate's factorisation take (with n and the spread).  What it does not
+// certify is reduced one-stage behind it, which loses against the reduction
+// alone.  900 drawn cells of 10 k, stiffnesses up to 3e3 apart, densities up to
+// 1e2, one part in 200 to 1 in volume, n = 98 .. 882: of the matrices with n spread
+// <= 90000 under 1 % are not certified in 12 rounds, above it 14 to 60 %.  Up to
+// 15000 as many are with 6 rounds; the launches of the other six, which return at
+// once, would cost 0.4 ms (n = 98, one wavevector: 1.86 ms with 6, 2.28 with 12).
+// 90 wavevectors, n = 882, 18 branches, a circle of 0.01, 100, 0.001 and 1000 times
+// the matrix's moduli: 27.6, 26.7, 162 and 162 ms (the last two reduced; with the
+// iteration before the reduction 625).
+constexpr double kSpreadEasy = 15000.0, kSpreadMost = 90000.0;
+bool bs_use_filter(int n, int nbands, double spread) {
   return g_reduction.load(std::memory_order_relaxed) == BS_REDUCE_AUTO && bs_bisect_sweeps() == 128 &&
-         bs_filter_fits(n, nbands);
+         bs_filter_fits(n, nbands) && n * spread <= kSpreadMost;
+}
+int bs_filter_rounds(int n, double spread) {
+  return n * spread <= kSpreadEasy ? 6 : BS_FILT_ROUNDS;
 }
 
 extern "C" int bs_set_reduction(int mode) {
@@ -398,6 +416,14 @@ static int create_common(const double h1[2], const double h2[2], double det, int
   }
   c->tol = 1e-6;
   c->floor2 = omega_floor2(c);
+  std::vector<double> vol(np, 0.0);   // of every phase
+  for (size_t i = 0; i < ph.size(); ++i) vol[ph[i]] += area ? (*area)[i] : 1.0;
+  SpeedSpread sp;
+  for (int i = 0; i < np; ++i) {
+    const double b = 2.0 * (raw[i] + raw[np + i]), g = 2.0 * raw[np + i];
+    if (vol[i] > 0.0) sp.add(vol[i], std::min(b, g), std::max(b, g), raw[2 * np + i]);
+  }
+  c->spread = sp.value();
   *out = c;
   return BS_OK;
 }
@@ -583,6 +609,16 @@ extern "C" int bs_set_stiffness(bs_cell* c, const double* C6) {
                 cudaMemcpyDeviceToHost), "bs_set_stiffness raw");
   // derived rows: S11, S22, rho, S12, S13, S23, S33 of S = C^-1 (Voigt)
   std::vector<double> tab(7 * (size_t)np);
+  // volume of every phase, for the spread of the wave speeds
+  std::vector<uint16_t> ph((size_t)c->nel);
+  std::vector<double> area(c->mesh ? c->nel : 0), vol(np, 0.0);
+  CK(cudaMemcpy(ph.data(), c->d_phase, ph.size() * 2, cudaMemcpyDeviceToHost),
+     "bs_set_stiffness phases");
+  if (c->mesh)
+    CK(cudaMemcpy(area.data(), c->d_area, area.size() * 8, cudaMemcpyDeviceToHost),
+       "bs_set_stiffness areas");
+  for (size_t i = 0; i < ph.size(); ++i) vol[ph[i]] += c->mesh ? area[i] : 1.0;
+  SpeedSpread sp;
   double c2min = 1e300;
   for (int i = 0; i < np; ++i) {
     const double* v = &cv[6 * (size_t)i];
@@ -621,6 +657,25 @@ extern "C" int bs_set_stiffness(bs_cell* c, const double* C6) {
       if (pd(mid)) lo = mid; else hi = mid;
     }
     c2min = std::min(c2min, lo / rho);
+    if (vol[i] > 0.0) {
+      // extreme eigenvalues of the tensor (third row and column by sqrt 2), to a
+      // percent, by the signs of the leading minors of t (C - x I), t = +1 or -1
+      const double q = sqrt(2.0);
+      auto extreme = [&](double t, double x0, double x1) {
+        for (int it = 0; it < 40 && x1 > 1.01 * x0; ++it) {
+          const double x = x0 > 0.0 ? sqrt(x0 * x1) : 0.01 * x1;
+          const double a = t * (C[0][0] - x), b = t * (C[1][1] - x), e = t * (2.0 * C[2][2] - x);
+          const double f = t * C[0][1], g = t * q * C[0][2], h = t * q * C[1][2];
+          const double d3 = a * (b * e - h * h) - f * (f * e - h * g) + g * (f * h - b * g);
+          const bool definite = a > 0.0 && a * b - f * f > 0.0 && d3 > 0.0;
+          if (definite == (t > 0.0)) x0 = x; else x1 = x;
+        }
+        return t > 0.0 ? x0 : x1;
+      };
+      const double tr = C[0][0] + C[1][1] + 2.0 * C[2][2];
+      const double big = extreme(-1.0, tr / 3.0, tr);
+      sp.add(vol[i], std::max(extreme(1.0, 0.0, tr / 3.0), 1e-12 * tr), big, rho);
+    }
   }
   if (!c->aniso) TRY(realloc_fields(c, 7));
   c->aniso = true;
@@ -629,6 +684,7 @@ extern "C" int bs_set_stiffness(bs_cell* c, const double* C6) {
   const double q2 = std::min(c->q1[0] * c->q1[0] + c->q1[1] * c->q1[1],
                              c->q2[0] * c->q2[0] + c->q2[1] * c->q2[1]);
   c->floor2 = c2min * q2 / 4.0;
+  c->spread = sp.value();
   c->assembled = false;
   return BS_OK;
 }
@@ -738,6 +794,14 @@ static int check_info(bs_cell* c, cudaStream_t s) {
   return BS_OK;
 }
 
+extern "C" int bs_filter_counts(const bs_cell* c, int counts[2]) {
+  if (!c || !counts) {
+    bs_set_error("bs_filter_counts: NULL argument");
+    return BS_EINVAL;
+  }
+  return bs_filter_read_counts(c->filt, counts);
+}
+
 extern "C" int bs_sync(bs_cell* c, void* stream) {
   if (!c) {
     bs_set_error("bs_sync: NULL cell");
@@ -787,20 +851,22 @@ static int solve_chunk_mixed(bs_cell* c, int kb, int nbands, cudaStream_t s) {
   return BS_OK;
 }
 
-static int solve_chunk(bs_cell* c, int kb, int nbands, cudaStream_t s) {
+// first: the first chunk of a solve
+static int solve_chunk(bs_cell* c, int kb, int nbands, bool first, cudaStream_t s) {
   if (c->precision == BS_PREC_MIXED) return solve_chunk_mixed(c, kb, nbands, s);
-  const bool filt = bs_use_filter(c->n, nbands);
+  const bool filt = bs_use_filter(c->n, nbands, c->spread);
   bs_phase_begin(c, PH_BUILD, s);
   TRY(bs_launch_builder(c->d_Cm, c->n, c->d_Q, kb, c->q1[0], c->q1[1], c->q2[0], c->q2[1], c->d_C,
                         s, filt));
   bs_phase_end(c, PH_BUILD, s);
   bs_phase_begin(c, PH_TRID, s);
   if (filt && !c->filt) c->filt = new FilterWs();
+  if (c->filt && first) c->filt->taken = 0;
   // no memory for its workspace: the reductions below need less
   if (filt && bs_filter_ws_alloc(c->filt, c->n, c->kcap) == BS_OK) {
     const FilterFallback fb{c->d_vec, c->d_part, c->d_de, c->d_tau, c->d_beta, c->d_count};
     TRY(bs_launch_eig_filter(c->d_C, c->n, kb, nbands, *c->filt, fb, c->d_w, c->d_stat,
-                             c->d_info + 1, s));
+                             c->d_info + 1, bs_filter_rounds(c->n, c->spread), s));
     c->band_used = false;
     bs_phase_end(c, PH_TRID, s);
     c->prof_ready[PH_BISECT] = false;
@@ -862,7 +928,7 @@ extern "C" int bs_solve_k(bs_cell* c, const double* Q, int nk, int nbands, doubl
     CK(cudaMemcpyAsync(c->d_Q, Q + 2 * (size_t)k0, 2 * kb * sizeof(double),
                        q_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s),
        "bs_solve_k Q");
-    TRY(solve_chunk(c, kb, nbands, s));
+    TRY(solve_chunk(c, kb, nbands, k0 == 0, s));
     if (!hst.empty())
       CK(cudaMemcpyAsync(hst.data() + k0, c->d_stat, kb * sizeof(int), cudaMemcpyDeviceToHost, s),
          "bs_solve_k status");

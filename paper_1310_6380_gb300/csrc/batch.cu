@@ -162,6 +162,7 @@ struct BatchGroup {
   zd* part64;
   BandWs* band;               // FP64 solver: two-stage reduction workspace (large n)
   FilterWs* filt;             // filtered iteration workspace (FP64 and dense solvers)
+  double spread, widest;      // of the wave speeds, of all cells but an eighth and of all
   SideStreams* side;
   // [0] tensor-core pipeline timeout of a main-stream product, [1] a Gram
   // Cholesky failed, [2] a tensor-core timeout during a cell's assembly
@@ -221,7 +222,7 @@ static void prof_mark(bs_batch* B, cudaStream_t s) {
 // n = 242 .. 578 x 30 k, 10 branches: 274 ms with the FP32 reduction and its
 // refinement, 145 ms so (results within 7e-11 of each other).
 static bool group_filter(const bs_batch* B, const BatchGroup& g) {
-  return g.filt && bs_use_filter(g.n, B->nbands) &&
+  return g.filt && bs_use_filter(g.n, B->nbands, g.spread) &&
          (B->solver == BS_SOLVER_FP64 || (B->solver == BS_SOLVER_DENSE && !g.forced && !B->d_vec));
 }
 
@@ -534,12 +535,14 @@ static int reduce_chunk_body(bs_batch* B, BatchGroup& g, int c0, int cn, int p, 
   const int K = cn * nk;
   const int* rows = g.d_rowidx + (size_t)c0 * nk;
   prof_mark(B, s);   // assembly ends, reduction begins
+  if (g.filt && c0 == 0) g.filt->taken = 0;
   if (B->solver == BS_SOLVER_FP64 || group_filter(B, g)) {
     // the plain FP64 path: filtered iteration, or Householder reduction and
     // Sturm multisection
     if (group_filter(B, g)) {
       const FilterFallback fb{g.vec64, g.part64, g.de, g.tau, g.beta, g.count};
-      TRY_LAUNCH(bs_launch_eig_filter(g.C64, n, K, B->nbands, *g.filt, fb, g.w, g.st, g.d_err, s));
+      TRY_LAUNCH(bs_launch_eig_filter(g.C64, n, K, B->nbands, *g.filt, fb, g.w, g.st, g.d_err,
+                                      bs_filter_rounds(n, g.widest), s));
       prof_mark(B, s);
     } else if (g.band) {
       BandBisect bis{B->nbands, g.w, g.st};
@@ -710,6 +713,7 @@ extern "C" int bs_batch_create(const bs_cell_desc* descs, int ncells, int nk, in
   B->cell_gi.assign(ncells, 0);
   std::vector<double> raw(rawn);
   std::map<int, std::vector<int>> byM;
+  std::vector<double> spread(ncells, 1.0);
   std::vector<uint16_t> ph(PP);
   for (int i = 0; !r && i < ncells; ++i) {
     const int np = descs[i].nphase;
@@ -729,6 +733,16 @@ extern "C" int bs_batch_create(const bs_cell_desc* descs, int ncells, int nk, in
     }
     std::vector<double> lmr(raw.begin() + B->raw_off[i], raw.begin() + B->raw_off[i] + 3 * np);
     r = validate(descs[i], i, lmr, ph);
+    if (!r) {
+      std::vector<double> vol(np, 0.0);
+      for (uint16_t p : ph) vol[p] += 1.0;
+      SpeedSpread sp;
+      for (int p = 0; p < np; ++p) {
+        const double b = 2.0 * (lmr[p] + lmr[np + p]), q = 2.0 * lmr[np + p];
+        if (vol[p] > 0.0) sp.add(vol[p], std::min(b, q), std::max(b, q), lmr[2 * np + p]);
+      }
+      spread[i] = sp.value();
+    }
     byM[descs[i].M].push_back(i);
   }
   if (!r) {
@@ -761,6 +775,13 @@ extern "C" int bs_batch_create(const bs_cell_desc* descs, int ncells, int nk, in
     g.b = bs_mixed_guard(nbands, g.n);
     int npmax = 1, ci0 = g.cells[0];
     for (int ci : g.cells) npmax = std::max(npmax, descs[ci].nphase);
+    // the group goes one way: that of its cells, the eighth of the widest spread
+    // left out (the reduction behind the iteration takes their matrices if need be)
+    std::vector<double> sp;
+    for (int ci : g.cells) sp.push_back(spread[ci]);
+    std::sort(sp.begin(), sp.end());
+    g.spread = sp[sp.size() - 1 - sp.size() / 8];
+    g.widest = sp.back();
     // worker cell: sized for the group's largest table
     bs_cell_desc wd = descs[ci0];
     std::vector<double> ones(npmax, 1.0);
@@ -868,7 +889,7 @@ static void drop_graph(bs_batch* B) {
 // the filtered iteration's workspace, and the buffers of the reduction behind
 // it; without memory for them the reductions take the group
 static void alloc_filter(bs_batch* B, BatchGroup& g) {
-  if (!bs_use_filter(g.n, B->nbands)) return;
+  if (!bs_use_filter(g.n, B->nbands, g.spread)) return;
   const size_t K = (size_t)g.chunk * B->nk;
   if (!g.vec64 && balloc(&g.vec64, K * bs_tridiag_vec_elems(g.n), "batch FP64 vectors")) return;
   if (!g.part64 && balloc(&g.part64, K * bs_tridiag_part_elems(g.n), "batch FP64 partials")) return;
@@ -999,6 +1020,21 @@ extern "C" int bs_batch_stats(const bs_batch* B, int* iters_out, int* fallback_o
     std::vector<int> fb(nq, 0);
     if (B->fb.size() == nq) fb = B->fb;
     CK(cudaMemcpy(fallback_out, fb.data(), nq * sizeof(int), cudaMemcpyDefault), "bs_batch_stats");
+  }
+  return BS_OK;
+}
+
+extern "C" int bs_batch_filter_counts(const bs_batch* B, int counts[2]) {
+  if (!B || !counts) {
+    bs_set_error("bs_batch_filter_counts: NULL argument");
+    return BS_EINVAL;
+  }
+  counts[0] = counts[1] = 0;
+  for (auto& g : B->groups) {
+    int c[2] = {0, 0};
+    TRY_LAUNCH(bs_filter_read_counts(g.filt, c));
+    counts[0] += c[0];
+    counts[1] += c[1];
   }
   return BS_OK;
 }

@@ -228,6 +228,7 @@ struct bs_cell {
   struct BandWs* band;  // two-stage reduction workspace (allocated on first use)
   bool band_used;       // the last FP64 solve took the two-stage reduction
   struct FilterWs* filt;  // filtered iteration workspace (allocated on first use)
+  double spread;          // of the phases' wave speeds (SpeedSpread)
   struct SideStreams* side;  // with the mixed workspace
 
   bool prof;
@@ -439,6 +440,7 @@ int bs_launch_rank2_update(const uint16_t* dA, const uint16_t* dB, const int* ex
 #define BS_FILT_MAX_BANDS 22   // wanted branches: at least 10 guard vectors remain
 #define BS_FILT_MIN_N 96
 #define BS_FILT_MAXDEG 12      // degrees of one filter
+#define BS_FILT_ROUNDS 12      // filters at most
 struct FilterWs {
   int n = 0, kf = 0;        // order, matrices per chunk
   zf* A = nullptr;          // kf x np x np scaled matrix, then its LDL^dagger (np: n padded to
@@ -467,6 +469,8 @@ struct FilterWs {
   float* rsum = nullptr;    // kf x np / 64 x np: row sums of |A^-1| by block column
   int* ord = nullptr;       // kf x BS_FILT_START
   float* w = nullptr;       // kf x np row scales
+  int* nred = nullptr;      // matrices of this solve that were reduced behind the iteration
+  int taken = 0;            // matrices of this solve (0 begins a new count)
   int* iw = nullptr;        // neg, flag, certified count, list (kf each), list length, fail, done, skip (kf)
 };
 // the buffers of the Householder reduction that takes what is not certified
@@ -479,14 +483,32 @@ struct FilterFallback {
   unsigned* count;
 };
 bool bs_filter_fits(int n, int nbands);
-// whether a solve of nbands branches takes it (BS_REDUCE_AUTO)
-bool bs_use_filter(int n, int nbands);
+// How far apart the wave speeds of a cell's phases are: the mean of c_max^2 over
+// that of 1 / c_min^2's inverse, by volume, c^2 the extreme eigenvalues of the
+// stiffness over the density.  1 or more; it goes with how far the wanted
+// eigenvalues lie below the diagonal of C(k), which decides how many rounds
+// the iteration takes (api.cu).
+struct SpeedSpread {
+  double hi = 0.0, inv = 0.0, vol = 0.0;
+  void add(double w, double lo_eig, double hi_eig, double rho) {
+    hi += w * hi_eig / rho;
+    inv += w * rho / lo_eig;
+    vol += w;
+  }
+  double value() const { return hi * inv / (vol * vol); }
+};
+// whether a solve of nbands branches takes it (BS_REDUCE_AUTO), and its rounds
+bool bs_use_filter(int n, int nbands, double spread);
+int bs_filter_rounds(int n, double spread);
 int bs_filter_ws_alloc(FilterWs* w, int n, int kb);
+// matrices that the last solve gave to the iteration, and those reduced behind it
+// (w may be null; waits for the device)
+int bs_filter_read_counts(const FilterWs* w, int counts[2]);
 void bs_filter_ws_free(FilterWs* w);
 // C: kb full Hermitian matrices (kept, but for those that take the fallback);
 // reduced (optional, kb): 1 where the fallback ran
 int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const FilterFallback& fb,
-                         double* omega, int* stat, int* err, cudaStream_t s,
+                         double* omega, int* stat, int* err, int rounds, cudaStream_t s,
                          int* reduced = nullptr);
 // tridiag.cu, bisect.cu: the matrices list[0 .. *nlist) of a batch (device list)
 int bs_launch_tridiag_list(zd* A, int n, zd* vec, zd* part, double* de, double* tau, zd* beta,

@@ -56,6 +56,7 @@ struct bs_cell3 {
   int* d_stat;
   BandWs* band;        // two-stage reduction workspace (allocated on first use)
   FilterWs* filt;      // filtered iteration workspace (allocated on first use)
+  double spread;       // of the phases' wave speeds (SpeedSpread)
 };
 
 namespace {
@@ -515,6 +516,14 @@ extern "C" int bs_create_cell3(const bs_cell3_desc* d, bs_cell3** out) {
     bs_destroy_cell3(c);
     return r;
   }
+  std::vector<double> share(np, 0.0);
+  for (size_t i = 0; i < P3; ++i) share[ph[i]] += 1.0;
+  SpeedSpread sp;
+  for (int i = 0; i < np; ++i) {
+    const double b = 3.0 * raw[i] + 2.0 * raw[np + i], g = 2.0 * raw[np + i];
+    if (share[i] > 0.0) sp.add(share[i], std::min(b, g), std::max(b, g), raw[2 * np + i]);
+  }
+  c->spread = sp.value();
   *out = c;
   return BS_OK;
 }
@@ -572,6 +581,14 @@ extern "C" int bs_assemble3(bs_cell3* c, void* stream) {
   return BS_OK;
 }
 
+extern "C" int bs_filter_counts3(const bs_cell3* c, int counts[2]) {
+  if (!c || !counts) {
+    bs_set_error("bs_filter_counts3: NULL argument");
+    return BS_EINVAL;
+  }
+  return bs_filter_read_counts(c->filt, counts);
+}
+
 extern "C" int bs_solve_k3(bs_cell3* c, const double* Q, int nk, int nbands, double* omega_out,
                            int* status_out, void* stream) {
   if (!c || nk < 0 || (nk > 0 && (!Q || !omega_out))) {
@@ -611,8 +628,9 @@ extern "C" int bs_solve_k3(bs_cell3* c, const double* Q, int nk, int nbands, dou
       break;
     }
     const size_t nn = (size_t)n * n;
-    bool filt = bs_use_filter(n, nbands);
+    bool filt = bs_use_filter(n, nbands, c->spread);
     if (filt && !c->filt) c->filt = new FilterWs();
+    if (c->filt && k0 == 0) c->filt->taken = 0;
     // no memory for its workspace: the reductions below need less
     filt = filt && bs_filter_ws_alloc(c->filt, n, c->kcap) == BS_OK;
     builder3_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(c->d_Cm, n, c->d_Q, kb, d_qv,
@@ -626,7 +644,7 @@ extern "C" int bs_solve_k3(bs_cell3* c, const double* Q, int nk, int nbands, dou
     if (filt) {
       const FilterFallback fb{c->d_vec, c->d_part, c->d_de, c->d_tau, c->d_beta, c->d_count};
       r = bs_launch_eig_filter(c->d_C, n, kb, nbands, *c->filt, fb, c->d_w, c->d_stat,
-                               c->d_info + 1, s);
+                               c->d_info + 1, bs_filter_rounds(n, c->spread), s);
     } else if (bs_use_band(n)) {
       if (!c->band) c->band = new BandWs();
       r = bs_band_ws_alloc(c->band, n, c->kcap, BS_SLICES_BAND);

@@ -1613,6 +1613,7 @@ __global__ void __launch_bounds__(1024) filt_decide_kernel(const int* __restrict
                                                            int* __restrict__ stat,
                                                            int* __restrict__ list,
                                                            int* __restrict__ nlist,
+                                                           int* __restrict__ nred,
                                                            int* __restrict__ reduced) {
   __shared__ int cnt[32], base;
   const int tid = threadIdx.x;
@@ -1633,7 +1634,10 @@ __global__ void __launch_bounds__(1024) filt_decide_kernel(const int* __restrict
       for (int w = 0; w < 32; ++w) base += cnt[w];
     __syncthreads();
   }
-  if (tid == 0) *nlist = base;
+  if (tid == 0) {
+    *nlist = base;
+    *nred += base;
+  }
 }
 
 }  // namespace
@@ -1653,7 +1657,7 @@ bool bs_filter_fits(int n, int nbands) {
 void bs_filter_ws_free(FilterWs* w) {
   void* p[] = {w->A, w->X, w->pA, w->pB, w->pD, w->eA, w->eB, w->Xb, w->CX, w->vec, w->vs, w->d, w->part,
                w->rpart, w->theta, w->rerr, w->W, w->coef, w->shift, w->cmax, w->sigma, w->kappa, w->rsum, w->ord, w->w,
-               w->iw};
+               w->iw, w->nred};
   for (void* q : p) cudaFree(q);
   *w = FilterWs();
 }
@@ -1707,6 +1711,7 @@ int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
       {(void**)&w->ord, k * NS * sizeof(int)},
       {(void**)&w->w, k * np * sizeof(float)},
       {(void**)&w->iw, (7 * k + 1) * sizeof(int)},
+      {(void**)&w->nred, sizeof(int)},
   };
   for (auto& it : items) {
     if (cudaMalloc(it.p, it.bytes) != cudaSuccess) {
@@ -1719,6 +1724,15 @@ int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
   w->n = n;
   w->kf = kf;
   return BS_OK;
+}
+
+int bs_filter_read_counts(const FilterWs* w, int counts[2]) {
+  counts[0] = w ? w->taken : 0;
+  counts[1] = 0;
+  if (!counts[0]) return BS_OK;
+  cudaError_t e = cudaDeviceSynchronize();   // the solve may be on any stream
+  if (e == cudaSuccess) e = cudaMemcpy(counts + 1, w->nred, sizeof(int), cudaMemcpyDeviceToHost);
+  return e == cudaSuccess ? BS_OK : bs_cuda_status(e, "filtered iteration counts");
 }
 
 // shared-memory opt-ins, per device
@@ -1800,19 +1814,26 @@ static int filter_ritz(FilterWs& w, int n, int np, int kf, cudaStream_t s) {
 }
 
 int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const FilterFallback& fb,
-                         double* omega, int* stat, int* err, cudaStream_t s, int* reduced) {
+                         double* omega, int* stat, int* err, int rounds, cudaStream_t s,
+                         int* reduced) {
   static_assert(TB == GR, "padded rows are covered by the row chunks");
   // filter degrees of the rounds: the first Ritz values come from plane
   // waves and misplace the cut, so the first filters are short; the later ones
   // are long because a Rayleigh-Ritz step costs as much as several products.
   // Matrices certified after the fourth round skip the others.
-  static const int degs[] = {4, 6, 8, 8, 8, 8};
-  constexpr int rounds = sizeof(degs) / sizeof(degs[0]), base = 4;
+  static const int degs[BS_FILT_ROUNDS] = {4, 6, 8, 8, 8, 8, 8, 8, 8, 8, 8, 8};
+  constexpr int base = 4;
+  rounds = std::max(base, std::min(rounds, BS_FILT_ROUNDS));
   if (w.n != n || w.kf < 1 || !bs_filter_fits(n, nbands)) {
     bs_set_error("filtered iteration: workspace for n = %d not set up", n);
     return BS_EINVAL;
   }
   TRY_LAUNCH(filter_attrs());
+  if (w.taken == 0) {
+    const cudaError_t e = cudaMemsetAsync(w.nred, 0, sizeof(int), s);
+    if (e != cudaSuccess) return bs_cuda_status(e, "filtered iteration count");
+  }
+  w.taken += kb;
   const int np = (n + TB - 1) / TB * TB, nt = np / TB, nch = (n + GR - 1) / GR;
   for (int k0 = 0; k0 < kb; k0 += w.kf) {
     const int kf = std::min(w.kf, kb - k0);
@@ -1870,7 +1891,7 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
         Ck, n, np, w.shift, sigma, level, w.theta, w.Xb, expect, w.w, w.A, neg, flag);
     BS_CHECK_LAUNCH("filt_lift_kernel");
     TRY_LAUNCH(filter_factor(w, np, kf, false, s, skip));
-    filt_decide_kernel<<<1, 1024, 0, s>>>(neg, flag, expect, kf, stat + k0, list, nlist,
+    filt_decide_kernel<<<1, 1024, 0, s>>>(neg, flag, expect, kf, stat + k0, list, nlist, w.nred,
                                           reduced ? reduced + k0 : nullptr);
     BS_CHECK_LAUNCH("filt_decide_kernel");
     TRY_LAUNCH(bs_launch_tridiag_list(Ck, n, fb.vec + (size_t)k0 * bs_tridiag_vec_elems(n),
@@ -1915,7 +1936,7 @@ extern "C" int bs_lowest_eigenvalues(const double* C, int n, int batch, int nban
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
     if (e == cudaSuccess)
       r = bs_launch_eig_filter((zd*)p[0], n, batch, nbands, w, fb, (double*)p[7], (int*)p[8], err,
-                               s, (int*)p[9]);
+                               BS_FILT_ROUNDS, s, (int*)p[9]);
     if (e == cudaSuccess) e = cudaMemcpyAsync(omega_out, p[7], bytes[7], cudaMemcpyDefault, s);
     if (e == cudaSuccess && reduced_out)
       e = cudaMemcpyAsync(reduced_out, p[9], bytes[9], cudaMemcpyDefault, s);
