@@ -88,21 +88,23 @@ bool bs_use_band(int n) {
 // takes, and the more of the gap above them the rounding errors of its
 // certificate's factorisation take (with n and the spread).  What it does not
 // certify is reduced one-stage behind it, which loses against the reduction
-// alone.  900 drawn cells of 10 k, stiffnesses up to 3e3 apart, densities up to
-// 1e2, one part in 200 to 1 in volume, n = 98 .. 882: of the matrices with n spread
-// <= 90000 under 1 % are not certified in 12 rounds, above it 14 to 60 %.  Up to
-// 15000 as many are with 6 rounds; the launches of the other six, which return at
-// once, would cost 0.4 ms (n = 98, one wavevector: 1.86 ms with 6, 2.28 with 12).
-// 90 wavevectors, n = 882, 18 branches, a circle of 0.01, 100, 0.001 and 1000 times
-// the matrix's moduli: 27.6, 26.7, 162 and 162 ms (the last two reduced; with the
-// iteration before the reduction 625).
-constexpr double kSpreadEasy = 15000.0, kSpreadMost = 90000.0;
+// alone.  Of the matrices of 700 drawn cells of two and more materials (10 k each,
+// stiffnesses up to 3e3 apart, densities up to 1e2, one part in 200 to 1 in
+// volume, n = 98 .. 882) none is refused in 6 rounds while n spread <= 30000 and none
+// in 8 while it is <= 60000; 1 % are in 12 rounds up to 90000, 10 to 55 % above.
+// Rounds that no matrix needs cost their launches, which return at once (six of
+// them 0.4 ms; n = 98, one wavevector, 1.86 ms without).  90 wavevectors, n = 882, 18
+// branches, a circle of 0.01, 100, 0.001 and 1000 times the matrix's moduli: 27.6,
+// 26.7, 162 and 162 ms (the last two reduced; with the iteration before the
+// reduction 625).
+constexpr double kSpreadRounds6 = 28000.0, kSpreadRounds8 = 56000.0, kSpreadMost = 90000.0;
 bool bs_use_filter(int n, int nbands, double spread) {
   return g_reduction.load(std::memory_order_relaxed) == BS_REDUCE_AUTO && bs_bisect_sweeps() == 128 &&
          bs_filter_fits(n, nbands) && n * spread <= kSpreadMost;
 }
 int bs_filter_rounds(int n, double spread) {
-  return n * spread <= kSpreadEasy ? 6 : BS_FILT_ROUNDS;
+  const double x = n * spread;
+  return x <= kSpreadRounds6 ? 6 : x <= kSpreadRounds8 ? 8 : BS_FILT_ROUNDS;
 }
 
 extern "C" int bs_set_reduction(int mode) {
