@@ -150,7 +150,9 @@ __device__ __forceinline__ void tri_index(int l, int& bi, int& bk) {
 // partials of four tiles are loaded together (instead of through global memory
 // at every stage: 1.2 us less per step at n = 882, mixed solve of 8 wavevectors
 // 44.6 -> 43.6 ms, of 90 77.0 -> 75.3 ms).  The sums take the same terms in the
-// same order as the general form in tridiag_tile.
+// same order as the general form in tridiag_tile, which FP64 keeps: there this
+// one is slower (n = 50, 98, 242, 338 with 60, 30, 70, 30 matrices: 1.66, 3.42, 16.6
+// and 20.4 ms against 1.49, 2.98, 15.2 and 18.4).
 constexpr int EPR = 4;
 template <typename R>
 __device__ __forceinline__ void column_step(typename Cplx<R>::T* a, int n, int r0,
@@ -377,7 +379,7 @@ __device__ __forceinline__ void tridiag_tile(typename Cplx<R>::T* __restrict__ A
   __threadfence();
 
   // ---- epilogue: one CTA per matrix
-  if (n - r0 <= EPR * NT) {
+  if constexpr (sizeof(R) == 4) if (n - r0 <= EPR * NT) {
     static_assert(2 * 16 * TS >= EPR * NT, "the column fits the reduction buffers");
     column_step<R>(a, n, r0, vcur, w, vprev, pt, t0, nt, de + (size_t)b * 2 * n,
                    tau + (size_t)b * n + j, tau + (size_t)b * n + r0, beta + (size_t)b * n + r0,
