@@ -282,7 +282,8 @@ int bs_set_iteration_limits(int lobpcg_maxit, int bisect_sweeps);
  *     Matrices it does not certify so are reduced (one-stage) in the same
  *     call, without a wait for the host.  Other solves: two-stage for
  *     n >= 400, one-stage below.
- * Process-wide; takes effect at the next solve.  The two-stage reduction
+ * Process-wide; takes effect at the next solve, which keeps to it (a batch's
+ * graph recorded in another mode is recorded again).  The two-stage reduction
  * needs an n x 8 complex panel in shared memory (n up to about 1800 on
  * GB300); larger n use the one-stage reduction in every mode.
  * Errors: BS_EINVAL for any other mode.

@@ -70,8 +70,9 @@ static std::atomic<int> g_reduction{BS_REDUCE_AUTO};
 // the reduction to tridiagonal form of the FP64 eigensolve for dimension n:
 // the two-stage (band) reduction from BS_BAND_AUTO_MIN on, where its
 // tensor-core products outrun the one-stage reduction's FP64 pipe
-bool bs_use_band(int n) {
-  const int mode = g_reduction.load(std::memory_order_relaxed);
+int bs_reduction_mode() { return g_reduction.load(std::memory_order_relaxed); }
+
+bool bs_use_band(int n, int mode) {
   if (!bs_band_supported(n)) return false;
   if (mode == BS_REDUCE_TWOSTAGE) return true;
   if (mode == BS_REDUCE_ONESTAGE) return false;
@@ -98,8 +99,8 @@ bool bs_use_band(int n) {
 // 26.7, 162 and 162 ms (the last two reduced; with the iteration before the
 // reduction 625).
 constexpr double kSpreadRounds6 = 28000.0, kSpreadRounds8 = 56000.0, kSpreadMost = 90000.0;
-bool bs_use_filter(int n, int nbands, double spread) {
-  return g_reduction.load(std::memory_order_relaxed) == BS_REDUCE_AUTO && bs_bisect_sweeps() == 128 &&
+bool bs_use_filter(int n, int nbands, double spread, int mode) {
+  return mode == BS_REDUCE_AUTO && bs_bisect_sweeps() == 128 &&
          bs_filter_fits(n, nbands) && n * spread <= kSpreadMost;
 }
 int bs_filter_rounds(int n, double spread) {
@@ -856,7 +857,8 @@ static int solve_chunk_mixed(bs_cell* c, int kb, int nbands, cudaStream_t s) {
 // first: the first chunk of a solve
 static int solve_chunk(bs_cell* c, int kb, int nbands, bool first, cudaStream_t s) {
   if (c->precision == BS_PREC_MIXED) return solve_chunk_mixed(c, kb, nbands, s);
-  const bool filt = bs_use_filter(c->n, nbands, c->spread);
+  const int mode = bs_reduction_mode();   // once: the build and the solve have to agree
+  const bool filt = bs_use_filter(c->n, nbands, c->spread, mode);
   bs_phase_begin(c, PH_BUILD, s);
   TRY(bs_launch_builder(c->d_Cm, c->n, c->d_Q, kb, c->q1[0], c->q1[1], c->q2[0], c->q2[1], c->d_C,
                         s, filt));
@@ -874,7 +876,7 @@ static int solve_chunk(bs_cell* c, int kb, int nbands, bool first, cudaStream_t 
     c->prof_ready[PH_BISECT] = false;
     return BS_OK;
   }
-  if (bs_use_band(c->n)) {
+  if (bs_use_band(c->n, mode)) {
     if (!c->band) c->band = new BandWs();
     TRY(bs_band_ws_alloc(c->band, c->n, c->kcap, BS_SLICES_BAND));
     c->band->prof = c->prof;

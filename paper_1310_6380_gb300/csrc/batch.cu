@@ -162,6 +162,7 @@ struct BatchGroup {
   zd* part64;
   BandWs* band;               // FP64 solver: two-stage reduction workspace (large n)
   FilterWs* filt;             // filtered iteration workspace (FP64 and dense solvers)
+  int route;                  // RT_*, decided once per solve (choose_route)
   double spread, widest;      // of the wave speeds, of all cells but an eighth and of all
   SideStreams* side;
   // [0] tensor-core pipeline timeout of a main-stream product, [1] a Gram
@@ -184,6 +185,7 @@ struct bs_batch {
   std::vector<BatchGroup> groups;
   bool use_graph;
   cudaGraphExec_t graph;
+  int graph_mode;         // reduction mode that the graph was recorded in
   cudaStream_t cap;       // non-blocking stream the graph is recorded and replayed on
   cudaEvent_t ev_in, ev_out;
   // profiling: event pairs per chunk and phase (assembly, reduction, shifts, refinement)
@@ -215,16 +217,10 @@ static void prof_mark(bs_batch* B, cudaStream_t s) {
   cudaEventRecord(B->pev[B->pev_used++], s);
 }
 
-// Whether a group's solves take the filtered iteration (bs_set_reduction): the
-// FP64 solver, and the dense one unless a reduction tile was chosen for it or
-// its eigenvectors are kept.  Its results are accurate to FP64, so the dense
-// solver's residual bound holds with room to spare.  Measured, 48 cells of
-// n = 242 .. 578 x 30 k, 10 branches: 274 ms with the FP32 reduction and its
-// refinement, 145 ms so (results within 7e-11 of each other).
-static bool group_filter(const bs_batch* B, const BatchGroup& g) {
-  return g.filt && bs_use_filter(g.n, B->nbands, g.spread) &&
-         (B->solver == BS_SOLVER_FP64 || (B->solver == BS_SOLVER_DENSE && !g.forced && !B->d_vec));
-}
+// What a group's chunks are built for and solved by: FP32 reduction or LOBPCG
+// (RT_OWN), or on FP64 matrices the filtered iteration, the two-stage and the
+// one-stage reduction.
+enum { RT_OWN, RT_FILTER, RT_BAND, RT_TRIDIAG };
 
 static void free_group(BatchGroup& g) {
   bs_side_free(g.side);
@@ -480,10 +476,10 @@ static int assemble_chunk(bs_batch* B, BatchGroup& g, int c0, int cn, int p) {
                           (size_t)g.N * g.N * sizeof(zd), cudaMemcpyDeviceToDevice, ws) == cudaSuccess
               ? BS_OK
               : bs_cuda_status(cudaGetLastError(), "batch L_R stash");
-    if (!r && (B->solver == BS_SOLVER_FP64 || group_filter(B, g)))
+    if (!r && g.route != RT_OWN)
       r = bs_launch_builder(wk->d_Cm, n, B->d_Q + (size_t)ci * nk * 2, nk, wk->q1[0], wk->q1[1],
                             wk->q2[0], wk->q2[1], g.C64 + (size_t)i * nk * nn, ws,
-                            group_filter(B, g));
+                            g.route == RT_FILTER);
     else if (!r)
       r = bs_launch_builder_mixed(wk->d_Cm, n, B->d_Q + (size_t)ci * nk * 2, nk, wk->q1[0],
                                   wk->q1[1], wk->q2[0], wk->q2[1], g.C64 + (size_t)i * nk * nn,
@@ -536,15 +532,15 @@ static int reduce_chunk_body(bs_batch* B, BatchGroup& g, int c0, int cn, int p, 
   const int* rows = g.d_rowidx + (size_t)c0 * nk;
   prof_mark(B, s);   // assembly ends, reduction begins
   if (g.filt && c0 == 0) g.filt->taken = 0;
-  if (B->solver == BS_SOLVER_FP64 || group_filter(B, g)) {
+  if (g.route != RT_OWN) {
     // the plain FP64 path: filtered iteration, or Householder reduction and
     // Sturm multisection
-    if (group_filter(B, g)) {
+    if (g.route == RT_FILTER) {
       const FilterFallback fb{g.vec64, g.part64, g.de, g.tau, g.beta, g.count};
       TRY_LAUNCH(bs_launch_eig_filter(g.C64, n, K, B->nbands, *g.filt, fb, g.w, g.st, g.d_err,
                                       bs_filter_rounds(n, g.widest), s));
       prof_mark(B, s);
-    } else if (g.band) {
+    } else if (g.route == RT_BAND) {
       BandBisect bis{B->nbands, g.w, g.st};
       TRY_LAUNCH(bs_launch_eig_band(g.C64, n, K, *g.band, g.de, g.d_err, s, &bis));
       prof_mark(B, s);
@@ -886,18 +882,42 @@ static void drop_graph(bs_batch* B) {
   }
 }
 
-// the filtered iteration's workspace, and the buffers of the reduction behind
-// it; without memory for them the reductions take the group
-static void alloc_filter(bs_batch* B, BatchGroup& g) {
-  if (!bs_use_filter(g.n, B->nbands, g.spread)) return;
+// The route of a group's solves in a reduction mode, with the workspace it needs.
+// The filtered iteration takes the FP64 solver's groups, and the dense one's
+// unless a reduction tile was chosen for it or its eigenvectors are kept: its
+// results are accurate to FP64, so the dense solver's residual bound holds with
+// room to spare (48 cells of n = 242 .. 578 x 30 k, 10 branches: 250 ms with the FP32
+// reduction and its refinement, 124 ms so).  Without memory for it the
+// reductions take the group.  Decided once per solve: the chunks' assembly and
+// their solve have to agree, whatever another thread sets meanwhile.
+static int choose_route(bs_batch* B, BatchGroup& g, int mode) {
+  g.route = RT_OWN;
+  const bool fp64 = B->solver == BS_SOLVER_FP64;
+  if (!fp64 && (B->solver != BS_SOLVER_DENSE || g.forced || B->d_vec)) return BS_OK;
+  const bool filter = bs_use_filter(g.n, B->nbands, g.spread, mode);
+  if (!fp64 && !filter) return BS_OK;
   const size_t K = (size_t)g.chunk * B->nk;
-  if (!g.vec64 && balloc(&g.vec64, K * bs_tridiag_vec_elems(g.n), "batch FP64 vectors")) return;
-  if (!g.part64 && balloc(&g.part64, K * bs_tridiag_part_elems(g.n), "batch FP64 partials")) return;
-  if (!g.filt) g.filt = new FilterWs();
-  if (bs_filter_ws_alloc(g.filt, g.n, (int)K) != BS_OK) {
+  int r = BS_OK;
+  if (!g.vec64) r = balloc(&g.vec64, K * bs_tridiag_vec_elems(g.n), "batch FP64 vectors");
+  if (!r && !g.part64) r = balloc(&g.part64, K * bs_tridiag_part_elems(g.n), "batch FP64 partials");
+  if (r) return fp64 ? r : BS_OK;
+  if (filter) {
+    if (!g.filt) g.filt = new FilterWs();
+    if (bs_filter_ws_alloc(g.filt, g.n, (int)K) == BS_OK) {
+      g.route = RT_FILTER;
+      return BS_OK;
+    }
     delete g.filt;
     g.filt = nullptr;
+    if (!fp64) return BS_OK;
   }
+  g.route = RT_TRIDIAG;
+  if (bs_use_band(g.n, mode)) {
+    if (!g.band) g.band = new BandWs();
+    TRY_LAUNCH(bs_band_ws_alloc(g.band, g.n, (int)K, BS_SLICES_BAND));
+    g.route = RT_BAND;
+  }
+  return BS_OK;
 }
 
 extern "C" int bs_batch_set_solver(bs_batch* B, int solver) {
@@ -917,25 +937,17 @@ extern "C" int bs_batch_set_solver(bs_batch* B, int solver) {
       }
     for (auto& g : B->groups) TRY_LAUNCH(alloc_lob(g, B->nk, B->nbands));
   }
-  if (solver == BS_SOLVER_FP64) {
-    for (auto& g : B->groups) {
-      const size_t K = (size_t)g.chunk * B->nk;
-      if (!g.vec64) TRY_LAUNCH(balloc(&g.vec64, K * bs_tridiag_vec_elems(g.n), "batch FP64 vectors"));
-      if (!g.part64)
-        TRY_LAUNCH(balloc(&g.part64, K * bs_tridiag_part_elems(g.n), "batch FP64 partials"));
-      if (bs_use_band(g.n)) {
-        if (!g.band) g.band = new BandWs();
-        TRY_LAUNCH(bs_band_ws_alloc(g.band, g.n, (int)K, BS_SLICES_BAND));
-      } else if (g.band) {
-        bs_band_ws_free(g.band);
-        delete g.band;
-        g.band = nullptr;
-      }
-      alloc_filter(B, g);
-    }
-  }
-  if (solver != B->solver) drop_graph(B);
+  const int before = B->solver;
+  if (solver != before) drop_graph(B);
   B->solver = solver;
+  if (solver == BS_SOLVER_FP64)   // its workspace now, so that a lack of memory shows here
+    for (auto& g : B->groups) {
+      const int r = choose_route(B, g, bs_reduction_mode());
+      if (r) {
+        B->solver = before;
+        return r;
+      }
+    }
   return BS_OK;
 }
 
@@ -1290,9 +1302,13 @@ extern "C" int bs_batch_solve(bs_batch* B, const double* Q, double* omega_out, i
   B->fb.assign(nq, 0);
   const bool prof = B->prof;
   B->prof = false;   // not while tuning or recording a graph
+  const int mode = bs_reduction_mode();
+  if (B->graph && B->graph_mode != mode) drop_graph(B);
+  const bool replay = B->use_graph && B->graph;
   for (auto& g : B->groups) {
-    if (B->solver == BS_SOLVER_DENSE && !g.forced && !B->d_vec && !g.filt) alloc_filter(B, g);
-    if (g.tuned || B->solver != BS_SOLVER_DENSE || group_filter(B, g)) continue;
+    if (replay) break;   // with the routes it was recorded with
+    TRY_LAUNCH(choose_route(B, g, mode));
+    if (g.tuned || B->solver != BS_SOLVER_DENSE || g.route != RT_OWN) continue;
     const auto key = tile_key(B, g);
     {
       std::lock_guard<std::mutex> lk(g_tile_mu);
@@ -1325,6 +1341,7 @@ extern "C" int bs_batch_solve(bs_batch* B, const double* Q, double* omega_out, i
       CK(cudaStreamBeginCapture(B->cap, cudaStreamCaptureModeThreadLocal), "bs_batch_solve capture");
       B->capturing = true;
       const int r = solve_all(B, floors, B->cap);
+      B->graph_mode = mode;
       B->capturing = false;
       cudaError_t ce = cudaStreamEndCapture(B->cap, &graph);
       if (r) return r;

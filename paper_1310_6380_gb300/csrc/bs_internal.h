@@ -402,7 +402,9 @@ struct BandWs {
 #define BS_BAND_GROUPS 5
 int bs_band_times(BandWs& w, double ms[BS_BAND_GROUPS]);
 bool bs_band_supported(int n);
-bool bs_use_band(int n);
+// the process's reduction mode (bs_set_reduction), read once per solve or chunk
+int bs_reduction_mode();
+bool bs_use_band(int n, int mode);
 int bs_band_ws_alloc(BandWs* w, int n, int kb, int S);
 void bs_band_ws_free(BandWs* w);
 // optional: the Sturm multisection of each part, run on the part's stream
@@ -498,7 +500,7 @@ struct SpeedSpread {
   double value() const { return hi * inv / (vol * vol); }
 };
 // whether a solve of nbands branches takes it (BS_REDUCE_AUTO), and its rounds
-bool bs_use_filter(int n, int nbands, double spread);
+bool bs_use_filter(int n, int nbands, double spread, int mode);
 int bs_filter_rounds(int n, double spread);
 int bs_filter_ws_alloc(FilterWs* w, int n, int kb);
 // matrices that the last solve gave to the iteration, and those reduced behind it

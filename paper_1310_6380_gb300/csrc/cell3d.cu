@@ -628,7 +628,8 @@ extern "C" int bs_solve_k3(bs_cell3* c, const double* Q, int nk, int nbands, dou
       break;
     }
     const size_t nn = (size_t)n * n;
-    bool filt = bs_use_filter(n, nbands, c->spread);
+    const int mode = bs_reduction_mode();
+    bool filt = bs_use_filter(n, nbands, c->spread, mode);
     if (filt && !c->filt) c->filt = new FilterWs();
     if (c->filt && k0 == 0) c->filt->taken = 0;
     // no memory for its workspace: the reductions below need less
@@ -645,7 +646,7 @@ extern "C" int bs_solve_k3(bs_cell3* c, const double* Q, int nk, int nbands, dou
       const FilterFallback fb{c->d_vec, c->d_part, c->d_de, c->d_tau, c->d_beta, c->d_count};
       r = bs_launch_eig_filter(c->d_C, n, kb, nbands, *c->filt, fb, c->d_w, c->d_stat,
                                c->d_info + 1, bs_filter_rounds(n, c->spread), s);
-    } else if (bs_use_band(n)) {
+    } else if (bs_use_band(n, mode)) {
       if (!c->band) c->band = new BandWs();
       r = bs_band_ws_alloc(c->band, n, c->kcap, BS_SLICES_BAND);
       BandBisect bis{nbands, c->d_w, c->d_stat};
