@@ -560,13 +560,19 @@ int bs_cell_dims(const bs_cell* cell, int* N, int* n);
  *           layout of bs_solve_k_lobpcg's vectors); host or device.
  *   S_out : nk x nvec x 3N complex128, index J*N + a with J in
  *           {S11, S22, S12}; host or device.
- * FP64 throughout, with the k-independent Gram factors of bs_assemble (any
- * precision); U need not be an eigenvector (the map is linear).  Requires
+ * Accurate to FP64 (the two Gram solves in eight 7-bit digits per operand under
+ * one scale per row and column, exactly summed), with the k-independent Gram
+ * factors of bs_assemble (any precision); U need not be an eigenvector (the map is linear).  Requires
  * bs_assemble (BS_ESTATE otherwise); 1 <= nvec <= 16384.  Asynchronous when
- * U and S_out are both device pointers; nk = 0 does nothing.
+ * U and S_out are both device pointers; nk = 0 does nothing.  Should a bounded
+ * wait of its tensor-core products run out, S_out is NaN and the call returns
+ * BS_ECUDA, or bs_sync does when the call was asynchronous; the next call
+ * starts afresh.  bs_set_late_wait: the cell's calls behave as if one had (a test
+ * of that handling; on = 0 ends it).
  */
 int bs_stress_coefficients(bs_cell* cell, const double* Q, int nk, int nvec,
                            const double* U, double* S_out, void* stream);
+int bs_set_late_wait(bs_cell* cell, int on);
 
 /*
  * bs_mode_field - fields of plane-wave expansions (Eq. (approximation2d)) on

@@ -106,6 +106,7 @@ def _load():
         "bs_reduction_times": [vp, dp],
         "bs_batch_set_tile": [vp, i32],
         "bs_stress_coefficients": [vp, dp, i32, i32, dp, dp, vp],
+        "bs_set_late_wait": [vp, i32],
         "bs_mode_field": [vp, dp, i32, i32, dp, i32, dp, vp],
         "bs_cnn_create": [i32, i32, i32, i32, ctypes.POINTER(vp)],
         "bs_cnn_destroy": [vp],
@@ -141,7 +142,7 @@ EXPORTED = ["bs_create_cell", "bs_assemble", "bs_solve_k", "bs_bands", "bs_form_
             "bs_assemble3", "bs_solve_k3", "bs_form_factors3", "bs_reduced_matrix3",
             "bs_cell3_dims", "bs_destroy_cell3", "bs_set_iteration_limits", "bs_probe_fp64",
             "bs_set_reduction", "bs_reduction_times", "bs_lowest_eigenvalues",
-            "bs_filter_counts", "bs_filter_counts3", "bs_batch_filter_counts"]
+            "bs_filter_counts", "bs_filter_counts3", "bs_batch_filter_counts", "bs_set_late_wait"]
 BS_SOLVER_DENSE, BS_SOLVER_LOBPCG, BS_SOLVER_FP64 = 0, 1, 2
 BS_LOB_MAX_BANDS, BS_LOB_MAXIT = 12, 80
 BS_REDUCE_AUTO, BS_REDUCE_ONESTAGE, BS_REDUCE_TWOSTAGE = 0, 1, 2
@@ -333,6 +334,10 @@ def bs_tridiag_eigenvalues(d, e, nbands: int, lam_out, stream=None):
     _check(_lib.bs_tridiag_eigenvalues(_ptr(d, np.float64), _ptr(e, np.float64), n, batch,
                                        int(nbands), _ptr(lam_out, np.float64), _stream(stream)))
     return lam_out
+
+
+def bs_set_late_wait(cell, on: bool):
+    _check(_lib.bs_set_late_wait(cell, int(bool(on))))
 
 
 def _counts(f, handle):

@@ -753,7 +753,7 @@ extern "C" int bs_assemble(bs_cell* c, void* stream) {
   }
   cudaStream_t s = (cudaStream_t)stream;
   const size_t NN = (size_t)c->N * c->N;
-  CK(cudaMemsetAsync(c->d_info, 0, 2 * sizeof(int), s), "bs_assemble");
+  CK(cudaMemsetAsync(c->d_info, 0, 3 * sizeof(int), s), "bs_assemble");
   for (int i = 0; i < PH_COUNT; ++i) c->prof_ready[i] = false;
   bs_phase_begin(c, PH_ASM, s);
   if (c->mesh)
@@ -782,15 +782,16 @@ extern "C" int bs_assemble(bs_cell* c, void* stream) {
   return BS_OK;
 }
 
-static int check_info(bs_cell* c, cudaStream_t s) {
-  int info[2] = {0, 0};
-  CK(cudaMemcpyAsync(info, c->d_info, 2 * sizeof(int), cudaMemcpyDeviceToHost, s), "info");
+// stress: also a wait of the last bs_stress_coefficients
+static int check_info(bs_cell* c, cudaStream_t s, bool stress = false) {
+  int info[3] = {0, 0, 0};
+  CK(cudaMemcpyAsync(info, c->d_info, 3 * sizeof(int), cudaMemcpyDeviceToHost, s), "info");
   CK(cudaStreamSynchronize(s), "sync");
   if (info[0]) {
     bs_set_error("Cholesky of a Gram matrix failed (not positive definite)");
     return BS_ENOTPD;
   }
-  if (info[1]) {
+  if (info[1] || (stress && info[2])) {
     bs_set_error("a tensor-core pipeline wait reached its limit");
     return BS_ECUDA;
   }
@@ -810,7 +811,7 @@ extern "C" int bs_sync(bs_cell* c, void* stream) {
     bs_set_error("bs_sync: NULL cell");
     return BS_EINVAL;
   }
-  return check_info(c, (cudaStream_t)stream);
+  return check_info(c, (cudaStream_t)stream, true);
 }
 
 // ------------------------------------------------------------------ solve

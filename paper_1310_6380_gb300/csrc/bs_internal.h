@@ -153,7 +153,8 @@ struct bs_cell {
   zd* d_F;             // 6 x N x N: F_X^a = L_R^-1 diag(G_a) L_X^-dagger
   zd* d_Pp;            // 12 x N x N: F_X^a F_X^b^dagger, a <= b
   zd* d_Cm;            // 6 x n x n monomial matrices of C(k)
-  int* d_info;         // [0] Cholesky failure, [1] tensor-core pipeline timeout
+  int* d_info;         // [0] Cholesky failure, [1] tensor-core pipeline timeout, [2] the same
+                       // of the last bs_stress_coefficients
   // exact-slice assembly operands
   uint16_t* d_sliceA;  // 3 S P x Kp digit planes of the fields
   uint16_t* d_sliceB;  // S 2D x Kp digit planes of the exponential table
@@ -229,6 +230,7 @@ struct bs_cell {
   bool band_used;       // the last FP64 solve took the two-stage reduction
   struct FilterWs* filt;  // filtered iteration workspace (allocated on first use)
   double spread;          // of the phases' wave speeds (SpeedSpread)
+  bool late_wait;         // bs_set_late_wait
   struct SideStreams* side;  // with the mixed workspace
 
   bool prof;

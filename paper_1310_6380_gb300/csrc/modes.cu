@@ -36,6 +36,8 @@
 // e^{2 pi i Q1} (A - i B), for half the multiply-adds.  The kernel is bound by
 // the FP32 pipe and its stores, not by any read (5400 fields of M = 10,
 // G = 256: 1.96 ms with every row summed by itself, 1.08 ms in pairs).
+#include <math_constants.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -228,9 +230,11 @@ __global__ void stress_rhs_kernel(const zd* __restrict__ U, const double* __rest
   Zm[(size_t)m * N + i] = zadd(zscale(u1, K2), zscale(u2, K1));
 }
 
-// S[j] = i V (Xk + Xm, Xk - Xm, X12) for column j
+// S[j] = i V (Xk + Xm, Xk - Xm, X12) for column j; NaN when late (optional) is set,
+// a tensor-core wait of the products that reached its limit
 __global__ void stress_combine_kernel(const zd* __restrict__ Xk, const zd* __restrict__ Xm,
-                                      int N, int m, double V, zd* __restrict__ S) {
+                                      int N, int m, double V, const int* __restrict__ late,
+                                      zd* __restrict__ S) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)N * m) return;
   const int a = (int)(i % N);
@@ -238,6 +242,7 @@ __global__ void stress_combine_kernel(const zd* __restrict__ Xk, const zd* __res
   const zd xk = Xk[i], xm = Xm[i], x12 = Xm[(size_t)m * N + i];
   const zd p = zadd(xk, xm), d = zsub(xk, xm);
   zd* s = S + (size_t)j * 3 * N;
+  if (late && *late) V = CUDART_NAN;
   s[a] = zmake(-V * p.y, V * p.x);
   s[N + a] = zmake(-V * d.y, V * d.x);
   s[2 * N + a] = zmake(-V * x12.y, V * x12.x);
@@ -368,7 +373,8 @@ int bs_launch_stress(bs_cell* c, const zd* U, const double* Q, int kc, int nvec,
   TRY_LAUNCH(gram_solve(c->d_Linv, N, m, Zk, Y, dg, s));
   TRY_LAUNCH(gram_solve(c->d_Linv + NN, N, 2 * m, Zm, Y, dg, s));
   stress_combine_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(Zk, Zm, N, m,
-                                                                     c->mesh ? 1.0 : c->V, S);
+                                                                     c->mesh ? 1.0 : c->V, dg.err,
+                                                                     S);
   BS_CHECK_LAUNCH("stress_combine_kernel");
   return BS_OK;
 }
@@ -411,10 +417,12 @@ extern "C" int bs_stress_coefficients(bs_cell* c, const double* Q, int nk, int n
       dg.wD = (float*)(p + d0);
       dg.eA = (int*)(dg.wD + nD);
       dg.eB = dg.eA + N;
-      dg.err = c->d_info + 1;
+      dg.err = c->d_info + 2;   // its own: an earlier call's says nothing about this one
     }
   }
   TRY_LAUNCH(mode_ws(c, need));
+  if (dg.wA)
+    MCK(cudaMemsetAsync(dg.err, c->late_wait ? 1 : 0, sizeof(int), s), "bs_stress_coefficients flag");
   double* dQ = c->d_mode;
   zd* Zk = (zd*)(dQ + zq);             // Zk, Zm: 3 N m contiguous (R3 of the anisotropic path)
   zd* Zm = Zk + (size_t)N * m;
@@ -461,6 +469,15 @@ extern "C" int bs_stress_coefficients(bs_cell* c, const double* Q, int nk, int n
       }
     }
   }
+  return BS_OK;
+}
+
+extern "C" int bs_set_late_wait(bs_cell* c, int on) {
+  if (!c) {
+    bs_set_error("bs_set_late_wait: NULL cell");
+    return BS_EINVAL;
+  }
+  c->late_wait = on != 0;
   return BS_OK;
 }
 
