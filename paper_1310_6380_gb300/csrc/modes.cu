@@ -78,7 +78,10 @@ __global__ void field_table_kernel(const double* __restrict__ Q, int nk, int M, 
 // every entry bounds the kernel above (99 us for 90 wavevectors of M = 10,
 // G = 256; 21 us here), so this one evaluates 2G + G of them per CTA, in
 // shared memory, and multiplies.  One CTA per wavevector and direction;
-// 2G <= ROOTS.
+// 2G <= ROOTS.  A CTA's 3G evaluations are a chain that few CTAs do not hide: with
+// few entries the kernel above is faster (M = 10, G = 256, both contractions
+// included: 1, 10, 30 and 90 wavevectors 57, 70, 87, 171 us with it, 70, 70, 72, 113
+// with this; G = 64: 37, 36, 43, 62 and 41, 42, 42, 45), hence the line.
 constexpr int ROOTS = 2048;
 __global__ void __launch_bounds__(256) field_roots_kernel(const double* __restrict__ Q, int M,
                                                           int WP, int G, zf* __restrict__ E) {
@@ -310,7 +313,7 @@ int bs_launch_mode_field(const zd* coef, const double* Q, long kbase, int nkt, l
   const int W = 2 * M + 1, WP = (W + 3) / 4 * 4, N = W * W;
   const size_t te = (size_t)nkt * 2 * WP * G;
   const double* Qt = Q + 2 * kbase;   // the table's wavevectors
-  if (2 * G <= ROOTS) {
+  if (2 * G <= ROOTS && te >= 49152 + 512 * (size_t)G) {
     field_roots_kernel<<<dim3(nkt, 2), 256, 2 * G * sizeof(zd), s>>>(Qt, M, WP, G, E);
     BS_CHECK_LAUNCH("field_roots_kernel");
   } else {
