@@ -19,6 +19,7 @@
 #include <algorithm>
 
 #include "bs_internal.h"
+#include "shrink_grid.h"
 
 namespace {
 
@@ -475,8 +476,13 @@ int bs_launch_tridiag_list(zd* A, int n, zd* vec, zd* part, double* de, double* 
   if (e != cudaSuccess) return bs_cuda_status(e, "tridiag_list_kernel");
   const int grid = std::max(1, per) * bs_sm_count();
   void* args[] = {&A, &n, &vec, &part, &de, &tau, &beta, &count, (void*)&list, (void*)&nlist};
-  e = cudaLaunchCooperativeKernel((const void*)tridiag_list_kernel, dim3(grid), dim3(NT), args, 0,
-                                  s);
+  // (the tiles and matrices go round whatever blocks there are)
+  e = bs_shrink_grid(grid, cudaErrorCooperativeLaunchTooLarge, [&](int g) {
+    const cudaError_t l =
+        cudaLaunchCooperativeKernel((const void*)tridiag_list_kernel, dim3(g), dim3(NT), args, 0, s);
+    if (l == cudaErrorCooperativeLaunchTooLarge) cudaGetLastError();
+    return l;
+  });
   if (e != cudaSuccess) return bs_cuda_status(e, "tridiag_list_kernel");
   BS_CHECK_LAUNCH("tridiag_list_kernel");
   return BS_OK;
