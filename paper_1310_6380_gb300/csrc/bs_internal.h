@@ -447,6 +447,7 @@ int bs_launch_rank2_update(const uint16_t* dA, const uint16_t* dB, const int* ex
 #define BS_FILT_ROUNDS 12      // filters at most
 struct FilterWs {
   int n = 0, kf = 0;        // order, matrices per chunk
+  int want = 0;             // the chunk it was asked for (kf is less when memory was short)
   zf* A = nullptr;          // kf x np x np scaled matrix, then its LDL^dagger (np: n padded to
                             // 64), then the BF16 split of the operator B (np x 4 np)
   zf* X = nullptr;          // kf x np x np inverse factor

@@ -51,6 +51,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <vector>
 
 #include "bs_internal.h"
 
@@ -1674,46 +1675,65 @@ static size_t filter_bytes(int n) {
 int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
   // chunks of at most about 8 GB of workspace, and of the slab launches' grid limit
   const int cap = (int)std::max<size_t>(1, std::min<size_t>(1000, ((size_t)8 << 30) / filter_bytes(n)));
-  const int kf = std::min(kb, cap);
-  if (w->n == n && w->kf >= kf) return BS_OK;
+  const int want = std::min(kb, cap);
+  if (w->n == n && w->want >= want) return BS_OK;
   bs_filter_ws_free(w);
   const size_t np = (n + TB - 1) / TB * TB, Kp = (2 * (size_t)n + 63) / 64 * 64;
   const size_t nch = (n + GR - 1) / GR;
-  const size_t k = kf;
-  struct Item { void** p; size_t bytes; } items[] = {
-      {(void**)&w->A, k * np * np * sizeof(zf)},
-      {(void**)&w->X, k * np * np * sizeof(zf)},
-      {(void**)&w->pA, k * n * 8 * Kp * 2},
-      {(void**)&w->pB, k * 2 * FB * 8 * Kp * 2},
-      // fewer digits can be cut into more slabs: room for either
-      {(void**)&w->pD, std::max(bs_slice_planes(8, (int)Kp, n, 2 * FB, kf),
-                                std::max(bs_slice_planes(STEER_DIGITS, (int)Kp, n, 2 * FB, kf),
-                                         bs_slice_planes(LAST_STEER_DIGITS, (int)Kp, n, 2 * FB, kf))) *
-                           n * 2 * FB * sizeof(float)},
-      {(void**)&w->eA, k * n * sizeof(int)},
-      {(void**)&w->eB, k * FB * sizeof(int)},
-      {(void**)&w->Xb, k * FB * n * sizeof(zd)},
-      {(void**)&w->CX, k * FB * n * sizeof(zd)},
-      {(void**)&w->vec, 3 * k * FB * np * sizeof(zf)},
-      {(void**)&w->vs, 2 * k * 2 * FB * 4 * np * sizeof(uint16_t)},
-      {(void**)&w->d, k * np * sizeof(float)},
-      {(void**)&w->part, k * nch * 2 * FB * FB * sizeof(zd)},
-      {(void**)&w->rpart, k * nch * 2 * FB * sizeof(float)},
-      {(void**)&w->theta, k * FB * sizeof(double)},
-      {(void**)&w->rerr, k * FB * sizeof(double)},
-      {(void**)&w->W, k * FB * FB * sizeof(zd)},
-      {(void**)&w->coef, k * BS_FILT_MAXDEG * 4 * FB * sizeof(float)},
-      {(void**)&w->shift, k * sizeof(double)},
-      {(void**)&w->cmax, k * sizeof(double)},
-      {(void**)&w->sigma, 2 * k * sizeof(double)},
-      {(void**)&w->kappa, k * sizeof(double)},
-      {(void**)&w->rsum, k * (np / TB) * np * sizeof(float)},
-      {(void**)&w->ord, k * NS * sizeof(int)},
-      {(void**)&w->w, k * np * sizeof(float)},
-      {(void**)&w->iw, (7 * k + 1) * sizeof(int)},
-      {(void**)&w->nred, sizeof(int)},
+  struct Item { void** p; size_t bytes; };
+  auto buffers = [&](int kf) {
+    const size_t k = kf;
+    return std::vector<Item>{
+        {(void**)&w->A, k * np * np * sizeof(zf)},
+        {(void**)&w->X, k * np * np * sizeof(zf)},
+        {(void**)&w->pA, k * n * 8 * Kp * 2},
+        {(void**)&w->pB, k * 2 * FB * 8 * Kp * 2},
+        // fewer digits can be cut into more slabs: room for either
+        {(void**)&w->pD, std::max(bs_slice_planes(8, (int)Kp, n, 2 * FB, kf),
+                                  std::max(bs_slice_planes(STEER_DIGITS, (int)Kp, n, 2 * FB, kf),
+                                           bs_slice_planes(LAST_STEER_DIGITS, (int)Kp, n, 2 * FB, kf))) *
+                             n * 2 * FB * sizeof(float)},
+        {(void**)&w->eA, k * n * sizeof(int)},
+        {(void**)&w->eB, k * FB * sizeof(int)},
+        {(void**)&w->Xb, k * FB * n * sizeof(zd)},
+        {(void**)&w->CX, k * FB * n * sizeof(zd)},
+        {(void**)&w->vec, 3 * k * FB * np * sizeof(zf)},
+        {(void**)&w->vs, 2 * k * 2 * FB * 4 * np * sizeof(uint16_t)},
+        {(void**)&w->d, k * np * sizeof(float)},
+        {(void**)&w->part, k * nch * 2 * FB * FB * sizeof(zd)},
+        {(void**)&w->rpart, k * nch * 2 * FB * sizeof(float)},
+        {(void**)&w->theta, k * FB * sizeof(double)},
+        {(void**)&w->rerr, k * FB * sizeof(double)},
+        {(void**)&w->W, k * FB * FB * sizeof(zd)},
+        {(void**)&w->coef, k * BS_FILT_MAXDEG * 4 * FB * sizeof(float)},
+        {(void**)&w->shift, k * sizeof(double)},
+        {(void**)&w->cmax, k * sizeof(double)},
+        {(void**)&w->sigma, 2 * k * sizeof(double)},
+        {(void**)&w->kappa, k * sizeof(double)},
+        {(void**)&w->rsum, k * (np / TB) * np * sizeof(float)},
+        {(void**)&w->ord, k * NS * sizeof(int)},
+        {(void**)&w->w, k * np * sizeof(float)},
+        {(void**)&w->iw, (7 * k + 1) * sizeof(int)},
+        {(void**)&w->nred, sizeof(int)},
+    };
   };
-  for (auto& it : items) {
+  // with less memory free, smaller chunks; no allocation is tried in vain
+  size_t room = 0, all = 0;
+  if (cudaMemGetInfo(&room, &all) != cudaSuccess) {
+    cudaGetLastError();
+    room = 0;
+  }
+  int kf = want;
+  for (;; kf /= 2) {
+    if (kf < 1) {
+      bs_set_error("out of device memory (filtered iteration, %zu bytes free)", room);
+      return BS_ENOMEM;
+    }
+    size_t total = 0;
+    for (const Item& it : buffers(kf)) total += (it.bytes + (2 << 20)) >> 21 << 21;   // 2 MB pages
+    if (total <= room) break;
+  }
+  for (const Item& it : buffers(kf)) {
     if (cudaMalloc(it.p, it.bytes) != cudaSuccess) {
       cudaGetLastError();
       bs_filter_ws_free(w);
@@ -1723,6 +1743,7 @@ int bs_filter_ws_alloc(FilterWs* w, int n, int kb) {
   }
   w->n = n;
   w->kf = kf;
+  w->want = want;
   return BS_OK;
 }
 

@@ -413,7 +413,9 @@ extern "C" int bs_stress_coefficients(bs_cell* c, const double* Q, int nk, int n
     bs_zgemm_tc_cols_elems(N, dg.cols, &nA, &nB, &nD);
     const size_t a = (need + 255) / 256 * 256, b = a + (nA + nB) * 2;
     const size_t d0 = (b + 255) / 256 * 256, e = d0 + (nD + N + dg.cols) * 4;
-    if (mode_ws(c, e) == BS_OK) {
+    size_t room = 0, all = 0;   // no allocation is tried in vain
+    if (c->mode_cap < e && cudaMemGetInfo(&room, &all) != cudaSuccess) cudaGetLastError();
+    if ((c->mode_cap >= e || c->mode_cap + room >= e) && mode_ws(c, e) == BS_OK) {
       char* p = (char*)c->d_mode;
       dg.wA = (uint16_t*)(p + a);
       dg.wB = dg.wA + nA;
