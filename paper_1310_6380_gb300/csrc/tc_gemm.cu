@@ -83,6 +83,14 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, in
       : "memory");
 }
 
+// The producer's last wait: for its copies of the last round of the ring, so that
+// none still writes to the CTA's shared memory when it ends, also where a
+// wait of the consumer ran out.  Where none did the consumer waits for them too.
+__device__ __forceinline__ void tma_drain(uint64_t* full, int stages, int issued, int* err) {
+  for (int i = issued > stages ? issued - stages : 0; i < issued; ++i)
+    mbar_wait(&full[i % stages], (uint32_t)(i / stages) & 1u, err);
+}
+
 // shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   uint64_t d = 0;
@@ -144,7 +152,8 @@ __global__ void __launch_bounds__(128, 2)
 
   if (warp == 0 && lane == 0) {
     // TMA producer
-    for (int kb = 0; kb < nk; ++kb) {
+    int kb = 0;
+    for (; kb < nk; ++kb) {
       const int s = kb % STAGES;
       const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
       if (kb >= STAGES && !mbar_wait(&empty[s], ph ^ 1u, err)) break;
@@ -152,6 +161,7 @@ __global__ void __launch_bounds__(128, 2)
       tma_load_3d(sA + s * TILE_A, &tmA, ka + kb * BK, m0, z, &full[s]);
       tma_load_3d(sB + s * TILE_B, &tmB, kbb + kb * BK, n0, z, &full[s]);
     }
+    tma_drain(full, STAGES, kb, err);
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
     for (int kb = 0; kb < nk; ++kb) {
@@ -282,13 +292,16 @@ __global__ void __launch_bounds__(NT, MINB)
     // TMA producer: B's eight blocks once, then A's digit blocks through the ring
     mbar_expect_tx(&bfull, R2_S * TILE_B);
     for (int b = 0; b < R2_S; ++b) tma_load_3d(sB + b * TILE_B, &tmB, b * BK, n0, z, &bfull);
-    for (int sd = 0; sd < R2_S; ++sd) {
+    int sd = 0;
+    for (; sd < R2_S; ++sd) {
       const int q = sd % R2_STAGES;
       const uint32_t ph = (uint32_t)(sd / R2_STAGES) & 1u;
       if (sd >= R2_STAGES && !mbar_wait(&empty[q], ph ^ 1u, err)) break;
       mbar_expect_tx(&full[q], TILE_A);
       tma_load_3d(sA + q * TILE_A, &tmA, sd * BK, m0, z, &full[q]);
     }
+    mbar_wait(&bfull, 0u, err);
+    tma_drain(full, R2_STAGES, sd, err);
   } else if (warp == 1 && lane == 0) {
     // MMA issuer: digit s of A against digits t = 0 .. 7-s of B into order s + t
     bool ok = mbar_wait(&bfull, 0u, err);
@@ -466,7 +479,8 @@ __global__ void __launch_bounds__(128, 2)
   const uint32_t tmem = tmem_base;
 
   if (warp == 0 && lane == 0) {
-    for (int kb = 0; kb < nk; ++kb) {
+    int kb = 0;
+    for (; kb < nk; ++kb) {
       const int s = kb % FP_STAGES;
       const uint32_t ph = (uint32_t)(kb / FP_STAGES) & 1u;
       if (kb >= FP_STAGES && !mbar_wait(&empty[s], ph ^ 1u, err)) break;
@@ -477,6 +491,7 @@ __global__ void __launch_bounds__(128, 2)
       tma_load_3d(st + 2 * TILE_A, &tmV, kb * BK, 0, z, &full[s]);
       tma_load_3d(st + 2 * TILE_A + TB_V, &tmV, K2 + kb * BK, 0, z, &full[s]);
     }
+    tma_drain(full, FP_STAGES, kb, err);
   } else if (warp == 1 && lane == 0) {
     for (int kb = 0; kb < nk; ++kb) {
       const int s = kb % FP_STAGES;
