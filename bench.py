@@ -466,6 +466,7 @@ def measure_c3(bs, torch, rep, args, ncell, steps, warmup, graph=True, oracle_ce
     status = st.cpu().numpy()
     ph = {k: statistics.mean(p[k] for p in phs) for k in phs[0]}
     tiles_chosen = bs.bs_batch_tiles(b)
+    counts = bs.bs_batch_filter_counts(b)
     _, fb_flags = bs.bs_batch_stats(b, ncell * nk)
     bs.bs_batch_destroy(b)
 
@@ -488,8 +489,8 @@ def measure_c3(bs, torch, rep, args, ncell, steps, warmup, graph=True, oracle_ce
            "d2h_bytes_per_step": hw.numel() * 8 + hs.numel() * 4,
            "api": "bs_batch_create (host arrays) + bs_batch_solve (host Q, outputs; first call "
                   "includes tile autotuning) + bs_batch_destroy"}
-    roofline = filter_roofline(np.repeat(ns, nk), ph["reduction"], device_peaks(torch),
-                               "one step's groups")
+    roofline = solve_roofline(counts, np.repeat(ns, nk), ph["reduction"], device_peaks(torch),
+                              "one step's groups", fp32=True)
     value = world * ncell * nk / (ms / 1e3)
     out = {
         "metric": METRIC, "value": value, "unit": "k-solves/s", "n_gpus": world,
@@ -504,7 +505,8 @@ def measure_c3(bs, torch, rep, args, ncell, steps, warmup, graph=True, oracle_ce
                    "cells_per_M": {int(m): Ms.count(m) for m in sorted(set(Ms))},
                    "l2": "flushed between timed steps (256 MiB write, untimed)"},
         "ms_per_step_plain": ms_plain, "ms_per_step_graph": ms_graph,
-        "tiles": tiles_chosen, "phases_ms": {k: round(v, 1) for k, v in ph.items()},
+        "tiles": tiles_chosen if counts[0] == 0 else None,   # (the iteration has none)
+        "phases_ms": {k: round(v, 1) for k, v in ph.items()},
         "status_nonzero": int(np.count_nonzero(status)),
         "fp64_fallbacks": int((fb_flags == 1).sum()), "gpu_launches_per_step": launches,
         "gpu_launches": launches * steps, "e2e": e2e, "roofline": roofline, "clocks": clocks,
@@ -632,15 +634,38 @@ def run_reference_batch(args):
 BAND_NB = 8
 
 
-def filter_taken(n, nb):
-    """The solves that the library routes to the filtered iteration by default."""
-    return 96 <= n <= 2048 and nb <= 22
+def solve_roofline(counts, ns, ms, peaks, what, fp32=False):
+    """The eigensolves' roofline by the route that they took: the library's
+    counts (matrices of the filtered iteration, reduced behind it) of the last
+    solve.  fp32: the reduction's precision where it ran."""
+    if counts[0] > 0:
+        roofline = filter_roofline(ns, ms, peaks, what)
+        roofline["matrices"], roofline["reduced_behind"] = counts
+        return roofline
+    ns = np.asarray(ns, float)
+    if fp32:
+        hbm_peak, _, note = measured_peaks()
+        achieved = 16.0 * float(np.sum(ns * (ns - 1) * (ns + 1) / 6)) / (ms / 1e3) / 1e9
+        return {"bound": "hbm", "kernel": f"tridiag_step_kernel<float> ({what})",
+                "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
+                "traffic": None, "peak_source": "copy bandwidth, " + note,
+                "algorithmic": "read + write (8 B each) of every trailing lower triangle, "
+                               f"{len(ns)} matrices, n = {int(min(ns))}..{int(max(ns))}"}
+    achieved = 16.0 / 3.0 * float(np.sum(ns ** 3)) / (ms / 1e3) / 1e12
+    peak = peaks["fp64_nominal_tflops"]
+    return {"bound": "alu", "kernel": f"FP64 reduction to tridiagonal form ({what})",
+            "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+            "traffic": None,
+            "peak_source": "nominal FP64: SMs (queried) x 2 FMA/clk x 2 flop x max SM clock",
+            "algorithmic": f"(16/3) n^3 real flops per matrix, {len(ns)} matrices, "
+                           f"n = {int(min(ns))}..{int(max(ns))}; the one-stage reduction's count, "
+                           "so above 1.0 means that the work left the FP64 pipe"}
 
 
 def filter_roofline(ns, ms, peaks, what):
     """Roofline of the filtered iteration on matrices of orders ns: its FP32
-    factorisation, triangular inverse, operator and inertia check (4/3 n^3 real
-    flops each) against the FP32 pipe, which its largest kernels run on; the
+    factorisation, triangular inverse, operator and the certificate's
+    factorisation (4/3 n^3 real flops each) against the FP32 pipe, which its largest kernels run on; the
     time also holds the tensor-core products and the Rayleigh-Ritz steps."""
     flops = 16.0 / 3.0 * float(np.sum(np.asarray(ns, float) ** 3))
     peak = peaks["fp32_nominal_tflops"]
@@ -840,9 +865,10 @@ def run_ours(args):
     red = {k: statistics.mean(r[k] for r in reds) for k in reds[0]}
     if prec == 0 and red["matrices"] > 0:
         roofline, reduction = band_roofline(red, n, nk, ph, peaks)
-    elif prec == 0 and filter_taken(n, nb):
+    elif prec == 0 and bs.bs_filter_counts(h)[0] > 0:
         reduction = None
-        roofline = filter_roofline([n] * nk, ph["tridiag"], peaks, "all launches of one step")
+        roofline = solve_roofline(bs.bs_filter_counts(h), [n] * nk, ph["tridiag"], peaks,
+                                  "all launches of one step")
     elif prec == 0:
         reduction = None
         trid_flops = nk * 16.0 / 3.0 * n ** 3
@@ -1503,8 +1529,8 @@ def run_3d(args):
     value = rep.value(nk, ms)
     omega = w.cpu().numpy()
     t_sol = statistics.mean(sol_ms)
-    roofline = filter_roofline([n] * nk, t_sol, device_peaks(torch),
-                               "bs_solve_k3 of one step, with the per-k builder")
+    roofline = solve_roofline(bs.bs_filter_counts3(h), [n] * nk, t_sol, device_peaks(torch),
+                              "bs_solve_k3 of one step, with the per-k builder")
     pin = lambda a: torch.from_numpy(np.ascontiguousarray(a)).pin_memory()
     hp, hl, hm, hr, hQ = (pin(cell.phase.astype(np.uint16)), pin(cell.lam), pin(cell.mu),
                           pin(cell.rho), pin(Q))

@@ -52,9 +52,11 @@ extern "C" {
 #define BS_ESTATE   -6   /* call out of order (e.g. solve before assemble)     */
 
 /* arithmetic of the eigen path */
-#define BS_PREC_FP64   0  /* results to float64 accuracy: every quantity that
-                             enters them is float64 or an exact-slice product of
-                             float64 operands (bs_set_reduction)              */
+#define BS_PREC_FP64   0  /* results to float64 accuracy: what enters them is
+                             float64, an exact-slice product of float64 operands
+                             or, in the filtered iteration's last products of 32
+                             vectors, held in 48 bits with its error counted
+                             (bs_set_reduction)                               */
 #define BS_PREC_MIXED  1  /* FP32 reduction + FP64 Rayleigh-Ritz refinement    */
 
 /* IBZ boundary paths for bs_bands (fractional corner points) */
@@ -438,9 +440,12 @@ int bs_tridiag_eigenvalues_static(const double* d, const double* e, int n, int b
  *   of the recording call must be reused); on == 0 drops the graph.
  * bs_batch_tiles - the reduction variant chosen for each truncation group
  *   and the group's eigen dimension n: 64 or 32 (tile edge of the
- *   per-step kernel).
- * bs_batch_set_tile - force that choice for every group (32 or 64) or,
- *   with -1, return to timing both on the next solve (BS_EINVAL for any
+ *   per-step kernel).  A group that takes the filtered iteration
+ *   (bs_batch_set_solver) uses no tile and is not tuned: its value is 64,
+ *   or the choice of an earlier solve that was reduced.
+ * bs_batch_set_tile - force that choice for every group (32 or 64), and with
+ *   it the reduction instead of the filtered iteration, or, with -1, return
+ *   to timing both on the next solve that is reduced (BS_EINVAL for any
  *   other value).  Drops a recorded graph.
  * bs_batch_set_profiling / bs_batch_phase_times - with profiling on, a
  *   solve that does not replay a graph records CUDA events around each
