@@ -1614,7 +1614,7 @@ __global__ void __launch_bounds__(1024) filt_decide_kernel(const int* __restrict
                                                            int* __restrict__ stat,
                                                            int* __restrict__ list,
                                                            int* __restrict__ nlist,
-                                                           int* __restrict__ nred,
+                                                           int* __restrict__ nred, bool first,
                                                            int* __restrict__ reduced) {
   __shared__ int cnt[32], base;
   const int tid = threadIdx.x;
@@ -1637,7 +1637,7 @@ __global__ void __launch_bounds__(1024) filt_decide_kernel(const int* __restrict
   }
   if (tid == 0) {
     *nlist = base;
-    *nred += base;
+    *nred = (first ? 0 : *nred) + base;
   }
 }
 
@@ -1850,10 +1850,7 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
     return BS_EINVAL;
   }
   TRY_LAUNCH(filter_attrs());
-  if (w.taken == 0) {
-    const cudaError_t e = cudaMemsetAsync(w.nred, 0, sizeof(int), s);
-    if (e != cudaSuccess) return bs_cuda_status(e, "filtered iteration count");
-  }
+  const bool first = w.taken == 0;
   w.taken += kb;
   const int np = (n + TB - 1) / TB * TB, nt = np / TB, nch = (n + GR - 1) / GR;
   for (int k0 = 0; k0 < kb; k0 += w.kf) {
@@ -1913,6 +1910,7 @@ int bs_launch_eig_filter(zd* C, int n, int kb, int nbands, FilterWs& w, const Fi
     BS_CHECK_LAUNCH("filt_lift_kernel");
     TRY_LAUNCH(filter_factor(w, np, kf, false, s, skip));
     filt_decide_kernel<<<1, 1024, 0, s>>>(neg, flag, expect, kf, stat + k0, list, nlist, w.nred,
+                                          first && k0 == 0,
                                           reduced ? reduced + k0 : nullptr);
     BS_CHECK_LAUNCH("filt_decide_kernel");
     TRY_LAUNCH(bs_launch_tridiag_list(Ck, n, fb.vec + (size_t)k0 * bs_tridiag_vec_elems(n),
