@@ -38,14 +38,15 @@
 //
 // Measured (one GB300, whole FP64 solve with its assembly, the reduction to
 // tridiagonal form before -> this): n = 882, 90 matrices, 18 branches
-// 171 -> 26 ms; n = 1029, 30 matrices, 12 branches 136 -> 18.3 ms; n = 242,
-// 70 matrices, 18 branches 16.9 -> 4.3 ms; n = 98, 65 matrices, 18 branches
-// 3.86 -> 2.52 ms.  What bounds it at n = 882 is the
-// FP32 pipe in the factorisations and the FP64 pipe in the Rayleigh-Ritz steps
-// (32-column products at 2 FMA per clock and SM).
+// 171 -> 26.2 ms; n = 1029, 30 matrices, 12 branches 136 -> 18.4 ms; n = 242,
+// 70 matrices, 18 branches 16.9 -> 4.2 ms; n = 98, 30 matrices, 8 branches
+// 3.86 -> 2.42 ms.  What bounds it at n = 882 is the FP32 factorisations (their
+// pipe is 58 % busy at most) and the FP64 pipe in the Rayleigh-Ritz steps (32-column
+// products at 2 FMA per clock and SM).
 //
-// Everything that enters a result (C X, the Gram matrices, the Ritz values,
-// the residuals) is FP64 or an exact-slice product of FP64 operands.
+// What enters a result: C X, an exact-slice product of FP64 operands; the Gram
+// matrices, FP64; the Ritz values, Rayleigh quotients in 48 bits with a bound; the
+// rotated block and its residuals, 48 bits.
 #include <float.h>
 #include <math.h>
 
