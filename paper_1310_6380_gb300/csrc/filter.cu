@@ -903,6 +903,11 @@ __device__ __forceinline__ void df_fma(df a, df b, df& acc) {
   acc.h = s;
   acc.l += fmaf(a.h, b.l, fmaf(a.l, b.h, e + t));
 }
+// a + b in two terms, exactly
+__device__ __forceinline__ df df_sum(float a, float b) {
+  const float s = a + b, t = s - a;
+  return {s, (a - (s - t)) + (b - t)};
+}
 __device__ __forceinline__ df df_neg(df a) { return {-a.h, -a.l}; }
 
 // operands of the rotation: FP32, or two FP32 terms (re, im) high, (re, im) low
@@ -1319,7 +1324,10 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
   float4(*L4)[FB + 1] = reinterpret_cast<float4(*)[FB + 1]>(&sm.H[0][0]);   // Li, two terms
   if constexpr (sizeof(R) == 8) {
     // V <- V + V F, F = (I - V^dagger V) / 2, columns to unit length.  F is 1e-6
-    // and needs no more than FP32; V^dagger V is summed in two FP32 terms
+    // and needs no more than FP32; V^dagger V is summed in two FP32 terms.  The sum is
+    // split anew: a low term of 1e-6 instead of 6e-8 of the high one, whose products
+    // with low terms df_fma leaves out, made Ritz values wrong by 1e-13 of
+    // themselves (up to 1e3 eps64 ||C|| in one of 1000 matrices of n = 98)
     zf(*F)[FB + 1] = sm.J.A[0];
     for (int e = tid; e < NT2; e += 256) {
       int r, c;
@@ -1351,7 +1359,8 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
 #pragma unroll 8
       for (int t = 0; t < FB; ++t) d = zfma(sm.J.V[r][t], F[t][c], d);
       const zf v = sm.J.V[r][c];
-      V4[r][c] = make_float4(v.x, v.y, d.x, d.y);
+      const df x = df_sum(v.x, d.x), y = df_sum(v.y, d.y);
+      V4[r][c] = make_float4(x.h, y.h, x.l, y.l);
     }
     __syncthreads();
     const int c = tid >> 3, q = tid & 7;

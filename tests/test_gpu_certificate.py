@@ -100,6 +100,34 @@ def test_lone_low_eigenvalues(n, low, top, angle):
     assert np.abs(got - lam[:, :len(low)]).max() <= (n + 128) * EPS * top
 
 
+@pytest.mark.parametrize("kind, n, nb, angle", [
+    ("even", 97, 22, 1.0), ("even", 98, 22, 0.3), ("even", 128, 15, 0.3), ("levels", 98, 7, 0.3),
+    ("levels", 129, 11, 0.1), ("lone", 98, 13, 0.3)])
+def test_ritz_values_keep_48_bits(kind, n, nb, angle):
+    """Many random spectra (even, on 41 levels, a low group far below the others): the
+    vectors of the small eigenproblem enter the Ritz values in 48 bits however
+    many rotations they went through.  Tolerance: (n + 4) eps64 ||C|| for the reference's
+    reduction, the certificate's 64 eps64 max C_rr."""
+    rng = np.random.default_rng(n)
+    count, top = 384, 1e4
+    C = np.empty((count, n, n), complex)
+    for i in range(count):
+        lam = top * rng.random(n)
+        if kind == "levels":
+            lam = np.round(lam / top * 40) * (top / 40)
+        elif kind == "lone":
+            lam = np.concatenate([10.0 ** rng.uniform(-6, 1, nb), rng.uniform(20, 40, n - nb)])
+        K = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+        V = np.linalg.qr(np.eye(n) + angle / np.sqrt(n) * (K - K.conj().T))[0]
+        C[i] = (V * np.sort(lam)) @ V.conj().T
+        C[i] = 0.5 * (C[i] + C[i].conj().T)
+    lam = np.linalg.eigvalsh(C)
+    got, _ = solve(C, nb)
+    err = np.abs(got - np.maximum(lam[:, :nb], 0.0)).max(1)
+    tol = EPS * ((n + 4) * lam[:, -1] + 64 * np.einsum("kii->ki", C).real.max(1))
+    assert (err / tol).max() <= 1.0
+
+
 @pytest.mark.parametrize("e", [-400, -120, -40, 40, 62, 124, 400])
 def test_any_unit(e):
     """A power of two as the unit changes no bit of any step: the same matrices
