@@ -1185,7 +1185,8 @@ __device__ __forceinline__ int jacobi32(JacobiSmem& sm, float offtol, int maxswe
 // whose block was far from diagonal (an ill-conditioned Gram matrix before it)
 // made Ritz values wrong by 1e4 eps64 ||C|| that no residual shows.  With
 // S = V^dagger A V, a Ritz value is within sum_j min(|S_ij|, 2 |S_ij|^2 / |S_ii - S_jj|) of
-// S_ii, and A itself within eps64 ||A|| / (smallest pivot of G).  The products
+// S_ii, and A itself within eps64 max C_rr / (smallest pivot of G), as C X errs by
+// eps64 of C's largest entries.  The products
 // take 48 bits, the off-diagonal part from U = A V - V diag(S) in FP32: 7 us.
 template <typename R>
 struct EigSmem {
@@ -1199,6 +1200,7 @@ struct EigCheckSmem : EigSmem<double> {
 template <typename R, bool CHECK>
 __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ part, int nch,
                                                        const double* __restrict__ shift,
+                                                       const double* __restrict__ cmax,
                                                        double* __restrict__ theta,
                                                        zd* __restrict__ W,
                                                        int* __restrict__ fail,
@@ -1439,19 +1441,17 @@ __global__ void __launch_bounds__(256) filt_eig_kernel(const zd* __restrict__ pa
         S[row + 8 * j][col] = fsqrt(fmaf(d[j].x, d[j].x, d[j].y * d[j].y));
       __syncthreads();
       {   // the bound of Ritz value c from its row of S, eight lanes per value
-        float e = 0.f, top = 0.f, ip = 0.f;
+        float e = 0.f, ip = 0.f;
         for (int r = q; r < FB; r += 8) {
-          top = fmaxf(top, fabsf((float)ev[r]));
           ip = fmaxf(ip, (float)pinv[r]);
           const float a = fmaxf(S[r][c], S[c][r]), g = fabsf((float)(ev[r] - ev[c]));
           if (r != c) e += 2.f * a < g ? 2.f * a * __fdividef(a, g) : a;
         }
         for (int o = 4; o > 0; o >>= 1) {
           e += __shfl_xor_sync(0xffffffffu, e, o);
-          top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
           ip = fmaxf(ip, __shfl_xor_sync(0xffffffffu, ip, o));
         }
-        e += (float)DBL_EPSILON * top * ip * ip;
+        e += (float)DBL_EPSILON * to_float(cmax[k], exponent(shift[k])) * ip * ip;
         if (q == 0) re_max[c] = e == e ? e : INFINITY;
       }
       __syncthreads();
@@ -1835,7 +1835,7 @@ static int filter_ritz(FilterWs& w, int n, int np, int kf, cudaStream_t s) {
                                                                   done);
   BS_CHECK_LAUNCH("filt_gram_kernel");
   filt_eig_kernel<R, CHECK><<<kf, 256, CHECK ? sizeof(EigCheckSmem) : sizeof(EigSmem<R>), s>>>(
-      w.part, nch, w.shift, w.theta, w.W, fail, w.rerr, done);
+      w.part, nch, w.shift, w.cmax, w.theta, w.W, fail, w.rerr, done);
   BS_CHECK_LAUNCH("filt_eig_kernel");
   // the rotation covers the padded rows as well (np <= nch GR)
   filt_rotate_kernel<R><<<dim3(nch, kf), 256, sizeof(RotSmem<R>), s>>>(w.Xb, w.CX, n, np, w.W, w.theta, w.shift,
