@@ -18,6 +18,8 @@
 // stop_rel > 4 eps ends the FP64 phase at stop_rel ||T||: the mixed path
 // needs the eigenvalues of its FP32-reduced T only as inverse-iteration
 // shifts, for which 1e-9 ||T|| is ample.
+#include <algorithm>
+
 #include <float.h>
 #include <math.h>
 
@@ -215,9 +217,11 @@ __global__ void __launch_bounds__(NTB) bisect_kernel(const double* __restrict__ 
 
 static int bisect_smem(int n, size_t* smem) {
   *smem = 2 * (size_t)n * sizeof(double) + 2 * (size_t)n * sizeof(float);
-  if (*smem > 48 * 1024) {
+  // 48 KB hold the kernel's static part too without the attribute; 200 KB at
+  // least, so that a thread with a smaller n does not lower it under another's launch
+  if (*smem + 1024 > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(bisect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)*smem);
+                                         std::max((int)*smem, 200 * 1024));
     if (e != cudaSuccess) return bs_cuda_status(e, "bisect smem");
   }
   return BS_OK;

@@ -55,6 +55,20 @@ def test_tridiagonal_eigenvalues(name):
             assert np.all(np.abs(lam[b] - ref) <= tol), (name, nb, b, np.abs(lam[b] - ref).max())
 
 
+@pytest.mark.parametrize("n", [2005, 2046, 2047, 2048, 2049])
+def test_rows_that_fill_48_kb(n):
+    """24 n bytes of shared memory beside the kernel's own: n = 2047 and 2048 are the
+    sizes whose rows fit 48 KB and whose sum does not."""
+    rng = np.random.default_rng(n)
+    d, e = rng.standard_normal((2, n)), rng.standard_normal((2, n - 1))
+    lam = np.empty((2, 5))
+    bs.bs_tridiag_eigenvalues(d, e, 5, lam)
+    for b in range(2):
+        ref = sla.eigvalsh_tridiagonal(d[b], e[b], select="i", select_range=(0, 4))
+        tol = 8 * np.finfo(float).eps * (np.abs(d[b]).max() + 2 * np.abs(e[b]).max())
+        assert np.all(np.abs(lam[b] - ref) <= tol)
+
+
 def test_device_buffers():
     d, e = _cases()["random"]
     dd = torch.tensor(d, device="cuda"); ed = torch.tensor(e, device="cuda")
